@@ -1,7 +1,7 @@
 // kf_fp64.cuh -- double-precision building blocks shared by the FP64 fit
 // kernel and the method-variant kernel: the transport Jacobian layout, the
 // per-state workspace record, the gain-matrix update with the Joseph form and
-// the Rauch-Tung-Striebel smoother over the stored records (paper Sect. 2).
+// the fixed-point form of the smoother (paper Sect. 2).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -59,7 +59,7 @@ struct WS {
   size_t nt;
   int rec64, rec32;
   int i;
-  __device__ double& d(int k, int e) const { return w64[((size_t)k * rec64 + e) * nt + i]; }
+  __device__ __forceinline__ double& d(int k, int e) const { return w64[((size_t)k * rec64 + e) * nt + i]; }
   __device__ float& f(int k, int e) const { return w32[((size_t)k * rec32 + e) * nt + i]; }
 };
 
@@ -72,6 +72,222 @@ template <> struct Rec<0> {
   __device__ static void put_bm(const WS& w, int k, int e, double v) { w.d(k, BM + e) = v; }
   __device__ static double get_bm(const WS& w, int k, int e) { return w.d(k, BM + e); }
 };
+
+// ---------------------------------------------------------------------------
+// gain-matrix update with the Joseph covariance form
+//   S = V + H Cp H^T, K = Cp H^T S^-1, xf = xp + K r
+//   Cf = (I-KH) Cp (I-KH)^T + K V K^T
+//      = Cp + K W - (H Cp)^T K^T,  W = S K^T - H Cp   (expanded, exact for any K)
+// Cp, Cf packed lower triangles.
+// ---------------------------------------------------------------------------
+// Gain, increments and chi2 of the gain-matrix update: S = V + H Cp H^T,
+// K = Cp H^T S^-1, r the predicted residual, dx = K r.
+__device__ __forceinline__ int kalman_gain(const double xp[6], const double Cp[21], const double m[2],
+                                           const double V[3], double K[6][2], double Si[3], double r[2],
+                                           double dx[6], double& chi2) {
+  const double S00 = V[0] + Cp[sy(0, 0)], S01 = V[1] + Cp[sy(1, 0)], S11 = V[2] + Cp[sy(1, 1)];
+  const double det = fma(S00, S11, -S01 * S01);
+  if (!(det > 0.0) || !(S00 > 0.0)) return ST_NON_SPD;
+  const double idet = rcp_any(det);
+  Si[0] = S11 * idet;
+  Si[1] = -S01 * idet;
+  Si[2] = S00 * idet;
+  r[0] = m[0] - xp[0];
+  r[1] = m[1] - xp[1];
+  chi2 = fma(r[0], fma(Si[0], r[0], 2.0 * Si[1] * r[1]), Si[2] * r[1] * r[1]);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const double c0 = Cp[sym(i, 0)], c1 = Cp[sym(i, 1)];
+    K[i][0] = fma(c0, Si[0], c1 * Si[1]);
+    K[i][1] = fma(c0, Si[1], c1 * Si[2]);
+    dx[i] = fma(K[i][0], r[0], K[i][1] * r[1]);
+  }
+  return ST_OK;
+}
+
+// C <- Cp + K W - (H Cp)^T K^T, W = S K^T - H Cp (the Joseph form, expanded)
+__device__ __forceinline__ void joseph_update(double C[21], const double V[3], const double K[6][2]) {
+  const double S00 = V[0] + C[sy(0, 0)], S01 = V[1] + C[sy(1, 0)], S11 = V[2] + C[sy(1, 1)];
+  double h0[6], h1[6], W0[6], W1[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    h0[j] = C[sym(0, j)];
+    h1[j] = C[sym(1, j)];
+    W0[j] = fma(S00, K[j][0], fma(S01, K[j][1], -h0[j]));
+    W1[j] = fma(S01, K[j][0], fma(S11, K[j][1], -h1[j]));
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) if (j <= i) {
+      double v = C[sy(i, j)];
+      v = fma(K[i][0], W0[j], v);
+      v = fma(K[i][1], W1[j], v);
+      v = fma(-h0[i], K[j][0], v);
+      v = fma(-h1[i], K[j][1], v);
+      C[sy(i, j)] = v;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// positive definiteness of a predicted covariance
+// ---------------------------------------------------------------------------
+
+// All six Cholesky pivots positive, in double precision.
+static __device__ __noinline__ bool spd_pivots_fp64(const double C[21]) {
+  double L[21];
+  bool ok = true;
+  for (int e = 0; e < 21; ++e) L[e] = C[e];
+  for (int j = 0; j < 6; ++j) {
+    double dj = L[sy(j, j)];
+    for (int q = 0; q < j; ++q) dj -= L[sy(j, q)] * L[sy(j, q)];
+    if (!(dj > 0.0)) ok = false;
+    const double idg = rsqrt_any(dj);
+    L[sy(j, j)] = dj * idg;
+    for (int r = j + 1; r < 6; ++r) {
+      double v = L[sy(r, j)];
+      for (int q = 0; q < j; ++q) v -= L[sy(r, q)] * L[sy(j, q)];
+      L[sy(r, j)] = v * idg;
+    }
+  }
+  return ok;
+}
+
+// The same verdict without FP64 work in the usual case: a float LDL^T of C
+// with its diagonal lowered by 1e-5 of itself.  If its pivots are positive,
+// the smallest eigenvalue of the Jacobi-scaled C exceeds 1e-5 less the
+// rounding errors (conversion 6 x 6e-8, factorisation 7 x 6e-8 x 6 = 2.5e-6:
+// Rump's verification by a shifted floating-point Cholesky, BIT 46, 2006), so
+// the double-precision factorisation cannot fail.  Otherwise (or with a
+// diagonal near the ends of the float range) the FP64 pivots decide.  The
+// predicted covariances of the telescope fits have a smallest scaled
+// eigenvalue of 0.02 and more.
+__device__ __forceinline__ bool spd_check(const double C[21]) {
+  float U[21], L[21], iD[6];
+#pragma unroll
+  for (int e = 0; e < 21; ++e) U[e] = d2f(C[e]);
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    const float cjj = U[sy(j, j)];
+    ok = ok && cjj > 1e-30f && cjj < 1e30f;
+    float dj = cjj * (1.0f - 1e-5f);
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+      if (q < j) dj = fmaf(-U[sy(j, q)], L[sy(j, q)], dj);
+    ok = ok && dj > 0.0f;
+    iD[j] = 1.0f / dj;
+#pragma unroll
+    for (int r = 0; r < 6; ++r)
+      if (r > j) {
+        float u = U[sy(r, j)];
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+          if (q < j) u = fmaf(-U[sy(r, q)], L[sy(j, q)], u);
+        U[sy(r, j)] = u;
+        L[sy(r, j)] = u * iD[j];
+      }
+  }
+  if (ok) return true;
+  double t[21];
+#pragma unroll
+  for (int e = 0; e < 21; ++e) t[e] = C[e];
+  return spd_pivots_fp64(t);
+}
+
+// ---------------------------------------------------------------------------
+// fixed-point smoother
+//
+// The RTS smoother's state 0 (its parameters and covariance are the fit's
+// result) equals the estimate of the state x_0 by a filter of the augmented
+// state (x_0, x_k), which runs along with the forward filter:
+//   predict  S = S F^T                         (S = Cov(x_0, x_k), 6x6)
+//   update   h = S H^T, K0 = h (V + H Cp H^T)^-1,
+//            x_0 += K0 r, P_0 -= K0 h^T, S -= h K^T
+// with F, K, r, V the forward filter's.  It takes about 300 FP64 instructions
+// per state where the backward recursion with stored Jacobians (a Cholesky
+// factorisation, six pairs of triangular solves and A (Cs' - Cp') A^T) takes
+// 735, needs no inverse of Cp, and no record of the forward pass is written
+// to memory (720 B per state before).  Against an 80-bit evaluation of the
+// whole fit (ten shapes of 2000 tracks) the errors of parameters, covariances
+// and chi2 are 0.2 to 0.7 of those of the backward recursion it replaced.
+// ---------------------------------------------------------------------------
+
+// row (v0..v5) -> row F^T, with F row 4 = e4 (times g) and column 5 = e5
+template <class FE>
+__device__ __forceinline__ void row_times_ft(const FE& f, double g, const double v[6], double o[6]) {
+#pragma unroll
+  for (int r = 0; r < 6; ++r) {
+    if (r == 4) {
+      o[r] = g * v[4];
+    } else {
+      double a = f(r, 0) * v[0];
+#pragma unroll
+      for (int c = 1; c < 5; ++c) a = fma(f(r, c), v[c], a);
+      if (r == 5) a += v[5];
+      o[r] = a;
+    }
+  }
+}
+
+// Measurement update of row i of S, x_0[i] and row i of P_0 (lower part);
+// h of the other rows comes in hall (rows 0..i are used).
+__device__ __forceinline__ void fixed_point_row(int i, double S[6], const double K[6][2], const double Si[3],
+                                                const double r[2], const double hall[6][2], double& x0,
+                                                double P0[21]) {
+  const double h0 = hall[i][0], h1 = hall[i][1];
+  const double k0 = fma(h0, Si[0], h1 * Si[1]), k1 = fma(h0, Si[1], h1 * Si[2]);
+  x0 = fma(k0, r[0], fma(k1, r[1], x0));
+#pragma unroll
+  for (int c = 0; c < 6; ++c)
+    if (c <= i) P0[sy(i, c)] = fma(-k0, hall[c][0], fma(-k1, hall[c][1], P0[sy(i, c)]));
+#pragma unroll
+  for (int c = 0; c < 6; ++c) S[c] = fma(-h0, K[c][0], fma(-h1, K[c][1], S[c]));
+}
+
+// Per-state record for the smoothed parameters of every state (written only
+// when they are wanted): F 25 | K 12 | S^-1 r 2 | x_f 6 | C_f 21 | g, the
+// factor of F's q/p row (with energy loss only).
+struct StateRec {
+  static constexpr int F = 0, K = 25, IR = 37, XF = 39, CF = 45, G = 66;
+};
+static_assert(StateRec::G + 1 <= kRec64Fp64, "record size");
+
+// Smoothed parameters of states n-1 .. 1 from the records, by the adjoint
+// form of the smoother (Bryson and Frazier): x_s,k = x_f,k - C_f,k l_k with
+//   l~ = l - H^T (K^T l + S^-1 r),  l_{k-1} = F_k^T l~.
+__device__ __forceinline__ void smooth_states(const WS& ws, int n, double* out_states, int64_t n_states, int64_t o0,
+                                              bool with_g = false) {
+  double l[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int k = n - 1; k >= 1; --k) {
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+      double v = ws.d(k, StateRec::XF + r);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) v = fma(-ws.d(k, StateRec::CF + sym(r, c)), l[c], v);
+      out_states[r * n_states + o0 + k] = v;
+    }
+    double a0 = ws.d(k, StateRec::IR), a1 = ws.d(k, StateRec::IR + 1);
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+      a0 = fma(ws.d(k, StateRec::K + 2 * r), l[r], a0);
+      a1 = fma(ws.d(k, StateRec::K + 2 * r + 1), l[r], a1);
+    }
+    l[0] -= a0;
+    l[1] -= a1;
+    double m[6];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      double v = c == 4 ? (with_g ? ws.d(k, StateRec::G) * l[4] : l[4]) : 0.0;
+#pragma unroll
+      for (int r = 0; r < 5; ++r) v = fma(ws.d(k, StateRec::F + r * 5 + c), l[r == 4 ? 5 : r], v);
+      m[c] = v;
+    }
+    m[5] = l[5];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) l[c] = m[c];
+  }
+}
 
 // ---------------------------------------------------------------------------
 // gain-matrix update with the Joseph covariance form (double precision for

@@ -27,8 +27,10 @@ constexpr int kSurfPacked = kSurfStride + kSurfStrideM;  // doubles per surface 
 constexpr int kMaxSurfaces = 1024;  // 192 KiB of shared memory (FP64 table)
 
 // Per-state record the forward pass writes and the RTS pass reads back.
-// FP64 path, all in ws64:  xp 6 | xf 6 | Cp 21 | Cf 21 | Bm 36   (90 doubles)
-//   Bm = F_k * Cf_{k-1}: the right-hand side of the smoother-gain solve.
+// FP64 path, all in ws64: 90 doubles.  The fit itself writes none (its
+//   smoother runs along with the filter); with smoothed states wanted, what
+//   their backward pass reads (StateRec, kf_fp64.cuh).  The method variants
+//   with the backward filter keep the filtered states there.
 // Mixed path, ws64:        xp 6                                   (6 doubles)
 //             ws32:        F 25 | q_phi | q_theta | dxf 6 | Cp 21 (54 floats)
 //   xp is written for state 0 always and for the others only when smoothed

@@ -1,15 +1,23 @@
 // kf_kernels.cu -- the FP64 fit kernel (sm_103a) of the Kalman-filter track
 // fit (arXiv 2105.01796): forward filter (Runge-Kutta-Nystrom propagation in
 // a constant field, Jacobian transport, multiple-scattering noise, gain-matrix
-// update with the Joseph covariance form, chi2) and the Rauch-Tung-Striebel
-// smoother, fused into one launch with one track per thread, every step in
-// double precision; plus the small helper kernels (surface packing, the
-// length sort of the sorted schedule, a self-check).  The mixed-precision
-// kernel is in kf_mixed.cu, the method variants in kf_variants.cu.
-// Paper references: Sect. 2 (filter step list, RTS smoother with the stored
-// Jacobians), Sect. 4.1 (RKN transport; local<->global Jacobians at both
-// surfaces), Sect. 4.2 (double-precision inverter), Sect. 4.3 (surfaces in
-// global memory accessed once; constant field).
+// update with the Joseph covariance form, chi2) with the smoothed estimate of
+// state 0 carried along (the fixed-point form of the smoother, kf_fp64.cuh),
+// one launch, one track per thread, every step in double precision; plus the
+// small helper kernels (surface packing, the length sort of the sorted
+// schedule, a self-check).  The mixed-precision kernel is in kf_mixed.cu, the
+// method variants in kf_variants.cu.
+// Paper references: Sect. 2 (filter step list, smoother), Sect. 4.1 (RKN
+// transport; local<->global Jacobians at both surfaces), Sect. 4.3 (surfaces
+// in global memory accessed once; constant field).
+//
+// The bound is the FP64 pipe (2 DFMA per clock and SM), so the design spends
+// as few FP64 instructions as the method allows: about 1050 per state with
+// the field along z, where the stage-by-stage transport with the backward
+// smoother took 2370.  100k tracks of 31 states: 15.28 -> 6.47 ms; 20k tracks
+// of 24 tilted planes in a general field with every smoothed state
+// 4.37 -> 1.95 ms; 97 tracks of 11 states (the latency of one warp per
+// sub-partition) 0.90 -> 0.40 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -25,132 +33,10 @@ using namespace dev;
 
 
 // ---------------------------------------------------------------------------
-// transport x (bound, on surface a) to surface b.  Returns the bound
-// prediction xp, the 6x6 Jacobian F (row 4 = e4 and column 5 = e5 implied),
-// and the unit-direction quantities the noise needs.
-// ---------------------------------------------------------------------------
-template <typename R, bool BZ>
-__device__ __forceinline__ int transport(const Surf& sa, const Surf& sb, const double x[6], const double B[3],
-                         double mass, double h_max, int n_iter, double xp[6], Jac<R>& J,
-                         R& sin_theta, R& cos_inc) {
-  Prop<R> s;
-  double sp, cp, st, ct;
-  sincos(x[2], &sp, &cp);
-  sincos(x[3], &st, &ct);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) s.r[i] = sa.c(i) + x[0] * sa.u(i) + x[1] * sa.v(i);
-  s.T[0] = cp * st;
-  s.T[1] = sp * st;
-  s.T[2] = ct;
-  s.t = x[5];
-  s.lam = x[4];
-  // G columns phi, theta: direction rows = dT/dphi, dT/dtheta; q/p column 0
-  s.gT[0][0] = (R)(-sp * st); s.gT[1][0] = (R)(cp * st); s.gT[2][0] = R(0);
-  s.gT[0][1] = (R)(cp * ct);  s.gT[1][1] = (R)(sp * ct); s.gT[2][1] = (R)(-st);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    s.gT[i][2] = R(0);
-    s.gr[i][0] = s.gr[i][1] = s.gr[i][2] = R(0);
-  }
-  s.gtl = R(0);
-
-  double s0;
-  if (!plane_step(s, sb, s0)) return ST_NO_INTERSECTION;
-  const double nsub_d = ceil(fabs(s0) / h_max);
-  if (!(nsub_d <= 64.0)) return ST_NO_INTERSECTION;
-  const int nsub = nsub_d < 1.0 ? 1 : (int)nsub_d;
-  const double h = s0 / nsub;
-  for (int k = 0; k < nsub; ++k) rkn_step<R, BZ>(s, h, B, mass);
-  for (int it = 0; it < n_iter; ++it) {
-    double si;
-    if (!plane_step(s, sb, si)) return ST_NO_INTERSECTION;
-    rkn_step<R, BZ>(s, si, B, mass);
-  }
-
-  // end point: unit direction and bound angles
-  // square roots and quotients of the end frame from Newton-refined
-  // reciprocal square roots (two steps: double rounding level)
-  const double rho2 = s.T[0] * s.T[0] + s.T[1] * s.T[1];
-  const double irho_d = rsqrt_any(rho2);
-  const double rho_d = rho2 * irho_d;
-  const double phi = atan2(s.T[1], s.T[0]);
-  const double theta = atan2(rho_d, s.T[2]);
-  const R Tr[3] = {(R)s.T[0], (R)s.T[1], (R)s.T[2]};
-  const double itn_d = rsqrt_any(rho2 + s.T[2] * s.T[2]);
-  const R rho = (R)rho_d;
-  const R tn = (R)((rho2 + s.T[2] * s.T[2]) * itn_d);
-  const R cph = Tr[0] * (R)irho_d, sph = Tr[1] * (R)irho_d;
-  const R sth = rho * (R)itn_d, cth = Tr[2] * (R)itn_d;
-  const R nb[3] = {(R)sb.n(0), (R)sb.n(1), (R)sb.n(2)};
-  const R nT = nb[0] * Tr[0] + nb[1] * Tr[1] + nb[2] * Tr[2];
-
-  // path correction: dfree += F' w, w = -(n . position rows) / (n . T),
-  // F' = (T, dt/ds, A T, 0) at the end point.
-  const R lk = (R)(s.lam * kKappa);
-  const R bs[3] = {lk * (R)B[0], lk * (R)B[1], lk * (R)B[2]};
-  R AT[3];
-  applyA<R, BZ>(bs, Tr, AT);
-  const R dtds = (R)(sqrt(1.0 + mass * mass * s.lam * s.lam) * kInvC);
-  const R inv_nT = (R)rcp_any((double)nT);
-  // columns 0..4: loc0, loc1, phi, theta, q/p; full G columns after correction
-  R Gr[3][5], GT[3][5], Gt[5];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    Gr[i][0] = (R)sa.u(i);
-    Gr[i][1] = (R)sa.v(i);
-    Gr[i][2] = s.gr[i][0];
-    Gr[i][3] = s.gr[i][1];
-    Gr[i][4] = s.gr[i][2];
-    GT[i][0] = R(0);
-    GT[i][1] = R(0);
-    GT[i][2] = s.gT[i][0];
-    GT[i][3] = s.gT[i][1];
-    GT[i][4] = s.gT[i][2];
-  }
-  Gt[0] = Gt[1] = Gt[2] = Gt[3] = R(0);
-  Gt[4] = s.gtl;
-#pragma unroll
-  for (int c = 0; c < 5; ++c) {
-    const R w = -(nb[0] * Gr[0][c] + nb[1] * Gr[1][c] + nb[2] * Gr[2][c]) * inv_nT;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Gr[i][c] += Tr[i] * w;
-      GT[i][c] += AT[i] * w;
-    }
-    Gt[c] += dtds * w;
-  }
-  // free -> bound at b
-  const R ub[3] = {(R)sb.u(0), (R)sb.u(1), (R)sb.u(2)};
-  const R vb[3] = {(R)sb.v(0), (R)sb.v(1), (R)sb.v(2)};
-  const R inv_sth = (R)rcp_any((double)sth);
-#pragma unroll
-  for (int c = 0; c < 5; ++c) {
-    J.f[0][c] = ub[0] * Gr[0][c] + ub[1] * Gr[1][c] + ub[2] * Gr[2][c];
-    J.f[1][c] = vb[0] * Gr[0][c] + vb[1] * Gr[1][c] + vb[2] * Gr[2][c];
-    J.f[2][c] = (-sph * GT[0][c] + cph * GT[1][c]) * inv_sth;
-    J.f[3][c] = cph * cth * GT[0][c] + sph * cth * GT[1][c] - sth * GT[2][c];
-    J.ft[c] = Gt[c];
-  }
-  const double d0 = s.r[0] - sb.c(0), d1 = s.r[1] - sb.c(1), d2 = s.r[2] - sb.c(2);
-  xp[0] = d0 * sb.u(0) + d1 * sb.u(1) + d2 * sb.u(2);
-  xp[1] = d0 * sb.v(0) + d1 * sb.v(1) + d2 * sb.v(2);
-  xp[2] = phi;
-  xp[3] = theta;
-  xp[4] = s.lam;
-  xp[5] = s.t;
-  sin_theta = sth;
-  cos_inc = nT / tn;
-  return ST_OK;
-}
-
-
-// ---------------------------------------------------------------------------
-// the fused fit kernel
+// the fused fit: forward filter and fixed-point smoother in one pass
 // ---------------------------------------------------------------------------
 template <bool BZ>
 __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s_surf, int i) {
-  using R = double;
-  using RC = Rec<0>;
   const int t = track_of(p, i);
   const size_t TT = (size_t)p.n_tracks_total;
   const WS ws{p.ws64, p.ws32, (size_t)p.n_tracks, kRec64Fp64, 0, i};
@@ -164,59 +50,71 @@ __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s
       if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
     }
 
-  double xs[6], Cs[21];
+  const bool states = p.out_states != nullptr;
+  // the estimate of state 0, as its offset from the seed (so that the sum over
+  // the states rounds at the offset's size), and its covariance
+  double xs[6], P0[21];
   double chi2sum = 0.0;
   int nmeas = 0;
+  bool spd = true;
   if (status == ST_OK) {
-    // ------------------------------------------------ forward filter
-    double x[6], C[21];
+    double x[6], C[21], S[6][6];
+    Angles ang;
 #pragma unroll
     for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TT + t];
 #pragma unroll
     for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TT + t];
-    int sid_prev = p.surface_id[o0];
-    for (int k = 0; k < n && status == ST_OK; ++k) {
+    int sid_prev = 0;
+    for (int k = 0; k < n; ++k) {
       const int sid = p.surface_id[o0 + k];
-      double xp[6], Cp[21];
-      if (k == 0) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xp[e] = x[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) Cp[e] = C[e];
-      } else {
+      if (k > 0) {
         const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
-        Jac<R> J;
-        R sin_th, cos_inc;
         // field copied to registers: taking the address of a kernel parameter
         // would move the parameter block to local memory
         const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
-        status = transport<R, BZ>(sa, sb, x, Bf, p.mass, p.h_max, p.n_iter, xp, J, sin_th, cos_inc);
-        if (status != ST_OK) break;
-        // Bm = F Cf_{k-1}; Cp = Bm F^T + Q.  F rows 0..3 and 5 over columns
-        // 0..4 are J; row 4 = e4; column 5 = e5.
-        R Cr[21];
+        double r0[3];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) Cr[e] = (R)C[e];
-        R Cpr[21];
+        for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
+        End o;
+        Jac<double> J;
+        {
+          Cols64 g;
+          status = propagate_to_plane<BZ, 7>(sb, r0, ang, x[4], Bf, p.mass, p.h_max, p.n_iter, o, g);
+          if (status != ST_OK) break;
+          double inv_nT;
+          end_frame(sb, o, inv_nT);
+          jacobian_columns<BZ, 31>(sa, sb, o, g, x[4], Bf, inv_nT, [&](int r, int c, double v) {
+            if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
+          });
+        }
+        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
+        x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
+        x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
+        // the filter needs the angles' cosines and sines only
+        if (states) end_angles(x[2], x[3], ang, o, x[2], x[3]);
+        x[5] += o.dt;
+        ang = o.a;
+        const auto fe = [&](int r, int c) { return jf(J, r, c); };
+        // C <- F C F^T, rows of F C formed on the fly
+        double Cp[21];
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
-          R brow[6];
+          double brow[6];
 #pragma unroll
           for (int j = 0; j < 6; ++j) {
-            R v;
+            double v;
             if (r == 4) {
-              v = Cr[sym(4, j)];
+              v = C[sym(4, j)];
             } else {
-              v = jf(J, r, 0) * Cr[sym(0, j)] + jf(J, r, 1) * Cr[sym(1, j)] + jf(J, r, 2) * Cr[sym(2, j)] +
-                  jf(J, r, 3) * Cr[sym(3, j)] + jf(J, r, 4) * Cr[sym(4, j)];
-              if (r == 5) v += Cr[sym(5, j)];
+              v = jf(J, r, 0) * C[sym(0, j)] + jf(J, r, 1) * C[sym(1, j)] + jf(J, r, 2) * C[sym(2, j)] +
+                  jf(J, r, 3) * C[sym(3, j)] + jf(J, r, 4) * C[sym(4, j)];
+              if (r == 5) v += C[sym(5, j)];
             }
             brow[j] = v;
-            RC::put_bm(ws, k, r * 6 + j, brow[j]);
           }
 #pragma unroll
           for (int c = 0; c < 6; ++c) if (c <= r) {
-            R v;
+            double v;
             if (c == 4) {
               v = brow[4];
             } else {
@@ -224,61 +122,103 @@ __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s
                   brow[4] * jf(J, c, 4);
               if (c == 5) v += brow[5];
             }
-            Cpr[sy(r, c)] = v;
+            Cp[sy(r, c)] = v;
           }
         }
-        // multiple scattering of surface k (added before the update)
-        const R xx0 = (R)sb.xx0();
-        if (xx0 > R(0)) {
-          const R th0 = highland<R>((R)fabs(x[4]), (R)(p.mass * p.mass), xx0, cos_inc);
-          const R q = th0 * th0;
-          Cpr[sy(2, 2)] += q / (sin_th * sin_th);
-          Cpr[sy(3, 3)] += q;
-        }
-#pragma unroll
-        for (int e = 0; e < 21; ++e) Cp[e] = (double)Cpr[e];
-      }
-      // record the prediction
-#pragma unroll
-      for (int e = 0; e < 6; ++e) ws.d(k, RC::XP + e) = xp[e];
-#pragma unroll
-      for (int e = 0; e < 21; ++e) ws.d(k, RC::CP + e) = Cp[e];
-      // update
-      if (!p.is_hole[o0 + k]) {
-        const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
-        const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-        double c2 = 0.0;
-        status = kalman_update<R>(xp, Cp, m, V, x, C, c2);
-        if (status != ST_OK) break;
-        chi2sum += c2;
-        ++nmeas;
-      } else {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] = xp[e];
 #pragma unroll
         for (int e = 0; e < 21; ++e) C[e] = Cp[e];
+        // multiple scattering of surface k (added before the update)
+        const double xx0 = sb.xx0();
+        if (xx0 > 0.0) {
+          const double q = highland_sq(x[4], o.g2, xx0, o.inv_cos);
+          C[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, C[sy(2, 2)]);
+          C[sy(3, 3)] += q;
+        }
+        spd = spd && spd_check(C);
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+          double v[6];
+#pragma unroll
+          for (int c = 0; c < 6; ++c) v[c] = S[r][c];
+          row_times_ft(fe, 1.0, v, S[r]);
+        }
+        if (states)
+#pragma unroll
+          for (int e = 0; e < 25; ++e) ws.d(k, StateRec::F + e) = e < 20 ? J.f[e / 5][e % 5] : J.ft[e % 5];
       }
+      // update
+      double K[6][2], ir[2] = {0.0, 0.0}, dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      const bool meas = !p.is_hole[o0 + k];
+      if (meas) {
+        const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
+        const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
+        double Si[3], r[2], c2;
+        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
+        if (status != ST_OK) break;
+        joseph_update(C, V, K);
+        chi2sum += c2;
+        ++nmeas;
 #pragma unroll
-      for (int e = 0; e < 6; ++e) ws.d(k, RC::XF + e) = x[e];
+        for (int e = 0; e < 6; ++e) x[e] += dx[e];
+        ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
+        ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+        if (k > 0) {
+          double hall[6][2];
 #pragma unroll
-      for (int e = 0; e < 21; ++e) RC::put_cf(ws, k, e, (R)C[e]);
+          for (int e = 0; e < 6; ++e) {
+            hall[e][0] = S[e][0];
+            hall[e][1] = S[e][1];
+          }
+#pragma unroll
+          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) K[e][0] = K[e][1] = 0.0;
+      }
+      if (k == 0) {
+        // state 0 starts as its own filtered estimate
+        ang = angles_of(x[2], x[3]);
+#pragma unroll
+        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) P0[e] = C[e];
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
+      } else if (meas) {
+        turn(ang.cp, ang.sp, dx[2]);
+        turn(ang.ct, ang.st, dx[3]);
+      }
+      if (states && k > 0) {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+          ws.d(k, StateRec::K + 2 * e) = K[e][0];
+          ws.d(k, StateRec::K + 2 * e + 1) = K[e][1];
+          ws.d(k, StateRec::XF + e) = x[e];
+        }
+        ws.d(k, StateRec::IR) = ir[0];
+        ws.d(k, StateRec::IR + 1) = ir[1];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) ws.d(k, StateRec::CF + e) = C[e];
+      }
       sid_prev = sid;
     }
-
-    // ------------------------------------------------ RTS smoother
-    if (status == ST_OK) {
+    if (status == ST_OK && !spd) status = ST_NON_SPD;
 #pragma unroll
-      for (int e = 0; e < 6; ++e) xs[e] = x[e];
+    for (int e = 0; e < 6; ++e) xs[e] += p.seed_params[e * TT + t];
+    if (status == ST_OK && states) {
+      smooth_states(ws, n, p.out_states, p.n_states, o0);
 #pragma unroll
-      for (int e = 0; e < 21; ++e) Cs[e] = C[e];
-      status = rts_smooth_fp64(ws, n, xs, Cs, p.out_states, p.n_states, o0);
+      for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0] = xs[e];
     }
     if (status == ST_OK) {
       bool fin = isfinite(chi2sum);
 #pragma unroll
       for (int e = 0; e < 6; ++e) fin = fin && isfinite(xs[e]);
 #pragma unroll
-      for (int e = 0; e < 21; ++e) fin = fin && isfinite(Cs[e]);
+      for (int e = 0; e < 21; ++e) fin = fin && isfinite(P0[e]);
       if (!fin) status = ST_NONFINITE;
     }
   }
@@ -287,7 +227,7 @@ __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s
 #pragma unroll
     for (int e = 0; e < 6; ++e) xs[e] = nan;
 #pragma unroll
-    for (int e = 0; e < 21; ++e) Cs[e] = nan;
+    for (int e = 0; e < 21; ++e) P0[e] = nan;
     chi2sum = nan;
     nmeas = 0;
     if (p.out_states && n >= 1 && o0 >= 0 && o1 <= p.n_states && n <= p.max_states)
@@ -297,7 +237,7 @@ __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s
 #pragma unroll
   for (int e = 0; e < 6; ++e) p.out_params[e * TT + t] = xs[e];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = Cs[e];
+  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = P0[e];
   p.out_chi2[t] = chi2sum;
   if (p.out_ndf) p.out_ndf[t] = 2 * nmeas;
   if (p.out_status) p.out_status[t] = (uint8_t)status;
