@@ -7,15 +7,24 @@
 //   * FP32: RKN stages, the step Jacobians, path correction, the 6x6
 //     transport F C F^T, the Highland noise, the gain K, the smoother gain
 //     algebra and the smoothed covariance.
-//   * FP64: the Joseph covariance update, chi2, the LDL^T factorisation
-//     of the predicted covariance and its solves (the smoother's inverse).
-//   * Double-float pairs of FP32 values (about 48 bits): the track's point,
-//     direction, angles, q/p and time between surfaces, which only receive
-//     FP32 increments and meet the plane geometry (split the same way in
-//     this kernel's own surface table) in dot products; no FP64 instruction
-//     is spent on them.
-//   * float<->double conversions run on the integer pipe (dev::f2d/d2f);
-//     FP64 1/sqrt and 1/x come from float seeds refined by a Newton step.
+//   * Double-float pairs of FP32 values (about 48 bits), on the FP32 pipe:
+//     the track's point, direction, angles, q/p and time between surfaces;
+//     the Joseph covariance update and chi2; the LDL^T factorisation of the
+//     predicted covariance and its solves (the smoother's inverse).  A warp's
+//     FP64 instruction holds the pipe of its sub-partition for 64 cycles, the
+//     pair form of the same operation takes 7 to 15 issue slots.  With these
+//     pieces in FP64 (about 145 instructions and 120 conversions per state)
+//     100k tracks of 31 states took 1.42 ms, with the pairs 0.80 ms; 1M uneven
+//     tracks 8.41 -> 5.28 ms, one event of 3001 tracks 0.209 -> 0.132 ms.
+//     Against an 80-bit evaluation of the fit the rms errors are the same
+//     (0.9 to 1.04 times the former; ten shapes of 2000 tracks): the float
+//     quantities set them.  What bounds it now is issue: 4950 instructions per
+//     state and warp, 59 % of the issue slots used, the rest waits for the
+//     records and for dependent results.
+//   * FP64 only for the seed: its direction's sines and cosines, and the
+//     update of state 0 where that is measured.
+//   * float<->double conversions run on the integer pipe (dev::f2d/d2f,
+//     df_cut).
 //   * The direction is carried as (phi, theta) with their cosines and
 //     sines; propagation and updates change them by small rotations, so no
 //     trigonometry of the carried angles runs after the seed.
@@ -26,8 +35,10 @@
 // and the smoothed covariance Cs = Cf + A (Cs' - Cp') A^T equals
 //   Cs = F^-1 (Q - Q Cp'^-1 Q) F^-T + A Cs' A^T,
 // a sum of two positive semi-definite terms (no cancellation against Cf).
-// Only the (phi, theta) columns of Cp'^-1 are needed: one FP64 LDL^T
-// factorisation of a 4x4 block and two FP64 triangular-solve pairs per state.
+// Only the (phi, theta) columns of Cp'^-1 are needed: one LDL^T
+// factorisation of a 4x4 block and two triangular-solve pairs per state; and
+// since I - Q Cp'^-1 differs from the identity in two rows, A Cs' A^T is two
+// row products and one sandwich with F^-1.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -42,8 +53,7 @@ using namespace dev;
 // per-state record: x_p in FP64 (written for state 0, and for every state
 // when the smoothed states are output); in FP32 the transport Jacobian, the
 // scattering variances, the filter increment and the predicted covariance
-// (its values are FP32 products, so the float copy is exact; the smoother
-// promotes them for its FP64 inverse)
+// (its values are FP32 products, so the float copy is exact)
 constexpr int XP = 0;                                           // ws64 fields
 constexpr int FJ = 0, QPHI = 25, QTH = 26, DXF = 27, CPF = 33;  // ws32 fields
 
@@ -96,6 +106,35 @@ __device__ __forceinline__ double df_to_d(DF x) { return f2d(x.hi) + f2d(x.lo); 
 __device__ __forceinline__ DF df_from_d(double v) {
   const float h = d2f(v);
   return {h, d2f(v - f2d(h))};
+}
+// from FP64 without an FP64 instruction: hi is the value cut to 24 bits, lo
+// the float of the 29 bits cut off (integer pipe), so hi + lo is within 2^-48
+// of the value; below 2^-96 the rest is dropped.  Zero, Inf and NaN as d2f.
+__device__ __forceinline__ DF df_cut(double v) {
+  const uint32_t w = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+  const uint32_t ah = w & 0x7fffffffu, sg = w & 0x80000000u;
+  if (ah < 0x38100000u || ah >= 0x47e00000u) return {d2f(v), 0.0f};
+  const uint32_t r = __funnelshift_l(l, ah, 3) + 0x40000000u;  // see d2f
+  const float hi = __uint_as_float(r | sg);
+  const uint32_t e = r >> 23;  // biased exponent of hi
+  if (e < 31u) return {hi, 0.0f};
+  // rest = (l mod 2^29) 2^-29 ulp(hi), ulp(hi) = 2^(e - 150)
+  const float ulp = __uint_as_float(((e - 23u) << 23) | sg);
+  return fast_two_sum(hi, (float)(l & 0x1fffffffu) * 0x1p-29f * ulp);
+}
+// acc - a * b
+__device__ __forceinline__ DF df_fnma(DF acc, DF a, DF b) {
+  const DF p = two_prod(a.hi, b.hi);
+  const float c = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
+  const DF s = two_sum(acc.hi, -p.hi);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(acc.lo, c)));
+}
+// 1 / x: a float reciprocal and one Newton step (relative error about 2^-44)
+__device__ __forceinline__ DF df_rcp(DF x) {
+  const float y = __frcp_rn(x.hi);
+  const DF p = two_prod(x.hi, y);
+  const float e = __fmaf_rn(-x.lo, y, __fsub_rn(__fsub_rn(1.0f, p.hi), p.lo));
+  return fast_two_sum(y, __fmul_rn(y, e));
 }
 // w . r - w0 for a vector w given as hi / lo float arrays and a df offset
 // w0: Dot2 (the products split exactly by FMA, the running sum by TwoSum,
@@ -200,6 +239,10 @@ __device__ __forceinline__ void cols_step(Cols& g, float h, const float bs[3], c
     applyA<float, BZ>(bs, b3, b4);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
+      if (BZ && i == 2) {  // the field turns the (x, y) components only
+        g.gr[i][c] += h * v[i];
+        continue;
+      }
       float dr = h * v[i] + h2 * b1[i] + h3 * b2[i] + h4 * b3[i];
       float nt = v[i] + h * b1[i] + h2 * b2[i] + h3 * b3[i] + h4 * b4[i];
       if (c == 2) {
@@ -225,6 +268,10 @@ __device__ __forceinline__ void value_step(float h, const float bs[3], const flo
   applyA<float, BZ>(bs, a3, a4);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
+    if (BZ && i == 2) {
+      dr[i] = dT[i] = 0.0f;
+      continue;
+    }
     dr[i] = h2 * a1[i] + h3 * a2[i] + h4 * a3[i];
     dT[i] = h * a1[i] + h2 * a2[i] + h3 * a3[i] + h4 * a4[i];
   }
@@ -585,86 +632,156 @@ __device__ __forceinline__ void invert_F(const float F[25], float Fi[6][6]) {
   Fi[5][5] = 1.0f;
 }
 
-// Columns phi and theta of Cp^-1 in FP64, by block elimination with the
-// angle block last: a = (loc0, loc1, q/p, t), b = (phi, theta).
+// Columns phi and theta of Cp^-1 in double-float arithmetic, by block
+// elimination with the angle block last: a = (loc0, loc1, q/p, t),
+// b = (phi, theta).
 //   X = Caa^-1 Cab (4x4 LDL^T, two solves), Sig = Cbb - Cab^T X (the 2x2
 //   Schur complement), then (Cp^-1)[b][b] = Sig^-1, (Cp^-1)[a][b] = -X Sig^-1.
-// Cp is SPD iff the four pivots of Caa and Sig are positive.  Returns false
-// otherwise.  w[0] = Cp^-1 e_phi, w[1] = Cp^-1 e_theta (6 each).
-__device__ __forceinline__ bool angle_columns_of_inverse(const double Cp[21], double w[2][6]) {
+// Cp (floats, exact) is SPD iff the four pivots of Caa and Sig are positive.
+// Returns false otherwise.  w[0] = Cp^-1 e_phi, w[1] = Cp^-1 e_theta.
+//
+// A warp DFMA takes the narrow FP64 pipe of a sub-partition for 64 cycles;
+// the double-float form of a multiply-subtract is 15 FP32 instructions, one
+// issue slot each.  The relative error of each operation is about 2^-46
+// against 2^-53, far below that of the float covariance itself.
+__device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF w[2][6]) {
   constexpr int ia[4] = {0, 1, 4, 5};
   // LDL^T of the 4x4 block (no square roots): U = L D below the diagonal
-  double L[4][4], U[4][4], iD[4];
+  DF L[4][4], U[4][4], iD[4];
   bool ok = true;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    double dj = Cp[sym(ia[j], ia[j])];
+    DF dj = {Cp[sym(ia[j], ia[j])], 0.0f};
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (q < j) dj = fma(-U[j][q], L[j][q], dj);
-    if (!dpos(dj)) {
+      if (q < j) dj = df_fnma(dj, U[j][q], L[j][q]);
+    if (!(dj.hi > 0.0f)) {
       ok = false;
-      dj = 1.0;
+      dj = {1.0f, 0.0f};
     }
-    iD[j] = rcp_nr<1>(dj);
+    iD[j] = df_rcp(dj);
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       if (r > j) {
-        double u = Cp[sym(ia[r], ia[j])];
+        DF u = {Cp[sym(ia[r], ia[j])], 0.0f};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q < j) u = fma(-U[r][q], L[j][q], u);
+          if (q < j) u = df_fnma(u, U[r][q], L[j][q]);
         U[r][j] = u;
-        L[r][j] = u * iD[j];
+        L[r][j] = df_mul(u, iD[j]);
       }
     }
   }
   // X = Caa^-1 Cab: unit-lower forward solve, scaling by D^-1, unit-upper
   // backward solve
-  double X[4][2];
+  DF X[4][2];
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
-    double y[4];
+    DF y[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      double v = Cp[sym(ia[r], 2 + m)];
+      DF v = {Cp[sym(ia[r], 2 + m)], 0.0f};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q < r) v = fma(-L[r][q], y[q], v);
+        if (q < r) v = df_fnma(v, L[r][q], y[q]);
       y[r] = v;
     }
 #pragma unroll
     for (int r = 3; r >= 0; --r) {
-      double v = y[r] * iD[r];
+      DF v = df_mul(y[r], iD[r]);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q > r) v = fma(-L[q][r], X[q][m], v);
+        if (q > r) v = df_fnma(v, L[q][r], X[q][m]);
       X[r][m] = v;
     }
   }
-  double s00 = Cp[sy(2, 2)], s01 = Cp[sy(3, 2)], s11 = Cp[sy(3, 3)];
+  DF s00 = {Cp[sy(2, 2)], 0.0f}, s01 = {Cp[sy(3, 2)], 0.0f}, s11 = {Cp[sy(3, 3)], 0.0f};
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
-    s00 = fma(-Cp[sym(ia[r], 2)], X[r][0], s00);
-    s01 = fma(-Cp[sym(ia[r], 2)], X[r][1], s01);
-    s11 = fma(-Cp[sym(ia[r], 3)], X[r][1], s11);
+    const DF c2 = {Cp[sym(ia[r], 2)], 0.0f}, c3 = {Cp[sym(ia[r], 3)], 0.0f};
+    s00 = df_fnma(s00, X[r][0], c2);
+    s01 = df_fnma(s01, X[r][1], c2);
+    s11 = df_fnma(s11, X[r][1], c3);
   }
-  const double det = fma(s00, s11, -s01 * s01);
-  if (!dpos(det) || !dpos(s00)) {
+  const DF det = df_fnma(df_mul(s00, s11), s01, s01);
+  if (!(det.hi > 0.0f) || !(s00.hi > 0.0f)) {
     ok = false;
   }
-  const double idet = rcp_nr<1>(det);
-  const double i00 = s11 * idet, i01 = -s01 * idet, i11 = s00 * idet;
+  const DF idet = df_rcp(det);
+  const DF i00 = df_mul(s11, idet), i01 = df_neg(df_mul(s01, idet)), i11 = df_mul(s00, idet);
   w[0][2] = i00;
   w[0][3] = i01;
   w[1][2] = i01;
   w[1][3] = i11;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
-    w[0][ia[r]] = -fma(X[r][0], i00, X[r][1] * i01);
-    w[1][ia[r]] = -fma(X[r][0], i01, X[r][1] * i11);
+    w[0][ia[r]] = df_fnma(df_neg(df_mul(X[r][0], i00)), X[r][1], i01);
+    w[1][ia[r]] = df_fnma(df_neg(df_mul(X[r][0], i01)), X[r][1], i11);
   }
   return ok;
+}
+
+// 1 - q w in float, without the cancellation a rounded w would leave
+__device__ __forceinline__ float one_minus(float q, DF w) {
+  const DF p = two_prod(q, w.hi);
+  return __fmaf_rn(-q, w.lo, __fsub_rn(__fsub_rn(1.0f, p.hi), p.lo));
+}
+
+// The update of state 0 where the seed's own plane measures: the seed
+// covariance comes in FP64, so this one update (out of line, once per track)
+// runs there.
+struct SeedUpdate {
+  float Cf[21], dx[6];
+  DF chi2;
+  bool ok;
+};
+static __device__ __noinline__ void update_seed(const double* __restrict__ seed_cov, size_t stride, double r0, double r1,
+                                                double V0, double V1, double V2, SeedUpdate* o) {
+  double Cp[21];
+  float Cpf[21];
+#pragma unroll
+  for (int e = 0; e < 21; ++e) {
+    Cp[e] = seed_cov[e * stride];
+    Cpf[e] = d2f(Cp[e]);
+  }
+  const double S00 = V0 + Cp[sy(0, 0)], S01 = V1 + Cp[sy(1, 0)], S11 = V2 + Cp[sy(1, 1)];
+  const double det = fma(S00, S11, -S01 * S01);
+  o->ok = dpos(det) && dpos(S00);
+  if (!o->ok) return;
+  const double idet = rcp_nr<1>(det);
+  const double u = fma(S11, r0, -S01 * r1), v = fma(S00, r1, -S01 * r0);
+  o->chi2 = df_from_d(fma(r0, u, r1 * v) * idet);
+  const float idf = d2f(idet);
+  const float i00 = d2f(S11) * idf, i01 = -d2f(S01) * idf, i11 = d2f(S00) * idf;
+  const float r0f = d2f(r0), r1f = d2f(r1);
+  double K[6][2];
+  float Kf[6][2];
+#pragma unroll
+  for (int e = 0; e < 6; ++e) {
+    const float c0 = Cpf[sym(e, 0)], c1 = Cpf[sym(e, 1)];
+    const float k0 = c0 * i00 + c1 * i01, k1 = c0 * i01 + c1 * i11;
+    Kf[e][0] = k0;
+    Kf[e][1] = k1;
+    K[e][0] = f2d(k0);
+    K[e][1] = f2d(k1);
+    o->dx[e] = k0 * r0f + k1 * r1f;
+  }
+  float Wf[2][6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    Wf[0][j] = d2f(fma(S00, K[j][0], fma(S01, K[j][1], -Cp[sym(0, j)])));
+    Wf[1][j] = d2f(fma(S01, K[j][0], fma(S11, K[j][1], -Cp[sym(1, j)])));
+  }
+#pragma unroll
+  for (int a = 0; a < 6; ++a)
+#pragma unroll
+    for (int b = 0; b < 6; ++b)
+      if (b <= a) {
+        double c = Cp[sy(a, b)];
+        c = fma(-Cp[sym(0, a)], K[b][0], c);
+        c = fma(-Cp[sym(1, a)], K[b][1], c);
+        o->Cf[sy(a, b)] = d2f(c) + (Kf[a][0] * Wf[0][b] + Kf[a][1] * Wf[1][b]);
+      }
 }
 
 template <bool BZ>
@@ -690,7 +807,7 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
 
   double xs[6];
   double Cs_out[21];
-  double chi2sum = 0.0;
+  DF chi2sum = {0.0f, 0.0f};
   int nmeas = 0;
   if (status == ST_OK) {
     // ------------------------------------------------ forward filter
@@ -698,7 +815,8 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
     // (point r, direction d, time x[5]) plus the filter's FP32 increments
     // in pd, which the next transport applies; the filtered q/p is x[4].
     // The filtered covariance is kept in FP32 between states: it only feeds
-    // the FP32 transport F Cf F^T (the Joseph update produces it in FP64).
+    // the FP32 transport F Cf F^T (the Joseph update produces it in
+    // double-float arithmetic).
     DF x[6], r[3];
     Pend pd = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, 0.0f, 0.0f, 0.0f};
     CS cs;  // float cosines / sines of the filtered direction
@@ -731,17 +849,13 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
     for (int k = 0; k < n && status == ST_OK; ++k) {
       const int sid = p.surface_id[o0 + k];
       DF xp[6], rp[3];
-      double Cp[21];
       float Cpf[21];
       Dir dp;
       if (k == 0) {
 #pragma unroll
         for (int e = 0; e < 6; ++e) xp[e] = x[e];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) {
-          Cp[e] = p.seed_cov[e * TT + t];
-          Cpf[e] = d2f(Cp[e]);
-        }
+        for (int e = 0; e < 21; ++e) Cpf[e] = d2f(p.seed_cov[e * TT + t]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) rp[c] = r[c];
         dp = d;
@@ -799,8 +913,6 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
         for (int e = 0; e < 5; ++e) ws.f(k, FJ + 20 + e) = J.ft[e];
         ws.f(k, QPHI) = qphi;
         ws.f(k, QTH) = qth;
-#pragma unroll
-        for (int e = 0; e < 21; ++e) Cp[e] = f2d(Cpf[e]);
       }
       if (k == 0 || p.out_states) {
 #pragma unroll
@@ -812,58 +924,80 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
       }
       const SurfM sk = surf_m(s_surf, sid);
       if (!p.is_hole[o0 + k]) {
-        // gain-matrix update: gain in FP32, Joseph covariance (but its K W term)
-        // and chi2 in FP64
         const double m0 = p.loc[o0 + k], m1 = p.loc[p.n_states + o0 + k];
         const double V0 = p.cov[o0 + k], V1 = p.cov[p.n_states + o0 + k], V2 = p.cov[2 * p.n_states + o0 + k];
-        const double S00 = V0 + Cp[sy(0, 0)], S01 = V1 + Cp[sy(1, 0)], S11 = V2 + Cp[sy(1, 1)];
-        const double det = fma(S00, S11, -S01 * S01);
-        if (!dpos(det) || !dpos(S00)) {
-          status = ST_NON_SPD;
-          break;
+        if (k == 0) {
+          SeedUpdate su;
+          update_seed(p.seed_cov + t, TT, (m0 - f2d(xp[0].hi)) - f2d(xp[0].lo), (m1 - f2d(xp[1].hi)) - f2d(xp[1].lo),
+                      V0, V1, V2, &su);
+          if (!su.ok) {
+            status = ST_NON_SPD;
+            break;
+          }
+          chi2sum = su.chi2;
+#pragma unroll
+          for (int e = 0; e < 6; ++e) dx[e] = su.dx[e];
+#pragma unroll
+          for (int e = 0; e < 21; ++e) Cf[e] = su.Cf[e];
+        } else {
+          // gain-matrix update: gain in FP32, the Joseph covariance and chi2
+          // in double-float arithmetic on the FP32 pipe.  The FP64 form took
+          // 90 FP64 instructions and 120 conversions per state.
+          const DF S00 = df_add_f(df_cut(V0), Cpf[sy(0, 0)]), S01 = df_add_f(df_cut(V1), Cpf[sy(1, 0)]),
+                   S11 = df_add_f(df_cut(V2), Cpf[sy(1, 1)]);
+          const DF det = df_fnma(df_mul(S00, S11), S01, S01);
+          if (!(det.hi > 0.0f) || !(S00.hi > 0.0f)) {
+            status = ST_NON_SPD;
+            break;
+          }
+          const DF idet = df_rcp(det);
+          const DF r0 = df_add(df_cut(m0), df_neg(xp[0])), r1 = df_add(df_cut(m1), df_neg(xp[1]));
+          const DF u = df_fnma(df_mul(S11, r0), S01, r1), v = df_fnma(df_mul(S00, r1), S01, r0);
+          chi2sum = df_add(chi2sum, df_mul(df_add(df_mul(r0, u), df_mul(r1, v)), idet));
+          const float idf = df_f(idet);
+          const float i00 = df_f(S11) * idf, i01 = -df_f(S01) * idf, i11 = df_f(S00) * idf;
+          const float r0f = df_f(r0), r1f = df_f(r1);
+          float Kf[6][2];
+#pragma unroll
+          for (int e = 0; e < 6; ++e) {
+            const float c0 = Cpf[sym(e, 0)], c1 = Cpf[sym(e, 1)];
+            const float k0 = c0 * i00 + c1 * i01, k1 = c0 * i01 + c1 * i11;
+            Kf[e][0] = k0;
+            Kf[e][1] = k1;
+            dx[e] = k0 * r0f + k1 * r1f;
+          }
+          // Joseph form, expanded: Cf = Cp - (H Cp)^T K^T + K W with
+          // W = S K^T - H Cp.  For the exact gain W = 0; here W is the
+          // residual of the gain equation left by the FP32 gain,
+          // O(eps32 |H Cp|).  Its products are exact (FMA splits), its
+          // cancelling sum is compensated (TwoSum); the element's own sum
+          // Cp - c0 K0 - c1 K1 likewise, with K W added to the low parts.
+          float Wf[2][6];
+          auto w_of = [](DF Sa, DF Sb, float k0, float k1, float c) {
+            const DF pa = two_prod(Sa.hi, k0), pb = two_prod(Sb.hi, k1);
+            const DF x1 = two_sum(pa.hi, -c);
+            const DF x2 = two_sum(x1.hi, pb.hi);
+            const float lo = __fadd_rn(__fadd_rn(x1.lo, x2.lo), __fadd_rn(pa.lo, pb.lo));
+            return __fadd_rn(x2.hi, __fmaf_rn(Sa.lo, k0, __fmaf_rn(Sb.lo, k1, lo)));
+          };
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            Wf[0][j] = w_of(S00, S01, Kf[j][0], Kf[j][1], Cpf[sym(0, j)]);
+            Wf[1][j] = w_of(S01, S11, Kf[j][0], Kf[j][1], Cpf[sym(1, j)]);
+          }
+#pragma unroll
+          for (int a = 0; a < 6; ++a)
+#pragma unroll
+            for (int b = 0; b < 6; ++b)
+              if (b <= a) {
+                const DF pa = two_prod(Cpf[sym(0, a)], Kf[b][0]), pb = two_prod(Cpf[sym(1, a)], Kf[b][1]);
+                const DF x1 = two_sum(Cpf[sy(a, b)], -pa.hi);
+                const DF x2 = two_sum(x1.hi, -pb.hi);
+                const float lo = __fsub_rn(__fsub_rn(__fadd_rn(x1.lo, x2.lo), pa.lo), pb.lo);
+                Cf[sy(a, b)] = __fadd_rn(x2.hi, __fmaf_rn(Kf[a][0], Wf[0][b], __fmaf_rn(Kf[a][1], Wf[1][b], lo)));
+              }
         }
-        const double idet = rcp_nr<1>(det);
-        const double r0 = (m0 - f2d(xp[0].hi)) - f2d(xp[0].lo), r1 = (m1 - f2d(xp[1].hi)) - f2d(xp[1].lo);
-        const double u = fma(S11, r0, -S01 * r1), v = fma(S00, r1, -S01 * r0);
-        chi2sum += fma(r0, u, r1 * v) * idet;
         ++nmeas;
-        const float idf = d2f(idet);
-        const float i00 = d2f(S11) * idf, i01 = -d2f(S01) * idf, i11 = d2f(S00) * idf;
-        const float r0f = d2f(r0), r1f = d2f(r1);
-        double K[6][2];
-        float Kf[6][2];
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          const float c0 = Cpf[sym(e, 0)], c1 = Cpf[sym(e, 1)];
-          const float k0 = c0 * i00 + c1 * i01, k1 = c0 * i01 + c1 * i11;
-          Kf[e][0] = k0;
-          Kf[e][1] = k1;
-          K[e][0] = f2d(k0);
-          K[e][1] = f2d(k1);
-          dx[e] = k0 * r0f + k1 * r1f;
-        }
-        // Joseph form, expanded: Cf = Cp - (H Cp)^T K^T + K W with
-        // W = S K^T - H Cp.  For the exact gain W = 0; here W is the residual
-        // of the gain equation left by the FP32 gain, O(eps32 |H Cp|), so
-        // the term K W is O(eps32 |Cp|).  FP64 takes the cancelling part
-        // (Cp - (H Cp)^T K^T, and W itself); K W is summed in FP32 onto the
-        // rounded result, which carries it to O(eps32^2 |Cp|).
-        float Wf[2][6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          Wf[0][j] = d2f(fma(S00, K[j][0], fma(S01, K[j][1], -Cp[sym(0, j)])));
-          Wf[1][j] = d2f(fma(S01, K[j][0], fma(S11, K[j][1], -Cp[sym(1, j)])));
-        }
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-          for (int b = 0; b < 6; ++b)
-            if (b <= a) {
-              double v = Cp[sy(a, b)];
-              v = fma(-Cp[sym(0, a)], K[b][0], v);
-              v = fma(-Cp[sym(1, a)], K[b][1], v);
-              Cf[sy(a, b)] = d2f(v) + (Kf[a][0] * Wf[0][b] + Kf[a][1] * Wf[1][b]);
-            }
         // the filtered state: the prediction plus the increments, which stay
         // pending in FP32 (the point moves in the plane by (dx0, dx1)); only
         // q/p is updated here
@@ -906,68 +1040,115 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
 #pragma unroll
         for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0 + n - 1] = ws.d(n - 1, XP + e) + f2d(dx[e]);
       for (int k = n - 2; k >= 0 && status == ST_OK; --k) {
-        // FP64: the (phi, theta) columns of Cp_{k+1}^-1
-        double Cp1[21];
+        // the (phi, theta) columns of Cp_{k+1}^-1
+        float Cp1[21];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) Cp1[e] = f2d(ws.f(k + 1, CPF + e));
-        double w[2][6];
+        for (int e = 0; e < 21; ++e) Cp1[e] = ws.f(k + 1, CPF + e);
+        DF w[2][6];
         if (!angle_columns_of_inverse(Cp1, w)) {
           status = ST_NON_SPD;
           break;
         }
-        // noise-rank pieces: Q Cp^-1 rows (phi, theta) and N = Q - Q Cp^-1 Q
+        // A = F^-1 M with M = I - Q Cp^-1, which differs from the identity in
+        // its rows phi (m0) and theta (m1) only; N = Q - Q Cp^-1 Q
         const float qp = ws.f(k + 1, QPHI), qt = ws.f(k + 1, QTH);
-        const double qpd = f2d(qp), qtd = f2d(qt);
-        float qw[2][6];
+        float m0[6], m1[6];
 #pragma unroll
         for (int e = 0; e < 6; ++e) {
-          qw[0][e] = qp * d2f(w[0][e]);
-          qw[1][e] = qt * d2f(w[1][e]);
+          m0[e] = -qp * df_f(w[0][e]);
+          m1[e] = -qt * df_f(w[1][e]);
         }
-        const float Npp = d2f(qpd * fma(-qpd, w[0][2], 1.0));
-        const float Ntt = d2f(qtd * fma(-qtd, w[1][3], 1.0));
-        const float Npt = d2f(-qpd * qtd * w[1][2]);
-        // F^-1 and the gain A = F^-1 - F^-1[:,phi] qw_phi^T - F^-1[:,theta] qw_theta^T
+        m0[2] = one_minus(qp, w[0][2]);
+        m1[3] = one_minus(qt, w[1][3]);
+        const float Npp = qp * m0[2], Ntt = qt * m1[3], Npt = qp * m1[2];
         float Fr[25];
 #pragma unroll
         for (int e = 0; e < 25; ++e) Fr[e] = ws.f(k + 1, FJ + e);
         float Fi[6][6];
         invert_F(Fr, Fi);
-        float A[6][6];
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-          for (int c = 0; c < 6; ++c) A[a][c] = Fi[a][c] - Fi[a][2] * qw[0][c] - Fi[a][3] * qw[1][c];
-        // off_k = A (dxf_{k+1} + off_{k+1})
+        // off_k = F^-1 M (dxf_{k+1} + off_{k+1})
         float dd[6];
 #pragma unroll
         for (int e = 0; e < 6; ++e) dd[e] = ws.f(k + 1, DXF + e) + off[e];
+        {
+          float d2 = 0.0f, d3 = 0.0f;
+#pragma unroll
+          for (int e = 0; e < 6; ++e) {
+            d2 += m0[e] * dd[e];
+            d3 += m1[e] * dd[e];
+          }
+          dd[2] = d2;
+          dd[3] = d3;
+        }
+        // F^-1 has row q/p = e4 and column t = e5
 #pragma unroll
         for (int a = 0; a < 6; ++a) {
-          float acc = 0.0f;
+          if (a == 4) {
+            off[a] = dd[4];
+            continue;
+          }
+          float acc = a == 5 ? dd[5] : 0.0f;
 #pragma unroll
-          for (int c = 0; c < 6; ++c) acc += A[a][c] * dd[c];
+          for (int c = 0; c < 5; ++c) acc += Fi[a][c] * dd[c];
           off[a] = acc;
         }
-        // Cs_k = F^-1 N F^-T (N on the (phi, theta) block) + A Cs_{k+1} A^T
+        // X = M Cs_{k+1} M^T + N: rows (and columns) phi and theta change
+        {
+          float y0[6], y1[6];
+#pragma unroll
+          for (int c = 0; c < 6; ++c) {
+            float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+              a0 += m0[q] * Cs[sym(q, c)];
+              a1 += m1[q] * Cs[sym(q, c)];
+            }
+            y0[c] = a0;
+            y1[c] = a1;
+          }
+          float x22 = Npp, x32 = Npt, x33 = Ntt;
+#pragma unroll
+          for (int q = 0; q < 6; ++q) {
+            x22 += m0[q] * y0[q];
+            x32 += m1[q] * y0[q];
+            x33 += m1[q] * y1[q];
+          }
+#pragma unroll
+          for (int c = 0; c < 6; ++c) {
+            if (c == 2 || c == 3) continue;
+            Cs[sym(2, c)] = y0[c];
+            Cs[sym(3, c)] = y1[c];
+          }
+          Cs[sy(2, 2)] = x22;
+          Cs[sy(3, 2)] = x32;
+          Cs[sy(3, 3)] = x33;
+        }
+        // Cs_k = F^-1 X F^-T
         float Cn[21];
 #pragma unroll
         for (int a = 0; a < 6; ++a) {
           float z[6];
 #pragma unroll
           for (int c = 0; c < 6; ++c) {
-            float acc = 0.0f;
+            if (a == 4) {
+              z[c] = Cs[sym(4, c)];
+              continue;
+            }
+            float acc = a == 5 ? Cs[sym(5, c)] : 0.0f;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) acc += A[a][q] * Cs[sym(q, c)];
+            for (int q = 0; q < 5; ++q) acc += Fi[a][q] * Cs[sym(q, c)];
             z[c] = acc;
           }
-          const float a2 = Fi[a][2] * Npp + Fi[a][3] * Npt, a3 = Fi[a][2] * Npt + Fi[a][3] * Ntt;
 #pragma unroll
           for (int c = 0; c < 6; ++c)
             if (c <= a) {
-              float acc = a2 * Fi[c][2] + a3 * Fi[c][3];
+              if (c == 4) {
+                Cn[sy(a, c)] = z[4];
+                continue;
+              }
+              float acc = c == 5 ? z[5] : 0.0f;
 #pragma unroll
-              for (int q = 0; q < 6; ++q) acc += z[q] * A[c][q];
+              for (int q = 0; q < 5; ++q) acc += z[q] * Fi[c][q];
               Cn[sy(a, c)] = acc;
             }
         }
@@ -996,7 +1177,7 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
       }
     }
     if (status == ST_OK) {
-      bool fin = isfinite(chi2sum);
+      bool fin = isfinite(chi2sum.hi);
 #pragma unroll
       for (int e = 0; e < 6; ++e) fin = fin && isfinite(xs[e]);
 #pragma unroll
@@ -1004,13 +1185,14 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
       if (!fin) status = ST_NONFINITE;
     }
   }
+  double chi2 = df_to_d(chi2sum);
   if (status != ST_OK) {
     const double nan = qnan();
 #pragma unroll
     for (int e = 0; e < 6; ++e) xs[e] = nan;
 #pragma unroll
     for (int e = 0; e < 21; ++e) Cs_out[e] = nan;
-    chi2sum = nan;
+    chi2 = nan;
     nmeas = 0;
     if (p.out_states && n >= 1 && o0 >= 0 && o1 <= p.n_states && n <= p.max_states)
       for (int k = 0; k < n; ++k)
@@ -1020,7 +1202,7 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
   for (int e = 0; e < 6; ++e) p.out_params[e * TT + t] = xs[e];
 #pragma unroll
   for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = Cs_out[e];
-  p.out_chi2[t] = chi2sum;
+  p.out_chi2[t] = chi2;
   if (p.out_ndf) p.out_ndf[t] = 2 * nmeas;
   if (p.out_status) p.out_status[t] = (uint8_t)status;
 }
