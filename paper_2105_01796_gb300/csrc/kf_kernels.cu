@@ -95,38 +95,7 @@ __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s
         x[5] += o.dt;
         ang = o.a;
         const auto fe = [&](int r, int c) { return jf(J, r, c); };
-        // C <- F C F^T, rows of F C formed on the fly
-        double Cp[21];
-#pragma unroll
-        for (int r = 0; r < 6; ++r) {
-          double brow[6];
-#pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            double v;
-            if (r == 4) {
-              v = C[sym(4, j)];
-            } else {
-              v = jf(J, r, 0) * C[sym(0, j)] + jf(J, r, 1) * C[sym(1, j)] + jf(J, r, 2) * C[sym(2, j)] +
-                  jf(J, r, 3) * C[sym(3, j)] + jf(J, r, 4) * C[sym(4, j)];
-              if (r == 5) v += C[sym(5, j)];
-            }
-            brow[j] = v;
-          }
-#pragma unroll
-          for (int c = 0; c < 6; ++c) if (c <= r) {
-            double v;
-            if (c == 4) {
-              v = brow[4];
-            } else {
-              v = brow[0] * jf(J, c, 0) + brow[1] * jf(J, c, 1) + brow[2] * jf(J, c, 2) + brow[3] * jf(J, c, 3) +
-                  brow[4] * jf(J, c, 4);
-              if (c == 5) v += brow[5];
-            }
-            Cp[sy(r, c)] = v;
-          }
-        }
-#pragma unroll
-        for (int e = 0; e < 21; ++e) C[e] = Cp[e];
+        cov_transport(J, 1.0, C);
         // multiple scattering of surface k (added before the update)
         const double xx0 = sb.xx0();
         if (xx0 > 0.0) {

@@ -12,6 +12,17 @@
 //     stages take the trilinearly interpolated field at their own points.
 // Any combination of the three runs here; the baseline method keeps its own
 // tuned FP64 and mixed kernels.
+//
+// The bound is the FP64 pipe, as for the FP64 fit, and the constant-field
+// variants share its transport and its fixed-point smoother (one kernel per
+// kind of field).  In a map the field of every stage is another, so the steps
+// stay stage by stage; the corrections after the first are tiny and take
+// their leading terms.  The backward filter's weighted mean (a 6x6
+// factorisation and six solves) is formed on the states that are output.
+// 50k tracks of 21 states with energy loss 7.54 -> 2.80 ms; 30k tracks of 31
+// states with map, energy loss and backward filter 16.9 -> 12.8 ms (5120 FP64
+// instructions per state, the pipe 98 % busy in the sub-partitions that the
+// 938 warps' two rounds keep occupied).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -19,6 +30,7 @@
 #include "kf_device.cuh"
 #include "kf_fp64.cuh"
 #include "kf_internal.h"
+#include "kf_transport.cuh"
 
 namespace kfgb {
 namespace {
@@ -28,16 +40,9 @@ using namespace dev;
 // field
 // ---------------------------------------------------------------------------
 
-// Field at r: the constant field, or the trilinear interpolation of the map's
-// 8 grid points around r (r clamped onto the grid; every index stays inside
+// Field at r: the trilinear interpolation of the map's 8 grid points around r (r clamped onto the grid; every index stays inside
 // [0, n-1], also for a non-finite r).
 __device__ __forceinline__ void field_at(const FitParams& p, const double r[3], double B[3]) {
-  if (p.map_b == nullptr) {
-    B[0] = p.bfield[0];
-    B[1] = p.bfield[1];
-    B[2] = p.bfield[2];
-    return;
-  }
   int idx[3];
   double w[3];
 #pragma unroll
@@ -79,8 +84,8 @@ __device__ __forceinline__ void cross3(const double a[3], const double b[3], dou
 // free-state accumulators plus the varying columns of G = D J_bf
 // (columns: 0 phi, 1 theta, 2 q/p)
 struct GProp {
-  double r[3], T[3], t, lam;
-  double gr[3][3], gT[3][3], gtl;
+  double r[3], T[3], lam, len;
+  double gr[3][3], gT[3][3];
 };
 
 // One 4-stage Nystrom step of length h:
@@ -90,7 +95,7 @@ struct GProp {
 //   r' = r + h T + h^2/6 (k1 + k2 + k3),  T' = T + h/6 (k1 + 2 k2 + 2 k3 + k4).
 // G advances by the derivative of this map with the three stage fields held
 // fixed (exact for a uniform field).
-__device__ __forceinline__ void rkn_step_field(const FitParams& p, GProp& s, double h, double mass) {
+__device__ __forceinline__ void rkn_step_field(const FitParams& p, GProp& s, double h) {
   const double lk = s.lam * kKappa;
   double B1[3], B2[3], B4[3];
   double TB1[3], TB2[3], TB3[3], TB4[3];  // T_s x B_s
@@ -143,16 +148,44 @@ __device__ __forceinline__ void rkn_step_field(const FitParams& p, GProp& s, dou
       s.gT[i][c] = g[i] + h / 6.0 * (d1[i] + 2.0 * d2[i] + 2.0 * d3[i] + d4[i]);
     }
   }
-  const double g2 = 1.0 + mass * mass * s.lam * s.lam;
-  const double igam = rsqrt_any(g2);
-  const double gam = g2 * igam;
-  s.gtl += h * mass * mass * s.lam * kInvC * igam;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     s.r[i] += h * s.T[i] + h * h / 6.0 * lk * (TB1[i] + TB2[i] + TB3[i]);
     s.T[i] += h / 6.0 * lk * (TB1[i] + 2.0 * TB2[i] + 2.0 * TB3[i] + TB4[i]);
   }
-  s.t += h * gam * kInvC;
+  s.len += h;
+}
+
+// The same step for a tiny h, to the order that double precision resolves:
+//   r += h T + h^2/2 a, T += h a, a = lk T x B(r)
+// and its derivative.  What it leaves out is (h lk B)^2 / 2 of the direction
+// (below 1e-17 under the caller's bound) and h^2 / 2 of the field's change
+// along the step (1e-16 for a field that changes by its own size over one
+// 25 mm grid cell at h = 2e-6 mm).  One field lookup instead of three and
+// about 60 FP64 instructions instead of 350; B is the field at r.
+__device__ __forceinline__ void tiny_step_field(GProp& s, double h, const double B[3]) {
+  const double hl = h * s.lam * kKappa, hk = h * kKappa;
+  double TB[3];
+  cross3(s.T, B, TB);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) s.gr[i][2] = fma(h, fma(0.5 * hk, TB[i], s.gT[i][2]), s.gr[i][2]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double g[3] = {s.gT[0][c], s.gT[1][c], s.gT[2][c]};
+    double x[3];
+    cross3(g, B, x);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (c < 2) s.gr[i][c] = fma(h, g[i], s.gr[i][c]);
+      s.gT[i][c] = fma(hl, x[i], g[i]) + (c == 2 ? hk * TB[i] : 0.0);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    s.r[i] = fma(h, fma(0.5 * hl, TB[i], s.T[i]), s.r[i]);
+    s.T[i] = fma(hl, TB[i], s.T[i]);
+  }
+  s.len += h;
 }
 
 __device__ __forceinline__ bool plane_distance(const GProp& s, const Surf& sb, double& out) {
@@ -163,147 +196,98 @@ __device__ __forceinline__ bool plane_distance(const GProp& s, const Surf& sb, d
   return true;
 }
 
-// Transport x (bound, surface a) to surface b in either direction (the path
-// length comes out negative when b lies behind): prediction xp, Jacobian J,
-// sin(theta) and the incidence cosine at b.
-__device__ __forceinline__ int transport_field(const FitParams& p, const Surf& sa, const Surf& sb,
-                                               const double x[6], double xp[6], Jac<double>& J,
-                                               double& sin_theta, double& cos_inc) {
+// Propagation to plane b through the field map (see propagate_to_plane for
+// the constant field); Be receives the field at the end point.
+__device__ __forceinline__ int propagate_map(const FitParams& p, const Surf& sb, const double r0[3], const Angles& a0,
+                                             double lam, End& o, Cols64& g, double Be[3]) {
   GProp s;
-  double sp, cp, st, ct;
-  sincos(x[2], &sp, &cp);
-  sincos(x[3], &st, &ct);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) s.r[i] = sa.c(i) + x[0] * sa.u(i) + x[1] * sa.v(i);
-  s.T[0] = cp * st;
-  s.T[1] = sp * st;
-  s.T[2] = ct;
-  s.t = x[5];
-  s.lam = x[4];
-  s.gT[0][0] = -sp * st; s.gT[1][0] = cp * st; s.gT[2][0] = 0.0;
-  s.gT[0][1] = cp * ct;  s.gT[1][1] = sp * ct; s.gT[2][1] = -st;
+  for (int i = 0; i < 3; ++i) s.r[i] = r0[i];
+  s.T[0] = a0.cp * a0.st;
+  s.T[1] = a0.sp * a0.st;
+  s.T[2] = a0.ct;
+  s.lam = lam;
+  s.len = 0.0;
+  s.gT[0][0] = -s.T[1]; s.gT[1][0] = s.T[0]; s.gT[2][0] = 0.0;
+  s.gT[0][1] = a0.cp * a0.ct;  s.gT[1][1] = a0.sp * a0.ct; s.gT[2][1] = -a0.st;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     s.gT[i][2] = 0.0;
     s.gr[i][0] = s.gr[i][1] = s.gr[i][2] = 0.0;
   }
-  s.gtl = 0.0;
-  const double mass = p.mass;
   double s0;
   if (!plane_distance(s, sb, s0)) return ST_NO_INTERSECTION;
   const double nsub_d = ceil(fabs(s0) / p.h_max);
   if (!(nsub_d <= 64.0)) return ST_NO_INTERSECTION;
   const int nsub = nsub_d < 1.0 ? 1 : (int)nsub_d;
-  const double h = s0 / nsub;
-  for (int k = 0; k < nsub; ++k) rkn_step_field(p, s, h, mass);
-  for (int it = 0; it < p.n_iter; ++it) {
-    double si;
-    if (!plane_distance(s, sb, si)) return ST_NO_INTERSECTION;
-    rkn_step_field(p, s, si, mass);
+  double h = s0 / nsub;
+  // one loop over main steps and corrections (one copy of the long step)
+  bool have_B = false;
+  int j = 0;
+  for (;;) {
+    if (j >= nsub) {
+      if (j == nsub + p.n_iter) break;
+      if (!plane_distance(s, sb, h)) return ST_NO_INTERSECTION;
+    }
+    ++j;
+    if (j > nsub && fabs(h) <= 2e-6) {
+      field_at(p, s.r, Be);
+      const double B2 = fma(Be[0], Be[0], fma(Be[1], Be[1], Be[2] * Be[2]));
+      const double x = h * lam * kKappa;
+      if (x * x * B2 <= 2e-17) {
+        have_B = fabs(h) <= 1e-12;  // the end point's field too
+        tiny_step_field(s, h, Be);
+        continue;
+      }
+    }
+    have_B = false;
+    rkn_step_field(p, s, h);
   }
-  // end point: bound angles and the unit direction
-  const double rho2 = s.T[0] * s.T[0] + s.T[1] * s.T[1];
-  const double irho = rsqrt_any(rho2);
-  const double rho = rho2 * irho;
-  const double phi = atan2(s.T[1], s.T[0]);
-  const double theta = atan2(rho, s.T[2]);
-  const double tn2 = rho2 + s.T[2] * s.T[2];
-  const double itn = rsqrt_any(tn2);
-  const double tn = tn2 * itn;
-  const double cph = s.T[0] * irho, sph = s.T[1] * irho;
-  const double sth = rho * itn, cth = s.T[2] * itn;
-  const double nT = sb.n(0) * s.T[0] + sb.n(1) * s.T[1] + sb.n(2) * s.T[2];
-  // path correction with F' = (T, dt/ds, (q/p) kappa T x B(end), 0)
-  double Be[3], TB[3];
-  field_at(p, s.r, Be);
-  cross3(s.T, Be, TB);
-  const double lk = s.lam * kKappa;
-  const double dtds = sqrt(1.0 + mass * mass * s.lam * s.lam) * kInvC;
-  const double inv_nT = rcp_any(nT);
-  double Gr[3][5], GT[3][5], Gt[5];
+  if (!have_B) field_at(p, s.r, Be);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    Gr[i][0] = sa.u(i);
-    Gr[i][1] = sa.v(i);
-    Gr[i][2] = s.gr[i][0];
-    Gr[i][3] = s.gr[i][1];
-    Gr[i][4] = s.gr[i][2];
-    GT[i][0] = 0.0;
-    GT[i][1] = 0.0;
-    GT[i][2] = s.gT[i][0];
-    GT[i][3] = s.gT[i][1];
-    GT[i][4] = s.gT[i][2];
-  }
-  Gt[0] = Gt[1] = Gt[2] = Gt[3] = 0.0;
-  Gt[4] = s.gtl;
+    o.r[i] = s.r[i];
+    o.T[i] = s.T[i];
 #pragma unroll
-  for (int c = 0; c < 5; ++c) {
-    const double w = -(sb.n(0) * Gr[0][c] + sb.n(1) * Gr[1][c] + sb.n(2) * Gr[2][c]) * inv_nT;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Gr[i][c] += s.T[i] * w;
-      GT[i][c] += lk * TB[i] * w;
+    for (int c = 0; c < 3; ++c) {
+      g.gr[i][c] = s.gr[i][c];
+      g.gT[i][c] = s.gT[i][c];
     }
-    Gt[c] += dtds * w;
   }
-  const double inv_sth = rcp_any(sth);
-#pragma unroll
-  for (int c = 0; c < 5; ++c) {
-    J.f[0][c] = sb.u(0) * Gr[0][c] + sb.u(1) * Gr[1][c] + sb.u(2) * Gr[2][c];
-    J.f[1][c] = sb.v(0) * Gr[0][c] + sb.v(1) * Gr[1][c] + sb.v(2) * Gr[2][c];
-    J.f[2][c] = (-sph * GT[0][c] + cph * GT[1][c]) * inv_sth;
-    J.f[3][c] = cph * cth * GT[0][c] + sph * cth * GT[1][c] - sth * GT[2][c];
-    J.ft[c] = Gt[c];
-  }
-  const double d0 = s.r[0] - sb.c(0), d1 = s.r[1] - sb.c(1), d2 = s.r[2] - sb.c(2);
-  xp[0] = d0 * sb.u(0) + d1 * sb.u(1) + d2 * sb.u(2);
-  xp[1] = d0 * sb.v(0) + d1 * sb.v(1) + d2 * sb.v(2);
-  xp[2] = phi;
-  xp[3] = theta;
-  xp[4] = s.lam;
-  xp[5] = s.t;
-  sin_theta = sth;
-  cos_inc = nT / tn;
+  const double mass = p.mass;
+  o.g2 = fma(mass * mass * lam, lam, 1.0);
+  const double igam = rsqrt_any(o.g2);
+  o.dtds = o.g2 * igam * kInvC;
+  o.dt = s.len * o.dtds;
+  g.gtl = s.len * (mass * mass * lam * kInvC) * igam;
   return ST_OK;
 }
 
-// C <- G F C F^T G^T with F from J (row 4 = e4, column 5 = e5) and
-// G = diag(1, 1, 1, 1, g, 1); the rows of Bm = G F C go to the record when
-// ws is given (the RTS smoother reads them back).
-__device__ __forceinline__ void cov_transport(const Jac<double>& J, double g, double C[21], const WS* ws, int k) {
-  double Cp[21];
+// FIELD: 0 constant along z, 1 constant, 2 map.
+// Transport x (bound, surface a, angles ang) to surface b in either direction
+// (the path length comes out negative when b lies behind): x becomes the
+// prediction but for its angles, which stay in ang and o.
+template <int FIELD>
+__device__ __forceinline__ int transport_variant(const FitParams& p, const Surf& sa, const Surf& sb, double x[6],
+                                                 const Angles& ang, End& o, Jac<double>& J) {
+  double r0[3], B[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
 #pragma unroll
-  for (int a = 0; a < 6; ++a) {
-    double brow[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      double v;
-      if (a == 4) {
-        v = g * C[sym(4, j)];
-      } else {
-        v = jf(J, a, 0) * C[sym(0, j)] + jf(J, a, 1) * C[sym(1, j)] + jf(J, a, 2) * C[sym(2, j)] +
-            jf(J, a, 3) * C[sym(3, j)] + jf(J, a, 4) * C[sym(4, j)];
-        if (a == 5) v += C[sym(5, j)];
-      }
-      brow[j] = v;
-      if (ws) Rec<0>::put_bm(*ws, k, a * 6 + j, v);
-    }
-#pragma unroll
-    for (int c = 0; c < 6; ++c)
-      if (c <= a) {
-        double v;
-        if (c == 4) {
-          v = g * brow[4];
-        } else {
-          v = brow[0] * jf(J, c, 0) + brow[1] * jf(J, c, 1) + brow[2] * jf(J, c, 2) + brow[3] * jf(J, c, 3) +
-              brow[4] * jf(J, c, 4);
-          if (c == 5) v += brow[5];
-        }
-        Cp[sy(a, c)] = v;
-      }
-  }
-#pragma unroll
-  for (int e = 0; e < 21; ++e) C[e] = Cp[e];
+  for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
+  Cols64 g;
+  const int st = FIELD == 2
+                     ? propagate_map(p, sb, r0, ang, x[4], o, g, B)
+                     : propagate_to_plane<FIELD == 0, 7>(sb, r0, ang, x[4], B, p.mass, p.h_max, p.n_iter, o, g);
+  if (st != ST_OK) return st;
+  double inv_nT;
+  end_frame(sb, o, inv_nT);
+  jacobian_columns<FIELD == 0, 31>(sa, sb, o, g, x[4], B, inv_nT, [&](int r, int c, double v) {
+    if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
+  });
+  const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
+  x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
+  x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
+  x[5] += o.dt;
+  return ST_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -313,64 +297,62 @@ __device__ __forceinline__ void cov_transport(const Jac<double>& J, double g, do
 // Sternheimer density effect, X = log10(beta gamma):
 //   X >= x1: 2 ln10 X - Cbar;  x0 <= X < x1: that + a (x1 - X)^k;
 //   X < x0: delta0 10^(2 (X - x0))
-__device__ __forceinline__ double density_effect(const FitParams& p, double bg) {
-  const double X = log10(bg);
-  const double two_ln10 = 2.0 * 2.302585092994045684;
+// ln_bg = ln(beta gamma).  (x1 - X)^k as exp(k ln(x1 - X)): the general
+// pow() costs over twice the FP64 instructions of both.
+__device__ __forceinline__ double density_effect(const FitParams& p, double ln_bg) {
+  const double X = ln_bg * 0.4342944819032518277;
   const double cbar = p.mat[3], x0 = p.mat[4], x1 = p.mat[5], a = p.mat[6], k = p.mat[7], d0 = p.mat[8];
-  if (X >= x1) return two_ln10 * X - cbar;
-  if (X >= x0) return two_ln10 * X - cbar + a * pow(x1 - X, k);
+  if (X >= x1) return fma(2.0, ln_bg, -cbar);
+  if (X >= x0) return fma(2.0, ln_bg, -cbar) + a * exp(k * log(x1 - X));
   return d0 * pow(10.0, 2.0 * (X - x0));
 }
 
 constexpr double kBetheK = 0.307075e-3;  // 4 pi N_A r_e^2 m_e c^2, GeV cm^2/mol
 constexpr double kMe = 0.51099895e-3;    // electron mass, GeV
 
-// mean stopping power, GeV cm^2/g (Bethe with the density effect)
-__device__ __forceinline__ double bethe(const FitParams& p, double bg, double mass) {
-  const double b2 = bg * bg / (1.0 + bg * bg);
-  const double gam = sqrt(1.0 + bg * bg);
-  const double r = kMe / mass;
-  const double wmax = 2.0 * kMe * bg * bg / (1.0 + 2.0 * gam * r + r * r);
-  const double I = p.mat[1];
-  const double arg = 2.0 * kMe * bg * bg * wmax / (I * I);
-  return kBetheK * p.mat[0] / b2 * (0.5 * log(arg) - b2 - 0.5 * density_effect(p, bg));
-}
-
 // The mean loss through a surface (dir = +1) or its restoration (dir = -1),
 // evaluated at the current momentum; thickness x/X0 * X0rho / cos.  qop
 // changes, jac = (p^3 E')/(p'^3 E), var_down = (E_d/p_d^3)^2 sigma_E^2 on the
 // downstream side with sigma_E = 4 xi / (2 sqrt(2 ln 2)) (the Gaussian of the
-// Landau FWHM).  ST_NONFINITE if the particle stops.
-__device__ __forceinline__ int energy_loss(const FitParams& p, double& qop, double xx0, double cos_inc, int dir,
+// Landau FWHM).  The stopping power is Bethe's formula with the density
+// effect.  ST_NONFINITE if the particle stops.
+// FP64 quotients and roots cost ten pipe slots and more each: they are
+// Newton-refined reciprocals here (5 to 6), and E, p', 1/p' and 1/E come from
+// two reciprocal square roots (about 170 slots per call against 420).
+__device__ __forceinline__ int energy_loss(const FitParams& p, double& qop, double xx0, double inv_cos, int dir,
                                            double& jac, double& var_down) {
-  jac = 1.0;
-  var_down = 0.0;
-  const double mass = p.mass;
-  const double thick = xx0 * p.mat[2] / fabs(cos_inc);
-  const double pm = 1.0 / fabs(qop);
-  const double E = sqrt(pm * pm + mass * mass);
-  const double beta = pm / E;
-  const double dE = bethe(p, pm / mass, mass) * thick;
+  const double mass = p.mass, im = rcp_any(mass);
+  const double thick = xx0 * p.mat[2] * fabs(inv_cos);
+  const double iq = fabs(qop), pm = rcp_any(iq);
+  const double bg = pm * im, bg2 = bg * bg;
+  const double Esq = fma(pm, pm, mass * mass), iE = rsqrt_any(Esq), E = Esq * iE;
+  const double ib2 = Esq * (iq * iq);  // 1 / beta^2
+  const double gam = E * im, r = kMe * im;
+  const double wden = fma(r, fma(2.0, gam, r), 1.0);  // wmax = 2 me bg^2 / wden
+  const double q = 2.0 * kMe * bg2, iI = rcp_any(p.mat[1]);
+  const double arg = (q * iI) * (q * iI) * rcp_any(wden);
+  const double b2 = pm * iE * (pm * iE);
+  const double dedx = kBetheK * p.mat[0] * ib2 * (0.5 * log(arg) - b2 - 0.5 * density_effect(p, log(bg)));
+  const double dE = dedx * thick;
   const double E2 = dir > 0 ? E - dE : E + dE;
   if (!(E2 > mass)) return ST_NONFINITE;
-  const double p2 = sqrt(E2 * E2 - mass * mass);
-  const double xi = 0.5 * kBetheK * p.mat[0] * thick / (beta * beta);
-  const double sigE = 4.0 * xi / (2.0 * sqrt(2.0 * 0.693147180559945309));
-  jac = (pm * pm * pm * E2) / (p2 * p2 * p2 * E);
-  const double Ed = dir > 0 ? E2 : E, pd = dir > 0 ? p2 : pm;
-  const double dqdE = Ed / (pd * pd * pd);
-  var_down = dqdE * dqdE * sigE * sigE;
-  qop = (qop > 0.0 ? 1.0 : -1.0) / p2;
+  const double ip2 = rsqrt_any(fma(E2, E2, -mass * mass));
+  const double xi = 0.5 * kBetheK * p.mat[0] * thick * ib2;
+  const double sigE = xi * (4.0 / 2.354820045030949327);  // 2 sqrt(2 ln 2)
+  const double ip2c = ip2 * ip2 * ip2;
+  jac = pm * pm * pm * iE * (E2 * ip2c);
+  const double dqdE = dir > 0 ? E2 * ip2c : E * (iq * iq * iq);
+  var_down = (dqdE * sigE) * (dqdE * sigE);
+  qop = qop > 0.0 ? ip2 : -ip2;
   return ST_OK;
 }
 
-// multiple-scattering variances of (phi, theta) for a state with |q/p| = la
-// crossing a surface of x/X0 = xx0 at incidence cos_inc
-__device__ __forceinline__ void add_scattering(const FitParams& p, double la, double xx0, double cos_inc,
-                                               double sin_th, double C[21]) {
-  const double th0 = highland<double>(la, p.mass * p.mass, xx0, cos_inc);
-  const double q = th0 * th0;
-  C[sy(2, 2)] += q / (sin_th * sin_th);
+// multiple-scattering variances of (phi, theta) for q/p = lam (g2 = 1 + m^2
+// lam^2) crossing a surface of x/X0 = xx0 at incidence 1/inv_cos
+__device__ __forceinline__ void add_scattering(double lam, double g2, double xx0, double inv_cos, double inv_st,
+                                               double C[21]) {
+  const double q = highland_sq(lam, g2, xx0, inv_cos);
+  C[sy(2, 2)] = fma(q, inv_st * inv_st, C[sy(2, 2)]);
   C[sy(3, 3)] += q;
 }
 
@@ -438,6 +420,13 @@ __device__ __forceinline__ int spd_solve_sym(const double S[21], const double B[
 // ---------------------------------------------------------------------------
 // the fused fit
 // ---------------------------------------------------------------------------
+
+// records of the backward-filter smoother: the forward-filtered states
+struct BackRec {
+  static constexpr int XF = 0, CF = 6;
+};
+
+template <int FIELD>
 __device__ __forceinline__ void fit_one_variants(const FitParams& p, const double* s_surf, int i) {
   const int t = track_of(p, i);
   const size_t TT = (size_t)p.n_tracks_total;
@@ -451,99 +440,153 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
       const int sid = p.surface_id[o0 + k];
       if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
     }
-  double xs[6], Cs[21];
+  const bool states = p.out_states != nullptr, back = p.smoother != 0;
+  double xs[6], P0[21];
   double chi2sum = 0.0;
   int nmeas = 0;
+  bool spd = true;
   if (status == ST_OK) {
-    // ------------------------------------------------ forward filter
-    double x[6], C[21];
+    // ------------------------------------------------ forward filter, with
+    // the fixed-point smoother (kf_fp64.cuh) unless the backward filter runs
+    double x[6], C[21], S[6][6];
+    Angles ang;
 #pragma unroll
     for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TT + t];
 #pragma unroll
     for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TT + t];
-    int sid_prev = p.surface_id[o0];
-    for (int k = 0; k < n && status == ST_OK; ++k) {
+    int sid_prev = 0;
+    for (int k = 0; k < n; ++k) {
       const int sid = p.surface_id[o0 + k];
-      double xp[6];
-      if (k == 0) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xp[e] = x[e];
-      } else {
+      if (k > 0) {
         const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
         Jac<double> J;
-        double sin_th, cos_inc;
-        status = transport_field(p, sa, sb, x, xp, J, sin_th, cos_inc);
+        End o;
+        const Angles a0 = ang;
+        status = transport_variant<FIELD>(p, sa, sb, x, a0, o, J);
         if (status != ST_OK) break;
+        if (states) end_angles(x[2], x[3], a0, o, x[2], x[3]);
+        ang = o.a;
         // material of surface k (before the update): scattering with the
         // arriving momentum, then the mean loss and its straggling
-        const double xx0 = sb.xx0();
-        const double la = fabs(xp[4]);
+        const double xx0 = sb.xx0(), lam = x[4];
         double g = 1.0, var_q = 0.0;
         if (p.energy_loss && xx0 > 0.0) {
-          status = energy_loss(p, xp[4], xx0, cos_inc, +1, g, var_q);
+          status = energy_loss(p, x[4], xx0, o.inv_cos, +1, g, var_q);
           if (status != ST_OK) break;
         }
-        cov_transport(J, g, C, &ws, k);
-        if (xx0 > 0.0) add_scattering(p, la, xx0, cos_inc, sin_th, C);
+        cov_transport(J, g, C);
+        if (xx0 > 0.0) add_scattering(lam, o.g2, xx0, o.inv_cos, o.inv_st, C);
         C[sy(4, 4)] += var_q;
+        if (!back) {
+          spd = spd && spd_check(C);
+          const auto fe = [&](int r, int c) { return jf(J, r, c); };
+#pragma unroll
+          for (int r = 0; r < 6; ++r) {
+            double v[6];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) v[c] = S[r][c];
+            row_times_ft(fe, g, v, S[r]);
+          }
+          if (states) {
+#pragma unroll
+            for (int e = 0; e < 25; ++e) ws.d(k, StateRec::F + e) = e < 20 ? J.f[e / 5][e % 5] : J.ft[e % 5];
+            ws.d(k, StateRec::G) = g;
+          }
+        }
       }
-      // record the prediction (C now holds Cp)
-#pragma unroll
-      for (int e = 0; e < 6; ++e) ws.d(k, Rec<0>::XP + e) = xp[e];
-#pragma unroll
-      for (int e = 0; e < 21; ++e) ws.d(k, Rec<0>::CP + e) = C[e];
-      if (!p.is_hole[o0 + k]) {
+      double K[6][2], ir[2] = {0.0, 0.0}, dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      const bool meas = !p.is_hole[o0 + k];
+      if (meas) {
         const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
         const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-        double c2 = 0.0, Cu[21];
-        status = kalman_update<double>(xp, C, m, V, x, Cu, c2);
+        double Si[3], r[2], c2;
+        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
         if (status != ST_OK) break;
-#pragma unroll
-        for (int e = 0; e < 21; ++e) C[e] = Cu[e];
+        joseph_update(C, V, K);
         chi2sum += c2;
         ++nmeas;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) x[e] += dx[e];
+        ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
+        ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+        if (k > 0 && !back) {
+          double hall[6][2];
+#pragma unroll
+          for (int e = 0; e < 6; ++e) {
+            hall[e][0] = S[e][0];
+            hall[e][1] = S[e][1];
+          }
+#pragma unroll
+          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
+        }
       } else {
 #pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] = xp[e];
+        for (int e = 0; e < 6; ++e) K[e][0] = K[e][1] = 0.0;
       }
+      if (k == 0) {
+        ang = angles_of(x[2], x[3]);
 #pragma unroll
-      for (int e = 0; e < 6; ++e) ws.d(k, Rec<0>::XF + e) = x[e];
+        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
 #pragma unroll
-      for (int e = 0; e < 21; ++e) Rec<0>::put_cf(ws, k, e, C[e]);
+        for (int e = 0; e < 21; ++e) P0[e] = C[e];
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
+      } else if (meas) {
+        turn(ang.cp, ang.sp, dx[2]);
+        turn(ang.ct, ang.st, dx[3]);
+      }
+      if (back) {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) ws.d(k, BackRec::XF + e) = x[e];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) ws.d(k, BackRec::CF + e) = C[e];
+      } else if (states && k > 0) {
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+          ws.d(k, StateRec::K + 2 * e) = K[e][0];
+          ws.d(k, StateRec::K + 2 * e + 1) = K[e][1];
+          ws.d(k, StateRec::XF + e) = x[e];
+        }
+        ws.d(k, StateRec::IR) = ir[0];
+        ws.d(k, StateRec::IR + 1) = ir[1];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) ws.d(k, StateRec::CF + e) = C[e];
+      }
       sid_prev = sid;
     }
 #pragma unroll
-    for (int e = 0; e < 6; ++e) xs[e] = x[e];
+    for (int e = 0; e < 6; ++e) xs[e] += p.seed_params[e * TT + t];
+    if (!back) {
+      if (status == ST_OK && !spd) status = ST_NON_SPD;
+      if (status == ST_OK && states) {
+        smooth_states(ws, n, p.out_states, p.n_states, o0, true);
 #pragma unroll
-    for (int e = 0; e < 21; ++e) Cs[e] = C[e];
-
-    if (status == ST_OK && p.smoother == 0) {
-      // ------------------------------------------------ RTS smoother
-      status = rts_smooth_fp64(ws, n, xs, Cs, p.out_states, p.n_states, o0);
+        for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0] = xs[e];
+      }
     } else if (status == ST_OK) {
       // ------------------------------------------------ backward filter
       // starts at the last state from the forward-filtered parameters with
       // bf_scale times their covariance; the last state keeps the forward
-      // filtered state
-      if (p.out_states)
+      // filtered state.  x, C and ang are the backward state from here on.
+      if (states)
 #pragma unroll
         for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0 + n - 1] = x[e];
-      double xb[6], Cb[21];
 #pragma unroll
-      for (int e = 0; e < 6; ++e) xb[e] = x[e];
-#pragma unroll
-      for (int e = 0; e < 21; ++e) Cb[e] = p.bf_scale * C[e];
-      for (int k = n - 1; k >= 1 && status == ST_OK; --k) {
+      for (int e = 0; e < 21; ++e) C[e] *= p.bf_scale;
+      for (int k = n - 1; k >= 1; --k) {
         if (!p.is_hole[o0 + k]) {
           const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
           const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-          double c2, xu[6], Cu[21];
-          status = kalman_update<double>(xb, Cb, m, V, xu, Cu, c2);
+          double c2, K[6][2], Si[3], r[2], dx[6];
+          status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
           if (status != ST_OK) break;
+          joseph_update(C, V, K);
 #pragma unroll
-          for (int e = 0; e < 6; ++e) xb[e] = xu[e];
-#pragma unroll
-          for (int e = 0; e < 21; ++e) Cb[e] = Cu[e];
+          for (int e = 0; e < 6; ++e) x[e] += dx[e];
+          turn(ang.cp, ang.sp, dx[2]);
+          turn(ang.ct, ang.st, dx[3]);
         }
         // material of surface k at the backward state: its scattering noise,
         // then the mean loss restored (straggling on the downstream side)
@@ -551,47 +594,55 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
         const Surf sj{s_surf + p.surface_id[o0 + k - 1] * kSurfStride};
         const double xx0 = sk.xx0();
         if (xx0 > 0.0) {
-          double sp, cp, st, ct;
-          sincos(xb[2], &sp, &cp);
-          sincos(xb[3], &st, &ct);
-          const double cos_inc = sk.n(0) * cp * st + sk.n(1) * sp * st + sk.n(2) * ct;
-          add_scattering(p, fabs(xb[4]), xx0, cos_inc, st, Cb);
+          const double inv_cos = rcp_any(fma(sk.n(0), ang.cp * ang.st, fma(sk.n(1), ang.sp * ang.st, sk.n(2) * ang.ct)));
+          const double lam = x[4];
+          add_scattering(lam, fma(p.mass * p.mass * lam, lam, 1.0), xx0, inv_cos, rcp_any(ang.st), C);
           if (p.energy_loss) {
             double g, var_q;
-            status = energy_loss(p, xb[4], xx0, cos_inc, -1, g, var_q);
+            status = energy_loss(p, x[4], xx0, inv_cos, -1, g, var_q);
             if (status != ST_OK) break;
-            Cb[sy(4, 4)] += var_q;
+            C[sy(4, 4)] += var_q;
 #pragma unroll
-            for (int j = 0; j < 6; ++j) Cb[sym(4, j)] *= g;
-            Cb[sy(4, 4)] *= g;
+            for (int j = 0; j < 6; ++j) C[sym(4, j)] *= g;
+            C[sy(4, 4)] *= g;
           }
         }
         // back-propagation to surface k-1
         Jac<double> J;
-        double xo[6], sin_th, cos_inc;
-        status = transport_field(p, sk, sj, xb, xo, J, sin_th, cos_inc);
+        End o;
+        status = transport_variant<FIELD>(p, sk, sj, x, ang, o, J);
         if (status != ST_OK) break;
-        cov_transport(J, 1.0, Cb, nullptr, 0);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xb[e] = xo[e];
+        ang = o.a;
+        cov_transport(J, 1.0, C);
         // weighted mean with the forward-filtered state k-1:
-        //   K = Cf (Cf + Cb)^-1, xs = xf + K (xb - xf), Cs = Cf - K Cf
-        double Cf[21], Ssum[21], xf[6];
+        //   K = Cf (Cf + Cb)^-1, xs = xf + K (xb - xf), Cs = Cf - K Cf,
+        // on the states that are output; the others only have to be
+        // positive definite
+        double Cf[21], Ssum[21];
 #pragma unroll
         for (int e = 0; e < 21; ++e) {
-          Cf[e] = Rec<0>::get_cf(ws, k - 1, e);
-          Ssum[e] = Cf[e] + Cb[e];
+          Cf[e] = ws.d(k - 1, BackRec::CF + e);
+          Ssum[e] = Cf[e] + C[e];
         }
+        if (k > 1 && !states) {
+          if (!spd_check(Ssum)) {
+            status = ST_NON_SPD;
+            break;
+          }
+          continue;
+        }
+        x[2] = atan2_call(o.T[1], o.T[0]);
+        x[3] = atan2_call(fma(o.a.cp, o.T[0], o.a.sp * o.T[1]), o.T[2]);
+        double X[6][6], xf[6];  // X = (Cf + Cb)^-1 Cf = K^T
 #pragma unroll
-        for (int e = 0; e < 6; ++e) xf[e] = ws.d(k - 1, Rec<0>::XF + e);
-        double X[6][6];  // (Cf + Cb)^-1 Cf = K^T
+        for (int e = 0; e < 6; ++e) xf[e] = ws.d(k - 1, BackRec::XF + e);
         status = spd_solve_sym(Ssum, Cf, X);
         if (status != ST_OK) break;
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
           double acc = 0.0;
 #pragma unroll
-          for (int q = 0; q < 6; ++q) acc += X[q][r] * (xb[q] - xf[q]);
+          for (int q = 0; q < 6; ++q) acc += X[q][r] * (x[q] - xf[q]);
           xs[r] = xf[r] + acc;
         }
 #pragma unroll
@@ -602,9 +653,9 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
               double acc = 0.0;
 #pragma unroll
               for (int q = 0; q < 6; ++q) acc += X[q][r] * Cf[sym(q, c)];
-              Cs[sy(r, c)] = Cf[sy(r, c)] - acc;
+              P0[sy(r, c)] = Cf[sy(r, c)] - acc;
             }
-        if (p.out_states)
+        if (states)
 #pragma unroll
           for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0 + k - 1] = xs[e];
       }
@@ -614,7 +665,7 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
 #pragma unroll
       for (int e = 0; e < 6; ++e) fin = fin && isfinite(xs[e]);
 #pragma unroll
-      for (int e = 0; e < 21; ++e) fin = fin && isfinite(Cs[e]);
+      for (int e = 0; e < 21; ++e) fin = fin && isfinite(P0[e]);
       if (!fin) status = ST_NONFINITE;
     }
   }
@@ -623,7 +674,7 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
 #pragma unroll
     for (int e = 0; e < 6; ++e) xs[e] = nan;
 #pragma unroll
-    for (int e = 0; e < 21; ++e) Cs[e] = nan;
+    for (int e = 0; e < 21; ++e) P0[e] = nan;
     chi2sum = nan;
     nmeas = 0;
     if (p.out_states && n >= 1 && o0 >= 0 && o1 <= p.n_states && n <= p.max_states)
@@ -633,16 +684,17 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
 #pragma unroll
   for (int e = 0; e < 6; ++e) p.out_params[e * TT + t] = xs[e];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = Cs[e];
+  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = P0[e];
   p.out_chi2[t] = chi2sum;
   if (p.out_ndf) p.out_ndf[t] = 2 * nmeas;
   if (p.out_status) p.out_status[t] = (uint8_t)status;
 }
 
+template <int FIELD>
 struct VariantBody {
   static constexpr int kStride = kSurfStride;
   static __device__ __forceinline__ void run(const FitParams& p, const double* s_surf, int i) {
-    fit_one_variants(p, s_surf, i);
+    fit_one_variants<FIELD>(p, s_surf, i);
   }
 };
 
@@ -651,7 +703,10 @@ struct VariantBody {
 cudaError_t launch_fit_variants(const FitParams& p, int block, cudaStream_t stream, int* launched) {
   if (launched) *launched = 0;
   if (p.n_tracks <= 0) return cudaSuccess;
-  return dev::launch_body<VariantBody, 1>(p, block ? block : 128, stream, launched);
+  const int b = block ? block : 128;
+  if (p.map_b) return dev::launch_body<VariantBody<2>, 1>(p, b, stream, launched);
+  if (p.bfield[0] == 0.0 && p.bfield[1] == 0.0) return dev::launch_body<VariantBody<0>, 1>(p, b, stream, launched);
+  return dev::launch_body<VariantBody<1>, 1>(p, b, stream, launched);
 }
 
 }  // namespace kfgb
