@@ -353,13 +353,12 @@ int kf_autotune(kf_handle* handle, const kf_tracks* tracks,
  *   out_chi2[T]       chi2 per track at this alignment (optional).
  *   grad_seed[6][T]   dL/d seed_params (optional).
  *   grad_align[6][S]  dL/d align (optional); overwritten.
- * Method: reverse mode throughout: a reverse sweep over the states with the
- * filtered states recomputed from checkpoints every 5 states, and inside it
- * every transport recomputed with its RKN stage inputs taped and swept
- * backwards.  Launch shape: opt->team_warps as for kf_grad; one thread per
- * track with opt->block threads per CTA (a multiple of 32 up to 256; 0, and
- * opt == NULL, choose CTAs of the warp count that covers the batch in nearly
- * full waves of one CTA per SM); the other launch options do not apply.  Device pointers; asynchronous on `stream`.  Tracks that fail
+ * Method: reverse mode throughout: a forward pass that stores the filtered
+ * states, then a reverse sweep over the states in which every transport is
+ * run again and swept backwards.  Launch shape: one thread per track with
+ * opt->block threads per CTA (a multiple of 32 up to 256; 0, and opt == NULL,
+ * choose CTAs of the warp count that covers the batch in nearly full waves
+ * of one CTA per SM); the other launch options do not apply.  Device pointers; asynchronous on `stream`.  Tracks that fail
  * get NaN chi2 and gradients and do not contribute to grad_align. */
 int kf_chi2_grad(kf_handle* handle, const kf_tracks* tracks,
                  const kf_surfaces* surfaces, const double* align,
@@ -392,33 +391,14 @@ typedef struct {
  * L above with respect to the seed parameters and the per-surface alignment,
  * in FP64 whatever opt->precision says.  align as for kf_chi2_grad.
  * Method: reverse mode throughout, one thread per track.
- *   1. forward filter, (x_f, C_f) checkpointed every 5 states;
- *   2. RTS smoother (when params, cov or the v / W terms are asked), from
- *      the last state down, each 5-state segment's filtered states and
- *      transports recomputed from its checkpoint; smoothed checkpoints at
- *      the segment starts;
- *   3. reverse of the smoother (when v or W is given), segment by segment
- *      upwards, each segment's filtered and smoothed states recomputed from
- *      the two kinds of checkpoint; each step's contributions to the
- *      adjoints of x_f, C_f, x_p, C_p and F (79 doubles per state) are kept
- *      in the handle's scratch for
- *   4. the reverse of the filter (as kf_chi2_grad) with those contributions
- *      added at every state.
- * No filtered or smoothed state is stored beyond the checkpoints.  Scratch
- * per track: 216 B per 5 states (filter checkpoints), plus with v or W 216 B
- * per 5 states (smoothed checkpoints) and 632 B per state; a batch whose
+ *   1. the forward filter with the smoothed state 0 carried along (the
+ *      cross-covariance of state 0 and the current state); the filtered
+ *      states, and with v or W those cross-covariances, are stored;
+ *   2. the reverse sweep over the states.
+ * Scratch per track: 224 B per state; charged with v or W 216 B per 5 states,
+ * 216 B per 5 states and 216 B more, and 632 B per state; a batch whose
  * scratch exceeds opt->workspace_bytes (0: 32 GiB) runs as several launches.
- * Launch shape: opt->team_warps 1 = one thread per track (CTAs as for
- * kf_chi2_grad); 2 = the pipelined form, for batches too small to fill the
- * GPU: two warps per 32 tracks, one running the forward half of the filter's
- * reverse sweep (the segments' recompute and the taped transports) one
- * transition ahead of the other, which runs the reverse half, and in the
- * smoother's passes recomputing each segment one segment ahead of the RTS
- * steps and their reverse, which the other runs (results equal
- * the one-thread form's, up to the summation order of the alignment
- * gradient); 0 (the default, and opt == NULL) = the pipelined form while
- * 2 x ceil(T / 32) warps fit in one warp per SM sub-partition (T <= 9728 on
- * 152 SMs), else one thread per track; others: KF_EUNSUPPORTED.
+ * opt->team_warps may be 0, 1 or 2 (no effect); others: KF_EUNSUPPORTED.
  * Failure behaviour as for kf_chi2_grad; a track whose smoother meets a
  * non-positive pivot gets NaN outputs and gradients.
  * Device pointers; asynchronous on `stream`. */

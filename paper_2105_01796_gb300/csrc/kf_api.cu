@@ -744,17 +744,8 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   // threads per CTA for min_blocks 1 / 3 / 4)
   const int grad_block = opt.block;
   if (grad_block < 0 || grad_block % 32 != 0 || grad_block > max_threads_of(opt.min_blocks)) return KF_EUNSUPPORTED;
-  // team_warps 2: the pipelined form (two warps per 32 tracks); 1: one
-  // thread per track; 0: the pipelined form while its two-warp teams fit in
-  // one warp per SM sub-partition (a batch too small to fill the GPU)
+  // 0, 1 and 2 are accepted and run the same kernel
   if (opt.team_warps != 0 && opt.team_warps != 1 && opt.team_warps != 2) return KF_EUNSUPPORTED;
-  bool pipelined = opt.team_warps == 2;
-  if (opt.team_warps == 0) {
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
-      pipelined = 2 * (((int64_t)tr->n_tracks + 31) / 32) <= 4 * (int64_t)nsm;
-  }
   opt.team_warps = 0;
   opt.block = 0;
   kf_outputs dummy;
@@ -767,7 +758,6 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   if (wants_variants(opt.smoother, opt.energy_loss, fi->map)) return KF_EUNSUPPORTED;
   GradArgs a;
   memset(&a, 0, sizeof(a));
-  a.align = align;
   if (wts) {
     a.dl_dchi2 = wts->dl_dchi2;
     a.dl_dparams = wts->dl_dparams;
@@ -789,15 +779,19 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   // as several launches over consecutive track ranges
   const bool want = a.grad_seed || a.grad_align;
   const bool sm_adj = want && (a.dl_dparams || a.dl_dcov);
-  const bool sm = sm_adj || a.params || a.cov;
-  const size_t per_track = sizeof(double) * grad_scratch_doubles(tr->max_states, sm, sm_adj, pipelined);
+  // charged against the cap as the header documents it (at least what the
+  // kernel uses), so that a given cap splits a batch the same way always
+  const size_t n_seg = ((size_t)tr->max_states + 4) / 5;
+  size_t per_track_d = sm_adj ? 27 * n_seg + 27 * (n_seg + 1) + 79 * (size_t)tr->max_states : 0;
+  if (per_track_d < grad_scratch_doubles(tr->max_states, sm_adj)) per_track_d = grad_scratch_doubles(tr->max_states, sm_adj);
+  const size_t per_track = sizeof(double) * per_track_d;
   const int64_t cap = opt.workspace_bytes > 0 ? opt.workspace_bytes : kDefaultWorkspace;
   int64_t chunk = cap / (int64_t)per_track;
   if (chunk < 1) chunk = 1;
   if (chunk > tr->n_tracks) chunk = tr->n_tracks;
-  // the alignment angles' cosines and sines ([6][S]) ahead of the tracks' scratch
-  const size_t trig_bytes = align_up(sizeof(double) * 6 * (size_t)su->n_surfaces, 256);
-  const size_t need = trig_bytes + per_track * (size_t)chunk;
+  // the surface tables ahead of the tracks' scratch
+  const size_t table_bytes = align_up(sizeof(double) * grad_table_doubles(su->n_surfaces), 256);
+  const size_t need = table_bytes + per_track * (size_t)chunk;
   if (h->ckpt_bytes < need) {
     if (h->ckpt) cudaFree(h->ckpt);
     h->ckpt = nullptr;
@@ -812,12 +806,9 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   e = launch_pack_surfaces(su->n_surfaces, su->center, su->rot, su->x_over_x0, h->surf, stream);
   if (e != cudaSuccess) return cuda_fail(e, "pack_surfaces launch");
   int launches = 1;
-  if (align) {
-    a.align_cs = (const double*)h->ckpt;
-    e = launch_align_trig(su->n_surfaces, align, (double*)h->ckpt, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "align trig launch");
-    ++launches;
-  }
+  e = launch_align_tables(su->n_surfaces, h->surf, align, (double*)h->ckpt, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "align tables launch");
+  ++launches;
   FitParams p;
   memset(&p, 0, sizeof(p));
   p.n_tracks_total = tr->n_tracks;
@@ -842,7 +833,8 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   for (int64_t t0 = 0; t0 < tr->n_tracks; t0 += chunk) {
     p.track0 = (int32_t)t0;
     p.n_tracks = (int32_t)((tr->n_tracks - t0) < chunk ? (tr->n_tracks - t0) : chunk);
-    e = launch_grad(p, a, (double*)((char*)h->ckpt + trig_bytes), grad_block, opt.min_blocks, pipelined, stream);
+    e = launch_grad(p, a, (const double*)h->ckpt, (double*)((char*)h->ckpt + table_bytes), grad_block, opt.min_blocks,
+                    stream);
     if (e != cudaSuccess) return cuda_fail(e, "grad launch");
     ++launches;
   }

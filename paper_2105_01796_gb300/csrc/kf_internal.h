@@ -148,8 +148,6 @@ cudaError_t launch_fit_variants(const FitParams& p, int block, cudaStream_t stre
 // smoothed parameters and packed covariance of state 0) and its gradient
 // with respect to the seeds and the per-surface alignment.
 struct GradArgs {
-  const double* align;       // [6][S] or null (zero)
-  const double* align_cs;    // [6][S] cosines and sines of its angles (launch_align_trig)
   const double* dl_dchi2;    // w [T] or null (ones)
   const double* dl_dparams;  // v [6][T] or null (zero)
   const double* dl_dcov;     // W [21][T] or null (zero)
@@ -160,21 +158,21 @@ struct GradArgs {
   double* grad_align;        // [6][S] or null: accumulated (the caller zeroes it)
 };
 
-// The cosines and sines of every surface's three alignment angles, out[6][S]
-// (cos alpha, sin alpha, cos beta, sin beta, cos gamma, sin gamma).
-cudaError_t launch_align_trig(int n_surfaces, const double* align, double* out, cudaStream_t stream);
+// Doubles of the adjoint's surface tables, and their computation from the
+// packed table: the surfaces moved by align ([6][S], null: zero) in the fit
+// kernels' layout, then the derivatives of their axes.
+size_t grad_table_doubles(int n_surfaces);
+cudaError_t launch_align_tables(int n_surfaces, const double* packed, const double* align, double* tables,
+                                cudaStream_t stream);
 
-// Scratch doubles per track of one adjoint launch: the filtered checkpoints,
-// with the smoother's adjoint the smoothed checkpoints and its per-state
-// contributions, and in the pipelined form two hand-off slots.
-size_t grad_scratch_doubles(int max_states, bool smoother, bool smoother_adjoint, bool pipelined);
+// Scratch doubles per track of one adjoint launch: the filtered states, with
+// the smoother's adjoint also their cross-covariances with state 0.
+size_t grad_scratch_doubles(int max_states, bool smoother_adjoint);
 
 // One launch over tracks [f.track0, f.track0 + f.n_tracks) of
 // f.n_tracks_total; scratch holds grad_scratch_doubles(...) x f.n_tracks.
-// pipelined: two warps per 32 tracks (the forward and the reverse half of
-// the filter's reverse sweep on separate warps), block ignored.
-cudaError_t launch_grad(const FitParams& f, const GradArgs& a, double* scratch, int block, int min_blocks,
-                        bool pipelined, cudaStream_t stream);
+cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tables, double* scratch, int block,
+                        int min_blocks, cudaStream_t stream);
 
 // Counting sort of the tracks by state count, longest first:
 // order[0..n_tracks) receives track indices.  hist needs max_states + 2 ints.
