@@ -452,6 +452,10 @@ int enqueue_fit(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const 
   p.waves = opt.schedule == KF_SCHEDULE_WAVES;
   p.team_warps = opt.team_warps;
   const bool variants = wants_variants(opt.smoother, opt.energy_loss, fi->map);
+  // (concurrent fits share the SMs: no launch of theirs has rounds of its own)
+  p.auto_team = !variants && !own_slice && opt.precision == KF_PRECISION_FP64 &&
+                shape_is_default(opt.schedule == KF_SCHEDULE_PERSISTENT, opt.block, opt.min_blocks,
+                                 opt.resident_warps, opt.team_warps);
   if (variants) fill_variants(&p, fi, opt);
   int c = 0;
   for (int64_t t0 = t_begin; t0 < t_end; t0 += chunk, ++c) {
@@ -629,10 +633,22 @@ int kf_autotune(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const 
       o.block = mixed ? shapes_mixed[bi][0] : shapes_fp64[bi][0];
       o.min_blocks = mixed ? shapes_mixed[bi][1] : shapes_fp64[bi][1];
       o.resident_warps = 0;
-      o.team_warps = 0;
+      o.team_warps = 1;
       o.use_graph = 0;
       cand[n_cand++] = o;
     }
+  if (!mixed && !variants) {
+    // the library's own choice (rounds of one-thread tracks, teams for a
+    // part-filled last one)
+    kf_options o = base;
+    o.schedule = KF_SCHEDULE_PERSISTENT;
+    o.block = 128;
+    o.min_blocks = 0;
+    o.resident_warps = 0;
+    o.team_warps = 0;
+    o.use_graph = 0;
+    cand[n_cand++] = o;
+  }
   if (!mixed && !variants)
     for (int tw = 2; tw <= 4; tw += 2) {
       // each track shared by a team of warps (small batches)
@@ -661,7 +677,7 @@ int kf_autotune(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const 
             o.min_blocks = mixed ? vars_mixed[vi] : 0;
             if (o.block > max_block(mixed, o.min_blocks)) continue;
             o.resident_warps = 0;
-            o.team_warps = 0;
+            o.team_warps = 1;
             o.use_graph = 0;
             cand[n_cand++] = o;
           }
@@ -676,7 +692,7 @@ int kf_autotune(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const 
       o.block = mixed ? waves_mixed[bi][0] : waves_fp64[bi][0];
       o.min_blocks = mixed ? waves_mixed[bi][1] : waves_fp64[bi][1];
       o.resident_warps = 0;
-      o.team_warps = 0;
+      o.team_warps = 1;
       o.use_graph = 0;
       cand[n_cand++] = o;
     }

@@ -102,9 +102,9 @@ __device__ __forceinline__ void applyA(const R bs[3], const R v[3], R out[3]) {
     out[1] = -v[0] * bs[2];
     out[2] = R(0);
   } else {
-    out[0] = v[1] * bs[2] - v[2] * bs[1];
-    out[1] = v[2] * bs[0] - v[0] * bs[2];
-    out[2] = v[0] * bs[1] - v[1] * bs[0];
+    out[0] = fma(v[1], bs[2], -(v[2] * bs[1]));
+    out[1] = fma(v[2], bs[0], -(v[0] * bs[2]));
+    out[2] = fma(v[0], bs[1], -(v[1] * bs[0]));
   }
 }
 

@@ -63,38 +63,44 @@ struct WS {
   __device__ float& f(int k, int e) const { return w32[((size_t)k * rec32 + e) * nt + i]; }
 };
 
-// C <- G F C F^T G^T with F from J (row 4 = e4, column 5 = e5) and
-// G = diag(1, 1, 1, 1, g, 1).
+// Row r of B = G F C, and element (r, c) of B F^T G from that row: F(r, c) by
+// f for rows 0..3 and 5 over columns 0..4 (row 4 = e4, column 5 = e5),
+// G = diag(1, 1, 1, 1, g, 1).  Written as FMA chains: the kernels that share
+// them give the same bits.
+template <class FE>
+__device__ __forceinline__ void fc_row(const FE& f, int r, double g, const double C[21], double b[6]) {
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    if (r == 4) {
+      b[j] = g * C[sym(4, j)];
+      continue;
+    }
+    double v = f(r, 0) * C[sym(0, j)];
+#pragma unroll
+    for (int q = 1; q < 5; ++q) v = fma(f(r, q), C[sym(q, j)], v);
+    b[j] = r == 5 ? v + C[sym(5, j)] : v;
+  }
+}
+template <class FE>
+__device__ __forceinline__ double fcf_element(const FE& f, int c, double g, const double b[6]) {
+  if (c == 4) return g * b[4];
+  double v = b[0] * f(c, 0);
+#pragma unroll
+  for (int q = 1; q < 5; ++q) v = fma(b[q], f(c, q), v);
+  return c == 5 ? v + b[5] : v;
+}
+
+// C <- G F C F^T G
 __device__ __forceinline__ void cov_transport(const Jac<double>& J, double g, double C[21]) {
+  const auto f = [&](int r, int c) { return jf(J, r, c); };
   double Cp[21];
 #pragma unroll
   for (int a = 0; a < 6; ++a) {
-    double brow[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      double v;
-      if (a == 4) {
-        v = g * C[sym(4, j)];
-      } else {
-        v = jf(J, a, 0) * C[sym(0, j)] + jf(J, a, 1) * C[sym(1, j)] + jf(J, a, 2) * C[sym(2, j)] +
-            jf(J, a, 3) * C[sym(3, j)] + jf(J, a, 4) * C[sym(4, j)];
-        if (a == 5) v += C[sym(5, j)];
-      }
-      brow[j] = v;
-    }
+    double b[6];
+    fc_row(f, a, g, C, b);
 #pragma unroll
     for (int c = 0; c < 6; ++c)
-      if (c <= a) {
-        double v;
-        if (c == 4) {
-          v = g * brow[4];
-        } else {
-          v = brow[0] * jf(J, c, 0) + brow[1] * jf(J, c, 1) + brow[2] * jf(J, c, 2) + brow[3] * jf(J, c, 3) +
-              brow[4] * jf(J, c, 4);
-          if (c == 5) v += brow[5];
-        }
-        Cp[sy(a, c)] = v;
-      }
+      if (c <= a) Cp[sy(a, c)] = fcf_element(f, c, g, b);
   }
 #pragma unroll
   for (int e = 0; e < 21; ++e) C[e] = Cp[e];

@@ -90,6 +90,7 @@ struct FitParams {
   int32_t resident_warps;  // persistent launch: warps per SM (0 = occupancy)
   int32_t waves;           // grid launch split into full waves + one spread wave (host side)
   int32_t team_warps;      // FP64 path: > 1 shares each track over that many warps (host side)
+  int32_t auto_team;       // FP64 path: teams for a last part-filled round (host side)
   // method variants (the FP64 variant kernel)
   int32_t smoother;        // 0 RTS, 1 backward filter + weighted mean
   int32_t energy_loss;     // 1: mean loss and straggling on q/p
@@ -138,6 +139,15 @@ cudaError_t launch_fit(const FitParams& p, int precision, int block, int min_blo
 // The FP64 fit with each track's work shared by a team of 2 or 4 warps
 // (kf_team.cu): one CTA per 32 tracks, grid schedule.
 cudaError_t launch_fit_team(const FitParams& p, int team_warps, cudaStream_t stream, int* launched = nullptr);
+// dynamic shared memory of one of its CTAs
+size_t team_smem_bytes(int n_surfaces);
+
+// Whether the options leave the FP64 fit's launch shape to the library
+// (every launch option at its default).
+inline bool shape_is_default(int schedule_is_persistent, int block, int min_blocks, int resident_warps, int team_warps) {
+  return schedule_is_persistent && (block == 0 || block == 128) && min_blocks == 0 && resident_warps == 0 &&
+         team_warps == 0;
+}
 
 // The FP64 kernel of the method variants (kf_variants.cu): backward-filter
 // smoother, energy loss, field map; same records as the FP64 path.

@@ -332,6 +332,51 @@ cudaError_t launch_pack_surfaces(int n_surfaces, const double* center, const dou
 
 cudaError_t launch_fit_mixed(const FitParams& p, int block, int min_blocks, cudaStream_t stream, int* launched);
 
+namespace {
+
+// The FP64 fit with the launch shape left to the library.  A sub-partition's
+// FP64 pipe is busy with one warp, so a batch takes whole rounds of one warp
+// (32 tracks) per sub-partition, and a last round that fills few of them
+// takes as long as a full one.  Its tracks go to teams of warps instead
+// (kf_team.cu; the same results bit for bit): with U warp units left over
+// after the full rounds, teams of 4 while they fit one per SM (U <= SMs:
+// 0.57 to 0.62 of a round's time, measured 465-505 against 815 us at 20
+// planes), teams of 2 up to two per SM (0.74, 605 us), else the round as it
+// is (3 U > 2 x 2 SMs would need a second round of teams: 0.92 and more).
+cudaError_t launch_fp64_auto(const FitParams& p, int block, int min_blocks, bool bz, cudaStream_t stream,
+                             int* launched) {
+  int dev = 0, nsm = 0, smem_max = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const long long units = ((long long)p.n_tracks + 31) / 32, round = 4LL * nsm;
+  const long long rest = units % round;
+  int team = rest == 0 ? 1 : rest <= nsm ? 4 : rest <= 2 * nsm ? 2 : 1;
+  if (team > 1 && (long long)team_smem_bytes(p.n_surfaces) + 1024 > smem_max) team = 1;
+  FitParams a = p;
+  if (team > 1) a.n_tracks = (int32_t)((units - rest) * 32);
+  int l = 0, count = 0;
+  if (a.n_tracks > 0) {
+    e = bz ? launch_fp64<true>(a, block, min_blocks, stream, &l) : launch_fp64<false>(a, block, min_blocks, stream, &l);
+    if (e != cudaSuccess) return e;
+    count = l;
+  }
+  if (team > 1) {
+    FitParams b = p;
+    b.track0 = p.track0 + a.n_tracks;
+    b.n_tracks = p.n_tracks - a.n_tracks;
+    b.work_counter = nullptr;
+    e = launch_fit_team(b, team, stream, &l);
+    if (e != cudaSuccess) return e;
+    count += l;
+  }
+  if (launched) *launched = count;
+  return cudaSuccess;
+}
+
+}  // namespace
+
 cudaError_t launch_fit(const FitParams& p, int precision, int block, int min_blocks, cudaStream_t stream,
                        int* launched) {
   if (launched) *launched = 0;
@@ -339,6 +384,7 @@ cudaError_t launch_fit(const FitParams& p, int precision, int block, int min_blo
   if (block <= 0) block = 128;
   const bool bz = p.bfield[0] == 0.0 && p.bfield[1] == 0.0;
   if (precision == 0 && p.team_warps > 1) return launch_fit_team(p, p.team_warps, stream, launched);
+  if (precision == 0 && p.auto_team) return launch_fp64_auto(p, block, min_blocks, bz, stream, launched);
   if (precision == 0) return bz ? launch_fp64<true>(p, block, min_blocks, stream, launched)
                                 : launch_fp64<false>(p, block, min_blocks, stream, launched);
   return launch_fit_mixed(p, block, min_blocks, stream, launched);

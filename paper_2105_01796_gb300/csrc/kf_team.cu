@@ -23,7 +23,8 @@
 // barriers per state and no second pass.  The 32 tracks of a CTA step through
 // the states in lockstep (a track with fewer states, or one that failed,
 // idles at its barriers).  The arithmetic of every element is that of the
-// one-thread-per-track FP64 kernel (kf_kernels.cu).  1000 tracks of 11 states,
+// one-thread-per-track FP64 kernel (kf_kernels.cu), bit for bit: the shared
+// functions write their fused multiply-adds out.  1000 tracks of 11 states,
 // 4 warps: 0.535 ms with the backward smoother as a second pass of two
 // barriers per state, 0.231 ms now.
 #include <cuda_runtime.h>
@@ -42,7 +43,7 @@ using namespace dev;
 constexpr int kTeamTracks = 32;
 // shared exchange buffers per CTA, [field][32 tracks] doubles
 // F 25 | Cp 21 | Cf 21 | the cosines and sines of the next transport's start
-// angles 4 | the scattering variances of phi and theta 2 | S H^T 12; at the
+// angles 4 | 1/sin^2(theta) and theta0^2 of the scattering 2 | S H^T 12; at the
 // end the smoothed state 0 and its covariance take the place of F
 constexpr int kShF = 0, kShCp = 25, kShCf = 46, kShTrig = 67, kShQ = 71, kShH = 73, kShFields = 85;
 constexpr int kShOut = 0;  // 27 fields
@@ -102,7 +103,7 @@ __device__ __forceinline__ int transport_warp(const Surf& sa, const Surf& sb, co
   if (w == noise_owner<W>()) {
     const double xx0 = sb.xx0();
     const double q = xx0 > 0.0 ? highland_sq(lam, o.g2, xx0, o.inv_cos) : 0.0;
-    sQ[0 * kTeamTracks + lane] = q * (o.inv_st * o.inv_st);
+    sQ[0 * kTeamTracks + lane] = o.inv_st * o.inv_st;
     sQ[1 * kTeamTracks + lane] = q;
   }
   return ST_OK;
@@ -179,7 +180,7 @@ __device__ __forceinline__ void fit_team(const FitParams& p, const double* s_sur
           ang = o.a;
         }
       }
-      team_sync<W>();  // F and the scattering variances complete
+      team_sync<W>();  // F and the scattering complete
       if (act) {
         const auto fe = [&](int r, int c) { return sF[((r == 5 ? 4 : r) * 5 + c) * kTeamTracks + lane]; };
         // the rows of F C F^T and of S F^T this warp owns
@@ -187,29 +188,11 @@ __device__ __forceinline__ void fit_team(const FitParams& p, const double* s_sur
         for (int r = 0; r < 6; ++r) {
           if (row_owner<W>(r) != w) continue;
           double brow[6];
-#pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            double v;
-            if (r == 4) {
-              v = C[sym(4, j)];
-            } else {
-              v = fe(r, 0) * C[sym(0, j)] + fe(r, 1) * C[sym(1, j)] + fe(r, 2) * C[sym(2, j)] +
-                  fe(r, 3) * C[sym(3, j)] + fe(r, 4) * C[sym(4, j)];
-              if (r == 5) v += C[sym(5, j)];
-            }
-            brow[j] = v;
-          }
+          fc_row(fe, r, 1.0, C, brow);
 #pragma unroll
           for (int c = 0; c <= r; ++c) {
-            double v;
-            if (c == 4) {
-              v = brow[4];
-            } else {
-              v = brow[0] * fe(c, 0) + brow[1] * fe(c, 1) + brow[2] * fe(c, 2) + brow[3] * fe(c, 3) +
-                  brow[4] * fe(c, 4);
-              if (c == 5) v += brow[5];
-            }
-            if (r == c && r == 2) v += sQ[0 * kTeamTracks + lane];
+            double v = fcf_element(fe, c, 1.0, brow);
+            if (r == c && r == 2) v = fma(sQ[1 * kTeamTracks + lane], sQ[0 * kTeamTracks + lane], v);
             if (r == c && r == 3) v += sQ[1 * kTeamTracks + lane];
             sCp[sy(r, c) * kTeamTracks + lane] = v;
           }
@@ -396,10 +379,17 @@ __global__ void __launch_bounds__(32 * W, 1) team_kernel(const FitParams p) {
   }
 }
 
+}  // namespace
+
+size_t team_smem_bytes(int n_surfaces) {
+  return (size_t)n_surfaces * kSurfStride * sizeof(double) + (size_t)kShFields * kTeamTracks * sizeof(double);
+}
+
+namespace {
+
 template <bool BZ, int W>
 cudaError_t launch_team_v(const FitParams& p, cudaStream_t stream) {
-  const size_t smem = (size_t)p.n_surfaces * kSurfStride * sizeof(double) +
-                      (size_t)kShFields * kTeamTracks * sizeof(double);
+  const size_t smem = team_smem_bytes(p.n_surfaces);
   auto kern = team_kernel<BZ, W>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -294,8 +294,8 @@ __device__ __forceinline__ int propagate_to_plane(const Surf& sb, const double r
     o.T[0] = st * z.e[0];
     o.T[1] = st * z.e[1];
     o.T[2] = ct;
-    o.r[0] = r0[0] + dr0;
-    o.r[1] = r0[1] + dr1;
+    o.r[0] = fma(st, z.q[0], r0[0]);
+    o.r[1] = fma(st, z.q[1], r0[1]);
     o.r[2] = fma(len, ct, r0[2]);
     // the phi column turns with the bend plane, the theta column is
     // (ct e, -st); neither needs a pass of its own
@@ -345,7 +345,7 @@ __device__ __forceinline__ int propagate_to_plane(const Surf& sb, const double r
   o.g2 = fma(mass * mass * lam, lam, 1.0);
   const double igam = rsqrt_any(o.g2);
   o.dtds = o.g2 * igam * kInvC;
-  o.dt = len * o.dtds;
+  o.dt = __dmul_rn(len, o.dtds);
   if (QP) g.gtl = len * (mass * mass * lam * kInvC) * igam;
   return ST_OK;
 }

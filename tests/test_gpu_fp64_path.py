@@ -93,3 +93,34 @@ def test_short_tracks(handle, team, length):  # noqa: F811
     compare(g, r, FP64)
     err = states_err(g["states"], r["states"], state_sigmas(ev))
     assert err.max() < 1e-9, err.max()
+
+
+@pytest.mark.parametrize("field", [(0.0, 0.0, 2.0), (0.3, -0.2, 2.0)])
+@pytest.mark.parametrize("states", [False, True])
+def test_library_shape_gives_the_same_bits(handle, field, states):  # noqa: F811
+    """The default launch shape (teams of 4 or 2 warps for a part-filled last
+    round of one warp per sub-partition) against one thread per track: small
+    batches, and full rounds with a remainder of one unit, of under and over
+    one team per SM, and of more than two."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rnd = 32 * 4 * sms
+    sizes = [1, 97, 32 * sms, 32 * sms + 1, 64 * sms, 64 * sms + 1, rnd, rnd + 1, rnd + 33 * sms]
+    ev = dict(synth.make_event(synth.scaled(synth.WORKLOADS["uneven30_1m"], max(sizes))))
+    ev["bfield"] = np.array(field)
+    for n in sizes:
+        sub = dict(ev)
+        m = int(ev["offsets"][n])
+        sub["n_tracks"], sub["offsets"] = n, ev["offsets"][:n + 1]
+        for k in ("seed_params", "seed_cov"):
+            sub[k] = np.ascontiguousarray(ev[k][:, :n])
+        for k in ("loc", "cov", "truth_states"):
+            if k in ev:
+                sub[k] = np.ascontiguousarray(ev[k][:, :m])
+        for k in ("surface_id", "is_hole"):
+            sub[k] = ev[k][:m]
+        a = gpu_fit(handle, sub, FP64, with_states=states)
+        b = gpu_fit(handle, sub, FP64, with_states=states, team_warps=1)
+        for k in a:
+            if a[k] is not None:
+                assert np.array_equal(a[k], b[k], equal_nan=True), (n, k)
