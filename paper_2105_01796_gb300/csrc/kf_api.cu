@@ -368,6 +368,7 @@ void fill_variants(FitParams* p, const kf_field* fi, const kf_options& opt) {
     for (int i = 0; i < 3; ++i) {
       p->map_origin[i] = f.origin[i];
       p->map_inv_spacing[i] = 1.0 / f.spacing[i];
+      p->map_off[i] = -f.origin[i] / f.spacing[i];
     }
     p->map_b = f.b;
   }

@@ -100,6 +100,7 @@ struct FitParams {
   int32_t map_n[3];        // field-map grid points per axis
   double map_origin[3];
   double map_inv_spacing[3];
+  double map_off[3];       // -origin / spacing
   const double* map_b;     // null: the constant field bfield
 };
 
