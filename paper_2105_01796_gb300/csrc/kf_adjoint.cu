@@ -47,15 +47,16 @@
 #include "kf_device.cuh"
 #include "kf_fp64.cuh"
 #include "kf_internal.h"
+#include "kf_team.cuh"
 #include "kf_transport.cuh"
 
 namespace kfgb {
 namespace {
 using namespace dev;
 
-// scratch per state and track: the filtered state (loc0, loc1, q/p, the
-// direction's cos phi, sin phi, cos theta, sin theta), its covariance, and S
-constexpr int kRX = 0, kRC = 7, kRS = 28, kRecFilter = 28, kRecWhole = 64;
+// scratch per state and track (kf_team.cuh)
+constexpr int kRX = AdjRec::X, kRC = AdjRec::C, kRS = AdjRec::S;
+constexpr int kRecFilter = AdjRec::kFilter, kRecWhole = AdjRec::kWhole;
 // derivative table per surface: R, then R dM/d(angle) for the three angles
 constexpr int kDTab = 36;
 
@@ -698,52 +699,19 @@ __device__ __forceinline__ void plane_gradient(const double* __restrict__ d, con
   }
 }
 
-// Register-cap variants as for the fit kernels: MINB 1 may use 255
-// registers (up to 8 warps per SM), 3 caps at 168 (12 warps) and 4 at 128
-// (16 warps).  SM: with the smoother's adjoint (v or W given).
-template <int MINB, bool BZ, bool SM>
-__global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const GradParams g) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  double* s_surf = reinterpret_cast<double*>(smem_raw);
-  __shared__ __align__(8) uint64_t s_mbar;
+// Pass B of track slot tl (in_range: a track of the launch; status: of its
+// forward pass).  All 32 lanes of a warp call it together.
+template <bool BZ, bool SM>
+__device__ __forceinline__ void grad_reverse(const GradParams& g, const double* s_surf, int tl, bool in_range,
+                                             int status) {
   const FitParams& p = g.f;
-  const bool staged = stage_surfaces(s_surf, p.surf, (uint32_t)(p.n_surfaces * kSurfStride * 8), &s_mbar,
-                                     p.error_flag, p.wait_limit, p.skip_stage_copy != 0);
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool in_range = t < p.n_tracks;
-  const int tl = in_range ? t : 0;
   const int tg = p.track0 + tl;
   const size_t TG = (size_t)p.n_tracks_total, TL = (size_t)p.n_tracks;
-  if (!staged) {
-    // a bounded wait of this call gave up: this CTA's tracks get NaN chi2,
-    // smoothed outputs and seed gradients and add nothing to the alignment
-    // gradient (the whole CTA returns here, so no warp-wide reduction below
-    // is entered)
-    if (in_range) {
-      if (g.chi2) g.chi2[tg] = qnan();
-      if (g.grad_seed)
-        for (int e = 0; e < 6; ++e) g.grad_seed[(size_t)e * TG + tg] = qnan();
-      if (g.out_params)
-        for (int e = 0; e < 6; ++e) g.out_params[(size_t)e * TG + tg] = qnan();
-      if (g.out_cov)
-        for (int e = 0; e < 21; ++e) g.out_cov[(size_t)e * TG + tg] = qnan();
-    }
-    return;
-  }
   constexpr int kRec = SM ? kRecWhole : kRecFilter;
   auto rec = [&](int k, int e) -> double& { return g.rec[((size_t)k * kRec + e) * TL + tl]; };
-  const int64_t o0 = p.offsets[tg], o1 = p.offsets[tg + 1];
-  const int n = (int)(o1 - o0);
-  int status = in_range ? ST_OK : ST_BAD_INPUT;
-  if (!(o1 > o0) || o0 < 0 || o1 > p.n_states || n > p.max_states) status = ST_BAD_INPUT;
-  if (status == ST_OK)
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
-    }
+  const int64_t o0 = p.offsets[tg];
+  const int n = (int)(p.offsets[tg + 1] - o0);
   const double w = (g.dl_dchi2 && in_range) ? g.dl_dchi2[tg] : 1.0;
-  const bool want = g.grad_seed || g.grad_align;
-  const bool sm_fwd = SM || g.out_params || g.out_cov;
   const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
   auto meas = [&](int k, double m[2], double V[3]) {
     m[0] = p.loc[o0 + k];
@@ -752,133 +720,6 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
     V[1] = p.cov[p.n_states + o0 + k];
     V[2] = p.cov[2 * p.n_states + o0 + k];
   };
-
-  // ---------------------------------------------------------- F: forward
-  if (status == ST_OK) {
-    double x[6], C[21], S[6][6], xs[6], P0[21];
-    double chi2sum = 0.0;
-    bool spd = true;
-    Angles ang;
-#pragma unroll
-    for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TG + tg];
-#pragma unroll
-    for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TG + tg];
-    int sid_prev = 0;
-#pragma unroll 1
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (k > 0) {
-        const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
-        double r0[3];
-#pragma unroll
-        for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
-        End o;
-        Jac<double> J;
-        {
-          Cols64 gc;
-          status = propagate_to_plane<BZ, 7>(sb, r0, ang, x[4], Bf, p.mass, p.h_max, p.n_iter, o, gc);
-          if (status != ST_OK) break;
-          double inv_nT;
-          end_frame(sb, o, inv_nT);
-          jacobian_columns<BZ, 31>(sa, sb, o, gc, x[4], Bf, inv_nT, [&](int r, int c, double v) {
-            if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
-          });
-        }
-        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
-        x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
-        x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
-        x[5] += o.dt;
-        ang = o.a;
-        cov_transport(J, 1.0, C);
-        const double xx0 = sb.xx0();
-        if (xx0 > 0.0) {
-          const double q = highland_sq(x[4], o.g2, xx0, o.inv_cos);
-          C[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, C[sy(2, 2)]);
-          C[sy(3, 3)] += q;
-        }
-        if (sm_fwd) {
-          spd = spd && spd_check(C);
-          const auto fe = [&](int r, int c) { return jf(J, r, c); };
-#pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            double v[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) v[c] = S[r][c];
-            row_times_ft(fe, 1.0, v, S[r]);
-          }
-        }
-      }
-      double dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const bool ms = !p.is_hole[o0 + k];
-      if (ms) {
-        double m[2], V[3], K[6][2], Si[3], r[2], c2;
-        meas(k, m, V);
-        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
-        if (status != ST_OK) break;
-        joseph_update(C, V, K);
-        chi2sum += c2;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] += dx[e];
-        if (sm_fwd && k > 0) {
-          double hall[6][2];
-#pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            hall[e][0] = S[e][0];
-            hall[e][1] = S[e][1];
-          }
-#pragma unroll
-          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
-        }
-      }
-      if (k == 0) {
-        ang = angles_of(x[2], x[3]);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) P0[e] = C[e];
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
-      } else if (ms) {
-        turn(ang.cp, ang.sp, dx[2]);
-        turn(ang.ct, ang.st, dx[3]);
-      }
-      if (want && k < n - 1) {
-        rec(k, kRX + 0) = x[0];
-        rec(k, kRX + 1) = x[1];
-        rec(k, kRX + 2) = x[4];
-        rec(k, kRX + 3) = ang.cp;
-        rec(k, kRX + 4) = ang.sp;
-        rec(k, kRX + 5) = ang.ct;
-        rec(k, kRX + 6) = ang.st;
-#pragma unroll
-        for (int e = 0; e < 21; ++e) rec(k, kRC + e) = C[e];
-        if (SM)
-#pragma unroll
-          for (int e = 0; e < 36; ++e) rec(k, kRS + e) = S[e / 6][e % 6];
-      }
-      sid_prev = sid;
-    }
-    if (status == ST_OK && !spd) status = ST_NON_SPD;
-    if (g.chi2) g.chi2[tg] = status == ST_OK ? chi2sum : qnan();
-    if (g.out_params)
-#pragma unroll
-      for (int e = 0; e < 6; ++e)
-        g.out_params[e * TG + tg] = status == ST_OK ? xs[e] + p.seed_params[e * TG + tg] : qnan();
-    if (g.out_cov)
-#pragma unroll
-      for (int e = 0; e < 21; ++e) g.out_cov[e * TG + tg] = status == ST_OK ? P0[e] : qnan();
-  } else if (in_range) {
-    if (g.chi2) g.chi2[tg] = qnan();
-    if (g.out_params)
-      for (int e = 0; e < 6; ++e) g.out_params[(size_t)e * TG + tg] = qnan();
-    if (g.out_cov)
-      for (int e = 0; e < 21; ++e) g.out_cov[(size_t)e * TG + tg] = qnan();
-  }
-  if (!want) return;
-
-  // ---------------------------------------------------------- B: reverse
   const double kB[3] = {kKappa * Bf[0], kKappa * Bf[1], kKappa * Bf[2]};
   const double nu2 = BZ ? kB[2] * kB[2] : dot3(kB, kB);
   double lf[6], Lf[21], LS[6][6], v[6], W[21];
@@ -1116,6 +957,223 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
   }
 }
 
+// outputs of a track whose CTA's staging wait gave up: NaN, and nothing is
+// added to the alignment gradient
+__device__ __forceinline__ void write_failed_grad(const GradParams& g, int tg) {
+  const size_t TG = (size_t)g.f.n_tracks_total;
+  if (g.chi2) g.chi2[tg] = qnan();
+  if (g.grad_seed)
+    for (int e = 0; e < 6; ++e) g.grad_seed[(size_t)e * TG + tg] = qnan();
+  if (g.out_params)
+    for (int e = 0; e < 6; ++e) g.out_params[(size_t)e * TG + tg] = qnan();
+  if (g.out_cov)
+    for (int e = 0; e < 21; ++e) g.out_cov[(size_t)e * TG + tg] = qnan();
+}
+
+// Register-cap variants as for the fit kernels: MINB 1 may use 255
+// registers (up to 8 warps per SM), 3 caps at 168 (12 warps) and 4 at 128
+// (16 warps).  SM: with the smoother's adjoint (v or W given).
+template <int MINB, bool BZ, bool SM>
+__global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const GradParams g) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  double* s_surf = reinterpret_cast<double*>(smem_raw);
+  __shared__ __align__(8) uint64_t s_mbar;
+  const FitParams& p = g.f;
+  const bool staged = stage_surfaces(s_surf, p.surf, (uint32_t)(p.n_surfaces * kSurfStride * 8), &s_mbar,
+                                     p.error_flag, p.wait_limit, p.skip_stage_copy != 0);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in_range = t < p.n_tracks;
+  const int tl = in_range ? t : 0;
+  const int tg = p.track0 + tl;
+  const size_t TG = (size_t)p.n_tracks_total, TL = (size_t)p.n_tracks;
+  if (!staged) {
+    // a bounded wait of this call gave up (the whole CTA returns here, so no
+    // warp-wide reduction below is entered)
+    if (in_range) write_failed_grad(g, tg);
+    return;
+  }
+  constexpr int kRec = SM ? kRecWhole : kRecFilter;
+  auto rec = [&](int k, int e) -> double& { return g.rec[((size_t)k * kRec + e) * TL + tl]; };
+  const int64_t o0 = p.offsets[tg], o1 = p.offsets[tg + 1];
+  const int n = (int)(o1 - o0);
+  int status = in_range ? ST_OK : ST_BAD_INPUT;
+  if (!(o1 > o0) || o0 < 0 || o1 > p.n_states || n > p.max_states) status = ST_BAD_INPUT;
+  if (status == ST_OK)
+    for (int k = 0; k < n; ++k) {
+      const int sid = p.surface_id[o0 + k];
+      if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
+    }
+  const bool want = g.grad_seed || g.grad_align;
+  const bool sm_fwd = SM || g.out_params || g.out_cov;
+  const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
+  auto meas = [&](int k, double m[2], double V[3]) {
+    m[0] = p.loc[o0 + k];
+    m[1] = p.loc[p.n_states + o0 + k];
+    V[0] = p.cov[o0 + k];
+    V[1] = p.cov[p.n_states + o0 + k];
+    V[2] = p.cov[2 * p.n_states + o0 + k];
+  };
+
+  // ---------------------------------------------------------- F: forward
+  if (status == ST_OK) {
+    double x[6], C[21], S[6][6], xs[6], P0[21];
+    double chi2sum = 0.0;
+    bool spd = true;
+    Angles ang;
+#pragma unroll
+    for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TG + tg];
+#pragma unroll
+    for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TG + tg];
+    int sid_prev = 0;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      const int sid = p.surface_id[o0 + k];
+      if (k > 0) {
+        const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
+        double r0[3];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
+        End o;
+        Jac<double> J;
+        {
+          Cols64 gc;
+          status = propagate_to_plane<BZ, 7>(sb, r0, ang, x[4], Bf, p.mass, p.h_max, p.n_iter, o, gc);
+          if (status != ST_OK) break;
+          double inv_nT;
+          end_frame(sb, o, inv_nT);
+          jacobian_columns<BZ, 31>(sa, sb, o, gc, x[4], Bf, inv_nT, [&](int r, int c, double v) {
+            if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
+          });
+        }
+        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
+        x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
+        x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
+        x[5] += o.dt;
+        ang = o.a;
+        cov_transport(J, 1.0, C);
+        const double xx0 = sb.xx0();
+        if (xx0 > 0.0) {
+          const double q = highland_sq(x[4], o.g2, xx0, o.inv_cos);
+          C[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, C[sy(2, 2)]);
+          C[sy(3, 3)] += q;
+        }
+        if (sm_fwd) {
+          spd = spd && spd_check(C);
+          const auto fe = [&](int r, int c) { return jf(J, r, c); };
+#pragma unroll
+          for (int r = 0; r < 6; ++r) {
+            double v[6];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) v[c] = S[r][c];
+            row_times_ft(fe, 1.0, v, S[r]);
+          }
+        }
+      }
+      double dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      const bool ms = !p.is_hole[o0 + k];
+      if (ms) {
+        double m[2], V[3], K[6][2], Si[3], r[2], c2;
+        meas(k, m, V);
+        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
+        if (status != ST_OK) break;
+        joseph_update(C, V, K);
+        chi2sum += c2;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) x[e] += dx[e];
+        if (sm_fwd && k > 0) {
+          double hall[6][2];
+#pragma unroll
+          for (int e = 0; e < 6; ++e) {
+            hall[e][0] = S[e][0];
+            hall[e][1] = S[e][1];
+          }
+#pragma unroll
+          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
+        }
+      }
+      if (k == 0) {
+        ang = angles_of(x[2], x[3]);
+#pragma unroll
+        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) P0[e] = C[e];
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
+      } else if (ms) {
+        turn(ang.cp, ang.sp, dx[2]);
+        turn(ang.ct, ang.st, dx[3]);
+      }
+      if (want && k < n - 1) {
+        rec(k, kRX + 0) = x[0];
+        rec(k, kRX + 1) = x[1];
+        rec(k, kRX + 2) = x[4];
+        rec(k, kRX + 3) = ang.cp;
+        rec(k, kRX + 4) = ang.sp;
+        rec(k, kRX + 5) = ang.ct;
+        rec(k, kRX + 6) = ang.st;
+#pragma unroll
+        for (int e = 0; e < 21; ++e) rec(k, kRC + e) = C[e];
+        if (SM)
+#pragma unroll
+          for (int e = 0; e < 36; ++e) rec(k, kRS + e) = S[e / 6][e % 6];
+      }
+      sid_prev = sid;
+    }
+    if (status == ST_OK && !spd) status = ST_NON_SPD;
+    if (g.chi2) g.chi2[tg] = status == ST_OK ? chi2sum : qnan();
+    if (g.out_params)
+#pragma unroll
+      for (int e = 0; e < 6; ++e)
+        g.out_params[e * TG + tg] = status == ST_OK ? xs[e] + p.seed_params[e * TG + tg] : qnan();
+    if (g.out_cov)
+#pragma unroll
+      for (int e = 0; e < 21; ++e) g.out_cov[e * TG + tg] = status == ST_OK ? P0[e] : qnan();
+  } else if (in_range) {
+    if (g.chi2) g.chi2[tg] = qnan();
+    if (g.out_params)
+      for (int e = 0; e < 6; ++e) g.out_params[(size_t)e * TG + tg] = qnan();
+    if (g.out_cov)
+      for (int e = 0; e < 21; ++e) g.out_cov[(size_t)e * TG + tg] = qnan();
+  }
+  if (!want) return;
+
+  grad_reverse<BZ, SM>(g, s_surf, tl, in_range, status);
+}
+
+// The same for batches that leave most sub-partitions idle: a CTA of 4 warps
+// per 32 tracks whose forward pass is the team fit's (kf_team.cuh: 0.57 of
+// one warp's time), then pass B in its first warp.  Up to one team per SM.
+// 2000 tracks x 21 states, forward and backward of the differentiable fit:
+// 3.57 -> 2.98 ms.
+template <bool BZ, bool SM>
+__global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  double* s_surf = reinterpret_cast<double*>(smem_raw);
+  __shared__ __align__(8) uint64_t s_mbar;
+  const FitParams& p = g.f;
+  double* sh = s_surf + (size_t)p.n_surfaces * kSurfStride;
+  const bool staged = stage_surfaces(s_surf, p.surf, (uint32_t)(p.n_surfaces * kSurfStride * 8), &s_mbar,
+                                     p.error_flag, p.wait_limit, p.skip_stage_copy != 0);
+  const int base = blockIdx.x * kTeamTracks, i = base + (int)(threadIdx.x & 31);
+  const bool in_range = i < p.n_tracks;
+  if (!staged) {
+    if (in_range && threadIdx.x < 32) write_failed_grad(g, p.track0 + i);
+    return;
+  }
+  constexpr int REC = SM ? 2 : 1;
+  switch (threadIdx.x >> 5) {
+    case 1: fit_team<BZ, 4, 1, REC>(p, s_surf, sh, base, g.rec); return;
+    case 2: fit_team<BZ, 4, 2, REC>(p, s_surf, sh, base, g.rec); return;
+    case 3: fit_team<BZ, 4, 3, REC>(p, s_surf, sh, base, g.rec); return;
+    default: break;
+  }
+  const int status = fit_team<BZ, 4, 0, REC>(p, s_surf, sh, base, g.rec);
+  __syncwarp();
+  if (g.grad_seed || g.grad_align) grad_reverse<BZ, SM>(g, s_surf, in_range ? i : 0, in_range, status);
+}
+
 template <int MINB, bool BZ, bool SM>
 cudaError_t launch_grad_v(const GradParams& g, int block, cudaStream_t stream) {
   const FitParams& f = g.f;
@@ -1144,6 +1202,18 @@ cudaError_t launch_grad_v(const GradParams& g, int block, cudaStream_t stream) {
   }
   const int grid = (f.n_tracks + block - 1) / block;
   kern<<<grid, block, smem, stream>>>(g);
+  return cudaGetLastError();
+}
+
+template <bool BZ, bool SM>
+cudaError_t launch_grad_team(const GradParams& g, cudaStream_t stream) {
+  const size_t smem = team_smem_bytes(g.f.n_surfaces);
+  auto kern = kf_grad_team_kernel<BZ, SM>;
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  kern<<<(g.f.n_tracks + kTeamTracks - 1) / kTeamTracks, 128, smem, stream>>>(g);
   return cudaGetLastError();
 }
 
@@ -1185,6 +1255,22 @@ cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tab
   g.grad_align = a.grad_align;
   g.rec = scratch;
   const bool sm = (a.grad_seed || a.grad_align) && (a.dl_dparams || a.dl_dcov);
+  // a batch of at most one team per SM, with the launch shape left to the
+  // library (above that two teams would share an SM's pipes)
+  int dev = 0, nsm = 0, smem_max = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  if (block <= 0 && min_blocks <= 1 && f.n_tracks <= 32 * nsm &&
+      (long long)team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
+    g.f.out_params = a.params;
+    g.f.out_cov = a.cov;
+    g.f.out_chi2 = a.chi2;
+    const bool bz = f.bfield[0] == 0.0 && f.bfield[1] == 0.0;
+    if (sm) return bz ? launch_grad_team<true, true>(g, stream) : launch_grad_team<false, true>(g, stream);
+    return bz ? launch_grad_team<true, false>(g, stream) : launch_grad_team<false, false>(g, stream);
+  }
   switch (min_blocks) {
     case 4: return launch_grad_m<4>(g, sm, block, stream);
     case 3: return launch_grad_m<3>(g, sm, block, stream);
