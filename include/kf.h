@@ -399,7 +399,7 @@ typedef struct {
  *      cross-covariance of state 0 and the current state); the filtered
  *      states, and with v or W those cross-covariances, are stored;
  *   2. the reverse sweep over the states.
- * Scratch per track: 224 B per state; charged with v or W 216 B per 5 states,
+ * Scratch per track: 176 B per state; charged with v or W 216 B per 5 states,
  * 216 B per 5 states and 216 B more, and 632 B per state; a batch whose
  * scratch exceeds opt->workspace_bytes (0: 32 GiB) runs as several launches.
  * opt->team_warps may be 0, 1 or 2 (no effect); others: KF_EUNSUPPORTED.

@@ -35,9 +35,10 @@
 // smoother's reverse is a few products with S instead of a backward pass of
 // its own with its recomputations.  Against the stage-by-stage reverse with
 // checkpoints every 5 states and a separate smoother adjoint: chi2 gradient
-// of 100k tracks x 21 states 50.3 -> 10.8 ms, fit and whole gradient of 2000
-// tracks x 21 states 14.8 -> 3.57 ms (there two warps shared 32 tracks).
-// Storing every filtered state (224 B, whole fit 512 B) costs 0.14 ms of
+// of 100k tracks x 21 states 50.3 -> 10.8 ms (9.6 ms without the time row), fit
+// and whole gradient of 2000 tracks x 21 states 14.8 -> 3.57 ms (there two
+// warps shared 32 tracks).
+// Storing every filtered state (176 B, whole fit 416 B) costs 0.14 ms of
 // memory traffic on the 100k tracks; recomputing them took a quarter of the
 // kernel.
 #include <cuda_runtime.h>
@@ -45,6 +46,7 @@
 #include <stdint.h>
 
 #include "kf_device.cuh"
+#include "kf_filter.cuh"
 #include "kf_fp64.cuh"
 #include "kf_internal.h"
 #include "kf_team.cuh"
@@ -54,7 +56,7 @@ namespace kfgb {
 namespace {
 using namespace dev;
 
-// scratch per state and track (kf_team.cuh)
+// scratch per state and track (kf_filter.cuh)
 constexpr int kRX = AdjRec::X, kRC = AdjRec::C, kRS = AdjRec::S;
 constexpr int kRecFilter = AdjRec::kFilter, kRecWhole = AdjRec::kWhole;
 // derivative table per surface: R, then R dM/d(angle) for the three angles
@@ -277,15 +279,16 @@ struct PlaneAdj {
 };
 
 // Reverse of a transport.  In: the forward's path, tape, end state, columns
-// and inv_nT; lxp (adjoint of x_p), lJ(r, c) (of F, rows 0..3 and 5 over
-// columns 0..4), lqp, lqt (of the scattering variances).  Out: lx; the
+// and inv_nT; lxp (adjoint of x_p), lJ(r, c) (of F, rows 0..3 over columns
+// 0..4), lqp, lqt (of the scattering variances).  The objective does not
+// depend on the time of any state but the seed's, so nothing here has a time.  Out: lx; the
 // adjoints of plane a (c, u, v) in pa, those of plane b added to pb.
 template <bool BZ, class LJ>
 __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb, const double x01[2],
                                                   const double r0[3], const Angles& a0, double lam, const double kB[3],
                                                   double nu2, double mass, double xx0, const Path& p, const Step* tape,
-                                                  const End& o, const Cols64& g, double inv_nT, const double lxp[6],
-                                                  LJ lJ, double lqp, double lqt, double lx[6], PlaneAdj& pa,
+                                                  const End& o, const Cols64& g, double inv_nT, const double lxp[5],
+                                                  LJ lJ, double lqp, double lqt, double lx[5], PlaneAdj& pa,
                                                   PlaneAdj& pb) {
   const double m2 = mass * mass;
   const double u[3] = {sb.u(0), sb.u(1), sb.u(2)}, v[3] = {sb.v(0), sb.v(1), sb.v(2)}, n[3] = {sb.n(0), sb.n(1), sb.n(2)};
@@ -299,10 +302,9 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
   for (int i = 0; i < 3; ++i) AT[i] = lam * NTe[i];
   const double uT = dot3(u, T), vT = dot3(v, T);
   const double fA = fma(fv[0], AT[0], fv[1] * AT[1]), hA = dot3(hv, AT);
-  const double igam = rsqrt_any(o.g2);
 
   double Tb[3] = {0.0, 0.0, 0.0}, rb[3], lamb = lxp[4];
-  double uTb = 0.0, vTb = 0.0, fAb = 0.0, hAb = 0.0, dtdsb = 0.0, nTb = 0.0;
+  double uTb = 0.0, vTb = 0.0, fAb = 0.0, hAb = 0.0, nTb = 0.0;
   double fvb[2] = {0.0, 0.0}, hvb[3] = {0.0, 0.0, 0.0};
   double pc[5][3], tc[3][3];  // adjoints of the columns
   // x_p = (u . d, v . d), d = r - c
@@ -320,14 +322,13 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
     const double q[3] = {c == 0 ? sa.u(0) : c == 1 ? sa.v(0) : g.gr[0][c < 2 ? 0 : c - 2],
                          c == 0 ? sa.u(1) : c == 1 ? sa.v(1) : g.gr[1][c < 2 ? 0 : c - 2],
                          c == 0 ? sa.u(2) : c == 1 ? sa.v(2) : g.gr[2][c < 2 ? 0 : c - 2]};
-    const double l0 = lJ(0, c), l1 = lJ(1, c), l2 = lJ(2, c), l3 = lJ(3, c), l5 = lJ(5, c);
+    const double l0 = lJ(0, c), l1 = lJ(1, c), l2 = lJ(2, c), l3 = lJ(3, c);
     const double w = -dot3(n, q) * inv_nT;
-    const double wb = fma(l0, uT, fma(l1, vT, fma(l2, fA, fma(l3, hA, l5 * o.dtds))));
+    const double wb = fma(l0, uT, fma(l1, vT, fma(l2, fA, l3 * hA)));
     uTb = fma(l0, w, uTb);
     vTb = fma(l1, w, vTb);
     fAb = fma(l2, w, fAb);
     hAb = fma(l3, w, hAb);
-    dtdsb = fma(l5, w, dtdsb);
     const double wi = -wb * inv_nT;
     nTb = fma(wi, w, nTb);
 #pragma unroll
@@ -345,7 +346,6 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
       for (int i = 0; i < 3; ++i) hvb[i] = fma(l3, g.gT[i][c - 2], hvb[i]);
     }
   }
-  const double gtlb = lJ(5, 4);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     pa.u[i] = pc[0][i];
@@ -361,7 +361,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
     const double qb = fma(lqp, is * is, lqt) * q;
     isb = 2.0 * lqp * q * is;
     const double ge = qb * (1.0 + il);
-    lamb = fma(2.0 * qb, rcp_any(lam), fma(ge, 2.0 * m2 * lam * (igam * igam), lamb));
+    lamb = fma(2.0 * qb, rcp_any(lam), fma(ge, 2.0 * m2 * lam * rcp_any(o.g2), lamb));
     tnb = ge;
     nTb = fma(-ge, inv_nT, nTb);
   }
@@ -400,12 +400,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
     Tb[1] += fma(phib, fv[1], fma(thb, hv[1], tt * T[1]));
     Tb[2] += fma(thb, hv[2], tt * T[2]);
   }
-  // t' = t + len dtds; gtl = len m^2 lam igam / c; dtds = sqrt(g2) / c
   CoefAdj a;
-  const double kt = m2 * kInvC * igam;
-  dtdsb = fma(lxp[5], p.w.len, dtdsb);
-  a.len = fma(lxp[5], o.dtds, gtlb * (kt * lam));
-  lamb = fma(dtdsb, kt * lam, fma(gtlb * p.w.len, kt * (igam * igam), lamb));
   // the operators on T, the phi and theta columns, and their lam derivatives
   // on T (the q/p column): out = (len + rb N + rg N^2) v to the position,
   // (1 + eb N + eg N^2) v to the direction
@@ -415,7 +410,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
   a.eg = dot3(Tb, p.NNT);
   a.rb = dot3(rb, p.NT);
   a.rg = dot3(rb, p.NNT);
-  a.len += dot3(rb, p.T0);
+  a.len = dot3(rb, p.T0);
   a.deb = dot3(tc[2], p.NT);
   a.deg = dot3(tc[2], p.NNT);
   a.drb = dot3(pc[4], p.NT);
@@ -542,7 +537,6 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
   lx[3] = fma(Vb[0][0], cpct, fma(Vb[0][1], spct, -Vb[0][2] * a0.st)) + fma(Vb[1][1], cpct, -Vb[1][0] * spct) -
           fma(Vb[2][0], cpst, fma(Vb[2][1], spst, Vb[2][2] * a0.ct));
   lx[4] = lamb;
-  lx[5] = lxp[5];
 }
 
 // ---------------------------------------------------------------------------
@@ -555,11 +549,11 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
 // and with SM the smoother's, h = Sp H^T (Sp = Cov(x_0, x_k) predicted):
 //   x0 += h y (weight v), P0 -= h Si h^T (weight W), Sf = Sp - h Si P^T.
 // lf, Lf (packed, full-matrix convention) and LS (adjoints of xf, Cf, Sf)
-// become those of xp, Cp, Sp.
-template <bool SM>
+// become those of xp, Cp, Sp.  N: parameters (5: without the time).
+template <bool SM, int N>
 __device__ __forceinline__ int update_reverse(const double xp[2], const double Cp[21], const double m[2],
                                               const double V[3], double w, const double hm[6][2], const double v[6],
-                                              const double W[21], double lf[6], double Lf[21], double LS[6][6]) {
+                                              const double W[21], double lf[6], double Lf[21], double LS[6][5]) {
   const double S00 = V[0] + Cp[sy(0, 0)], S01 = V[1] + Cp[sy(1, 0)], S11 = V[2] + Cp[sy(1, 1)];
   const double idet = rcp_any(fma(S00, S11, -S01 * S01));
   const double Si[3] = {S11 * idet, -S01 * idet, S00 * idet};
@@ -569,10 +563,10 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
   double U[6][2], yb[2] = {0.0, 0.0};
   double G00 = w * r[0] * r[0], G01 = w * r[0] * r[1], G11 = w * r[1] * r[1];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < N; ++i) {
     double u0 = 0.0, u1 = 0.0;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
+    for (int j = 0; j < N; ++j) {
       u0 = fma(Lf[sym(i, j)], Cp[sym(j, 0)], u0);
       u1 = fma(Lf[sym(i, j)], Cp[sym(j, 1)], u1);
     }
@@ -586,7 +580,7 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
   }
   double Z[6][2];  // 2 U + LS^T h
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < N; ++i) {
     Z[i][0] = 2.0 * U[i][0];
     Z[i][1] = 2.0 * U[i][1];
   }
@@ -604,6 +598,9 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
       for (int j = 0; j < 6; ++j) {
         a0 = fma(W[sym(i, j)], hm[j][0], a0);
         a1 = fma(W[sym(i, j)], hm[j][1], a1);
+      }
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
         q0 = fma(LS[i][j], Cp[sym(j, 0)], q0);
         q1 = fma(LS[i][j], Cp[sym(j, 1)], q1);
         Z[j][0] = fma(LS[i][j], hm[i][0], Z[j][0]);
@@ -630,7 +627,7 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
   Lf[sy(1, 1)] -= fma(Si[1], t01, Si[2] * t11);
   // adjoint of P: lf y^T - Z Si, into columns 0 and 1 (symmetrised)
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < N; ++i) {
     const double P0 = fma(lf[i], y[0], -fma(Z[i][0], Si[0], Z[i][1] * Si[1]));
     const double P1 = fma(lf[i], y[1], -fma(Z[i][0], Si[1], Z[i][1] * Si[2]));
     Lf[sym(i, 0)] += i == 0 ? P0 : 0.5 * P0;
@@ -713,16 +710,10 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
   const int n = (int)(p.offsets[tg + 1] - o0);
   const double w = (g.dl_dchi2 && in_range) ? g.dl_dchi2[tg] : 1.0;
   const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
-  auto meas = [&](int k, double m[2], double V[3]) {
-    m[0] = p.loc[o0 + k];
-    m[1] = p.loc[p.n_states + o0 + k];
-    V[0] = p.cov[o0 + k];
-    V[1] = p.cov[p.n_states + o0 + k];
-    V[2] = p.cov[2 * p.n_states + o0 + k];
-  };
   const double kB[3] = {kKappa * Bf[0], kKappa * Bf[1], kKappa * Bf[2]};
   const double nu2 = BZ ? kB[2] * kB[2] : dot3(kB, kB);
-  double lf[6], Lf[21], LS[6][6], v[6], W[21];
+  // adjoints of x_f, C_f (packed, full-matrix convention) and S of state k
+  double lf[6], Lf[21], LS[6][5], v[6], W[21];
 #pragma unroll
   for (int e = 0; e < 6; ++e) {
     lf[e] = 0.0;
@@ -732,7 +723,7 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
   for (int i = 0; i < 6; ++i)
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      LS[i][j] = 0.0;
+      if (j < 5) LS[i][j] = 0.0;
       if (j <= i) {
         Lf[sy(i, j)] = 0.0;
         // the weight of a packed element (i, j), i > j, stands for both C_ij
@@ -794,23 +785,21 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
           }
         }
         o.g2 = fma(p.mass * p.mass * lam, lam, 1.0);
-        const double igam = rsqrt_any(o.g2);
-        o.dtds = o.g2 * igam * kInvC;
-        gc.gtl = q.len * (p.mass * p.mass * lam * kInvC) * igam;
+        o.dtds = gc.gtl = 0.0;  // (no time row)
       }
       double inv_nT;
       end_frame(sb, o, inv_nT);
       Jac<double> J;
       jacobian_columns<BZ, 31>(sa, sb, o, gc, lam, Bf, inv_nT, [&](int r, int c, double q) {
-        if (r == 5) J.ft[c] = q; else J.f[r][c] = q;
+        if (r < 4) J.f[r][c] = q;
       });
       const double xx0 = sb.xx0();
       // reverse of the update at k
       if (!p.is_hole[o0 + k]) {
         double Cp[21];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) Cp[e] = rec(k - 1, kRC + e);
-        cov_transport(J, 1.0, Cp);
+        for (int e = 0; e < 15; ++e) Cp[e] = rec(k - 1, kRC + e);
+        cov_transport<5>(J, 1.0, Cp);
         if (xx0 > 0.0) {
           const double q = highland_sq(lam, o.g2, xx0, o.inv_cos);
           Cp[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, Cp[sy(2, 2)]);
@@ -823,7 +812,7 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
             double h0 = 0.0, h1 = 0.0;
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
-              const double s = rec(k - 1, kRS + 6 * i + c);
+              const double s = rec(k - 1, kRS + 5 * i + c);
               h0 = fma(J.f[0][c], s, h0);
               h1 = fma(J.f[1][c], s, h1);
             }
@@ -835,55 +824,53 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
         const double xp[2] = {fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2))),
                               fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)))};
         double m[2], V[3];
-        meas(k, m, V);
-        update_reverse<SM>(xp, Cp, m, V, w, hm, v, W, lf, Lf, LS);
+        hit_of(p, o0 + k, m, V);
+        update_reverse<SM, 5>(xp, Cp, m, V, w, hm, v, W, lf, Lf, LS);
       }
       // reverse of Cp = F C F^T + Q and Sp = S F^T:
       //   l_F = 2 Lp F C + LSp^T S, L_C = F^T Lp F, LS = LSp F
-      double lF[5][5];  // rows loc0, loc1, phi, theta, time
+      double lF[4][5];  // rows loc0, loc1, phi, theta
       {
-        double LF[6][6];
+        double LF[5][5];
 #pragma unroll
-        for (int a = 0; a < 6; ++a) {
+        for (int a = 0; a < 5; ++a)
 #pragma unroll
           for (int c = 0; c < 5; ++c) {
             double q = c == 4 ? Lf[sym(a, 4)] : 0.0;
 #pragma unroll
             for (int r = 0; r < 4; ++r) q = fma(Lf[sym(a, r)], J.f[r][c], q);
-            LF[a][c] = fma(Lf[sym(a, 5)], J.ft[c], q);
+            LF[a][c] = q;
           }
-          LF[a][5] = Lf[sym(a, 5)];
-        }
         {
-          double Cq[21];
+          double Cq[15];
 #pragma unroll
-          for (int e = 0; e < 21; ++e) Cq[e] = rec(k - 1, kRC + e);
+          for (int e = 0; e < 15; ++e) Cq[e] = rec(k - 1, kRC + e);
 #pragma unroll
-          for (int r = 0; r < 5; ++r)
+          for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
               double q = 0.0;
 #pragma unroll
-              for (int j = 0; j < 6; ++j) q = fma(LF[r == 4 ? 5 : r][j], Cq[sym(j, c)], q);
+              for (int j = 0; j < 5; ++j) q = fma(LF[r][j], Cq[sym(j, c)], q);
               lF[r][c] = 2.0 * q;
             }
         }
         if (SM) {
 #pragma unroll
           for (int i = 0; i < 6; ++i) {
-            double s[5], o5[6];
+            double s[5], o5[5];
 #pragma unroll
-            for (int c = 0; c < 5; ++c) s[c] = rec(k - 1, kRS + 6 * i + c);
+            for (int c = 0; c < 5; ++c) s[c] = rec(k - 1, kRS + 5 * i + c);
 #pragma unroll
-            for (int r = 0; r < 5; ++r)
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-              for (int c = 0; c < 5; ++c) lF[r][c] = fma(LS[i][r == 4 ? 5 : r], s[c], lF[r][c]);
+              for (int c = 0; c < 5; ++c) lF[r][c] = fma(LS[i][r], s[c], lF[r][c]);
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
               double q = c == 4 ? LS[i][4] : 0.0;
 #pragma unroll
               for (int r = 0; r < 4; ++r) q = fma(LS[i][r], J.f[r][c], q);
-              o5[c] = fma(LS[i][5], J.ft[c], q);
+              o5[c] = q;
             }
 #pragma unroll
             for (int c = 0; c < 5; ++c) LS[i][c] = o5[c];
@@ -891,31 +878,22 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
         }
         const double lqp = Lf[sy(2, 2)], lqt = Lf[sy(3, 3)];
         // L_C before the transport's reverse, which needs lqp, lqt only
-        double Ln[21];
 #pragma unroll
-        for (int a = 0; a < 6; ++a)
+        for (int a = 0; a < 5; ++a)
 #pragma unroll
-          for (int b = 0; b < 6; ++b)
+          for (int b = 0; b < 5; ++b)
             if (b <= a) {
-              double q;
-              if (a == 5) {
-                q = LF[5][b];
-              } else {
-                q = a == 4 ? LF[4][b] : 0.0;
+              double q = a == 4 ? LF[4][b] : 0.0;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) q = fma(J.f[r][a], LF[r][b], q);
-                q = fma(J.ft[a], LF[5][b], q);
-              }
-              Ln[sy(a, b)] = q;
+              for (int r = 0; r < 4; ++r) q = fma(J.f[r][a], LF[r][b], q);
+              Lf[sy(a, b)] = q;
             }
-#pragma unroll
-        for (int e = 0; e < 21; ++e) Lf[e] = Ln[e];
-        double lx[6];
+        double lx[5];
         PlaneAdj na;
         transport_reverse<BZ>(sa, sb, x01, r0, a0, lam, kB, nu2, p.mass, xx0, path, tape, o, gc, inv_nT, lf,
-                              [&](int r, int c) { return lF[r == 5 ? 4 : r][c]; }, lqp, lqt, lx, na, adj);
+                              [&](int r, int c) { return lF[r][c]; }, lqp, lqt, lx, na, adj);
 #pragma unroll
-        for (int e = 0; e < 6; ++e) lf[e] = lx[e];
+        for (int e = 0; e < 5; ++e) lf[e] = lx[e];
         if (g.grad_align) plane_gradient(g.dtab + (size_t)sid * kDTab, adj, ga);
         adj = na;
       }
@@ -942,14 +920,18 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
 #pragma unroll
           for (int i = 0; i < 6; ++i)
 #pragma unroll
-            for (int j = 0; j <= i; ++j) Lf[sy(i, j)] += W[sy(i, j)] + 0.5 * (LS[i][j] + LS[j][i]);
+            for (int j = 0; j <= i; ++j) {
+              double q = j < 5 ? LS[i][j] : 0.0;
+              if (i < 5) q += LS[j][i];
+              Lf[sy(i, j)] += fma(0.5, q, W[sy(i, j)]);
+            }
         double m[2], V[3], xp0[2], Cp0[21];
-        meas(0, m, V);
+        hit_of(p, o0, m, V);
         xp0[0] = p.seed_params[tg];
         xp0[1] = p.seed_params[TG + tg];
 #pragma unroll
         for (int e = 0; e < 21; ++e) Cp0[e] = p.seed_cov[e * TG + tg];
-        update_reverse<false>(xp0, Cp0, m, V, w, nullptr, nullptr, nullptr, lf, Lf, LS);
+        update_reverse<false, 6>(xp0, Cp0, m, V, w, nullptr, nullptr, nullptr, lf, Lf, LS);
       }
     }
 #pragma unroll
@@ -992,150 +974,36 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
     if (in_range) write_failed_grad(g, tg);
     return;
   }
-  constexpr int kRec = SM ? kRecWhole : kRecFilter;
-  auto rec = [&](int k, int e) -> double& { return g.rec[((size_t)k * kRec + e) * TL + tl]; };
-  const int64_t o0 = p.offsets[tg], o1 = p.offsets[tg + 1];
-  const int n = (int)(o1 - o0);
-  int status = in_range ? ST_OK : ST_BAD_INPUT;
-  if (!(o1 > o0) || o0 < 0 || o1 > p.n_states || n > p.max_states) status = ST_BAD_INPUT;
-  if (status == ST_OK)
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
-    }
   const bool want = g.grad_seed || g.grad_align;
-  const bool sm_fwd = SM || g.out_params || g.out_cov;
-  const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
-  auto meas = [&](int k, double m[2], double V[3]) {
-    m[0] = p.loc[o0 + k];
-    m[1] = p.loc[p.n_states + o0 + k];
-    V[0] = p.cov[o0 + k];
-    V[1] = p.cov[p.n_states + o0 + k];
-    V[2] = p.cov[2 * p.n_states + o0 + k];
-  };
+  const bool smooth = SM || g.out_params || g.out_cov;
+  int64_t o0, o1;
+  int n;
+  int status = in_range ? track_input(p, tg, o0, o1, n) : ST_BAD_INPUT;
 
   // ---------------------------------------------------------- F: forward
+  Filter f;
+  if (status == ST_OK) status = filter_first(p, tg, o0, f);
   if (status == ST_OK) {
-    double x[6], C[21], S[6][6], xs[6], P0[21];
-    double chi2sum = 0.0;
-    bool spd = true;
-    Angles ang;
-#pragma unroll
-    for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TG + tg];
-#pragma unroll
-    for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TG + tg];
-    int sid_prev = 0;
-#pragma unroll 1
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (k > 0) {
-        const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
-        double r0[3];
-#pragma unroll
-        for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
-        End o;
-        Jac<double> J;
-        {
-          Cols64 gc;
-          status = propagate_to_plane<BZ, 7>(sb, r0, ang, x[4], Bf, p.mass, p.h_max, p.n_iter, o, gc);
-          if (status != ST_OK) break;
-          double inv_nT;
-          end_frame(sb, o, inv_nT);
-          jacobian_columns<BZ, 31>(sa, sb, o, gc, x[4], Bf, inv_nT, [&](int r, int c, double v) {
-            if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
-          });
-        }
-        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
-        x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
-        x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
-        x[5] += o.dt;
-        ang = o.a;
-        cov_transport(J, 1.0, C);
-        const double xx0 = sb.xx0();
-        if (xx0 > 0.0) {
-          const double q = highland_sq(x[4], o.g2, xx0, o.inv_cos);
-          C[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, C[sy(2, 2)]);
-          C[sy(3, 3)] += q;
-        }
-        if (sm_fwd) {
-          spd = spd && spd_check(C);
-          const auto fe = [&](int r, int c) { return jf(J, r, c); };
-#pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            double v[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) v[c] = S[r][c];
-            row_times_ft(fe, 1.0, v, S[r]);
-          }
-        }
-      }
-      double dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const bool ms = !p.is_hole[o0 + k];
-      if (ms) {
-        double m[2], V[3], K[6][2], Si[3], r[2], c2;
-        meas(k, m, V);
-        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
-        if (status != ST_OK) break;
-        joseph_update(C, V, K);
-        chi2sum += c2;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] += dx[e];
-        if (sm_fwd && k > 0) {
-          double hall[6][2];
-#pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            hall[e][0] = S[e][0];
-            hall[e][1] = S[e][1];
-          }
-#pragma unroll
-          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
-        }
-      }
-      if (k == 0) {
-        ang = angles_of(x[2], x[3]);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) P0[e] = C[e];
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
-      } else if (ms) {
-        turn(ang.cp, ang.sp, dx[2]);
-        turn(ang.ct, ang.st, dx[3]);
-      }
-      if (want && k < n - 1) {
-        rec(k, kRX + 0) = x[0];
-        rec(k, kRX + 1) = x[1];
-        rec(k, kRX + 2) = x[4];
-        rec(k, kRX + 3) = ang.cp;
-        rec(k, kRX + 4) = ang.sp;
-        rec(k, kRX + 5) = ang.ct;
-        rec(k, kRX + 6) = ang.st;
-#pragma unroll
-        for (int e = 0; e < 21; ++e) rec(k, kRC + e) = C[e];
-        if (SM)
-#pragma unroll
-          for (int e = 0; e < 36; ++e) rec(k, kRS + e) = S[e / 6][e % 6];
-      }
-      sid_prev = sid;
+    constexpr int REC = SM ? 2 : 1;
+    const WS ws{nullptr, nullptr, TL, 0, 0, tl};
+    if (!smooth || time_is_settled(f.C)) {
+      status = filter_states<BZ, 5, false, REC>(p, s_surf, ws, o0, n, smooth, g.rec, f);
+    } else {
+      Filter q = f;
+      status = filter_states_with_time<BZ, REC>(p, s_surf, ws, o0, n, smooth, g.rec, &q);
+      f = q;
     }
-    if (status == ST_OK && !spd) status = ST_NON_SPD;
-    if (g.chi2) g.chi2[tg] = status == ST_OK ? chi2sum : qnan();
+    if (status == ST_OK && !f.spd) status = ST_NON_SPD;
+  }
+  if (in_range) {
+    if (g.chi2) g.chi2[tg] = status == ST_OK ? f.chi2 : qnan();
     if (g.out_params)
 #pragma unroll
       for (int e = 0; e < 6; ++e)
-        g.out_params[e * TG + tg] = status == ST_OK ? xs[e] + p.seed_params[e * TG + tg] : qnan();
+        g.out_params[e * TG + tg] = status == ST_OK ? f.xs[e] + p.seed_params[e * TG + tg] : qnan();
     if (g.out_cov)
 #pragma unroll
-      for (int e = 0; e < 21; ++e) g.out_cov[e * TG + tg] = status == ST_OK ? P0[e] : qnan();
-  } else if (in_range) {
-    if (g.chi2) g.chi2[tg] = qnan();
-    if (g.out_params)
-      for (int e = 0; e < 6; ++e) g.out_params[(size_t)e * TG + tg] = qnan();
-    if (g.out_cov)
-      for (int e = 0; e < 21; ++e) g.out_cov[(size_t)e * TG + tg] = qnan();
+      for (int e = 0; e < 21; ++e) g.out_cov[e * TG + tg] = status == ST_OK ? f.P0[e] : qnan();
   }
   if (!want) return;
 
@@ -1146,7 +1014,7 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
 // per 32 tracks whose forward pass is the team fit's (kf_team.cuh: 0.57 of
 // one warp's time), then pass B in its first warp.  Up to one team per SM.
 // 2000 tracks x 21 states, forward and backward of the differentiable fit:
-// 3.57 -> 2.98 ms.
+// 3.57 -> 2.98 ms (2.66 ms without the time row).
 template <bool BZ, bool SM>
 __global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g) {
   extern __shared__ __align__(128) unsigned char smem_raw[];

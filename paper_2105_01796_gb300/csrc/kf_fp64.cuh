@@ -67,10 +67,14 @@ struct WS {
 // f for rows 0..3 and 5 over columns 0..4 (row 4 = e4, column 5 = e5),
 // G = diag(1, 1, 1, 1, g, 1).  Written as FMA chains: the kernels that share
 // them give the same bits.
-template <class FE>
+//
+// N here and below: 6, or 5 for the parameters without the time (the last one;
+// the packed elements 0..14 are the leading 5x5 block).  Nothing else depends
+// on the time: it is not measured and moves no other parameter.
+template <int N, class FE>
 __device__ __forceinline__ void fc_row(const FE& f, int r, double g, const double C[21], double b[6]) {
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
+  for (int j = 0; j < N; ++j) {
     if (r == 4) {
       b[j] = g * C[sym(4, j)];
       continue;
@@ -91,19 +95,20 @@ __device__ __forceinline__ double fcf_element(const FE& f, int c, double g, cons
 }
 
 // C <- G F C F^T G
+template <int N>
 __device__ __forceinline__ void cov_transport(const Jac<double>& J, double g, double C[21]) {
   const auto f = [&](int r, int c) { return jf(J, r, c); };
   double Cp[21];
 #pragma unroll
-  for (int a = 0; a < 6; ++a) {
+  for (int a = 0; a < N; ++a) {
     double b[6];
-    fc_row(f, a, g, C, b);
+    fc_row<N>(f, a, g, C, b);
 #pragma unroll
-    for (int c = 0; c < 6; ++c)
+    for (int c = 0; c < N; ++c)
       if (c <= a) Cp[sy(a, c)] = fcf_element(f, c, g, b);
   }
 #pragma unroll
-  for (int e = 0; e < 21; ++e) C[e] = Cp[e];
+  for (int e = 0; e < sy(N, 0); ++e) C[e] = Cp[e];
 }
 
 // ---------------------------------------------------------------------------
@@ -115,6 +120,7 @@ __device__ __forceinline__ void cov_transport(const Jac<double>& J, double g, do
 // ---------------------------------------------------------------------------
 // Gain, increments and chi2 of the gain-matrix update: S = V + H Cp H^T,
 // K = Cp H^T S^-1, r the predicted residual, dx = K r.
+template <int N>
 __device__ __forceinline__ int kalman_gain(const double xp[6], const double Cp[21], const double m[2],
                                            const double V[3], double K[6][2], double Si[3], double r[2],
                                            double dx[6], double& chi2) {
@@ -129,7 +135,7 @@ __device__ __forceinline__ int kalman_gain(const double xp[6], const double Cp[2
   r[1] = m[1] - xp[1];
   chi2 = fma(r[0], fma(Si[0], r[0], 2.0 * Si[1] * r[1]), Si[2] * r[1] * r[1]);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
+  for (int i = 0; i < N; ++i) {
     const double c0 = Cp[sym(i, 0)], c1 = Cp[sym(i, 1)];
     K[i][0] = fma(c0, Si[0], c1 * Si[1]);
     K[i][1] = fma(c0, Si[1], c1 * Si[2]);
@@ -139,20 +145,21 @@ __device__ __forceinline__ int kalman_gain(const double xp[6], const double Cp[2
 }
 
 // C <- Cp + K W - (H Cp)^T K^T, W = S K^T - H Cp (the Joseph form, expanded)
+template <int N>
 __device__ __forceinline__ void joseph_update(double C[21], const double V[3], const double K[6][2]) {
   const double S00 = V[0] + C[sy(0, 0)], S01 = V[1] + C[sy(1, 0)], S11 = V[2] + C[sy(1, 1)];
   double h0[6], h1[6], W0[6], W1[6];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
+  for (int j = 0; j < N; ++j) {
     h0[j] = C[sym(0, j)];
     h1[j] = C[sym(1, j)];
     W0[j] = fma(S00, K[j][0], fma(S01, K[j][1], -h0[j]));
     W1[j] = fma(S01, K[j][0], fma(S11, K[j][1], -h1[j]));
   }
 #pragma unroll
-  for (int i = 0; i < 6; ++i)
+  for (int i = 0; i < N; ++i)
 #pragma unroll
-    for (int j = 0; j < 6; ++j) if (j <= i) {
+    for (int j = 0; j < N; ++j) if (j <= i) {
       double v = C[sy(i, j)];
       v = fma(K[i][0], W0[j], v);
       v = fma(K[i][1], W1[j], v);
@@ -166,18 +173,18 @@ __device__ __forceinline__ void joseph_update(double C[21], const double V[3], c
 // positive definiteness of a predicted covariance
 // ---------------------------------------------------------------------------
 
-// All six Cholesky pivots positive, in double precision.
-static __device__ __noinline__ bool spd_pivots_fp64(const double C[21]) {
+// All Cholesky pivots of the leading n x n block positive, in double precision.
+static __device__ __noinline__ bool spd_pivots_fp64(const double C[21], int n) {
   double L[21];
   bool ok = true;
-  for (int e = 0; e < 21; ++e) L[e] = C[e];
-  for (int j = 0; j < 6; ++j) {
+  for (int e = 0; e < sy(n, 0); ++e) L[e] = C[e];
+  for (int j = 0; j < n; ++j) {
     double dj = L[sy(j, j)];
     for (int q = 0; q < j; ++q) dj -= L[sy(j, q)] * L[sy(j, q)];
     if (!(dj > 0.0)) ok = false;
     const double idg = rsqrt_any(dj);
     L[sy(j, j)] = dj * idg;
-    for (int r = j + 1; r < 6; ++r) {
+    for (int r = j + 1; r < n; ++r) {
       double v = L[sy(r, j)];
       for (int q = 0; q < j; ++q) v -= L[sy(r, q)] * L[sy(j, q)];
       L[sy(r, j)] = v * idg;
@@ -195,37 +202,57 @@ static __device__ __noinline__ bool spd_pivots_fp64(const double C[21]) {
 // diagonal near the ends of the float range) the FP64 pivots decide.  The
 // predicted covariances of the telescope fits have a smallest scaled
 // eigenvalue of 0.02 and more.
-__device__ __forceinline__ bool spd_check(const double C[21]) {
+template <int N>
+__device__ __forceinline__ bool spd_certificate(const double C[21]) {
   float U[21], L[21], iD[6];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) U[e] = d2f(C[e]);
+  for (int e = 0; e < sy(N, 0); ++e) U[e] = d2f(C[e]);
   bool ok = true;
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
+  for (int j = 0; j < N; ++j) {
     const float cjj = U[sy(j, j)];
     ok = ok && cjj > 1e-30f && cjj < 1e30f;
     float dj = cjj * (1.0f - 1e-5f);
 #pragma unroll
-    for (int q = 0; q < 6; ++q)
+    for (int q = 0; q < N; ++q)
       if (q < j) dj = fmaf(-U[sy(j, q)], L[sy(j, q)], dj);
     ok = ok && dj > 0.0f;
     iD[j] = 1.0f / dj;
 #pragma unroll
-    for (int r = 0; r < 6; ++r)
+    for (int r = 0; r < N; ++r)
       if (r > j) {
         float u = U[sy(r, j)];
 #pragma unroll
-        for (int q = 0; q < 6; ++q)
+        for (int q = 0; q < N; ++q)
           if (q < j) u = fmaf(-U[sy(r, q)], L[sy(j, q)], u);
         U[sy(r, j)] = u;
         L[sy(r, j)] = u * iD[j];
       }
   }
-  if (ok) return true;
+  return ok;
+}
+
+template <int N>
+__device__ __forceinline__ bool spd_check(const double C[21]) {
+  if (spd_certificate<N>(C)) return true;
   double t[21];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) t[e] = C[e];
-  return spd_pivots_fp64(t);
+  for (int e = 0; e < sy(N, 0); ++e) t[e] = C[e];
+  return spd_pivots_fp64(t, N);
+}
+
+// Whether the time's pivot can be taken as positive in every prediction of a
+// track that starts from C, so that the other five parameters decide.  The
+// time of state k is the part of t_0 that is independent of the other
+// parameters (of variance at least 1e-5 C_tt once C is certified) plus a
+// function of the path: its pivot never falls below the former, and fails in
+// double precision only if the path's contribution to its variance is some
+// 1e8 times C_tt.  That contribution is about the position's variance over
+// c^2; the bound allows positions uncertain by the seed's widths over 10 m of
+// path, a thousandfold.
+__device__ __forceinline__ bool time_is_settled(const double C[21]) {
+  const double path = (C[sy(0, 0)] + C[sy(1, 1)]) + 1e8 * (C[sy(2, 2)] + C[sy(3, 3)]);
+  return spd_certificate<6>(C) && C[sy(5, 5)] > 1e-6 * (kInvC * kInvC) * path;
 }
 
 // ---------------------------------------------------------------------------
@@ -234,10 +261,10 @@ __device__ __forceinline__ bool spd_check(const double C[21]) {
 // The RTS smoother's state 0 (its parameters and covariance are the fit's
 // result) equals the estimate of the state x_0 by a filter of the augmented
 // state (x_0, x_k), which runs along with the forward filter:
-//   predict  S = S F^T                         (S = Cov(x_0, x_k), 6x6)
+//   predict  S = S F^T       (S = Cov(x_0, x_k), 6x5: x_k's time is not needed)
 //   update   h = S H^T, K0 = h (V + H Cp H^T)^-1,
 //            x_0 += K0 r, P_0 -= K0 h^T, S -= h K^T
-// with F, K, r, V the forward filter's.  It takes about 300 FP64 instructions
+// with F, K, r, V the forward filter's.  It takes about 250 FP64 instructions
 // per state where the backward recursion with stored Jacobians (a Cholesky
 // factorisation, six pairs of triangular solves and A (Cs' - Cp') A^T) takes
 // 735, needs no inverse of Cp, and no record of the forward pass is written
@@ -246,26 +273,25 @@ __device__ __forceinline__ bool spd_check(const double C[21]) {
 // and chi2 are 0.2 to 0.7 of those of the backward recursion it replaced.
 // ---------------------------------------------------------------------------
 
-// row (v0..v5) -> row F^T, with F row 4 = e4 (times g) and column 5 = e5
+// row (v0..v4) -> row F^T over the columns 0..4, with F row 4 = g e4
 template <class FE>
-__device__ __forceinline__ void row_times_ft(const FE& f, double g, const double v[6], double o[6]) {
+__device__ __forceinline__ void row_times_ft(const FE& f, double g, double v[5]) {
+  double o[4];
 #pragma unroll
-  for (int r = 0; r < 6; ++r) {
-    if (r == 4) {
-      o[r] = g * v[4];
-    } else {
-      double a = f(r, 0) * v[0];
+  for (int r = 0; r < 4; ++r) {
+    double a = f(r, 0) * v[0];
 #pragma unroll
-      for (int c = 1; c < 5; ++c) a = fma(f(r, c), v[c], a);
-      if (r == 5) a += v[5];
-      o[r] = a;
-    }
+    for (int c = 1; c < 5; ++c) a = fma(f(r, c), v[c], a);
+    o[r] = a;
   }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) v[r] = o[r];
+  v[4] = g * v[4];
 }
 
 // Measurement update of row i of S, x_0[i] and row i of P_0 (lower part);
 // h of the other rows comes in hall (rows 0..i are used).
-__device__ __forceinline__ void fixed_point_row(int i, double S[6], const double K[6][2], const double Si[3],
+__device__ __forceinline__ void fixed_point_row(int i, double S[5], const double K[6][2], const double Si[3],
                                                 const double r[2], const double hall[6][2], double& x0,
                                                 double P0[21]) {
   const double h0 = hall[i][0], h1 = hall[i][1];
@@ -275,7 +301,7 @@ __device__ __forceinline__ void fixed_point_row(int i, double S[6], const double
   for (int c = 0; c < 6; ++c)
     if (c <= i) P0[sy(i, c)] = fma(-k0, hall[c][0], fma(-k1, hall[c][1], P0[sy(i, c)]));
 #pragma unroll
-  for (int c = 0; c < 6; ++c) S[c] = fma(-h0, K[c][0], fma(-h1, K[c][1], S[c]));
+  for (int c = 0; c < 5; ++c) S[c] = fma(-h0, K[c][0], fma(-h1, K[c][1], S[c]));
 }
 
 // Per-state record for the smoothed parameters of every state (written only

@@ -12,20 +12,21 @@
 // in global memory accessed once; constant field).
 //
 // The bound is the FP64 pipe (2 DFMA per clock and SM), so the design spends
-// as few FP64 instructions as the method allows: about 1050 per state with
-// the field along z, where the stage-by-stage transport with the backward
-// smoother took 2370.  100k tracks of 31 states: 15.28 -> 6.47 ms; 20k tracks
-// of 24 tilted planes in a general field with every smoothed state
-// 4.37 -> 1.95 ms; 97 tracks of 11 states (the latency of one warp per
-// sub-partition) 0.90 -> 0.40 ms.
+// as few FP64 instructions as the method allows: about 900 per state with the
+// field along z, where the stage-by-stage transport with the backward
+// smoother took 2370.  100k tracks of 31 states: 15.28 -> 6.47 ms with the
+// closed-form transport and the fixed-point smoother, 6.22 ms with teams for
+// the last round, 5.44 ms without the time row (kf_filter.cuh); 20k tracks of
+// 24 tilted planes in a general field with every smoothed state 3.56 -> 1.65
+// ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include "kf_device.cuh"
+#include "kf_filter.cuh"
 #include "kf_fp64.cuh"
 #include "kf_internal.h"
-#include "kf_transport.cuh"
 
 namespace kfgb {
 namespace {
@@ -35,180 +36,64 @@ using namespace dev;
 // ---------------------------------------------------------------------------
 // the fused fit: forward filter and fixed-point smoother in one pass
 // ---------------------------------------------------------------------------
-template <bool BZ>
+// STATES: the smoothed parameters of every state are wanted.
+template <bool BZ, bool STATES>
 __device__ __forceinline__ void fit_one_fp64(const FitParams& p, const double* s_surf, int i) {
   const int t = track_of(p, i);
   const size_t TT = (size_t)p.n_tracks_total;
   const WS ws{p.ws64, p.ws32, (size_t)p.n_tracks, kRec64Fp64, 0, i};
-  const int64_t o0 = p.offsets[t], o1 = p.offsets[t + 1];
-  const int n = (int)(o1 - o0);
-  int status = ST_OK;
-  if (!(o1 > o0) || o0 < 0 || o1 > p.n_states || n > p.max_states) status = ST_BAD_INPUT;
-  if (status == ST_OK)
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
-    }
-
-  const bool states = p.out_states != nullptr;
-  // the estimate of state 0, as its offset from the seed (so that the sum over
-  // the states rounds at the offset's size), and its covariance
-  double xs[6], P0[21];
-  double chi2sum = 0.0;
-  int nmeas = 0;
-  bool spd = true;
+  int64_t o0, o1;
+  int n;
+  int status = track_input(p, t, o0, o1, n);
+  Filter f;
+  if (status == ST_OK) status = filter_first(p, t, o0, f);
   if (status == ST_OK) {
-    double x[6], C[21], S[6][6];
-    Angles ang;
-#pragma unroll
-    for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TT + t];
-#pragma unroll
-    for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TT + t];
-    int sid_prev = 0;
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (k > 0) {
-        const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
-        // field copied to registers: taking the address of a kernel parameter
-        // would move the parameter block to local memory
-        const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
-        double r0[3];
-#pragma unroll
-        for (int e = 0; e < 3; ++e) r0[e] = fma(x[0], sa.u(e), fma(x[1], sa.v(e), sa.c(e)));
-        End o;
-        Jac<double> J;
-        {
-          Cols64 g;
-          status = propagate_to_plane<BZ, 7>(sb, r0, ang, x[4], Bf, p.mass, p.h_max, p.n_iter, o, g);
-          if (status != ST_OK) break;
-          double inv_nT;
-          end_frame(sb, o, inv_nT);
-          jacobian_columns<BZ, 31>(sa, sb, o, g, x[4], Bf, inv_nT, [&](int r, int c, double v) {
-            if (r == 5) J.ft[c] = v; else J.f[r][c] = v;
-          });
-        }
-        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
-        x[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
-        x[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
-        // the filter needs the angles' cosines and sines only
-        if (states) end_angles(x[2], x[3], ang, o, x[2], x[3]);
-        x[5] += o.dt;
-        ang = o.a;
-        const auto fe = [&](int r, int c) { return jf(J, r, c); };
-        cov_transport(J, 1.0, C);
-        // multiple scattering of surface k (added before the update)
-        const double xx0 = sb.xx0();
-        if (xx0 > 0.0) {
-          const double q = highland_sq(x[4], o.g2, xx0, o.inv_cos);
-          C[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, C[sy(2, 2)]);
-          C[sy(3, 3)] += q;
-        }
-        spd = spd && spd_check(C);
-#pragma unroll
-        for (int r = 0; r < 6; ++r) {
-          double v[6];
-#pragma unroll
-          for (int c = 0; c < 6; ++c) v[c] = S[r][c];
-          row_times_ft(fe, 1.0, v, S[r]);
-        }
-        if (states)
-#pragma unroll
-          for (int e = 0; e < 25; ++e) ws.d(k, StateRec::F + e) = e < 20 ? J.f[e / 5][e % 5] : J.ft[e % 5];
-      }
-      // update
-      double K[6][2], ir[2] = {0.0, 0.0}, dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const bool meas = !p.is_hole[o0 + k];
-      if (meas) {
-        const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
-        const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-        double Si[3], r[2], c2;
-        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
-        if (status != ST_OK) break;
-        joseph_update(C, V, K);
-        chi2sum += c2;
-        ++nmeas;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] += dx[e];
-        ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
-        ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
-        if (k > 0) {
-          double hall[6][2];
-#pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            hall[e][0] = S[e][0];
-            hall[e][1] = S[e][1];
-          }
-#pragma unroll
-          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) K[e][0] = K[e][1] = 0.0;
-      }
-      if (k == 0) {
-        // state 0 starts as its own filtered estimate
-        ang = angles_of(x[2], x[3]);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) P0[e] = C[e];
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
-      } else if (meas) {
-        turn(ang.cp, ang.sp, dx[2]);
-        turn(ang.ct, ang.st, dx[3]);
-      }
-      if (states && k > 0) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          ws.d(k, StateRec::K + 2 * e) = K[e][0];
-          ws.d(k, StateRec::K + 2 * e + 1) = K[e][1];
-          ws.d(k, StateRec::XF + e) = x[e];
-        }
-        ws.d(k, StateRec::IR) = ir[0];
-        ws.d(k, StateRec::IR + 1) = ir[1];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) ws.d(k, StateRec::CF + e) = C[e];
-      }
-      sid_prev = sid;
+    if (STATES) {
+      status = filter_states<BZ, 6, true, 0>(p, s_surf, ws, o0, n, true, nullptr, f);
+    } else if (time_is_settled(f.C)) {
+      status = filter_states<BZ, 5, false, 0>(p, s_surf, ws, o0, n, true, nullptr, f);
+    } else {
+      Filter g = f;
+      status = filter_states_with_time<BZ, 0>(p, s_surf, ws, o0, n, true, nullptr, &g);
+      f = g;
     }
-    if (status == ST_OK && !spd) status = ST_NON_SPD;
+  }
+  if (status == ST_OK) {
+    if (!f.spd) status = ST_NON_SPD;
 #pragma unroll
-    for (int e = 0; e < 6; ++e) xs[e] += p.seed_params[e * TT + t];
-    if (status == ST_OK && states) {
-      smooth_states(ws, n, p.out_states, p.n_states, o0);
+    for (int e = 0; e < 6; ++e) f.xs[e] += p.seed_params[e * TT + t];
+  }
+  if (STATES && status == ST_OK) {
+    smooth_states(ws, n, p.out_states, p.n_states, o0);
 #pragma unroll
-      for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0] = xs[e];
-    }
-    if (status == ST_OK) {
-      bool fin = isfinite(chi2sum);
+    for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0] = f.xs[e];
+  }
+  if (status == ST_OK) {
+    bool fin = isfinite(f.chi2);
 #pragma unroll
-      for (int e = 0; e < 6; ++e) fin = fin && isfinite(xs[e]);
+    for (int e = 0; e < 6; ++e) fin = fin && isfinite(f.xs[e]);
 #pragma unroll
-      for (int e = 0; e < 21; ++e) fin = fin && isfinite(P0[e]);
-      if (!fin) status = ST_NONFINITE;
-    }
+    for (int e = 0; e < 21; ++e) fin = fin && isfinite(f.P0[e]);
+    if (!fin) status = ST_NONFINITE;
   }
   if (status != ST_OK) {
     const double nan = qnan();
 #pragma unroll
-    for (int e = 0; e < 6; ++e) xs[e] = nan;
+    for (int e = 0; e < 6; ++e) f.xs[e] = nan;
 #pragma unroll
-    for (int e = 0; e < 21; ++e) P0[e] = nan;
-    chi2sum = nan;
-    nmeas = 0;
-    if (p.out_states && n >= 1 && o0 >= 0 && o1 <= p.n_states && n <= p.max_states)
+    for (int e = 0; e < 21; ++e) f.P0[e] = nan;
+    f.chi2 = nan;
+    f.nmeas = 0;
+    if (STATES && n >= 1 && o0 >= 0 && o1 <= p.n_states && n <= p.max_states)
       for (int k = 0; k < n; ++k)
         for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0 + k] = nan;
   }
 #pragma unroll
-  for (int e = 0; e < 6; ++e) p.out_params[e * TT + t] = xs[e];
+  for (int e = 0; e < 6; ++e) p.out_params[e * TT + t] = f.xs[e];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = P0[e];
-  p.out_chi2[t] = chi2sum;
-  if (p.out_ndf) p.out_ndf[t] = 2 * nmeas;
+  for (int e = 0; e < 21; ++e) p.out_cov[e * TT + t] = f.P0[e];
+  p.out_chi2[t] = f.chi2;
+  if (p.out_ndf) p.out_ndf[t] = 2 * f.nmeas;
   if (p.out_status) p.out_status[t] = (uint8_t)status;
 }
 
@@ -270,18 +155,19 @@ __global__ void pack_surfaces_kernel(int n, const double* __restrict__ center, c
   m[31] = 0.0f;
 }
 
-template <bool BZ>
+template <bool BZ, bool STATES>
 struct Fp64Body {
   static constexpr int kStride = kSurfStride;
   static __device__ __forceinline__ void run(const FitParams& p, const double* s_surf, int i) {
-    fit_one_fp64<BZ>(p, s_surf, i);
+    fit_one_fp64<BZ, STATES>(p, s_surf, i);
   }
 };
 
 template <bool BZ>
 cudaError_t launch_fp64(const FitParams& p, int block, int min_blocks, cudaStream_t stream, int* launched) {
   (void)min_blocks;  // a register cap below 255 spills this kernel heavily
-  return launch_body<Fp64Body<BZ>, 1>(p, block, stream, launched);
+  if (p.out_states) return launch_body<Fp64Body<BZ, true>, 1>(p, block, stream, launched);
+  return launch_body<Fp64Body<BZ, false>, 1>(p, block, stream, launched);
 }
 
 // counting sort of tracks by state count (longest first)
@@ -340,9 +226,9 @@ namespace {
 // takes as long as a full one.  Its tracks go to teams of warps instead
 // (kf_team.cu; the same results bit for bit): with U warp units left over
 // after the full rounds, teams of 4 while they fit one per SM (U <= SMs:
-// 0.57 to 0.62 of a round's time, measured 465-505 against 815 us at 20
-// planes), teams of 2 up to two per SM (0.74, 605 us), else the round as it
-// is (3 U > 2 x 2 SMs would need a second round of teams: 0.92 and more).
+// 0.60 to 0.64 of a round's time, measured 421-453 against 706 us at 20
+// planes), teams of 2 up to two per SM (0.72 to 0.75, 510-531 us), else the
+// round as it is (a second round of teams takes 0.9 and more).
 cudaError_t launch_fp64_auto(const FitParams& p, int block, int min_blocks, bool bz, cudaStream_t stream,
                              int* launched) {
   int dev = 0, nsm = 0, smem_max = 0;

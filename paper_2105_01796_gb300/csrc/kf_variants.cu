@@ -19,7 +19,7 @@
 // stay stage by stage; the corrections after the first are tiny and take
 // their leading terms.  The backward filter's weighted mean (a 6x6
 // factorisation and six solves) is formed on the states that are output.
-// 50k tracks of 21 states with energy loss 7.54 -> 2.80 ms; 30k tracks of 31
+// 50k tracks of 21 states with energy loss 7.54 -> 2.48 ms; 30k tracks of 31
 // states with map, energy loss and backward filter 16.9 -> 11.0 ms (4540 FP64
 // instructions per state, the pipe all but fully busy in the sub-partitions
 // that the 938 warps' two rounds on 608 keep occupied).
@@ -28,6 +28,7 @@
 #include <stdint.h>
 
 #include "kf_device.cuh"
+#include "kf_filter.cuh"
 #include "kf_fp64.cuh"
 #include "kf_internal.h"
 #include "kf_transport.cuh"
@@ -473,146 +474,160 @@ struct BackRec {
   static constexpr int XF = 0, CF = 6;
 };
 
+// What a launch wants besides the smoothed state 0 by the fixed-point
+// smoother: nothing, the smoothed parameters of every state, or the backward
+// filter in its place.
+enum : int { kState0 = 0, kEveryState = 1, kBackward = 2 };
+
+// States 1 .. n-1 of the forward filter (N as in filter_states).
+template <int FIELD, int N, int MODE>
+__device__ __forceinline__ int variant_states(const FitParams& p, const double* s_surf, const WS& ws, int64_t o0, int n,
+                                              Filter& f) {
+  int sid_prev = p.surface_id[o0];
+#pragma unroll 1
+  for (int k = 1; k < n; ++k) {
+    const int sid = p.surface_id[o0 + k];
+    const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
+    Jac<double> J;
+    End o;
+    const Angles a0 = f.ang;
+    int status = transport_variant<FIELD>(p, sa, sb, f.x, a0, o, J);
+    if (status != ST_OK) return status;
+    if (MODE == kEveryState || (MODE == kBackward && p.out_states))
+      end_angles(f.x[2], f.x[3], a0, o, f.x[2], f.x[3]);
+    f.ang = o.a;
+    // material of surface k (before the update): scattering with the
+    // arriving momentum, then the mean loss and its straggling
+    const double xx0 = sb.xx0(), lam = f.x[4];
+    double g = 1.0, var_q = 0.0;
+    if (p.energy_loss && xx0 > 0.0) {
+      status = energy_loss(p, f.x[4], xx0, o.inv_cos, +1, g, var_q);
+      if (status != ST_OK) return status;
+    }
+    cov_transport<N>(J, g, f.C);
+    if (xx0 > 0.0) add_scattering(lam, o.g2, xx0, o.inv_cos, o.inv_st, f.C);
+    f.C[sy(4, 4)] += var_q;
+    if (MODE != kBackward) {
+      f.spd = f.spd && spd_check<N>(f.C);
+      const auto fe = [&](int r, int c) { return jf(J, r, c); };
+#pragma unroll
+      for (int r = 0; r < 6; ++r) row_times_ft(fe, g, f.S[r]);
+    }
+    if (MODE == kEveryState) {
+#pragma unroll
+      for (int e = 0; e < 25; ++e) ws.d(k, StateRec::F + e) = e < 20 ? J.f[e / 5][e % 5] : J.ft[e % 5];
+      ws.d(k, StateRec::G) = g;
+    }
+    double K[6][2], ir[2] = {0.0, 0.0};
+    if (!p.is_hole[o0 + k]) {
+      double m[2], V[3], Si[3], r[2], dx[6], c2;
+      hit_of(p, o0 + k, m, V);
+      status = kalman_gain<N>(f.x, f.C, m, V, K, Si, r, dx, c2);
+      if (status != ST_OK) return status;
+      joseph_update<N>(f.C, V, K);
+      f.chi2 += c2;
+      ++f.nmeas;
+#pragma unroll
+      for (int e = 0; e < N; ++e) f.x[e] += dx[e];
+      ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
+      ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+      if (MODE != kBackward) {
+        double hall[6][2];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+          hall[e][0] = f.S[e][0];
+          hall[e][1] = f.S[e][1];
+        }
+#pragma unroll
+        for (int e = 0; e < 6; ++e) fixed_point_row(e, f.S[e], K, Si, r, hall, f.xs[e], f.P0);
+      }
+      turn(f.ang.cp, f.ang.sp, dx[2]);
+      turn(f.ang.ct, f.ang.st, dx[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 6; ++e) K[e][0] = K[e][1] = 0.0;
+    }
+    if (MODE == kBackward) {
+#pragma unroll
+      for (int e = 0; e < 6; ++e) ws.d(k, BackRec::XF + e) = f.x[e];
+#pragma unroll
+      for (int e = 0; e < 21; ++e) ws.d(k, BackRec::CF + e) = f.C[e];
+    } else if (MODE == kEveryState) {
+#pragma unroll
+      for (int e = 0; e < 6; ++e) {
+        ws.d(k, StateRec::K + 2 * e) = K[e][0];
+        ws.d(k, StateRec::K + 2 * e + 1) = K[e][1];
+        ws.d(k, StateRec::XF + e) = f.x[e];
+      }
+      ws.d(k, StateRec::IR) = ir[0];
+      ws.d(k, StateRec::IR + 1) = ir[1];
+#pragma unroll
+      for (int e = 0; e < 21; ++e) ws.d(k, StateRec::CF + e) = f.C[e];
+    }
+    sid_prev = sid;
+  }
+  return ST_OK;
+}
+
+// The same with the time, out of line (see filter_states_with_time).
 template <int FIELD>
+__device__ __noinline__ int variant_states_with_time(const FitParams& p, const double* s_surf, const WS& ws, int64_t o0,
+                                                     int n, Filter* f) {
+  Filter t = *f;
+  const int st = variant_states<FIELD, 6, kState0>(p, s_surf, ws, o0, n, t);
+  *f = t;
+  return st;
+}
+
+template <int FIELD, int MODE>
 __device__ __forceinline__ void fit_one_variants(const FitParams& p, const double* s_surf, int i) {
   const int t = track_of(p, i);
   const size_t TT = (size_t)p.n_tracks_total;
   const WS ws{p.ws64, p.ws32, (size_t)p.n_tracks, kRec64Fp64, 0, i};
-  const int64_t o0 = p.offsets[t], o1 = p.offsets[t + 1];
-  const int n = (int)(o1 - o0);
-  int status = ST_OK;
-  if (!(o1 > o0) || o0 < 0 || o1 > p.n_states || n > p.max_states) status = ST_BAD_INPUT;
-  if (status == ST_OK)
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (sid < 0 || sid >= p.n_surfaces) status = ST_BAD_INPUT;
-    }
-  const bool states = p.out_states != nullptr, back = p.smoother != 0;
+  int64_t o0, o1;
+  int n;
+  int status = track_input(p, t, o0, o1, n);
+  const bool states = p.out_states != nullptr;
   double xs[6], P0[21];
   double chi2sum = 0.0;
   int nmeas = 0;
-  bool spd = true;
   if (status == ST_OK) {
-    // ------------------------------------------------ forward filter, with
-    // the fixed-point smoother (kf_fp64.cuh) unless the backward filter runs
-    double x[6], C[21], S[6][6];
-    Angles ang;
+    Filter f;
+    status = filter_first(p, t, o0, f);
+    if (status == ST_OK) {
+      if (MODE == kBackward) {
 #pragma unroll
-    for (int e = 0; e < 6; ++e) x[e] = p.seed_params[e * TT + t];
+        for (int e = 0; e < 6; ++e) ws.d(0, BackRec::XF + e) = f.x[e];
 #pragma unroll
-    for (int e = 0; e < 21; ++e) C[e] = p.seed_cov[e * TT + t];
-    int sid_prev = 0;
-    for (int k = 0; k < n; ++k) {
-      const int sid = p.surface_id[o0 + k];
-      if (k > 0) {
-        const Surf sa{s_surf + sid_prev * kSurfStride}, sb{s_surf + sid * kSurfStride};
-        Jac<double> J;
-        End o;
-        const Angles a0 = ang;
-        status = transport_variant<FIELD>(p, sa, sb, x, a0, o, J);
-        if (status != ST_OK) break;
-        if (states) end_angles(x[2], x[3], a0, o, x[2], x[3]);
-        ang = o.a;
-        // material of surface k (before the update): scattering with the
-        // arriving momentum, then the mean loss and its straggling
-        const double xx0 = sb.xx0(), lam = x[4];
-        double g = 1.0, var_q = 0.0;
-        if (p.energy_loss && xx0 > 0.0) {
-          status = energy_loss(p, x[4], xx0, o.inv_cos, +1, g, var_q);
-          if (status != ST_OK) break;
-        }
-        cov_transport(J, g, C);
-        if (xx0 > 0.0) add_scattering(lam, o.g2, xx0, o.inv_cos, o.inv_st, C);
-        C[sy(4, 4)] += var_q;
-        if (!back) {
-          spd = spd && spd_check(C);
-          const auto fe = [&](int r, int c) { return jf(J, r, c); };
-#pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            double v[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) v[c] = S[r][c];
-            row_times_ft(fe, g, v, S[r]);
-          }
-          if (states) {
-#pragma unroll
-            for (int e = 0; e < 25; ++e) ws.d(k, StateRec::F + e) = e < 20 ? J.f[e / 5][e % 5] : J.ft[e % 5];
-            ws.d(k, StateRec::G) = g;
-          }
-        }
-      }
-      double K[6][2], ir[2] = {0.0, 0.0}, dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const bool meas = !p.is_hole[o0 + k];
-      if (meas) {
-        const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
-        const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-        double Si[3], r[2], c2;
-        status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
-        if (status != ST_OK) break;
-        joseph_update(C, V, K);
-        chi2sum += c2;
-        ++nmeas;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) x[e] += dx[e];
-        ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
-        ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
-        if (k > 0 && !back) {
-          double hall[6][2];
-#pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            hall[e][0] = S[e][0];
-            hall[e][1] = S[e][1];
-          }
-#pragma unroll
-          for (int e = 0; e < 6; ++e) fixed_point_row(e, S[e], K, Si, r, hall, xs[e], P0);
-        }
+        for (int e = 0; e < 21; ++e) ws.d(0, BackRec::CF + e) = f.C[e];
+        status = variant_states<FIELD, 6, MODE>(p, s_surf, ws, o0, n, f);
+      } else if (MODE == kEveryState) {
+        status = variant_states<FIELD, 6, MODE>(p, s_surf, ws, o0, n, f);
+      } else if (time_is_settled(f.C)) {
+        status = variant_states<FIELD, 5, kState0>(p, s_surf, ws, o0, n, f);
       } else {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) K[e][0] = K[e][1] = 0.0;
+        Filter q = f;
+        status = variant_states_with_time<FIELD>(p, s_surf, ws, o0, n, &q);
+        f = q;
       }
-      if (k == 0) {
-        ang = angles_of(x[2], x[3]);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) xs[e] = dx[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) P0[e] = C[e];
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-          for (int c = 0; c < 6; ++c) S[r][c] = C[sym(r, c)];
-      } else if (meas) {
-        turn(ang.cp, ang.sp, dx[2]);
-        turn(ang.ct, ang.st, dx[3]);
-      }
-      if (back) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) ws.d(k, BackRec::XF + e) = x[e];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) ws.d(k, BackRec::CF + e) = C[e];
-      } else if (states && k > 0) {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          ws.d(k, StateRec::K + 2 * e) = K[e][0];
-          ws.d(k, StateRec::K + 2 * e + 1) = K[e][1];
-          ws.d(k, StateRec::XF + e) = x[e];
-        }
-        ws.d(k, StateRec::IR) = ir[0];
-        ws.d(k, StateRec::IR + 1) = ir[1];
-#pragma unroll
-        for (int e = 0; e < 21; ++e) ws.d(k, StateRec::CF + e) = C[e];
-      }
-      sid_prev = sid;
     }
+    chi2sum = f.chi2;
+    nmeas = f.nmeas;
 #pragma unroll
-    for (int e = 0; e < 6; ++e) xs[e] += p.seed_params[e * TT + t];
-    if (!back) {
-      if (status == ST_OK && !spd) status = ST_NON_SPD;
-      if (status == ST_OK && states) {
+    for (int e = 0; e < 6; ++e) xs[e] = f.xs[e] + p.seed_params[e * TT + t];
+#pragma unroll
+    for (int e = 0; e < 21; ++e) P0[e] = f.P0[e];
+    if (MODE != kBackward) {
+      if (status == ST_OK && !f.spd) status = ST_NON_SPD;
+      if (MODE == kEveryState && status == ST_OK) {
         smooth_states(ws, n, p.out_states, p.n_states, o0, true);
 #pragma unroll
         for (int e = 0; e < 6; ++e) p.out_states[e * p.n_states + o0] = xs[e];
       }
     } else if (status == ST_OK) {
+      double (&x)[6] = f.x;
+      double (&C)[21] = f.C;
+      Angles& ang = f.ang;
       // ------------------------------------------------ backward filter
       // starts at the last state from the forward-filtered parameters with
       // bf_scale times their covariance; the last state keeps the forward
@@ -627,9 +642,9 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
           const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
           const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
           double c2, K[6][2], Si[3], r[2], dx[6];
-          status = kalman_gain(x, C, m, V, K, Si, r, dx, c2);
+          status = kalman_gain<6>(x, C, m, V, K, Si, r, dx, c2);
           if (status != ST_OK) break;
-          joseph_update(C, V, K);
+          joseph_update<6>(C, V, K);
 #pragma unroll
           for (int e = 0; e < 6; ++e) x[e] += dx[e];
           turn(ang.cp, ang.sp, dx[2]);
@@ -660,7 +675,7 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
         status = transport_variant<FIELD>(p, sk, sj, x, ang, o, J);
         if (status != ST_OK) break;
         ang = o.a;
-        cov_transport(J, 1.0, C);
+        cov_transport<6>(J, 1.0, C);
         // weighted mean with the forward-filtered state k-1:
         //   K = Cf (Cf + Cb)^-1, xs = xf + K (xb - xf), Cs = Cf - K Cf,
         // on the states that are output; the others only have to be
@@ -672,7 +687,7 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
           Ssum[e] = Cf[e] + C[e];
         }
         if (k > 1 && !states) {
-          if (!spd_check(Ssum)) {
+          if (!spd_check<6>(Ssum)) {
             status = ST_NON_SPD;
             break;
           }
@@ -737,13 +752,20 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
   if (p.out_status) p.out_status[t] = (uint8_t)status;
 }
 
-template <int FIELD>
+template <int FIELD, int MODE>
 struct VariantBody {
   static constexpr int kStride = kSurfStride;
   static __device__ __forceinline__ void run(const FitParams& p, const double* s_surf, int i) {
-    fit_one_variants<FIELD>(p, s_surf, i);
+    fit_one_variants<FIELD, MODE>(p, s_surf, i);
   }
 };
+
+template <int FIELD>
+cudaError_t launch_mode(const FitParams& p, int block, cudaStream_t stream, int* launched) {
+  if (p.smoother != 0) return launch_body<VariantBody<FIELD, kBackward>, 1>(p, block, stream, launched);
+  if (p.out_states) return launch_body<VariantBody<FIELD, kEveryState>, 1>(p, block, stream, launched);
+  return launch_body<VariantBody<FIELD, kState0>, 1>(p, block, stream, launched);
+}
 
 }  // namespace
 
@@ -751,9 +773,9 @@ cudaError_t launch_fit_variants(const FitParams& p, int block, cudaStream_t stre
   if (launched) *launched = 0;
   if (p.n_tracks <= 0) return cudaSuccess;
   const int b = block ? block : 128;
-  if (p.map_b) return dev::launch_body<VariantBody<2>, 1>(p, b, stream, launched);
-  if (p.bfield[0] == 0.0 && p.bfield[1] == 0.0) return dev::launch_body<VariantBody<0>, 1>(p, b, stream, launched);
-  return dev::launch_body<VariantBody<1>, 1>(p, b, stream, launched);
+  if (p.map_b) return launch_mode<2>(p, b, stream, launched);
+  if (p.bfield[0] == 0.0 && p.bfield[1] == 0.0) return launch_mode<0>(p, b, stream, launched);
+  return launch_mode<1>(p, b, stream, launched);
 }
 
 }  // namespace kfgb

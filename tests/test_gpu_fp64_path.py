@@ -124,3 +124,24 @@ def test_library_shape_gives_the_same_bits(handle, field, states):  # noqa: F811
         for k in a:
             if a[k] is not None:
                 assert np.array_equal(a[k], b[k], equal_nan=True), (n, k)
+
+
+@pytest.mark.parametrize("team", TEAMS)
+def test_time_carried_or_not(handle, team):  # noqa: F811
+    """The fit leaves the time row out where the seed settles its pivot: seeds
+    with correlated times, and with time errors so small (1e-6 ns) that the
+    row is carried, give the oracle's results and the bits of the fit that
+    keeps every state (which always carries it)."""
+    ev = _event(97)
+    c = ev["seed_cov"].copy()
+    sd = np.sqrt(c[[0, 2, 5, 9, 14, 20]])
+    sd[5, 0::3] = 1e-6
+    for e, (i, j) in enumerate((i, j) for i in range(6) for j in range(i + 1)):
+        rho = 1.0 if i == j else 0.3 if (i, j) in ((5, 0), (5, 3), (2, 0)) else 0.0
+        c[e] = rho * sd[i] * sd[j]
+    ev["seed_cov"] = c
+    g = gpu_fit(handle, ev, FP64, team_warps=team)
+    compare(g, oracle.fit_batch(ev), FP64)
+    s = gpu_fit(handle, ev, FP64, with_states=True, team_warps=team)
+    for k in ("params", "cov", "chi2", "status"):
+        assert np.array_equal(g[k], s[k]), k
