@@ -14,13 +14,16 @@
 //     FP64 instruction holds the pipe of its sub-partition for 64 cycles, the
 //     pair form of the same operation takes 7 to 15 issue slots.  With these
 //     pieces in FP64 (about 145 instructions and 120 conversions per state)
-//     100k tracks of 31 states took 1.42 ms, with the pairs 0.80 ms; 1M uneven
-//     tracks 8.41 -> 5.28 ms, one event of 3001 tracks 0.209 -> 0.132 ms.
+//     100k tracks of 31 states took 1.42 ms, with the pairs 0.80 ms, and 0.755
+//     ms with what only the outputs need (the angles' own values, the time)
+//     left to launches that output every state, sums of products normalised
+//     once and the first state ahead of the loop; 1M uneven tracks 8.41 ->
+//     5.14 ms, one event of 3001 tracks 0.209 -> 0.121 ms.
 //     Against an 80-bit evaluation of the fit the rms errors are the same
 //     (0.9 to 1.04 times the former; ten shapes of 2000 tracks): the float
 //     quantities set them.  What bounds it now is issue: 4950 instructions per
 //     state and warp, 59 % of the issue slots used, the rest waits for the
-//     records and for dependent results.
+//     records and for dependent results (counted before the last of these).
 //   * FP64 only for the seed: its direction's sines and cosines, and the
 //     update of state 0 where that is measured.
 //   * float<->double conversions run on the integer pipe (dev::f2d/d2f,
@@ -122,12 +125,22 @@ __device__ __forceinline__ DF df_cut(double v) {
   const float ulp = __uint_as_float(((e - 23u) << 23) | sg);
   return fast_two_sum(hi, (float)(l & 0x1fffffffu) * 0x1p-29f * ulp);
 }
-// acc - a * b
-__device__ __forceinline__ DF df_fnma(DF acc, DF a, DF b) {
+// acc - a * b, the sum left unnormalised: a chain of these ends with df_norm
+__device__ __forceinline__ DF df_fnma_acc(DF acc, DF a, DF b) {
   const DF p = two_prod(a.hi, b.hi);
   const float c = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
   const DF s = two_sum(acc.hi, -p.hi);
-  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(acc.lo, c)));
+  return {s.hi, __fadd_rn(s.lo, __fsub_rn(acc.lo, c))};
+}
+__device__ __forceinline__ DF df_norm(DF x) { return fast_two_sum(x.hi, x.lo); }
+__device__ __forceinline__ DF df_fnma(DF acc, DF a, DF b) { return df_norm(df_fnma_acc(acc, a, b)); }
+// x + a * b + f
+__device__ __forceinline__ DF df_muladd(DF x, DF a, DF b, float f) {
+  const DF p = two_prod(a.hi, b.hi);
+  const float c = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
+  const DF s = two_sum(x.hi, p.hi);
+  const DF t = two_sum(s.hi, f);
+  return two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(s.lo, __fadd_rn(x.lo, c))));
 }
 // 1 / x: a float reciprocal and one Newton step (relative error about 2^-44)
 __device__ __forceinline__ DF df_rcp(DF x) {
@@ -341,8 +354,8 @@ __device__ __forceinline__ void turn_inc(CS& cs, float a, float b, float out[3])
 template <bool BZ>
 __device__ __forceinline__ int transport_mixed(const SurfM& sa, const SurfM& sb, const DF r0[3], const DF x[6],
                                const Dir& d, const Pend& pd, CS& cs, const float Bf[3], float m2, float h_max,
-                               int n_iter, DF xp[6], DF rp[3], Dir& dp, JacF& J, float& sin_th,
-                               float& cos_inc) {
+                               int n_iter, bool outputs, DF xp[6], DF rp[3], Dir& dp, JacF& J,
+                               float& sin_th, float& cos_inc) {
   // The point and the direction stay df (predicted values of surface a);
   // everything that moves them here (the pending filter increments, the RKN
   // curvature terms, the direction change accT, the plane corrections) is
@@ -452,20 +465,21 @@ __device__ __forceinline__ int transport_mixed(const SurfM& sa, const SurfM& sb,
     const float drem = dmf - (nb[0] * orr[0] + nb[1] * orr[1] + nb[2] * orr[2]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      r[i] = df_add_f(df_add(r[i], df_mul(s0d, Td[i])), off[i] + orr[i] + drem * nb[i]);
+      r[i] = df_muladd(r[i], s0d, Td[i], off[i] + orr[i] + drem * nb[i]);
       accT[i] += oT[i];
     }
     tinc += ot;
   }
-  const DF t = df_add_f(x[5], pd.t + tinc);
-  // end angles: the rotation from the start to the end direction, computed in
-  // FP32 from the start direction c and its change a = accT (no cancellation
-  // of large terms):
-  //   tan dphi = (c0 a1 - c1 a0) / (rho^2 + c0 a0 + c1 a1),
-  //   tan dtheta = (c2 drho - rho a2) / (c2 (c2 + a2) + rho (rho + drho)),
-  // with rho = |(c0, c1)| and drho the change of rho; the df angles and
-  // their cosines / sines then turn by these increments.
-  {
+  // the angles themselves and the time are only read for output
+  if (outputs) {
+    xp[5] = df_add_f(x[5], pd.t + tinc);
+    // end angles: the rotation from the start to the end direction, computed in
+    // FP32 from the start direction c and its change a = accT (no cancellation
+    // of large terms):
+    //   tan dphi = (c0 a1 - c1 a0) / (rho^2 + c0 a0 + c1 a1),
+    //   tan dtheta = (c2 drho - rho a2) / (c2 (c2 + a2) + rho (rho + drho)),
+    // with rho = |(c0, c1)| and drho the change of rho; the df angles and
+    // their cosines / sines then turn by these increments.
     const float c0 = T0f[0], c1 = T0f[1], c2 = T0f[2];
     const float a0 = accT[0], a1 = accT[1], a2 = accT[2];
     const float rho_sq = c0 * c0 + c1 * c1;
@@ -483,18 +497,17 @@ __device__ __forceinline__ int transport_mixed(const SurfM& sa, const SurfM& sb,
       phi = df_add(phi, DF{2.0f * kPiHi, 2.0f * kPiLo});
     dp.phi = phi;
     dp.theta = df_add_f(d.theta, pd.theta + dth);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) dp.T[i] = df_add_f(Td[i], pd.T[i] + accT[i]);
+    xp[2] = dp.phi;
+    xp[3] = dp.theta;
   }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) dp.T[i] = df_add_f(Td[i], pd.T[i] + accT[i]);
   rp[0] = r[0];
   rp[1] = r[1];
   rp[2] = r[2];
   xp[0] = df_dot(sb.uh(), sb.ul(), sb.uc(), r);
   xp[1] = df_dot(sb.vh(), sb.vl(), sb.vc(), r);
-  xp[2] = dp.phi;
-  xp[3] = dp.theta;
   xp[4] = x[4];
-  xp[5] = t;
 
   // path correction and free -> bound Jacobian (FP32)
   float cph, sph, cth, sth;
@@ -654,7 +667,8 @@ __device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF 
     DF dj = {Cp[sym(ia[j], ia[j])], 0.0f};
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (q < j) dj = df_fnma(dj, U[j][q], L[j][q]);
+      if (q < j) dj = df_fnma_acc(dj, U[j][q], L[j][q]);
+    if (j > 0) dj = df_norm(dj);
     if (!(dj.hi > 0.0f)) {
       ok = false;
       dj = {1.0f, 0.0f};
@@ -666,7 +680,8 @@ __device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF 
         DF u = {Cp[sym(ia[r], ia[j])], 0.0f};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q < j) u = df_fnma(u, U[r][q], L[j][q]);
+          if (q < j) u = df_fnma_acc(u, U[r][q], L[j][q]);
+        if (j > 0) u = df_norm(u);
         U[r][j] = u;
         L[r][j] = df_mul(u, iD[j]);
       }
@@ -683,7 +698,8 @@ __device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF 
       DF v = {Cp[sym(ia[r], 2 + m)], 0.0f};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q < r) v = df_fnma(v, L[r][q], y[q]);
+        if (q < r) v = df_fnma_acc(v, L[r][q], y[q]);
+      if (r > 0) v = df_norm(v);
       y[r] = v;
     }
 #pragma unroll
@@ -691,7 +707,8 @@ __device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF 
       DF v = df_mul(y[r], iD[r]);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q > r) v = df_fnma(v, L[q][r], X[q][m]);
+        if (q > r) v = df_fnma_acc(v, L[q][r], X[q][m]);
+      if (r < 3) v = df_norm(v);
       X[r][m] = v;
     }
   }
@@ -699,10 +716,13 @@ __device__ __forceinline__ bool angle_columns_of_inverse(const float Cp[21], DF 
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const DF c2 = {Cp[sym(ia[r], 2)], 0.0f}, c3 = {Cp[sym(ia[r], 3)], 0.0f};
-    s00 = df_fnma(s00, X[r][0], c2);
-    s01 = df_fnma(s01, X[r][1], c2);
-    s11 = df_fnma(s11, X[r][1], c3);
+    s00 = df_fnma_acc(s00, X[r][0], c2);
+    s01 = df_fnma_acc(s01, X[r][1], c2);
+    s11 = df_fnma_acc(s11, X[r][1], c3);
   }
+  s00 = df_norm(s00);
+  s01 = df_norm(s01);
+  s11 = df_norm(s11);
   const DF det = df_fnma(df_mul(s00, s11), s01, s01);
   if (!(det.hi > 0.0f) || !(s00.hi > 0.0f)) {
     ok = false;
@@ -865,8 +885,41 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
       for (int e = 0; e < 3; ++e) q.V[e] = p.cov[e * p.n_states + o0 + k];
     };
     Hit hit, next;
-    if (AHEAD) load_hit(0, next);
-    for (int k = 0; k < n && status == ST_OK; ++k) {
+    // state 0: x_p is the seed
+#pragma unroll
+    for (int e = 0; e < 6; ++e) ws.d(0, XP + e) = df_to_d(x[e]);
+    load_hit(0, hit);
+    if (!hit.hole) {
+      SeedUpdate su;
+      update_seed(p.seed_cov + t, TT, (hit.m[0] - f2d(x[0].hi)) - f2d(x[0].lo),
+                  (hit.m[1] - f2d(x[1].hi)) - f2d(x[1].lo), hit.V[0], hit.V[1], hit.V[2], &su);
+      if (su.ok) {
+        chi2sum = su.chi2;
+        ++nmeas;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) dx[e] = su.dx[e];
+#pragma unroll
+        for (int e = 0; e < 21; ++e) Cf[e] = su.Cf[e];
+        const SurfM s0 = surf_m(s_surf, sid_prev);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) pd.r[c] = dx[0] * s0.uf(c) + dx[1] * s0.vf(c);
+        turn_inc(cs, dx[2], dx[3], pd.T);
+        pd.phi = dx[2];
+        pd.theta = dx[3];
+        pd.t = dx[5];
+        x[4] = df_add_f(x[4], dx[4]);
+      } else {
+        status = ST_NON_SPD;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 21; ++e) Cf[e] = d2f(p.seed_cov[e * TT + t]);
+    }
+#pragma unroll
+    for (int e = 0; e < 6; ++e) ws.f(0, DXF + e) = dx[e];
+    if (AHEAD && n > 1) load_hit(1, next);
+#pragma unroll 1
+    for (int k = 1; k < n && status == ST_OK; ++k) {
       if (AHEAD) {
         hit = next;
         if (k + 1 < n) load_hit(k + 1, next);
@@ -875,152 +928,125 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
       DF xp[6], rp[3];
       float Cpf[21];
       Dir dp;
-      if (k == 0) {
+      const SurfM sa = surf_m(s_surf, sid_prev), sb = surf_m(s_surf, sid);
+      JacF J;
+      float sin_th, cos_inc;
+      status = transport_mixed<BZ>(sa, sb, r, x, d, pd, cs, Bf, m2, h_max, p.n_iter, p.out_states != nullptr,
+                                   xp, rp, dp, J, sin_th, cos_inc);
+      if (status != ST_OK) break;
+      const float* Cr = Cf;
+      // Cp = F Cf F^T, rows of Bm = F Cf formed on the fly
 #pragma unroll
-        for (int e = 0; e < 6; ++e) xp[e] = x[e];
+      for (int a = 0; a < 6; ++a) {
+        float brow[6];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) Cpf[e] = d2f(p.seed_cov[e * TT + t]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) rp[c] = r[c];
-        dp = d;
-      } else {
-        const SurfM sa = surf_m(s_surf, sid_prev), sb = surf_m(s_surf, sid);
-        JacF J;
-        float sin_th, cos_inc;
-        status = transport_mixed<BZ>(sa, sb, r, x, d, pd, cs, Bf, m2, h_max, p.n_iter, xp, rp, dp, J, sin_th,
-                                     cos_inc);
-        if (status != ST_OK) break;
-        const float* Cr = Cf;
-        // Cp = F Cf F^T, rows of Bm = F Cf formed on the fly
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-          float brow[6];
-#pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            float v;
-            if (a == 4) {
-              v = Cr[sym(4, j)];
-            } else {
-              v = jf(J, a, 0) * Cr[sym(0, j)] + jf(J, a, 1) * Cr[sym(1, j)] + jf(J, a, 2) * Cr[sym(2, j)] +
-                  jf(J, a, 3) * Cr[sym(3, j)] + jf(J, a, 4) * Cr[sym(4, j)];
-              if (a == 5) v += Cr[sym(5, j)];
-            }
-            brow[j] = v;
+        for (int j = 0; j < 6; ++j) {
+          float v;
+          if (a == 4) {
+            v = Cr[sym(4, j)];
+          } else {
+            v = jf(J, a, 0) * Cr[sym(0, j)] + jf(J, a, 1) * Cr[sym(1, j)] + jf(J, a, 2) * Cr[sym(2, j)] +
+                jf(J, a, 3) * Cr[sym(3, j)] + jf(J, a, 4) * Cr[sym(4, j)];
+            if (a == 5) v += Cr[sym(5, j)];
           }
+          brow[j] = v;
+        }
 #pragma unroll
-          for (int c = 0; c < 6; ++c)
-            if (c <= a) {
-              float v;
-              if (c == 4) {
-                v = brow[4];
-              } else {
-                v = brow[0] * jf(J, c, 0) + brow[1] * jf(J, c, 1) + brow[2] * jf(J, c, 2) +
-                    brow[3] * jf(J, c, 3) + brow[4] * jf(J, c, 4);
-                if (c == 5) v += brow[5];
-              }
-              Cpf[sy(a, c)] = v;
+        for (int c = 0; c < 6; ++c)
+          if (c <= a) {
+            float v;
+            if (c == 4) {
+              v = brow[4];
+            } else {
+              v = brow[0] * jf(J, c, 0) + brow[1] * jf(J, c, 1) + brow[2] * jf(J, c, 2) +
+                  brow[3] * jf(J, c, 3) + brow[4] * jf(J, c, 4);
+              if (c == 5) v += brow[5];
             }
-        }
-        // multiple scattering of surface k, added before the update
-        float qphi = 0.0f, qth = 0.0f;
-        const float xx0 = sb.xx0f();
-        if (xx0 > 0.0f) {
-          const float th0 = highland<float>(fabsf(x[4].hi), m2, xx0, cos_inc);
-          qth = th0 * th0;
-          qphi = qth / (sin_th * sin_th);
-          Cpf[sy(2, 2)] += qphi;
-          Cpf[sy(3, 3)] += qth;
-        }
-#pragma unroll
-        for (int e = 0; e < 20; ++e) ws.f(k, FJ + e) = J.f[e / 5][e % 5];
-#pragma unroll
-        for (int e = 0; e < 5; ++e) ws.f(k, FJ + 20 + e) = J.ft[e];
-        ws.f(k, QPHI) = qphi;
-        ws.f(k, QTH) = qth;
+            Cpf[sy(a, c)] = v;
+          }
       }
-      if (k == 0 || p.out_states) {
+      // multiple scattering of surface k, added before the update
+      float qphi = 0.0f, qth = 0.0f;
+      const float xx0 = sb.xx0f();
+      if (xx0 > 0.0f) {
+        const float th0 = highland<float>(fabsf(x[4].hi), m2, xx0, cos_inc);
+        qth = th0 * th0;
+        qphi = qth / (sin_th * sin_th);
+        Cpf[sy(2, 2)] += qphi;
+        Cpf[sy(3, 3)] += qth;
+      }
+#pragma unroll
+      for (int e = 0; e < 20; ++e) ws.f(k, FJ + e) = J.f[e / 5][e % 5];
+#pragma unroll
+      for (int e = 0; e < 5; ++e) ws.f(k, FJ + 20 + e) = J.ft[e];
+      ws.f(k, QPHI) = qphi;
+      ws.f(k, QTH) = qth;
+      if (p.out_states) {
 #pragma unroll
         for (int e = 0; e < 6; ++e) ws.d(k, XP + e) = df_to_d(xp[e]);
       }
-      if (k > 0) {
 #pragma unroll
-        for (int e = 0; e < 21; ++e) ws.f(k, CPF + e) = Cpf[e];
-      }
+      for (int e = 0; e < 21; ++e) ws.f(k, CPF + e) = Cpf[e];
       const SurfM sk = surf_m(s_surf, sid);
       if (AHEAD ? !hit.hole : !p.is_hole[o0 + k]) {
         if (!AHEAD) load_hit(k, hit);
         const double m0 = hit.m[0], m1 = hit.m[1], V0 = hit.V[0], V1 = hit.V[1], V2 = hit.V[2];
-        if (k == 0) {
-          SeedUpdate su;
-          update_seed(p.seed_cov + t, TT, (m0 - f2d(xp[0].hi)) - f2d(xp[0].lo), (m1 - f2d(xp[1].hi)) - f2d(xp[1].lo),
-                      V0, V1, V2, &su);
-          if (!su.ok) {
-            status = ST_NON_SPD;
-            break;
-          }
-          chi2sum = su.chi2;
-#pragma unroll
-          for (int e = 0; e < 6; ++e) dx[e] = su.dx[e];
-#pragma unroll
-          for (int e = 0; e < 21; ++e) Cf[e] = su.Cf[e];
-        } else {
-          // gain-matrix update: gain in FP32, the Joseph covariance and chi2
-          // in double-float arithmetic on the FP32 pipe.  The FP64 form took
-          // 90 FP64 instructions and 120 conversions per state.
-          const DF S00 = df_add_f(df_cut(V0), Cpf[sy(0, 0)]), S01 = df_add_f(df_cut(V1), Cpf[sy(1, 0)]),
-                   S11 = df_add_f(df_cut(V2), Cpf[sy(1, 1)]);
-          const DF det = df_fnma(df_mul(S00, S11), S01, S01);
-          if (!(det.hi > 0.0f) || !(S00.hi > 0.0f)) {
-            status = ST_NON_SPD;
-            break;
-          }
-          const DF idet = df_rcp(det);
-          const DF r0 = df_add(df_cut(m0), df_neg(xp[0])), r1 = df_add(df_cut(m1), df_neg(xp[1]));
-          const DF u = df_fnma(df_mul(S11, r0), S01, r1), v = df_fnma(df_mul(S00, r1), S01, r0);
-          chi2sum = df_add(chi2sum, df_mul(df_add(df_mul(r0, u), df_mul(r1, v)), idet));
-          const float idf = df_f(idet);
-          const float i00 = df_f(S11) * idf, i01 = -df_f(S01) * idf, i11 = df_f(S00) * idf;
-          const float r0f = df_f(r0), r1f = df_f(r1);
-          float Kf[6][2];
-#pragma unroll
-          for (int e = 0; e < 6; ++e) {
-            const float c0 = Cpf[sym(e, 0)], c1 = Cpf[sym(e, 1)];
-            const float k0 = c0 * i00 + c1 * i01, k1 = c0 * i01 + c1 * i11;
-            Kf[e][0] = k0;
-            Kf[e][1] = k1;
-            dx[e] = k0 * r0f + k1 * r1f;
-          }
-          // Joseph form, expanded: Cf = Cp - (H Cp)^T K^T + K W with
-          // W = S K^T - H Cp.  For the exact gain W = 0; here W is the
-          // residual of the gain equation left by the FP32 gain,
-          // O(eps32 |H Cp|).  Its products are exact (FMA splits), its
-          // cancelling sum is compensated (TwoSum); the element's own sum
-          // Cp - c0 K0 - c1 K1 likewise, with K W added to the low parts.
-          float Wf[2][6];
-          auto w_of = [](DF Sa, DF Sb, float k0, float k1, float c) {
-            const DF pa = two_prod(Sa.hi, k0), pb = two_prod(Sb.hi, k1);
-            const DF x1 = two_sum(pa.hi, -c);
-            const DF x2 = two_sum(x1.hi, pb.hi);
-            const float lo = __fadd_rn(__fadd_rn(x1.lo, x2.lo), __fadd_rn(pa.lo, pb.lo));
-            return __fadd_rn(x2.hi, __fmaf_rn(Sa.lo, k0, __fmaf_rn(Sb.lo, k1, lo)));
-          };
-#pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            Wf[0][j] = w_of(S00, S01, Kf[j][0], Kf[j][1], Cpf[sym(0, j)]);
-            Wf[1][j] = w_of(S01, S11, Kf[j][0], Kf[j][1], Cpf[sym(1, j)]);
-          }
-#pragma unroll
-          for (int a = 0; a < 6; ++a)
-#pragma unroll
-            for (int b = 0; b < 6; ++b)
-              if (b <= a) {
-                const DF pa = two_prod(Cpf[sym(0, a)], Kf[b][0]), pb = two_prod(Cpf[sym(1, a)], Kf[b][1]);
-                const DF x1 = two_sum(Cpf[sy(a, b)], -pa.hi);
-                const DF x2 = two_sum(x1.hi, -pb.hi);
-                const float lo = __fsub_rn(__fsub_rn(__fadd_rn(x1.lo, x2.lo), pa.lo), pb.lo);
-                Cf[sy(a, b)] = __fadd_rn(x2.hi, __fmaf_rn(Kf[a][0], Wf[0][b], __fmaf_rn(Kf[a][1], Wf[1][b], lo)));
-              }
+        // gain-matrix update: gain in FP32, the Joseph covariance and chi2
+        // in double-float arithmetic on the FP32 pipe.  The FP64 form took
+        // 90 FP64 instructions and 120 conversions per state.
+        const DF S00 = df_add_f(df_cut(V0), Cpf[sy(0, 0)]), S01 = df_add_f(df_cut(V1), Cpf[sy(1, 0)]),
+                 S11 = df_add_f(df_cut(V2), Cpf[sy(1, 1)]);
+        const DF det = df_fnma(df_mul(S00, S11), S01, S01);
+        if (!(det.hi > 0.0f) || !(S00.hi > 0.0f)) {
+          status = ST_NON_SPD;
+          break;
         }
+        const DF idet = df_rcp(det);
+        const DF r0 = df_add(df_cut(m0), df_neg(xp[0])), r1 = df_add(df_cut(m1), df_neg(xp[1]));
+        const DF u = df_fnma(df_mul(S11, r0), S01, r1), v = df_fnma(df_mul(S00, r1), S01, r0);
+        chi2sum = df_add(chi2sum, df_mul(df_add(df_mul(r0, u), df_mul(r1, v)), idet));
+        const float idf = df_f(idet);
+        const float i00 = df_f(S11) * idf, i01 = -df_f(S01) * idf, i11 = df_f(S00) * idf;
+        const float r0f = df_f(r0), r1f = df_f(r1);
+        float Kf[6][2];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+          const float c0 = Cpf[sym(e, 0)], c1 = Cpf[sym(e, 1)];
+          const float k0 = c0 * i00 + c1 * i01, k1 = c0 * i01 + c1 * i11;
+          Kf[e][0] = k0;
+          Kf[e][1] = k1;
+          dx[e] = k0 * r0f + k1 * r1f;
+        }
+        // Joseph form, expanded: Cf = Cp - (H Cp)^T K^T + K W with
+        // W = S K^T - H Cp.  For the exact gain W = 0; here W is the
+        // residual of the gain equation left by the FP32 gain,
+        // O(eps32 |H Cp|).  Its products are exact (FMA splits), its
+        // cancelling sum is compensated (TwoSum); the element's own sum
+        // Cp - c0 K0 - c1 K1 likewise, with K W added to the low parts.
+        float Wf[2][6];
+        auto w_of = [](DF Sa, DF Sb, float k0, float k1, float c) {
+          const DF pa = two_prod(Sa.hi, k0), pb = two_prod(Sb.hi, k1);
+          const DF x1 = two_sum(pa.hi, -c);
+          const DF x2 = two_sum(x1.hi, pb.hi);
+          const float lo = __fadd_rn(__fadd_rn(x1.lo, x2.lo), __fadd_rn(pa.lo, pb.lo));
+          return __fadd_rn(x2.hi, __fmaf_rn(Sa.lo, k0, __fmaf_rn(Sb.lo, k1, lo)));
+        };
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          Wf[0][j] = w_of(S00, S01, Kf[j][0], Kf[j][1], Cpf[sym(0, j)]);
+          Wf[1][j] = w_of(S01, S11, Kf[j][0], Kf[j][1], Cpf[sym(1, j)]);
+        }
+#pragma unroll
+        for (int a = 0; a < 6; ++a)
+#pragma unroll
+          for (int b = 0; b < 6; ++b)
+            if (b <= a) {
+              const DF pa = two_prod(Cpf[sym(0, a)], Kf[b][0]), pb = two_prod(Cpf[sym(1, a)], Kf[b][1]);
+              const DF x1 = two_sum(Cpf[sy(a, b)], -pa.hi);
+              const DF x2 = two_sum(x1.hi, -pb.hi);
+              const float lo = __fsub_rn(__fsub_rn(__fadd_rn(x1.lo, x2.lo), pa.lo), pb.lo);
+              Cf[sy(a, b)] = __fadd_rn(x2.hi, __fmaf_rn(Kf[a][0], Wf[0][b], __fmaf_rn(Kf[a][1], Wf[1][b], lo)));
+            }
         ++nmeas;
         // the filtered state: the prediction plus the increments, which stay
         // pending in FP32 (the point moves in the plane by (dx0, dx1)); only
