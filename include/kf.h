@@ -226,10 +226,11 @@ typedef struct {
                                   Jacobian columns and the matrix rows, for
                                   batches too small to fill the GPU; grid
                                   schedule, block ignored; 0 = one thread per
-                                  track, and with every launch option at its
-                                  default a last round that would fill at
-                                  most half of the GPU goes to teams; the
-                                  results are the same bits) */
+                                  track, and with the other launch options
+                                  but the schedule at their defaults (and a
+                                  schedule other than waves) a last round
+                                  that would fill at most half of the GPU
+                                  goes to teams; the same bits) */
   int32_t test_wait_timeout;   /* diagnostic of the timeout path (0 = off):
                                   1 announces the surface table's copy on
                                   each CTA's barrier without issuing it, so

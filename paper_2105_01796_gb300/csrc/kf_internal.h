@@ -143,10 +143,11 @@ cudaError_t launch_fit_team(const FitParams& p, int team_warps, cudaStream_t str
 // dynamic shared memory of one of its CTAs
 size_t team_smem_bytes(int n_surfaces);
 
-// Whether the options leave the FP64 fit's launch shape to the library
-// (every launch option at its default).
-inline bool shape_is_default(int schedule_is_persistent, int block, int min_blocks, int resident_warps, int team_warps) {
-  return schedule_is_persistent && (block == 0 || block == 128) && min_blocks == 0 && resident_warps == 0 &&
+// Whether the options leave the FP64 fit's launch shape to the library (every
+// launch option but the schedule at its default; the wave-split schedule
+// spreads its last round itself).
+inline bool shape_is_default(bool waves, int block, int min_blocks, int resident_warps, int team_warps) {
+  return !waves && (block == 0 || block == 128) && min_blocks == 0 && resident_warps == 0 &&
          team_warps == 0;
 }
 

@@ -228,7 +228,10 @@ namespace {
 // after the full rounds, teams of 4 while they fit one per SM (U <= SMs:
 // 0.60 to 0.64 of a round's time, measured 421-453 against 706 us at 20
 // planes), teams of 2 up to two per SM (0.72 to 0.75, 510-531 us), else the
-// round as it is (a second round of teams takes 0.9 and more).
+// round as it is (a second round of teams takes 0.9 and more).  On the
+// length-sorted schedule the last round holds the shortest tracks; without
+// teams its CTAs share SMs with some of the longest (20k tracks of 6 to 25
+// states: 2.07-2.41 ms by the luck of the placement, 1.58-1.64 ms with them).
 cudaError_t launch_fp64_auto(const FitParams& p, int block, int min_blocks, bool bz, cudaStream_t stream,
                              int* launched) {
   int dev = 0, nsm = 0, smem_max = 0;
