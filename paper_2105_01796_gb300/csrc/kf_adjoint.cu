@@ -543,25 +543,55 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
 // the update
 // ---------------------------------------------------------------------------
 
+// What the smoother adds to the reverse of a transition: with h = Sp H^T
+// (Sp = Cov(x_0, x_k) predicted) its update is
+//   x0 += h y (weight v), P0 -= h Si h^T (weight W), Sf = Sp - h Si P^T,
+// and its prediction Sp = S F^T.  Contributions to the adjoints of y (yb), Si
+// (G: 00, 01, 11) and F (lF), and LS^T h for that of P (Z).
+struct SmOut {
+  double yb[2], G[3], Z[5][2], lF[4][5];
+};
+
+// Si and y = Si r of the update at a state
+struct Innov {
+  double Si[3], r[2], y[2];
+};
+__device__ __forceinline__ Innov innovation(const double xp[2], const double Cp[21], const double m[2],
+                                            const double V[3]) {
+  const double S00 = V[0] + Cp[sy(0, 0)], S01 = V[1] + Cp[sy(1, 0)], S11 = V[2] + Cp[sy(1, 1)];
+  const double idet = rcp_any(fma(S00, S11, -S01 * S01));
+  Innov q;
+  q.Si[0] = S11 * idet;
+  q.Si[1] = -S01 * idet;
+  q.Si[2] = S00 * idet;
+  q.r[0] = m[0] - xp[0];
+  q.r[1] = m[1] - xp[1];
+  q.y[0] = fma(q.Si[0], q.r[0], q.Si[1] * q.r[1]);
+  q.y[1] = fma(q.Si[1], q.r[0], q.Si[2] * q.r[1]);
+  return q;
+}
+
 // Reverse through one measured update:
 //   P = Cp H^T, S = V + H Cp H^T, Si = S^-1, r = m - H xp, y = Si r,
 //   xf = xp + P y, Cf = Cp - P Si P^T, chi2 = r^T y (weight w),
-// and with SM the smoother's, h = Sp H^T (Sp = Cov(x_0, x_k) predicted):
-//   x0 += h y (weight v), P0 -= h Si h^T (weight W), Sf = Sp - h Si P^T.
-// lf, Lf (packed, full-matrix convention) and LS (adjoints of xf, Cf, Sf)
-// become those of xp, Cp, Sp.  N: parameters (5: without the time).
+// with the smoother's contributions if SM.  lf, Lf (packed, full-matrix
+// convention; adjoints of xf, Cf) become those of xp, Cp.  N: parameters
+// (5: without the time).
 template <bool SM, int N>
-__device__ __forceinline__ int update_reverse(const double xp[2], const double Cp[21], const double m[2],
-                                              const double V[3], double w, const double hm[6][2], const double v[6],
-                                              const double W[21], double lf[6], double Lf[21], double LS[6][5]) {
-  const double S00 = V[0] + Cp[sy(0, 0)], S01 = V[1] + Cp[sy(1, 0)], S11 = V[2] + Cp[sy(1, 1)];
-  const double idet = rcp_any(fma(S00, S11, -S01 * S01));
-  const double Si[3] = {S11 * idet, -S01 * idet, S00 * idet};
-  const double r[2] = {m[0] - xp[0], m[1] - xp[1]};
-  const double y[2] = {fma(Si[0], r[0], Si[1] * r[1]), fma(Si[1], r[0], Si[2] * r[1])};
+__device__ __forceinline__ void update_reverse(const Innov& q, const double Cp[21], double w, const SmOut& sm,
+                                               double lf[6], double Lf[21]) {
   // U = Lf P; yb = P^T lf (+ h^T v); G = adjoint of Si (symmetric)
-  double U[6][2], yb[2] = {0.0, 0.0};
+  const double* Si = q.Si;
+  const double* r = q.r;
+  double Z[6][2], yb[2] = {0.0, 0.0};
   double G00 = w * r[0] * r[0], G01 = w * r[0] * r[1], G11 = w * r[1] * r[1];
+  if (SM) {
+    yb[0] = sm.yb[0];
+    yb[1] = sm.yb[1];
+    G00 += sm.G[0];
+    G01 += sm.G[1];
+    G11 += sm.G[2];
+  }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     double u0 = 0.0, u1 = 0.0;
@@ -570,51 +600,13 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
       u0 = fma(Lf[sym(i, j)], Cp[sym(j, 0)], u0);
       u1 = fma(Lf[sym(i, j)], Cp[sym(j, 1)], u1);
     }
-    U[i][0] = u0;
-    U[i][1] = u1;
     yb[0] = fma(Cp[sym(i, 0)], lf[i], yb[0]);
     yb[1] = fma(Cp[sym(i, 1)], lf[i], yb[1]);
     G00 = fma(-Cp[sym(i, 0)], u0, G00);
     G01 = fma(-Cp[sym(i, 0)], u1, G01);
     G11 = fma(-Cp[sym(i, 1)], u1, G11);
-  }
-  double Z[6][2];  // 2 U + LS^T h
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    Z[i][0] = 2.0 * U[i][0];
-    Z[i][1] = 2.0 * U[i][1];
-  }
-  if (SM) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      yb[0] = fma(hm[i][0], v[i], yb[0]);
-      yb[1] = fma(hm[i][1], v[i], yb[1]);
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      // row i of W h and of LS P
-      double a0 = 0.0, a1 = 0.0, q0 = 0.0, q1 = 0.0;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        a0 = fma(W[sym(i, j)], hm[j][0], a0);
-        a1 = fma(W[sym(i, j)], hm[j][1], a1);
-      }
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        q0 = fma(LS[i][j], Cp[sym(j, 0)], q0);
-        q1 = fma(LS[i][j], Cp[sym(j, 1)], q1);
-        Z[j][0] = fma(LS[i][j], hm[i][0], Z[j][0]);
-        Z[j][1] = fma(LS[i][j], hm[i][1], Z[j][1]);
-      }
-      const double b0 = a0 + q0, b1 = a1 + q1;
-      G00 = fma(-hm[i][0], b0, G00);
-      G11 = fma(-hm[i][1], b1, G11);
-      G01 = fma(-0.5, fma(hm[i][0], b1, hm[i][1] * b0), G01);
-      const double c0 = fma(2.0, a0, q0), c1 = fma(2.0, a1, q1);
-      // adjoint of h: v y^T - (2 W h + LS P) Si
-      LS[i][0] += fma(v[i], y[0], -fma(c0, Si[0], c1 * Si[1]));
-      LS[i][1] += fma(v[i], y[1], -fma(c0, Si[1], c1 * Si[2]));
-    }
+    Z[i][0] = SM && i < 5 ? fma(2.0, u0, sm.Z[i < 5 ? i : 0][0]) : 2.0 * u0;
+    Z[i][1] = SM && i < 5 ? fma(2.0, u1, sm.Z[i < 5 ? i : 0][1]) : 2.0 * u1;
   }
   G00 = fma(yb[0], r[0], G00);
   G11 = fma(yb[1], r[1], G11);
@@ -628,15 +620,14 @@ __device__ __forceinline__ int update_reverse(const double xp[2], const double C
   // adjoint of P: lf y^T - Z Si, into columns 0 and 1 (symmetrised)
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const double P0 = fma(lf[i], y[0], -fma(Z[i][0], Si[0], Z[i][1] * Si[1]));
-    const double P1 = fma(lf[i], y[1], -fma(Z[i][0], Si[1], Z[i][1] * Si[2]));
+    const double P0 = fma(lf[i], q.y[0], -fma(Z[i][0], Si[0], Z[i][1] * Si[1]));
+    const double P1 = fma(lf[i], q.y[1], -fma(Z[i][0], Si[1], Z[i][1] * Si[2]));
     Lf[sym(i, 0)] += i == 0 ? P0 : 0.5 * P0;
     Lf[sym(i, 1)] += i == 1 ? P1 : 0.5 * P1;
   }
   // adjoint of r: Si (yb + 2 w r)
-  lf[0] -= fma(2.0 * w, y[0], fma(Si[0], yb[0], Si[1] * yb[1]));
-  lf[1] -= fma(2.0 * w, y[1], fma(Si[1], yb[0], Si[2] * yb[1]));
-  return ST_OK;
+  lf[0] -= fma(2.0 * w, q.y[0], fma(Si[0], yb[0], Si[1] * yb[1]));
+  lf[1] -= fma(2.0 * w, q.y[1], fma(Si[1], yb[0], Si[2] * yb[1]));
 }
 
 struct GradParams {
@@ -696,216 +687,325 @@ __device__ __forceinline__ void plane_gradient(const double* __restrict__ d, con
   }
 }
 
-// Pass B of track slot tl (in_range: a track of the launch; status: of its
-// forward pass).  All 32 lanes of a warp call it together.
-template <bool BZ, bool SM>
-__device__ __forceinline__ void grad_reverse(const GradParams& g, const double* s_surf, int tl, bool in_range,
-                                             int status) {
-  const FitParams& p = g.f;
-  const int tg = p.track0 + tl;
-  const size_t TG = (size_t)p.n_tracks_total, TL = (size_t)p.n_tracks;
-  constexpr int kRec = SM ? kRecWhole : kRecFilter;
-  auto rec = [&](int k, int e) -> double& { return g.rec[((size_t)k * kRec + e) * TL + tl]; };
-  const int64_t o0 = p.offsets[tg];
-  const int n = (int)(p.offsets[tg + 1] - o0);
-  const double w = (g.dl_dchi2 && in_range) ? g.dl_dchi2[tg] : 1.0;
-  const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
-  const double kB[3] = {kKappa * Bf[0], kKappa * Bf[1], kKappa * Bf[2]};
-  const double nu2 = BZ ? kB[2] * kB[2] : dot3(kB, kB);
-  // adjoints of x_f, C_f (packed, full-matrix convention) and S of state k
-  double lf[6], Lf[21], LS[6][5], v[6], W[21];
+// One track of a launch as pass B sees it.
+template <bool SM>
+struct TrackB {
+  const GradParams* g;
+  const double* s_surf;
+  int64_t o0;
+  int tl, tg;
+  double kB[3], nu2;
+  __device__ __forceinline__ TrackB(const GradParams& gp, const double* surf, int slot, bool bz)
+      : g(&gp), s_surf(surf), tl(slot), tg(gp.f.track0 + slot) {
+    o0 = gp.f.offsets[tg];
 #pragma unroll
-  for (int e = 0; e < 6; ++e) {
-    lf[e] = 0.0;
-    v[e] = SM && g.dl_dparams && status == ST_OK ? g.dl_dparams[e * TG + tg] : 0.0;
+    for (int e = 0; e < 3; ++e) kB[e] = kKappa * gp.f.bfield[e];
+    nu2 = bz ? kB[2] * kB[2] : dot3(kB, kB);
   }
+  __device__ __forceinline__ double rec(int k, int e) const {
+    return g->rec[((size_t)k * (SM ? kRecWhole : kRecFilter) + e) * (size_t)g->f.n_tracks + tl];
+  }
+  __device__ __forceinline__ Surf surf(int k) const { return Surf{s_surf + g->f.surface_id[o0 + k] * kSurfStride}; }
+  __device__ __forceinline__ bool hole(int k) const { return g->f.is_hole[o0 + k] != 0; }
+};
+
+// the filtered state a transition starts from
+struct StartB {
+  double x01[2], lam, r0[3];
+  Angles a0;
+};
+template <bool SM>
+__device__ __forceinline__ StartB start_of(const TrackB<SM>& t, int k) {
+  StartB s;
+  s.x01[0] = t.rec(k - 1, kRX + 0);
+  s.x01[1] = t.rec(k - 1, kRX + 1);
+  s.lam = t.rec(k - 1, kRX + 2);
+  s.a0 = {t.rec(k - 1, kRX + 3), t.rec(k - 1, kRX + 4), t.rec(k - 1, kRX + 5), t.rec(k - 1, kRX + 6)};
+  const Surf sa = t.surf(k - 1);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) s.r0[e] = fma(s.x01[0], sa.u(e), fma(s.x01[1], sa.v(e), sa.c(e)));
+  return s;
+}
+
+// Transition k-1 -> k run again.
+struct FwdB {
+  Path path;
+  End o;
+  Cols64 gc;
+  double inv_nT, F[4][5], xp[2], Cp[21], hm[6][2];
+};
+
+// every double of it that another warp needs (the tape apart)
+template <bool SM, class V>
+__device__ __forceinline__ void visit(FwdB& f, V v) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    v(f.path.T0[i]); v(f.path.NT[i]); v(f.path.NNT[i]);
+    v(f.o.r[i]); v(f.o.T[i]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      v(f.gc.gr[i][c]);
+      v(f.gc.gT[i][c]);
+    }
+  }
+  v(f.path.p00); v(f.path.pN); v(f.path.pNN); v(f.path.d0); v(f.path.s0);
+  PathG<true>& w = f.path.w;
+  v(w.eb); v(w.eg); v(w.rb); v(w.rg); v(w.deb); v(w.deg); v(w.drb); v(w.drg); v(w.len);
+  v(f.o.a.cp); v(f.o.a.sp); v(f.o.a.ct); v(f.o.a.st); v(f.o.inv_st); v(f.o.inv_cos); v(f.o.g2);
+  v(f.inv_nT);
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v(f.F[r][c]);
+  v(f.xp[0]); v(f.xp[1]);
+#pragma unroll
+  for (int e = 0; e < 15; ++e) v(f.Cp[e]);
+  if (SM)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      v(f.hm[i][0]);
+      v(f.hm[i][1]);
+    }
+}
+
+template <bool BZ, bool SM>
+__device__ __forceinline__ void forward_part(const TrackB<SM>& t, int k, const StartB& st, FwdB& f, Step* tape) {
+  const FitParams& p = t.g->f;
+  const Surf sa = t.surf(k - 1), sb = t.surf(k);
+  const double Bf[3] = {p.bfield[0], p.bfield[1], p.bfield[2]};
+  Path& path = f.path;
+  End& o = f.o;
+  Cols64& gc = f.gc;
+  path_forward<BZ>(sb, st.r0, st.a0, st.lam, t.kB, t.nu2, p.h_max, p.n_iter, path, tape);
+  const PathG<true>& q = path.w;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    o.r[i] = st.r0[i] + fma(q.len, path.T0[i], fma(q.rb, path.NT[i], q.rg * path.NNT[i]));
+    o.T[i] = path.T0[i] + fma(q.eb, path.NT[i], q.eg * path.NNT[i]);
+    gc.gr[i][2] = fma(q.drb, path.NT[i], q.drg * path.NNT[i]);
+    gc.gT[i][2] = fma(q.deb, path.NT[i], q.deg * path.NNT[i]);
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const double vc[3] = {c == 0 ? -path.T0[1] : st.a0.cp * st.a0.ct, c == 0 ? path.T0[0] : st.a0.sp * st.a0.ct,
+                          c == 0 ? 0.0 : -st.a0.st};
+    double Nv[3], NNv[3];
+    applyA<double, BZ>(t.kB, vc, Nv);
+    applyA<double, BZ>(t.kB, Nv, NNv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      gc.gr[i][c] = fma(q.len, vc[i], fma(q.rb, Nv[i], q.rg * NNv[i]));
+      gc.gT[i][c] = vc[i] + fma(q.eb, Nv[i], q.eg * NNv[i]);
+    }
+  }
+  o.g2 = fma(p.mass * p.mass * st.lam, st.lam, 1.0);
+  o.dtds = gc.gtl = 0.0;  // (no time row)
+  end_frame(sb, o, f.inv_nT);
+  Jac<double> J;
+  jacobian_columns<BZ, 31>(sa, sb, o, gc, st.lam, Bf, f.inv_nT, [&](int r, int c, double x) {
+    if (r < 4) J.f[r][c] = f.F[r][c] = x;
+  });
+  if (t.hole(k)) return;
+#pragma unroll
+  for (int e = 0; e < 15; ++e) f.Cp[e] = t.rec(k - 1, kRC + e);
+  cov_transport<5>(J, 1.0, f.Cp);
+  const double xx0 = sb.xx0();
+  if (xx0 > 0.0) {
+    const double z = highland_sq(st.lam, o.g2, xx0, o.inv_cos);
+    f.Cp[sy(2, 2)] = fma(z, o.inv_st * o.inv_st, f.Cp[sy(2, 2)]);
+    f.Cp[sy(3, 3)] += z;
+  }
+  if (SM)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      double h0 = 0.0, h1 = 0.0;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        const double z = t.rec(k - 1, kRS + 5 * i + c);
+        h0 = fma(f.F[0][c], z, h0);
+        h1 = fma(f.F[1][c], z, h1);
+      }
+      f.hm[i][0] = h0;
+      f.hm[i][1] = h1;
+    }
+  const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
+  f.xp[0] = fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2)));
+  f.xp[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
+}
+
+// The smoother's part of the reverse of transition k: LS (adjoint of S_k)
+// becomes that of S_k-1; it depends on nothing else of the reverse.
+__device__ __forceinline__ void smoother_part(const TrackB<true>& t, int k, const double F[4][5], const double Cp[21],
+                                              const double xp[2], const double hm[6][2], const double v[6],
+                                              const double W[21], double LS[6][5], SmOut& o) {
+  if (!t.hole(k)) {
+    double m[2], V[3];
+    hit_of(t.g->f, t.o0 + k, m, V);
+    const Innov q = innovation(xp, Cp, m, V);
+    o.yb[0] = o.yb[1] = o.G[0] = o.G[1] = o.G[2] = 0.0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) o.Z[j][0] = o.Z[j][1] = 0.0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      o.yb[0] = fma(hm[i][0], v[i], o.yb[0]);
+      o.yb[1] = fma(hm[i][1], v[i], o.yb[1]);
+      // row i of W h and of LS P
+      double a0 = 0.0, a1 = 0.0, q0 = 0.0, q1 = 0.0;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {
+        a0 = fma(W[sym(i, j)], hm[j][0], a0);
+        a1 = fma(W[sym(i, j)], hm[j][1], a1);
+      }
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        q0 = fma(LS[i][j], Cp[sym(j, 0)], q0);
+        q1 = fma(LS[i][j], Cp[sym(j, 1)], q1);
+        o.Z[j][0] = fma(LS[i][j], hm[i][0], o.Z[j][0]);
+        o.Z[j][1] = fma(LS[i][j], hm[i][1], o.Z[j][1]);
+      }
+      const double b0 = a0 + q0, b1 = a1 + q1;
+      o.G[0] = fma(-hm[i][0], b0, o.G[0]);
+      o.G[2] = fma(-hm[i][1], b1, o.G[2]);
+      o.G[1] = fma(-0.5, fma(hm[i][0], b1, hm[i][1] * b0), o.G[1]);
+      const double c0 = fma(2.0, a0, q0), c1 = fma(2.0, a1, q1);
+      // adjoint of h: v y^T - (2 W h + LS P) Si
+      LS[i][0] += fma(v[i], q.y[0], -fma(c0, q.Si[0], c1 * q.Si[1]));
+      LS[i][1] += fma(v[i], q.y[1], -fma(c0, q.Si[1], c1 * q.Si[2]));
+    }
+  }
+  // Sp = S F^T
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) o.lF[r][c] = 0.0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    double s[5], o5[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) s[c] = t.rec(k - 1, kRS + 5 * i + c);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) o.lF[r][c] = fma(LS[i][r], s[c], o.lF[r][c]);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      double q = c == 4 ? LS[i][4] : 0.0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) q = fma(LS[i][r], F[r][c], q);
+      o5[c] = q;
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) LS[i][c] = o5[c];
+  }
+}
+
+// The rest of the reverse of transition k: lf, Lf (adjoints of x_f,k and
+// C_f,k) become those of k-1; adj enters with what transition k+1 contributed
+// to the adjoint of surface k and leaves with what this one contributes to
+// that of k-1; ga receives surface k's alignment derivatives.
+template <bool BZ, bool SM>
+__device__ __forceinline__ void reverse_part(const TrackB<SM>& t, int k, double w, const StartB& st, const FwdB& f,
+                                             const Step* tape, const SmOut& sm, double lf[6], double Lf[21],
+                                             PlaneAdj& adj, double ga[6]) {
+  const FitParams& p = t.g->f;
+  const Surf sa = t.surf(k - 1), sb = t.surf(k);
+  if (!t.hole(k)) {
+    double m[2], V[3];
+    hit_of(p, t.o0 + k, m, V);
+    update_reverse<SM, 5>(innovation(f.xp, f.Cp, m, V), f.Cp, w, sm, lf, Lf);
+  }
+  // reverse of Cp = F C F^T + Q (and Sp = S F^T):
+  //   l_F = 2 Lp F C (+ LSp^T S), L_C = F^T Lp F
+  double lF[4][5];  // rows loc0, loc1, phi, theta
+  double LF[5][5];
+#pragma unroll
+  for (int a = 0; a < 5; ++a)
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      double q = c == 4 ? Lf[sym(a, 4)] : 0.0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) q = fma(Lf[sym(a, r)], f.F[r][c], q);
+      LF[a][c] = q;
+    }
+  {
+    double Cq[15];
+#pragma unroll
+    for (int e = 0; e < 15; ++e) Cq[e] = t.rec(k - 1, kRC + e);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        double q = 0.0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) q = fma(LF[r][j], Cq[sym(j, c)], q);
+        lF[r][c] = SM ? fma(2.0, q, sm.lF[r][c]) : 2.0 * q;
+      }
+  }
+  const double lqp = Lf[sy(2, 2)], lqt = Lf[sy(3, 3)];
+#pragma unroll
+  for (int a = 0; a < 5; ++a)
+#pragma unroll
+    for (int b = 0; b < 5; ++b)
+      if (b <= a) {
+        double q = a == 4 ? LF[4][b] : 0.0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) q = fma(f.F[r][a], LF[r][b], q);
+        Lf[sy(a, b)] = q;
+      }
+  double lx[5];
+  PlaneAdj na;
+  transport_reverse<BZ>(sa, sb, st.x01, st.r0, st.a0, st.lam, t.kB, t.nu2, p.mass, sb.xx0(), f.path, tape, f.o, f.gc,
+                        f.inv_nT, lf, [&](int r, int c) { return lF[r][c]; }, lqp, lqt, lx, na, adj);
+#pragma unroll
+  for (int e = 0; e < 5; ++e) lf[e] = lx[e];
+  if (t.g->grad_align) plane_gradient(t.g->dtab + (size_t)p.surface_id[t.o0 + k] * kDTab, adj, ga);
+  adj = na;
+}
+
+// weights of the smoothed state 0 (zero for a track without status ST_OK);
+// the weight of a packed element (i, j), i > j, of the covariance stands for
+// both C_ij and C_ji in the full-matrix convention: half each
+template <bool SM>
+__device__ __forceinline__ void smoother_weights(const GradParams& g, int tg, bool ok, double v[6], double W[21]) {
+  const size_t TG = (size_t)g.f.n_tracks_total;
+#pragma unroll
+  for (int e = 0; e < 6; ++e) v[e] = SM && g.dl_dparams && ok ? g.dl_dparams[e * TG + tg] : 0.0;
 #pragma unroll
   for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (j < 5) LS[i][j] = 0.0;
+    for (int j = 0; j < 6; ++j)
       if (j <= i) {
-        Lf[sy(i, j)] = 0.0;
-        // the weight of a packed element (i, j), i > j, stands for both C_ij
-        // and C_ji in the full-matrix convention: half each
-        const double q = SM && g.dl_dcov && status == ST_OK ? g.dl_dcov[sy(i, j) * TG + tg] : 0.0;
+        const double q = SM && g.dl_dcov && ok ? g.dl_dcov[sy(i, j) * TG + tg] : 0.0;
         W[sy(i, j)] = i == j ? q : 0.5 * q;
       }
-    }
-  PlaneAdj adj;  // of surface k: what the transition k -> k+1 contributed
+}
+
+// The reverse's own state, and its end: surface and update of state 0.
+struct RevB {
+  double lf[6], Lf[21];  // adjoints of x_f, C_f (packed, full-matrix convention)
+  PlaneAdj adj;
+  double w;
+};
+__device__ __forceinline__ void reverse_begin(const GradParams& g, int tg, bool in_range, RevB& b) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i) adj.c[i] = adj.u[i] = adj.v[i] = adj.n[i] = 0.0;
-  // in lock-step over the warp's longest track, so that the reduction of the
-  // alignment gradient sees whole warps
-  const int n_ok = status == ST_OK ? n : 0;
-  int nmax = n_ok;
+  for (int e = 0; e < 6; ++e) b.lf[e] = 0.0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-#pragma unroll 1
-  for (int k = nmax - 1; k >= 1; --k) {
-    const bool act = k < n_ok;
-    double ga[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    int sid = 0;
-    if (act) {
-      sid = p.surface_id[o0 + k];
-      const int sid_a = p.surface_id[o0 + k - 1];
-      const Surf sa{s_surf + sid_a * kSurfStride}, sb{s_surf + sid * kSurfStride};
-      const double x01[2] = {rec(k - 1, kRX + 0), rec(k - 1, kRX + 1)};
-      const double lam = rec(k - 1, kRX + 2);
-      const Angles a0 = {rec(k - 1, kRX + 3), rec(k - 1, kRX + 4), rec(k - 1, kRX + 5), rec(k - 1, kRX + 6)};
-      double r0[3];
+  for (int e = 0; e < 21; ++e) b.Lf[e] = 0.0;
 #pragma unroll
-      for (int e = 0; e < 3; ++e) r0[e] = fma(x01[0], sa.u(e), fma(x01[1], sa.v(e), sa.c(e)));
-      // the transport again, with its tape
-      Step tape[kMaxSteps];
-      Path path;
-      path_forward<BZ>(sb, r0, a0, lam, kB, nu2, p.h_max, p.n_iter, path, tape);
-      End o;
-      Cols64 gc;
-      {
-        const PathG<true>& q = path.w;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          o.r[i] = r0[i] + fma(q.len, path.T0[i], fma(q.rb, path.NT[i], q.rg * path.NNT[i]));
-          o.T[i] = path.T0[i] + fma(q.eb, path.NT[i], q.eg * path.NNT[i]);
-          gc.gr[i][2] = fma(q.drb, path.NT[i], q.drg * path.NNT[i]);
-          gc.gT[i][2] = fma(q.deb, path.NT[i], q.deg * path.NNT[i]);
-        }
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const double vc[3] = {c == 0 ? -path.T0[1] : a0.cp * a0.ct, c == 0 ? path.T0[0] : a0.sp * a0.ct,
-                                c == 0 ? 0.0 : -a0.st};
-          double Nv[3], NNv[3];
-          applyA<double, BZ>(kB, vc, Nv);
-          applyA<double, BZ>(kB, Nv, NNv);
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            gc.gr[i][c] = fma(q.len, vc[i], fma(q.rb, Nv[i], q.rg * NNv[i]));
-            gc.gT[i][c] = vc[i] + fma(q.eb, Nv[i], q.eg * NNv[i]);
-          }
-        }
-        o.g2 = fma(p.mass * p.mass * lam, lam, 1.0);
-        o.dtds = gc.gtl = 0.0;  // (no time row)
-      }
-      double inv_nT;
-      end_frame(sb, o, inv_nT);
-      Jac<double> J;
-      jacobian_columns<BZ, 31>(sa, sb, o, gc, lam, Bf, inv_nT, [&](int r, int c, double q) {
-        if (r < 4) J.f[r][c] = q;
-      });
-      const double xx0 = sb.xx0();
-      // reverse of the update at k
-      if (!p.is_hole[o0 + k]) {
-        double Cp[21];
-#pragma unroll
-        for (int e = 0; e < 15; ++e) Cp[e] = rec(k - 1, kRC + e);
-        cov_transport<5>(J, 1.0, Cp);
-        if (xx0 > 0.0) {
-          const double q = highland_sq(lam, o.g2, xx0, o.inv_cos);
-          Cp[sy(2, 2)] = fma(q, o.inv_st * o.inv_st, Cp[sy(2, 2)]);
-          Cp[sy(3, 3)] += q;
-        }
-        double hm[6][2];
-        if (SM) {
-#pragma unroll
-          for (int i = 0; i < 6; ++i) {
-            double h0 = 0.0, h1 = 0.0;
-#pragma unroll
-            for (int c = 0; c < 5; ++c) {
-              const double s = rec(k - 1, kRS + 5 * i + c);
-              h0 = fma(J.f[0][c], s, h0);
-              h1 = fma(J.f[1][c], s, h1);
-            }
-            hm[i][0] = h0;
-            hm[i][1] = h1;
-          }
-        }
-        const double d0 = o.r[0] - sb.c(0), d1 = o.r[1] - sb.c(1), d2 = o.r[2] - sb.c(2);
-        const double xp[2] = {fma(d0, sb.u(0), fma(d1, sb.u(1), d2 * sb.u(2))),
-                              fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)))};
-        double m[2], V[3];
-        hit_of(p, o0 + k, m, V);
-        update_reverse<SM, 5>(xp, Cp, m, V, w, hm, v, W, lf, Lf, LS);
-      }
-      // reverse of Cp = F C F^T + Q and Sp = S F^T:
-      //   l_F = 2 Lp F C + LSp^T S, L_C = F^T Lp F, LS = LSp F
-      double lF[4][5];  // rows loc0, loc1, phi, theta
-      {
-        double LF[5][5];
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-          for (int c = 0; c < 5; ++c) {
-            double q = c == 4 ? Lf[sym(a, 4)] : 0.0;
-#pragma unroll
-            for (int r = 0; r < 4; ++r) q = fma(Lf[sym(a, r)], J.f[r][c], q);
-            LF[a][c] = q;
-          }
-        {
-          double Cq[15];
-#pragma unroll
-          for (int e = 0; e < 15; ++e) Cq[e] = rec(k - 1, kRC + e);
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 5; ++c) {
-              double q = 0.0;
-#pragma unroll
-              for (int j = 0; j < 5; ++j) q = fma(LF[r][j], Cq[sym(j, c)], q);
-              lF[r][c] = 2.0 * q;
-            }
-        }
-        if (SM) {
-#pragma unroll
-          for (int i = 0; i < 6; ++i) {
-            double s[5], o5[5];
-#pragma unroll
-            for (int c = 0; c < 5; ++c) s[c] = rec(k - 1, kRS + 5 * i + c);
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-              for (int c = 0; c < 5; ++c) lF[r][c] = fma(LS[i][r], s[c], lF[r][c]);
-#pragma unroll
-            for (int c = 0; c < 5; ++c) {
-              double q = c == 4 ? LS[i][4] : 0.0;
-#pragma unroll
-              for (int r = 0; r < 4; ++r) q = fma(LS[i][r], J.f[r][c], q);
-              o5[c] = q;
-            }
-#pragma unroll
-            for (int c = 0; c < 5; ++c) LS[i][c] = o5[c];
-          }
-        }
-        const double lqp = Lf[sy(2, 2)], lqt = Lf[sy(3, 3)];
-        // L_C before the transport's reverse, which needs lqp, lqt only
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-          for (int b = 0; b < 5; ++b)
-            if (b <= a) {
-              double q = a == 4 ? LF[4][b] : 0.0;
-#pragma unroll
-              for (int r = 0; r < 4; ++r) q = fma(J.f[r][a], LF[r][b], q);
-              Lf[sy(a, b)] = q;
-            }
-        double lx[5];
-        PlaneAdj na;
-        transport_reverse<BZ>(sa, sb, x01, r0, a0, lam, kB, nu2, p.mass, xx0, path, tape, o, gc, inv_nT, lf,
-                              [&](int r, int c) { return lF[r][c]; }, lqp, lqt, lx, na, adj);
-#pragma unroll
-        for (int e = 0; e < 5; ++e) lf[e] = lx[e];
-        if (g.grad_align) plane_gradient(g.dtab + (size_t)sid * kDTab, adj, ga);
-        adj = na;
-      }
-    }
-    if (g.grad_align) add_align_grad(g.grad_align, p.n_surfaces, sid, ga, act);
-  }
-  // surface of state 0
+  for (int i = 0; i < 3; ++i) b.adj.c[i] = b.adj.u[i] = b.adj.v[i] = b.adj.n[i] = 0.0;
+  b.w = (g.dl_dchi2 && in_range) ? g.dl_dchi2[tg] : 1.0;
+}
+template <bool SM>
+__device__ __forceinline__ void reverse_end(const TrackB<SM>& t, bool in_range, int status, RevB& b,
+                                            const double LS[6][5]) {
+  const GradParams& g = *t.g;
+  const FitParams& p = g.f;
+  const size_t TG = (size_t)p.n_tracks_total;
   if (g.grad_align) {
-    const bool act = n_ok > 0;
-    const int sid = act ? p.surface_id[o0] : 0;
+    const bool act = status == ST_OK;
+    const int sid = act ? p.surface_id[t.o0] : 0;
     double ga[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (act) plane_gradient(g.dtab + (size_t)sid * kDTab, adj, ga);
+    if (act) plane_gradient(g.dtab + (size_t)sid * kDTab, b.adj, ga);
     add_align_grad(g.grad_align, p.n_surfaces, sid, ga, act);
   }
   // state 0: x_s0, P_0 and S start as the filtered state 0 (S = P_0 = C_f,0);
@@ -913,9 +1013,11 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
   // directly
   if (in_range && g.grad_seed) {
     if (status == ST_OK) {
+      double v[6], W[21];
+      smoother_weights<SM>(g, t.tg, true, v, W);
 #pragma unroll
-      for (int e = 0; e < 6; ++e) lf[e] += v[e];
-      if (!p.is_hole[o0]) {
+      for (int e = 0; e < 6; ++e) b.lf[e] += v[e];
+      if (!t.hole(0)) {
         if (SM)
 #pragma unroll
           for (int i = 0; i < 6; ++i)
@@ -923,20 +1025,196 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
             for (int j = 0; j <= i; ++j) {
               double q = j < 5 ? LS[i][j] : 0.0;
               if (i < 5) q += LS[j][i];
-              Lf[sy(i, j)] += fma(0.5, q, W[sy(i, j)]);
+              b.Lf[sy(i, j)] += fma(0.5, q, W[sy(i, j)]);
             }
         double m[2], V[3], xp0[2], Cp0[21];
-        hit_of(p, o0, m, V);
-        xp0[0] = p.seed_params[tg];
-        xp0[1] = p.seed_params[TG + tg];
+        hit_of(p, t.o0, m, V);
+        xp0[0] = p.seed_params[t.tg];
+        xp0[1] = p.seed_params[TG + t.tg];
 #pragma unroll
-        for (int e = 0; e < 21; ++e) Cp0[e] = p.seed_cov[e * TG + tg];
-        update_reverse<false, 6>(xp0, Cp0, m, V, w, nullptr, nullptr, nullptr, lf, Lf, LS);
+        for (int e = 0; e < 21; ++e) Cp0[e] = p.seed_cov[e * TG + t.tg];
+        SmOut none;
+        update_reverse<false, 6>(innovation(xp0, Cp0, m, V), Cp0, b.w, none, b.lf, b.Lf);
       }
     }
 #pragma unroll
-    for (int e = 0; e < 6; ++e) g.grad_seed[e * TG + tg] = status == ST_OK ? lf[e] : qnan();
+    for (int e = 0; e < 6; ++e) g.grad_seed[e * TG + t.tg] = status == ST_OK ? b.lf[e] : qnan();
   }
+}
+
+// states of a track that pass B reverses, and the most of a warp's tracks: the
+// warps step through them together, so that the reduction of the alignment
+// gradient sees whole warps
+__device__ __forceinline__ int states_of(const FitParams& p, int tg, int status, int& nmax) {
+  const int n = status == ST_OK ? (int)(p.offsets[tg + 1] - p.offsets[tg]) : 0;
+  nmax = n;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+  return n;
+}
+
+// Pass B of track slot tl (in_range: a track of the launch; status: of its
+// forward pass).  All 32 lanes of a warp call it together.
+template <bool BZ, bool SM>
+__device__ __forceinline__ void grad_reverse(const GradParams& g, const double* s_surf, int tl, bool in_range,
+                                             int status) {
+  const TrackB<SM> t(g, s_surf, tl, BZ);
+  RevB b;
+  reverse_begin(g, t.tg, in_range, b);
+  double LS[6][5], v[6], W[21];  // LS: adjoint of S of state k
+  smoother_weights<SM>(g, t.tg, status == ST_OK, v, W);
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = 0; j < 5; ++j) LS[i][j] = 0.0;
+  int nmax;
+  const int n = states_of(g.f, t.tg, status, nmax);
+#pragma unroll 1
+  for (int k = nmax - 1; k >= 1; --k) {
+    const bool act = k < n;
+    double ga[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (act) {
+      const StartB st = start_of(t, k);
+      Step tape[kMaxSteps];
+      FwdB f;
+      SmOut sm;
+      forward_part<BZ, SM>(t, k, st, f, tape);
+      if constexpr (SM) smoother_part(t, k, f.F, f.Cp, f.xp, f.hm, v, W, LS, sm);
+      reverse_part<BZ, SM>(t, k, b.w, st, f, tape, sm, b.lf, b.Lf, b.adj, ga);
+    }
+    if (g.grad_align) add_align_grad(g.grad_align, g.f.n_surfaces, act ? g.f.surface_id[t.o0 + k] : 0, ga, act);
+  }
+  reverse_end<SM>(t, in_range, status, b, LS);
+}
+
+// Pass B of 32 tracks by three warps in a pipeline (two without the
+// smoother's adjoint, which has no part in it then): at stage j warp 1 runs
+// transition j of the sweep again, warp 2 the smoother's part of transition
+// j - 1, and warp 0 the rest of the reverse of j - 2, each from what the
+// others left in shared memory; one barrier per stage.  Every value is
+// computed as in grad_reverse.
+constexpr int kPipeFwd = 92, kPipeHm = 12, kPipeTape = 13, kPipeSm = 35;
+constexpr int kPipeFields = 3 * (kPipeFwd + kPipeHm + kPipeTape) + 2 * kPipeSm + 30;
+template <bool BZ, bool SM, int w>
+__device__ __forceinline__ void grad_reverse_pipe(const GradParams& g, const double* s_surf, double* sh, int tl,
+                                                  bool in_range, int status) {
+  constexpr int kLag = SM ? 2 : 1, kThreads = SM ? 96 : 64;
+  constexpr int kSlot = kPipeFwd + kPipeHm + kPipeTape;
+  const int lane = threadIdx.x & 31;
+  auto sync = [] {
+    __syncwarp();
+    asm volatile("barrier.cta.sync 2, %0;" ::"n"(kThreads) : "memory");
+  };
+  const TrackB<SM> t(g, s_surf, tl, BZ);
+  double* slot[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) slot[i] = sh + (size_t)i * kSlot * 32 + lane;
+  double* sm_slot = sh + (size_t)3 * kSlot * 32 + lane;
+  double* s_LS = sm_slot + (size_t)2 * kPipeSm * 32;
+  RevB b;
+  double LS[6][5], v[6], W[21];
+  if (w == 0) reverse_begin(g, t.tg, in_range, b);
+  if (w == 2) {
+    smoother_weights<SM>(g, t.tg, status == ST_OK, v, W);
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+      for (int j = 0; j < 5; ++j) LS[i][j] = 0.0;
+  }
+  int nmax;
+  const int n = states_of(g.f, t.tg, status, nmax);
+  const int steps = nmax - 1;
+#pragma unroll 1
+  for (int j = 0; j < steps + kLag; ++j) {
+    const int mine = w == 1 ? j : w == 2 ? j - 1 : j - kLag;  // transition of the sweep
+    const int k = nmax - 1 - mine;
+    const bool go = mine >= 0 && mine < steps, act = go && k < n;
+    double* q = slot[0] + (size_t)(mine >= 0 ? mine % 3 : 0) * kSlot * 32;
+    double* qs = sm_slot + (size_t)(mine >= 0 ? mine & 1 : 0) * kPipeSm * 32;
+    if (w == 1 && act) {
+      const StartB st = start_of(t, k);
+      Step tape[kMaxSteps];
+      FwdB f;
+      forward_part<BZ, SM>(t, k, st, f, tape);
+      int e = 0;
+      visit<SM>(f, [&](double x) { q[(e++) * 32] = x; });
+      double* z = q + (size_t)(kPipeFwd + kPipeHm) * 32;
+      z[0] = (double)f.path.nsub;
+      z[32] = (double)f.path.n_steps;
+      if (f.path.n_steps == 2) {
+        const Step& s = tape[1];
+        z[2 * 32] = s.w.eb; z[3 * 32] = s.w.eg; z[4 * 32] = s.w.rb; z[5 * 32] = s.w.rg;
+        z[6 * 32] = s.w.deb; z[7 * 32] = s.w.deg; z[8 * 32] = s.w.drb; z[9 * 32] = s.w.drg;
+        z[10 * 32] = s.w.len; z[11 * 32] = s.s; z[12 * 32] = (double)s.m;
+      }
+    }
+    if constexpr (SM && w == 2) {
+      if (act) {
+        FwdB f;
+        SmOut o;
+        int e = 0;
+        visit<SM>(f, [&](double& x) { x = q[(e++) * 32]; });  // (what is not used is not loaded)
+        smoother_part(t, k, f.F, f.Cp, f.xp, f.hm, v, W, LS, o);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) qs[i * 32] = o.yb[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) qs[(2 + i) * 32] = o.G[i];
+#pragma unroll
+        for (int i = 0; i < 10; ++i) qs[(5 + i) * 32] = o.Z[i / 2][i % 2];
+#pragma unroll
+        for (int i = 0; i < 20; ++i) qs[(15 + i) * 32] = o.lF[i / 5][i % 5];
+      }
+    }
+    if (w == 0) {
+      double ga[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      if (act) {
+        const StartB st = start_of(t, k);
+        Step tape[kMaxSteps];
+        FwdB f;
+        SmOut sm;
+        int e = 0;
+        visit<SM>(f, [&](double& x) { x = q[(e++) * 32]; });
+        const double* z = q + (size_t)(kPipeFwd + kPipeHm) * 32;
+        f.path.nsub = (int)z[0];
+        f.path.n_steps = (int)z[32];
+        if (f.path.n_steps <= 2) {
+          tape[0].s = f.path.nsub == 1 ? f.path.s0 : f.path.s0 / f.path.nsub;
+          tape[0].m = 0;
+          Step& s = tape[1];
+          s.w.eb = z[2 * 32]; s.w.eg = z[3 * 32]; s.w.rb = z[4 * 32]; s.w.rg = z[5 * 32];
+          s.w.deb = z[6 * 32]; s.w.deg = z[7 * 32]; s.w.drb = z[8 * 32]; s.w.drg = z[9 * 32];
+          s.w.len = z[10 * 32]; s.s = z[11 * 32]; s.m = f.path.n_steps == 2 ? (int)z[12 * 32] : 0;
+        } else {
+          Path again;  // more steps: their records are not passed on
+          path_forward<BZ>(t.surf(k), st.r0, st.a0, st.lam, t.kB, t.nu2, g.f.h_max, g.f.n_iter, again, tape);
+        }
+        if (SM) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) sm.yb[i] = qs[i * 32];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) sm.G[i] = qs[(2 + i) * 32];
+#pragma unroll
+          for (int i = 0; i < 10; ++i) sm.Z[i / 2][i % 2] = qs[(5 + i) * 32];
+#pragma unroll
+          for (int i = 0; i < 20; ++i) sm.lF[i / 5][i % 5] = qs[(15 + i) * 32];
+        }
+        reverse_part<BZ, SM>(t, k, b.w, st, f, tape, sm, b.lf, b.Lf, b.adj, ga);
+      }
+      if (g.grad_align && go)
+        add_align_grad(g.grad_align, g.f.n_surfaces, act ? g.f.surface_id[t.o0 + k] : 0, ga, act);
+    }
+    sync();
+  }
+  if (SM) {
+    if (w == 2)
+#pragma unroll
+      for (int i = 0; i < 30; ++i) s_LS[i * 32] = LS[i / 5][i % 5];
+    sync();
+    if (w == 0)
+#pragma unroll
+      for (int i = 0; i < 30; ++i) LS[i / 5][i % 5] = s_LS[i * 32];
+  }
+  if (w == 0) reverse_end<SM>(t, in_range, status, b, LS);
 }
 
 // outputs of a track whose CTA's staging wait gave up: NaN, and nothing is
@@ -1011,10 +1289,11 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
 }
 
 // The same for batches that leave most sub-partitions idle: a CTA of 4 warps
-// per 32 tracks whose forward pass is the team fit's (kf_team.cuh: 0.57 of
-// one warp's time), then pass B in its first warp.  Up to one team per SM.
-// 2000 tracks x 21 states, forward and backward of the differentiable fit:
-// 3.57 -> 2.98 ms (2.66 ms without the time row).
+// per 32 tracks whose forward pass is the team fit's (kf_team.cuh: 0.6 of one
+// warp's time) and whose pass B is a pipeline over its warps.  Up to one team
+// per SM.  2000 tracks x 21 states, forward and backward of the
+// differentiable fit: 3.57 -> 2.98 ms with the team's forward pass (2.66
+// without the time row), 1.90 ms with the pipeline.
 template <bool BZ, bool SM>
 __global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1031,15 +1310,28 @@ __global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g
     return;
   }
   constexpr int REC = SM ? 2 : 1;
-  switch (threadIdx.x >> 5) {
-    case 1: fit_team<BZ, 4, 1, REC>(p, s_surf, sh, base, g.rec); return;
-    case 2: fit_team<BZ, 4, 2, REC>(p, s_surf, sh, base, g.rec); return;
-    case 3: fit_team<BZ, 4, 3, REC>(p, s_surf, sh, base, g.rec); return;
-    default: break;
+  __shared__ int s_status[32];
+  const int wid = threadIdx.x >> 5;
+  switch (wid) {
+    case 0: s_status[threadIdx.x] = fit_team<BZ, 4, 0, REC>(p, s_surf, sh, base, g.rec); break;
+    case 1: fit_team<BZ, 4, 1, REC>(p, s_surf, sh, base, g.rec); break;
+    case 2: fit_team<BZ, 4, 2, REC>(p, s_surf, sh, base, g.rec); break;
+    default: fit_team<BZ, 4, 3, REC>(p, s_surf, sh, base, g.rec); break;
   }
-  const int status = fit_team<BZ, 4, 0, REC>(p, s_surf, sh, base, g.rec);
-  __syncwarp();
-  if (g.grad_seed || g.grad_align) grad_reverse<BZ, SM>(g, s_surf, in_range ? i : 0, in_range, status);
+  if (!g.grad_seed && !g.grad_align) return;
+  __threadfence_block();
+  __syncthreads();  // the records and the verdicts; the exchange buffers are free
+  const int status = s_status[threadIdx.x & 31], tl = in_range ? i : 0;
+  if (wid == 0) grad_reverse_pipe<BZ, SM, 0>(g, s_surf, sh, tl, in_range, status);
+  if (wid == 1) grad_reverse_pipe<BZ, SM, 1>(g, s_surf, sh, tl, in_range, status);
+  if constexpr (SM)
+    if (wid == 2) grad_reverse_pipe<BZ, SM, 2>(g, s_surf, sh, tl, in_range, status);
+}
+
+// dynamic shared memory of one of its CTAs
+size_t grad_team_smem_bytes(int n_surfaces) {
+  static_assert(kPipeFields >= kShFields, "the exchange buffers are reused");
+  return ((size_t)n_surfaces * kSurfStride + (size_t)kPipeFields * 32) * sizeof(double);
 }
 
 template <int MINB, bool BZ, bool SM>
@@ -1075,7 +1367,7 @@ cudaError_t launch_grad_v(const GradParams& g, int block, cudaStream_t stream) {
 
 template <bool BZ, bool SM>
 cudaError_t launch_grad_team(const GradParams& g, cudaStream_t stream) {
-  const size_t smem = team_smem_bytes(g.f.n_surfaces);
+  const size_t smem = grad_team_smem_bytes(g.f.n_surfaces);
   auto kern = kf_grad_team_kernel<BZ, SM>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1131,7 +1423,7 @@ cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tab
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   if (block <= 0 && min_blocks <= 1 && f.n_tracks <= 32 * nsm &&
-      (long long)team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
+      (long long)grad_team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
     g.f.out_params = a.params;
     g.f.out_cov = a.cov;
     g.f.out_chi2 = a.chi2;
