@@ -163,8 +163,11 @@ __device__ __forceinline__ float d2f(double x) {
 // range: a float seed refined by Newton-Raphson steps in double,
 //   rsqrt: y <- y + y (1 - x y^2) / 2,   rcp: y <- y + y (1 - x y).
 // One step leaves a relative error below 1e-13 (the seed is accurate to a few
-// float ulps and each step squares the error); two steps reach double
-// rounding level.
+// float ulps and the step squares the error).  STEPS = 2 reaches double
+// rounding level: one step of third order (e + e^2, e/2 + 3 e^2/8), whose
+// error is that of the seed cubed, for one FP64 instruction less than two
+// steps of second order (FP64 fit of 100k tracks of 10 planes 5.43 -> 5.39 ms,
+// of 97 tracks 211 -> 207 us).
 // y / 2 for a positive normal double, by decrementing the exponent field on
 // the integer pipe
 __device__ __forceinline__ double half_pos(double y) {
@@ -173,13 +176,9 @@ __device__ __forceinline__ double half_pos(double y) {
 
 template <int STEPS>
 __device__ __forceinline__ double rsqrt_nr(double x) {
-  double y = f2d(rsqrtf(d2f(x)));
-#pragma unroll
-  for (int i = 0; i < STEPS; ++i) {
-    const double e = fma(-x * y, y, 1.0);
-    y = fma(half_pos(y), e, y);
-  }
-  return y;
+  const double y = f2d(rsqrtf(d2f(x)));
+  const double e = fma(-x * y, y, 1.0);
+  return STEPS == 1 ? fma(half_pos(y), e, y) : fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // x > 0 (false for NaN), decided on the integer pipe: positive doubles order
@@ -191,13 +190,9 @@ __device__ __forceinline__ bool dpos(double x) {
 
 template <int STEPS>
 __device__ __forceinline__ double rcp_nr(double x) {
-  double y = f2d(__frcp_rn(d2f(x)));
-#pragma unroll
-  for (int i = 0; i < STEPS; ++i) {
-    const double e = fma(-x, y, 1.0);
-    y = fma(y, e, y);
-  }
-  return y;
+  const double y = f2d(__frcp_rn(d2f(x)));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, STEPS == 1 ? e : fma(e, e, e), y);
 }
 
 __device__ __forceinline__ double qnan() { return __longlong_as_double(0x7ff8000000000000ULL); }
