@@ -160,8 +160,8 @@ typedef struct {
 } kf_material;
 
 typedef enum {
-  KF_SMOOTHER_RTS = 0,             /* Rauch-Tung-Striebel with the stored
-                                      Jacobians (Sect. 2) */
+  KF_SMOOTHER_RTS = 0,             /* the Rauch-Tung-Striebel estimate with the
+                                      filter's own Jacobians (Sect. 2) */
   KF_SMOOTHER_BACKWARD_FILTER = 1  /* a second Kalman filter run from the
                                       last state to the first with its own
                                       propagation, combined with the forward
@@ -432,7 +432,8 @@ const char* kf_last_cuda_error(void);
  * [1] double->float (round to nearest even), [2] 1/sqrt one step beyond 1e-13
  * relative, [3] 1/x one step beyond 1e-13, [4] two-step forms beyond 4 ulp,
  * [5] the full-range forms of the FP64 path (any normal double) beyond
- * 4 ulp.  All zero means the helpers behave as documented.  Synchronous. */
+ * 4 ulp, and its logarithm beyond 1.5e-14 |log m| (m the mantissa) plus
+ * rounding.  All zero means the helpers behave as documented.  Synchronous. */
 int kf_selftest(int64_t n_patterns, uint64_t* counts);
 
 /* Diagnostic: device self-check of the mixed path's double-float arithmetic

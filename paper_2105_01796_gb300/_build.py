@@ -12,7 +12,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkfgb.so")
 SOURCES = ["kf_kernels.cu", "kf_team.cu", "kf_mixed.cu", "kf_adjoint.cu", "kf_variants.cu", "kf_api.cu",
            "kf_static.cu"]
-HEADERS = ["kf_internal.h", "kf_device.cuh", "kf_fp64.cuh", "kf_transport.cuh", "kf_team.cuh", "kf_filter.cuh",
+HEADERS = ["kf_internal.h", "kf_device.cuh", "kf_fp64.cuh", "kf_transport.cuh", "kf_team.cuh", "kf_filter.cuh", "kf_df.cuh",
            os.path.join("..", "..", "include", "kf.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # per-file flags: the mixed kernel's FP32 divisions and square roots (step

@@ -35,9 +35,10 @@
 // smoother's reverse is a few products with S instead of a backward pass of
 // its own with its recomputations.  Against the stage-by-stage reverse with
 // checkpoints every 5 states and a separate smoother adjoint: chi2 gradient
-// of 100k tracks x 21 states 50.3 -> 10.8 ms (9.6 ms without the time row), fit
-// and whole gradient of 2000 tracks x 21 states 14.8 -> 3.57 ms (there two
-// warps shared 32 tracks).
+// of 100k tracks x 21 states 50.3 -> 10.8 ms (9.6 ms without the time row,
+// 9.4 ms with the cheaper logarithm), fit and whole gradient of 2000 tracks x
+// 21 states 14.8 -> 3.57 ms (there two warps shared 32 tracks; 1.89 ms with
+// the team kernel below).
 // Storing every filtered state (176 B, whole fit 416 B) costs 0.14 ms of
 // memory traffic on the 100k tracks; recomputing them took a quarter of the
 // kernel.
@@ -356,7 +357,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
   double isb = 0.0, tnb = 0.0;  // tnb: adjoint of ln |T|
   if (xx0 > 0.0) {
     const double eps = xx0 * fabs(o.inv_cos), a = 0.0136 * lam;
-    const double l = fma(0.038, log(eps * o.g2), 1.0), il = 0.076 * rcp_any(l);
+    const double l = fma(0.038, log_df(eps * o.g2), 1.0), il = 0.076 * rcp_any(l);
     const double q = a * a * o.g2 * eps * (l * l);
     const double qb = fma(lqp, is * is, lqt) * q;
     isb = 2.0 * lqp * q * is;

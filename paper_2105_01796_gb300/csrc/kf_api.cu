@@ -36,7 +36,7 @@ struct kf_handle {
   int64_t order_cap = 0;
   int32_t* hist = nullptr;
   int hist_cap = 0;
-  // adjoint checkpoints
+  // adjoint scratch: the surface tables and the filtered states
   double* ckpt = nullptr;
   size_t ckpt_bytes = 0;
   // autotuner cache: best launch options per batch shape

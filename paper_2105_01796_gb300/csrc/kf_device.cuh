@@ -166,7 +166,7 @@ __device__ __forceinline__ float d2f(double x) {
 // float ulps and the step squares the error).  STEPS = 2 reaches double
 // rounding level: one step of third order (e + e^2, e/2 + 3 e^2/8), whose
 // error is that of the seed cubed, for one FP64 instruction less than two
-// steps of second order (FP64 fit of 100k tracks of 10 planes 5.43 -> 5.39 ms,
+// steps of second order (FP64 fit of 100k tracks of 30 planes 5.43 -> 5.39 ms,
 // of 97 tracks 211 -> 207 us).
 // y / 2 for a positive normal double, by decrementing the exponent field on
 // the integer pipe

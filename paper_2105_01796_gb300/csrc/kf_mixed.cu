@@ -47,6 +47,7 @@
 #include <stdint.h>
 
 #include "kf_device.cuh"
+#include "kf_df.cuh"
 #include "kf_internal.h"
 
 namespace kfgb {
@@ -60,95 +61,6 @@ using namespace dev;
 constexpr int XP = 0;                                           // ws64 fields
 constexpr int FJ = 0, QPHI = 25, QTH = 26, DXF = 27, CPF = 33;  // ws32 fields
 
-// ---- double-float ("df") values: an unevaluated sum hi + lo of two floats
-// with |lo| <= ulp(hi) / 2, about 48 significant bits.  Error-free
-// transformations: Knuth's TwoSum, Dekker's Fast2Sum and the exact product
-// from one FMA; sums and products of df values as in Dekker (1971), dot
-// products as Dot2 of Ogita, Rump and Oishi (2005).  The _rn intrinsics keep
-// the compiler from contracting or reassociating these steps.
-struct DF {
-  float hi, lo;
-};
-__device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-// exact for |a| >= |b| or a = 0
-__device__ __forceinline__ DF fast_two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ DF two_prod(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-// x + f (the final TwoSum keeps the pair normalised under cancellation)
-__device__ __forceinline__ DF df_add_f(DF x, float f) {
-  const DF s = two_sum(x.hi, f);
-  return two_sum(s.hi, __fadd_rn(s.lo, x.lo));
-}
-// x + y, with the low parts summed exactly as well
-__device__ __forceinline__ DF df_add(DF x, DF y) {
-  const DF s = two_sum(x.hi, y.hi);
-  const DF t = two_sum(x.lo, y.lo);
-  const DF u = two_sum(s.hi, __fadd_rn(s.lo, t.hi));
-  return two_sum(u.hi, __fadd_rn(u.lo, t.lo));
-}
-__device__ __forceinline__ DF df_neg(DF x) { return {-x.hi, -x.lo}; }
-// x * y (the lo * lo term is below the pair's resolution)
-__device__ __forceinline__ DF df_mul(DF x, DF y) {
-  const DF p = two_prod(x.hi, y.hi);
-  return fast_two_sum(p.hi, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p.lo)));
-}
-// float value (hi + lo rounded)
-__device__ __forceinline__ float df_f(DF x) { return __fadd_rn(x.hi, x.lo); }
-// conversions: to FP64 exactly, from FP64 as the nearest float and the
-// nearest float to the rest
-__device__ __forceinline__ double df_to_d(DF x) { return f2d(x.hi) + f2d(x.lo); }
-__device__ __forceinline__ DF df_from_d(double v) {
-  const float h = d2f(v);
-  return {h, d2f(v - f2d(h))};
-}
-// from FP64 without an FP64 instruction: hi is the value cut to 24 bits, lo
-// the float of the 29 bits cut off (integer pipe), so hi + lo is within 2^-48
-// of the value; below 2^-96 the rest is dropped.  Zero, Inf and NaN as d2f.
-__device__ __forceinline__ DF df_cut(double v) {
-  const uint32_t w = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
-  const uint32_t ah = w & 0x7fffffffu, sg = w & 0x80000000u;
-  if (ah < 0x38100000u || ah >= 0x47e00000u) return {d2f(v), 0.0f};
-  const uint32_t r = __funnelshift_l(l, ah, 3) + 0x40000000u;  // see d2f
-  const float hi = __uint_as_float(r | sg);
-  const uint32_t e = r >> 23;  // biased exponent of hi
-  if (e < 31u) return {hi, 0.0f};
-  // rest = (l mod 2^29) 2^-29 ulp(hi), ulp(hi) = 2^(e - 150)
-  const float ulp = __uint_as_float(((e - 23u) << 23) | sg);
-  return fast_two_sum(hi, (float)(l & 0x1fffffffu) * 0x1p-29f * ulp);
-}
-// acc - a * b, the sum left unnormalised: a chain of these ends with df_norm
-__device__ __forceinline__ DF df_fnma_acc(DF acc, DF a, DF b) {
-  const DF p = two_prod(a.hi, b.hi);
-  const float c = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
-  const DF s = two_sum(acc.hi, -p.hi);
-  return {s.hi, __fadd_rn(s.lo, __fsub_rn(acc.lo, c))};
-}
-__device__ __forceinline__ DF df_norm(DF x) { return fast_two_sum(x.hi, x.lo); }
-__device__ __forceinline__ DF df_fnma(DF acc, DF a, DF b) { return df_norm(df_fnma_acc(acc, a, b)); }
-// x + a * b + f
-__device__ __forceinline__ DF df_muladd(DF x, DF a, DF b, float f) {
-  const DF p = two_prod(a.hi, b.hi);
-  const float c = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
-  const DF s = two_sum(x.hi, p.hi);
-  const DF t = two_sum(s.hi, f);
-  return two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(s.lo, __fadd_rn(x.lo, c))));
-}
-// 1 / x: a float reciprocal and one Newton step (relative error about 2^-44)
-__device__ __forceinline__ DF df_rcp(DF x) {
-  const float y = __frcp_rn(x.hi);
-  const DF p = two_prod(x.hi, y);
-  const float e = __fmaf_rn(-x.lo, y, __fsub_rn(__fsub_rn(1.0f, p.hi), p.lo));
-  return fast_two_sum(y, __fmul_rn(y, e));
-}
 // w . r - w0 for a vector w given as hi / lo float arrays and a df offset
 // w0: Dot2 (the products split exactly by FMA, the running sum by TwoSum,
 // every error term gathered in one float), as accurate as a dot product in

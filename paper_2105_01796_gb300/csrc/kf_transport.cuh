@@ -30,6 +30,7 @@
 #include <math.h>
 
 #include "kf_device.cuh"
+#include "kf_df.cuh"
 #include "kf_fp64.cuh"
 
 namespace kfgb {
@@ -417,7 +418,7 @@ __device__ __forceinline__ void jacobian_columns(const Surf& sa, const Surf& sb,
 // the width enters squared.
 __device__ __forceinline__ double highland_sq(double lam, double g2, double xx0, double inv_cos) {
   const double eps = xx0 * fabs(inv_cos);
-  const double a = 0.0136 * lam, l = fma(0.038, log(eps * g2), 1.0);
+  const double a = 0.0136 * lam, l = fma(0.038, log_df(eps * g2), 1.0);
   return a * a * g2 * eps * (l * l);
 }
 

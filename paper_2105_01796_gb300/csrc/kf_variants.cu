@@ -19,8 +19,8 @@
 // stay stage by stage; the corrections after the first are tiny and take
 // their leading terms.  The backward filter's weighted mean (a 6x6
 // factorisation and six solves) is formed on the states that are output.
-// 50k tracks of 21 states with energy loss 7.54 -> 2.48 ms; 30k tracks of 31
-// states with map, energy loss and backward filter 16.9 -> 11.0 ms (4540 FP64
+// 50k tracks of 21 states with energy loss 7.54 -> 2.31 ms; 30k tracks of 31
+// states with map, energy loss and backward filter 16.9 -> 10.6 ms (4540 FP64
 // instructions per state, the pipe all but fully busy in the sub-partitions
 // that the 938 warps' two rounds on 608 keep occupied).
 #include <cuda_runtime.h>
@@ -351,7 +351,7 @@ __device__ __forceinline__ double density_effect(const FitParams& p, double ln_b
   const double X = ln_bg * 0.4342944819032518277;
   const double cbar = p.mat[3], x0 = p.mat[4], x1 = p.mat[5], a = p.mat[6], k = p.mat[7], d0 = p.mat[8];
   if (X >= x1) return fma(2.0, ln_bg, -cbar);
-  if (X >= x0) return fma(2.0, ln_bg, -cbar) + a * exp(k * log(x1 - X));
+  if (X >= x0) return fma(2.0, ln_bg, -cbar) + a * exp(k * log_df(x1 - X));
   return d0 * pow(10.0, 2.0 * (X - x0));
 }
 
@@ -380,7 +380,7 @@ __device__ __forceinline__ int energy_loss(const FitParams& p, double& qop, doub
   const double q = 2.0 * kMe * bg2, iI = rcp_any(p.mat[1]);
   const double arg = (q * iI) * (q * iI) * rcp_any(wden);
   const double b2 = pm * iE * (pm * iE);
-  const double dedx = kBetheK * p.mat[0] * ib2 * (0.5 * log(arg) - b2 - 0.5 * density_effect(p, log(bg)));
+  const double dedx = kBetheK * p.mat[0] * ib2 * (0.5 * log_df(arg) - b2 - 0.5 * density_effect(p, log_df(bg)));
   const double dE = dedx * thick;
   const double E2 = dir > 0 ? E - dE : E + dE;
   if (!(E2 > mass)) return ST_NONFINITE;
