@@ -454,9 +454,9 @@ int enqueue_fit(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const 
   p.team_warps = opt.team_warps;
   const bool variants = wants_variants(opt.smoother, opt.energy_loss, fi->map);
   // (concurrent fits share the SMs: no launch of theirs has rounds of its own)
-  p.auto_team = !variants && !own_slice && opt.precision == KF_PRECISION_FP64 &&
-                shape_is_default(opt.schedule == KF_SCHEDULE_WAVES, opt.block, opt.min_blocks,
-                                 opt.resident_warps, opt.team_warps);
+  p.auto_shape = !own_slice && opt.precision == KF_PRECISION_FP64 &&
+                 shape_is_default(opt.schedule == KF_SCHEDULE_WAVES, opt.block, opt.min_blocks,
+                                  opt.resident_warps, opt.team_warps);
   if (variants) fill_variants(&p, fi, opt);
   int c = 0;
   for (int64_t t0 = t_begin; t0 < t_end; t0 += chunk, ++c) {

@@ -90,7 +90,7 @@ struct FitParams {
   int32_t resident_warps;  // persistent launch: warps per SM (0 = occupancy)
   int32_t waves;           // grid launch split into full waves + one spread wave (host side)
   int32_t team_warps;      // FP64 path: > 1 shares each track over that many warps (host side)
-  int32_t auto_team;       // FP64 path: teams for a last part-filled round (host side)
+  int32_t auto_shape;      // FP64 kernels: the launch shape is the library's choice (host side)
   // method variants (the FP64 variant kernel)
   int32_t smoother;        // 0 RTS, 1 backward filter + weighted mean
   int32_t energy_loss;     // 1: mean loss and straggling on q/p
@@ -102,6 +102,8 @@ struct FitParams {
   double map_inv_spacing[3];
   double map_off[3];       // -origin / spacing
   const double* map_b;     // null: the constant field bfield
+  // every track of the batch has max_states states
+  bool uniform() const { return (long long)n_tracks_total * max_states == (long long)n_states; }
 };
 
 // Record a failed CUDA call for kf_last_cuda_error() and map it to a
@@ -149,6 +151,46 @@ size_t team_smem_bytes(int n_surfaces);
 inline bool shape_is_default(bool waves, int block, int min_blocks, int resident_warps, int team_warps) {
   return !waves && (block == 0 || block == 128) && min_blocks == 0 && resident_warps == 0 &&
          team_warps == 0;
+}
+
+// How an FP64 batch of equally long tracks is spread when the launch shape is
+// left to the library: full waves of one CTA of `warps` warps per SM (255
+// registers leave room for 8), then one last wave of CTAs of `last` warps.
+// The FP64 pipe is the bound, yet a wave's time does not step with the warps
+// per sub-partition: in units of the time of 1 to 4 warps per SM (one per
+// sub-partition, 932 us at 31 states) 5 warps take 1.45, 6 1.53, 7 1.76 and 8
+// 2.0.  So a batch of 10.3 warps per SM, which took three rounds of 4 (two
+// CTAs per SM), takes a wave of 7 and one of 4: 2.76; 20.6 warps per SM take
+// three waves of 7: 5.28 instead of 5 rounds and a team's 0.62.  With teams
+// (kf_team.cu) a last wave of one or two warps per SM takes 0.62 or 0.74.
+// All tracks equally long is what the host can see (n_states = n_tracks x
+// max_states); uneven ones keep the work counter's order of smaller CTAs.
+struct WavePlan {
+  long long main = 0;  // 32-track units of the full waves
+  int warps = 0, last = 0;
+};
+inline WavePlan plan_waves(long long units, int nsm, bool teams) {
+  const double cost[9] = {0.0, teams ? 0.62 : 1.0, teams ? 0.74 : 1.0, 1.0, 1.0, 1.45, 1.53, 1.76, 2.0};
+  WavePlan best;
+  double best_cost = 1e300;
+  for (int w = 8; w >= 6; --w) {
+    const long long wave = (long long)w * nsm;
+    long long k = (units - 8LL * nsm + wave - 1) / wave;  // the last wave takes what is left
+    if (k < 0) k = 0;
+    for (; ; ++k) {
+      const long long rest = units - k * wave;
+      const int b = rest > 0 ? (int)((rest + nsm - 1) / nsm) : 0;
+      const double c = (double)k * cost[w] + cost[b];
+      if (c < best_cost - 1e-9) {
+        best_cost = c;
+        best.main = rest > 0 ? k * wave : units;
+        best.warps = w;
+        best.last = b;
+      }
+      if (rest <= 0) break;
+    }
+  }
+  return best;
 }
 
 // The FP64 kernel of the method variants (kf_variants.cu): backward-filter

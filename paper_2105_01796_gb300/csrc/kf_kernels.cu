@@ -17,8 +17,8 @@
 // smoother took 2370.  100k tracks of 31 states: 15.28 -> 6.47 ms with the
 // closed-form transport and the fixed-point smoother, 6.22 ms with teams for
 // the last round, 5.43 ms without the time row (kf_filter.cuh), 5.29 ms with
-// cheaper reciprocals and logarithms; 20k tracks of 24 tilted planes in a
-// general field with every smoothed state 3.56 -> 1.58 ms.
+// cheaper reciprocals and logarithms, 4.90 ms in waves of 7 warps per SM; 20k tracks of 24 tilted planes in a
+// general field with every smoothed state 3.56 -> 1.57 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -229,11 +229,13 @@ cudaError_t launch_fit_mixed(const FitParams& p, int block, int min_blocks, cuda
 
 namespace {
 
-// The FP64 fit with the launch shape left to the library.  A sub-partition's
-// FP64 pipe is busy with one warp, so a batch takes whole rounds of one warp
-// (32 tracks) per sub-partition, and a last round that fills few of them
-// takes as long as a full one.  Its tracks go to teams of warps instead
-// (kf_team.cu; the same results bit for bit): with U warp units left over
+// The FP64 fit with the launch shape left to the library.  Equally long tracks
+// run in waves of one CTA per SM (plan_waves; 100k tracks of 31 states 5.29 ->
+// 4.90 ms).  Else a sub-partition's FP64 pipe is busy with one warp, so a batch
+// takes rounds of one warp (32 tracks) per sub-partition, and a last round
+// that fills few of them takes as long as a full one.  The tracks of a last
+// round go to teams of warps instead (kf_team.cu; the same results bit for
+// bit): with U warp units left over
 // after the full rounds, teams of 4 while they fit one per SM (U <= SMs:
 // 0.60 to 0.64 of a round's time, measured 421-453 against 706 us at 20
 // planes), teams of 2 up to two per SM (0.72 to 0.75, 510-531 us), else the
@@ -249,10 +251,34 @@ cudaError_t launch_fp64_auto(const FitParams& p, int block, int min_blocks, bool
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   const long long units = ((long long)p.n_tracks + 31) / 32, round = 4LL * nsm;
-  const long long rest = units % round;
-  int team = rest == 0 ? 1 : rest <= nsm ? 4 : rest <= 2 * nsm ? 2 : 1;
-  if (team > 1 && (long long)team_smem_bytes(p.n_surfaces) + 1024 > smem_max) team = 1;
+  long long rest = units % round;
+  const bool teams = (long long)team_smem_bytes(p.n_surfaces) + 1024 <= smem_max;
+  int team = rest == 0 || !teams ? 1 : rest <= nsm ? 4 : rest <= 2 * nsm ? 2 : 1;
   FitParams a = p;
+  if (p.uniform() && !p.order) {
+    const WavePlan plan = plan_waves(units, nsm, teams);
+    rest = units - plan.main;
+    team = plan.last == 1 && teams ? 4 : plan.last == 2 && teams ? 2 : 1;
+    a.work_counter = nullptr;
+    block = 32 * plan.warps;
+    if (team == 1 && rest > 0) {
+      a.n_tracks = (int32_t)(plan.main * 32);
+      int l = 0;
+      if (a.n_tracks > 0) {
+        e = bz ? launch_fp64<true>(a, block, min_blocks, stream, &l)
+               : launch_fp64<false>(a, block, min_blocks, stream, &l);
+        if (e != cudaSuccess) return e;
+      }
+      if (launched) *launched = l;
+      a.track0 = p.track0 + a.n_tracks;
+      a.n_tracks = p.n_tracks - a.n_tracks;
+      block = 32 * plan.last;
+      e = bz ? launch_fp64<true>(a, block, min_blocks, stream, &l)
+             : launch_fp64<false>(a, block, min_blocks, stream, &l);
+      if (launched) *launched += l;
+      return e;
+    }
+  }
   if (team > 1) a.n_tracks = (int32_t)((units - rest) * 32);
   int l = 0, count = 0;
   if (a.n_tracks > 0) {
@@ -282,7 +308,7 @@ cudaError_t launch_fit(const FitParams& p, int precision, int block, int min_blo
   if (block <= 0) block = 128;
   const bool bz = p.bfield[0] == 0.0 && p.bfield[1] == 0.0;
   if (precision == 0 && p.team_warps > 1) return launch_fit_team(p, p.team_warps, stream, launched);
-  if (precision == 0 && p.auto_team) return launch_fp64_auto(p, block, min_blocks, bz, stream, launched);
+  if (precision == 0 && p.auto_shape) return launch_fp64_auto(p, block, min_blocks, bz, stream, launched);
   if (precision == 0) return bz ? launch_fp64<true>(p, block, min_blocks, stream, launched)
                                 : launch_fp64<false>(p, block, min_blocks, stream, launched);
   return launch_fit_mixed(p, block, min_blocks, stream, launched);

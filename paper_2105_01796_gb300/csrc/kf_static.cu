@@ -149,8 +149,8 @@ extern "C" int kf_fit_static(const kf_tracks* tr, const kf_surfaces* su, const k
   p.skip_stage_copy = opt.test_wait_timeout;
   // persistent launches share one work counter, re-zeroed before each chunk
   const bool persistent = opt.schedule != KF_SCHEDULE_GRID;
-  p.auto_team = opt.precision == KF_PRECISION_FP64 &&
-                shape_is_default(false, opt.block, opt.min_blocks, opt.resident_warps, opt.team_warps);
+  p.auto_shape = opt.precision == KF_PRECISION_FP64 &&
+                 shape_is_default(false, opt.block, opt.min_blocks, opt.resident_warps, opt.team_warps);
   for (size_t t0 = 0; t0 < (size_t)tr->n_tracks; t0 += chunk) {
     p.track0 = (int32_t)t0;
     p.n_tracks = (int32_t)(((size_t)tr->n_tracks - t0) < chunk ? ((size_t)tr->n_tracks - t0) : chunk);

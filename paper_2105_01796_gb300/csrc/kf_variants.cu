@@ -19,10 +19,9 @@
 // stay stage by stage; the corrections after the first are tiny and take
 // their leading terms.  The backward filter's weighted mean (a 6x6
 // factorisation and six solves) is formed on the states that are output.
-// 50k tracks of 21 states with energy loss 7.54 -> 2.31 ms; 30k tracks of 31
-// states with map, energy loss and backward filter 16.9 -> 10.6 ms (4540 FP64
-// instructions per state, the pipe all but fully busy in the sub-partitions
-// that the 938 warps' two rounds on 608 keep occupied).
+// 50k tracks of 21 states with energy loss 7.54 -> 2.17 ms; 30k tracks of 31
+// states with map, energy loss and backward filter 16.9 -> 9.58 ms (4290 FP64
+// instructions per state; the 938 warps run as one wave of 7 per SM).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -773,6 +772,31 @@ cudaError_t launch_fit_variants(const FitParams& p, int block, cudaStream_t stre
   if (launched) *launched = 0;
   if (p.n_tracks <= 0) return cudaSuccess;
   const int b = block ? block : 128;
+  if (p.auto_shape && p.uniform() && !p.order) {
+    // waves of one CTA per SM (plan_waves): 30k tracks with map, energy loss
+    // and backward filter 10.6 -> 9.58 ms, 50k with energy loss 2.31 -> 2.17 ms
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const WavePlan plan = plan_waves(((long long)p.n_tracks + 31) / 32, nsm, false);
+    FitParams a = p;
+    a.auto_shape = 0;
+    a.work_counter = nullptr;
+    int l = 0, count = 0;
+    if (plan.main > 0) {
+      const long long n = plan.main * 32;
+      a.n_tracks = (int32_t)(n < p.n_tracks ? n : p.n_tracks);
+      e = launch_fit_variants(a, 32 * plan.warps, stream, &l);
+      if (e != cudaSuccess) return e;
+      count = l;
+      a.track0 = p.track0 + a.n_tracks;
+      a.n_tracks = p.n_tracks - a.n_tracks;
+    }
+    e = launch_fit_variants(a, 32 * (plan.last > 0 ? plan.last : 1), stream, &l);
+    if (launched) *launched = count + l;
+    return e;
+  }
   if (p.map_b) return launch_mode<2>(p, b, stream, launched);
   if (p.bfield[0] == 0.0 && p.bfield[1] == 0.0) return launch_mode<0>(p, b, stream, launched);
   return launch_mode<1>(p, b, stream, launched);
