@@ -3,7 +3,7 @@
 Workload: 100,000 synthetic muon tracks through a telescope of 30 planes
 (25 mm spacing, 1 % X0 each), Bz = 2 T, p log-uniform 0.5-100 GeV, 30 um hits
 (one state on the reference plane plus 30 measured states per track).
-A step is one complete fit of the batch: forward filter + RTS smoother of
+A step is one complete fit of the batch: forward filter and smoother of
 every track.  Prints one JSON line (rank 0).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -37,36 +37,37 @@ SM_COUNT, SM_MAX_MHZ = 152, 2070.0
 FP64_PEAK_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12      # 1.259
 FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12    # 80.5
 
-# DRAM traffic of the mixed kernel (dram__bytes_read.sum + dram__bytes_write.sum)
-# from one ncu capture of both wave-split launches of a 100k-track, 3.1M-state
-# step of the same workload: launch A 442.7 + 356.2 MB, launch B 372.7 +
-# 309.2 MB.  Traffic grows in proportion to the states, so a launch's traffic
-# is this per-state figure times its states.  It holds only for the kernel
-# sources and build flags that were captured: any change to them makes the
-# figure null.
-MIXED_TRAFFIC_BYTES_PER_STATE = (442.68288e6 + 356.226304e6 + 372.705536e6 + 309.217792e6) / 3.1e6
-MIXED_TRAFFIC_SOURCES_SHA256 = "97aced5b5c14c3999e2f1739b2b6d73320a1d0671d27f427ceaa7a9bae368779"
-# the same for the FP64 path's kernel (one launch of the 100k-track step:
-# 2301.875 + 2223.671 MB)
-FP64_TRAFFIC_BYTES_PER_STATE = (2301.875e6 + 2223.671e6) / 3.1e6
-FP64_TRAFFIC_SOURCES_SHA256 = "021253bb834cb2d2d256b0a9917e45781ba32226a69ae9577eb6016de1512920"
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) and the flops the
+# hardware counted (2 x FMA + ADD + MUL thread instructions), per state, from
+# one ncu capture each: the mixed kernel's launch of a 100k-track, 3.1M-state
+# fit of the same workload, and the FP64 kernel's of its first 97 280 tracks
+# (3 015 680 states).  Both grow in proportion to the states.  They hold only
+# for the kernel sources and build flags that were captured: any change to them
+# makes the figures null.
+MIXED_TRAFFIC_BYTES_PER_STATE = (700.33e6 + 665.54e6) / 3.1e6
+MIXED_FLOPS_PER_STATE = (2 * 4189804071 + 5358001003 + 1848603186) / 3.1e6    # FP32
+MIXED_TRAFFIC_SOURCES_SHA256 = "d8c6abc03831e8bc3e9a52143ac687d07f35536d90eee69f32ac054619b64122"
+FP64_TRAFFIC_BYTES_PER_STATE = (161.02e6 + 12.50e6) / 3015680
+FP64_FLOPS_PER_STATE = (2 * 1830282709 + 70924384 + 730438129) / 3015680    # FP64
+FP64_TRAFFIC_SOURCES_SHA256 = "9def4ae28b9b04333262edb2678b912d8e1ae21f35c73a5c96614c18ed47ff27"
 
 
 # FP64 flops the hardware counted (ncu: 2 x DFMA + DADD + DMUL thread
-# instructions) per track in one 100k-track launch of the variant kernel
+# instructions) per track in one 30k-track launch of the variant kernel
 # (fringe30, 31 states, all three variants) and of the adjoint kernel
 # (align20, 21 states; the chi2 objective and the whole-fit objective);
 # reported while those kernels' sources match
-EXT_FLOPS_PER_TRACK = {"variants": (2 * 12582105289 + 2760501554 + 5733751583) / 1e5,
-                       "adjoint_chi2": (2 * 14277599975 + 1627200021 + 7860000013) / 1e5,
-                       "adjoint_whole": (2 * 27684800044 + 2716200085 + 11449099947) / 1e5}
-EXT_SOURCES_SHA256 = "3a16bfd21128941923a73fcc50dc8a0a20e200ebe1a9e8fd66701d3eb829c210"
+EXT_FLOPS_PER_TRACK = {"variants": (2 * 1998482340 + 463353310 + 886198499) / 3e4,
+                       "adjoint_chi2": (2 * 983610000 + 122860160 + 451470000) / 3e4,
+                       "adjoint_whole": (2 * 1482240000 + 126130080 + 492750000) / 3e4}
+EXT_SOURCES_SHA256 = "b0ee6640d6ec29f79cb8d89b60f4b8c28910eb1da23ff018769d18050bfaa075"
 
 
 def ext_kernel_sources_sha256():
     import hashlib
     h = hashlib.sha256()
-    for f in ("csrc/kf_variants.cu", "csrc/kf_adjoint.cu", "csrc/kf_fp64.cuh", "csrc/kf_device.cuh",
+    for f in ("csrc/kf_variants.cu", "csrc/kf_adjoint.cu", "csrc/kf_filter.cuh", "csrc/kf_transport.cuh",
+              "csrc/kf_fp64.cuh", "csrc/kf_team.cuh", "csrc/kf_df.cuh", "csrc/kf_device.cuh",
               "csrc/kf_internal.h", "_build.py"):
         with open(os.path.join(ROOT, "paper_2105_01796_gb300", f), "rb") as fh:
             h.update(fh.read())
@@ -82,7 +83,7 @@ def ext_roofline(kind, tracks, ms):
     achieved = flops / (ms / 1e3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS, "flops_per_launch": flops,
-            "flops_source": "hardware-counted FP64 flops (ncu) of a 100k-track launch, per track"}
+            "flops_source": "hardware-counted FP64 flops (ncu) of a 30k-track launch, per track"}
 
 
 def kernel_sources_sha256(files):
@@ -95,11 +96,13 @@ def kernel_sources_sha256(files):
 
 
 def mixed_kernel_sources_sha256():
-    return kernel_sources_sha256(("csrc/kf_mixed.cu", "csrc/kf_device.cuh", "csrc/kf_internal.h", "_build.py"))
+    return kernel_sources_sha256(("csrc/kf_mixed.cu", "csrc/kf_df.cuh", "csrc/kf_device.cuh", "csrc/kf_internal.h",
+                                  "_build.py"))
 
 
 def fp64_kernel_sources_sha256():
-    return kernel_sources_sha256(("csrc/kf_kernels.cu", "csrc/kf_transport.cuh", "csrc/kf_fp64.cuh",
+    return kernel_sources_sha256(("csrc/kf_kernels.cu", "csrc/kf_filter.cuh", "csrc/kf_transport.cuh",
+                                  "csrc/kf_fp64.cuh", "csrc/kf_team.cu", "csrc/kf_team.cuh", "csrc/kf_df.cuh",
                                   "csrc/kf_device.cuh", "csrc/kf_internal.h", "_build.py"))
 
 
@@ -470,15 +473,33 @@ CONFIGS = (("tel10_1k", "fp64", "all"), ("uneven30_1m", "mixed", "all"))
 
 
 def fit_roofline(roofline, offsets, is_hole, prec_id, ms, hbm):
-    """Roofline entry of a fit from the required flops of its own states."""
-    f64, f32 = roofline.batch_flops(offsets, is_hole, prec_id)
+    """Roofline entry of a fit: the flops the hardware counted per state of
+    the 100k-track fit (null once the kernel has changed) on the pipe that
+    carries them, FP32 for the mixed path.  The method's stage-by-stage count
+    stands beside it: the kernels reach the same result in fewer operations."""
+    mixed = prec_id == 1
+    captured = ((mixed_kernel_sources_sha256() == MIXED_TRAFFIC_SOURCES_SHA256) if mixed
+                else (fp64_kernel_sources_sha256() == FP64_TRAFFIC_SOURCES_SHA256))
+    states = int(np.asarray(offsets)[-1])
+    peak = FP32_PEAK_TFLOPS if mixed else FP64_PEAK_TFLOPS
+    t64, t32 = roofline.batch_flops(offsets, is_hole, prec_id)
     nbytes = roofline.algorithmic_bytes(offsets, is_hole)
-    achieved = f64 / (ms / 1e3) / 1e12
-    t_roof = max(f64 / (FP64_PEAK_TFLOPS * 1e12), f32 / (FP32_PEAK_TFLOPS * 1e12), nbytes / (hbm * 1e9))
-    return {"bound": "alu", "pipe": "fp64", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "peak_source": "derived: 152 SM x 2 DFMA/clk x 2070 MHz",
-            "fp64_flops_per_launch": f64, "fp32_flops_per_launch": f32, "algorithmic_bytes_per_launch": nbytes,
-            "t_roof_ms": 1e3 * t_roof, "roof_frac": 1e3 * t_roof / ms, "traffic": None}
+    out = {"bound": "alu", "pipe": "fp32" if mixed else "fp64", "achieved": None, "peak": peak, "unit": "TFLOP/s",
+           "frac": None,
+           "peak_source": "derived: 152 SM x %d FMA/clk x 2070 MHz" % (128 if mixed else 2),
+           "flops_per_launch": None, "traffic": None,
+           "flops_source": "hardware-counted flops (ncu) per state of the 100k-track fit" if captured
+           else "kernel changed since the last ncu capture",
+           "stage_by_stage_fp64_flops": t64, "stage_by_stage_fp32_flops": t32,
+           "algorithmic_bytes_per_launch": nbytes}
+    if captured:
+        flops = (MIXED_FLOPS_PER_STATE if mixed else FP64_FLOPS_PER_STATE) * states
+        achieved = flops / (ms / 1e3) / 1e12
+        t_roof = max(flops / (peak * 1e12), nbytes / (hbm * 1e9))
+        out.update(achieved=achieved, frac=achieved / peak, flops_per_launch=flops,
+                   traffic=(MIXED_TRAFFIC_BYTES_PER_STATE if mixed else FP64_TRAFFIC_BYTES_PER_STATE) * states,
+                   t_roof_ms=1e3 * t_roof, roof_frac=1e3 * t_roof / ms)
+    return out
 
 
 def time_config(h, kf, synth, roofline, torch, stream, l2_flush, steps, warmup, name, prec, hbm, rank):
@@ -741,14 +762,8 @@ def run_ours(args, rank, world, local):
             dist.destroy_process_group()
         return
 
-    f64, f32 = roofline.batch_flops(ev["offsets"], ev["is_hole"], prec_id[args.precision])
-    nbytes = roofline.algorithmic_bytes(ev["offsets"], ev["is_hole"])
-    kern_s = step_ms / 1e3
-    achieved = f64 / kern_s / 1e12
-    t_roof = max(f64 / (FP64_PEAK_TFLOPS * 1e12), f32 / (FP32_PEAK_TFLOPS * 1e12), nbytes / (hbm * 1e9))
-    traffic = None
-    if args.precision == "mixed" and mixed_kernel_sources_sha256() == MIXED_TRAFFIC_SOURCES_SHA256:
-        traffic = MIXED_TRAFFIC_BYTES_PER_STATE * M
+    head = fit_roofline(roofline, ev["offsets"], ev["is_hole"], prec_id[args.precision], step_ms, hbm)
+    head["kernel"] = "fit_kernel<MixedBody>" if args.precision == "mixed" else "fit_kernel<Fp64Body>"
     cpu = None
     acc = None
     if not args.no_cpu:
@@ -800,23 +815,10 @@ def run_ours(args, rank, world, local):
         "fp64_path" if args.precision == "mixed" else "mixed_path": {
             "value": world * T / (other_ms / 1e3), "ms_per_step": other_ms, "step_ms": step_stats(ms_other),
             "ok_tracks": int((st_other == 0).sum()),
-            "roofline": dict(fit_roofline(roofline, ev["offsets"], ev["is_hole"], prec_id[other], other_ms, hbm),
-                             traffic=(FP64_TRAFFIC_BYTES_PER_STATE * M
-                                      if other == "fp64" and fp64_kernel_sources_sha256() == FP64_TRAFFIC_SOURCES_SHA256
-                                      else None))},
+            "roofline": fit_roofline(roofline, ev["offsets"], ev["is_hole"], prec_id[other], other_ms, hbm)},
         "ok_tracks": int((st == 0).sum()),
         "launch_shape": tuned,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                     "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic,
-                     "kernel": "fit_kernel<MixedBody>" if args.precision == "mixed" else "fit_kernel<Fp64Body>",
-                     "pipe": "fp64",
-                     "peak_source": "derived: 152 SM x 2 DFMA/clk x 2070 MHz",
-                     "t_roof_ms": 1e3 * t_roof, "roof_frac": 1e3 * t_roof / step_ms,
-                     "fp64_flops_per_launch": f64, "fp32_flops_per_launch": f32,
-                     "algorithmic_bytes_per_launch": nbytes,
-                     "traffic_note": ("ncu capture of both launches of a 100k-track step of this kernel (wave split, 168 registers); "
-                                      "mostly the smoother's per-state record round trip (216 B each way)")
-                     if traffic else "kernel changed since the last ncu capture"},
+        "roofline": head,
         "cpu_baseline": cpu,
         "accuracy": acc,
         "scale": scale,
@@ -827,10 +829,10 @@ def run_ours(args, rank, world, local):
         "gpu_launches": launches,
         "clocks": clocks,
     }
-    if clocks and clocks.get("sm_mhz"):
+    if clocks and clocks.get("sm_mhz") and head["achieved"] is not None:
         # the same derived peak at the median SM clock sampled under load
-        pk = FP64_PEAK_TFLOPS * clocks["sm_mhz"] / 2070.0
-        line["roofline"].update(peak_at_sampled_clock=pk, frac_at_sampled_clock=achieved / pk)
+        pk = head["peak"] * clocks["sm_mhz"] / SM_MAX_MHZ
+        head.update(peak_at_sampled_clock=pk, frac_at_sampled_clock=head["achieved"] / pk)
     print(json.dumps(line), flush=True)
     if dist is not None:
         dist.destroy_process_group()

@@ -187,7 +187,10 @@ typedef struct {
                                   straight-line estimate, which the mixed
                                   path takes in FP32 (~1e-4 sigma from FP64);
                                   every end point is projected onto its plane */
-  int32_t block;               /* threads per CTA, a multiple of 32 (0 = 128):
+  int32_t block;               /* threads per CTA, a multiple of 32 (0 = 128;
+                                  an FP64 fit with every launch option at its
+                                  default and tracks of equal length takes
+                                  the size that fills the SMs best):
                                   up to 256, or 384 / 512 for the mixed
                                   path's min_blocks 3 / 4 variants */
   int64_t workspace_bytes;     /* cap on the handle's workspace (0 = 32 GiB);

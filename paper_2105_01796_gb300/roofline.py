@@ -1,10 +1,15 @@
 """Algorithmic work of the fit, for roofline accounting.
 
 Counts are floating-point operations (an FMA counts 2; a square root,
-reciprocal or transcendental call counts 1) of the arithmetic the method
-needs in the structure-exploiting form the kernels use: covariances stored
+reciprocal or transcendental call counts 1) of the method carried out step by
+step -- the RKN stages with their Jacobian columns, then the smoother's
+backward recursion -- in its structure-exploiting form: covariances stored
 as 21 values, H a projection onto (loc0, loc1), F with its trivial q/p row and
 time column, constant field along z, solves instead of explicit inverses.
+The kernels need fewer operations for the same fit (operators of a whole step
+in closed form, the smoother carried along with the filter) and the mixed
+kernel's double-precision part runs as pairs of floats, so these counts measure
+the method, not the kernels' load.
 
 Per track: n states, n-1 transitions (state k-1 -> k), m measured states and
 n-1 smoother steps.
