@@ -908,17 +908,19 @@ __device__ __forceinline__ void fit_one_mixed(const FitParams& p, const double* 
         // 90 FP64 instructions and 120 conversions per state.
         const DF S00 = df_add_f(df_cut(V0), Cpf[sy(0, 0)]), S01 = df_add_f(df_cut(V1), Cpf[sy(1, 0)]),
                  S11 = df_add_f(df_cut(V2), Cpf[sy(1, 1)]);
-        const DF det = df_fnma(df_mul(S00, S11), S01, S01);
-        if (!(det.hi > 0.0f) || !(S00.hi > 0.0f)) {
+        // S = L D L^T, L = (1, 0; l, 1): no product of two variances is formed,
+        // so that a hit with no information (1e20 in both coordinates, say)
+        // stays in the floats' range, as it did with the determinant in FP64
+        const DF is0 = df_rcp(S00), l = df_mul(S01, is0), d1 = df_fnma(S11, l, S01);
+        if (!(d1.hi > 0.0f) || !(S00.hi > 0.0f)) {
           status = ST_NON_SPD;
           break;
         }
-        const DF idet = df_rcp(det);
+        const DF id1 = df_rcp(d1);
         const DF r0 = df_add(df_cut(m0), df_neg(xp[0])), r1 = df_add(df_cut(m1), df_neg(xp[1]));
-        const DF u = df_fnma(df_mul(S11, r0), S01, r1), v = df_fnma(df_mul(S00, r1), S01, r0);
-        chi2sum = df_add(chi2sum, df_mul(df_add(df_mul(r0, u), df_mul(r1, v)), idet));
-        const float idf = df_f(idet);
-        const float i00 = df_f(S11) * idf, i01 = -df_f(S01) * idf, i11 = df_f(S00) * idf;
+        const DF q1 = df_fnma(r1, l, r0);
+        chi2sum = df_add(chi2sum, df_add(df_mul(r0, df_mul(r0, is0)), df_mul(q1, df_mul(q1, id1))));
+        const float lf = df_f(l), i11 = df_f(id1), i01 = -lf * i11, i00 = df_f(is0) - lf * i01;
         const float r0f = df_f(r0), r1f = df_f(r1);
         float Kf[6][2];
 #pragma unroll
