@@ -18,10 +18,12 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # per-file flags: the mixed kernel's FP32 divisions and square roots (step
 # lengths, Jacobian normalisations, angle increments) need no IEEE rounding;
 # its FP64 helpers use explicit intrinsics and are unaffected
-# the one-thread and the team kernel of the FP64 fit give the same bits: their
-# fused multiply-adds are written out, and the compiler contracts nothing more
+# the warps of a track team each compute the state on their own and must take
+# the same decisions, and the one-thread and the team kernels of the FP64 fit
+# and of the adjoint give the same bits: their fused multiply-adds are written
+# out, and the compiler contracts nothing more
 FILE_FLAGS = {"kf_mixed.cu": ["-prec-div=false", "-prec-sqrt=false"],
-              "kf_kernels.cu": ["-fmad=false"], "kf_team.cu": ["-fmad=false"]}
+              "kf_kernels.cu": ["-fmad=false"], "kf_team.cu": ["-fmad=false"], "kf_adjoint.cu": ["-fmad=false"]}
 
 
 def nvcc() -> str:

@@ -42,6 +42,9 @@
 // Storing every filtered state (176 B, whole fit 416 B) costs 0.14 ms of
 // memory traffic on the 100k tracks; recomputing them took a quarter of the
 // kernel.
+// The fused multiply-adds are written out and the compiler contracts nothing
+// more (as in kf_kernels.cu and kf_team.cu): the warps of a team agree, and
+// both kernels give the same bits and those of the FP64 fit.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -265,11 +268,17 @@ template <bool BZ>
 __device__ __forceinline__ void add_transposed(const double kB[3], const double y1[3], const double y2[3],
                                                double out[3]) {
   // out += N^T y1 + (N^2)^T y2 = -N (y1 - N y2)
+  if (BZ) {
+    const double z0 = fma(-y2[1], kB[2], y1[0]), z1 = fma(y2[0], kB[2], y1[1]);
+    out[0] = fma(-z1, kB[2], out[0]);
+    out[1] = fma(z0, kB[2], out[1]);
+    return;
+  }
   double z[3], q[3];
-  applyA<double, BZ>(kB, y2, z);
+  applyA<double, false>(kB, y2, z);
 #pragma unroll
   for (int i = 0; i < 3; ++i) z[i] = y1[i] - z[i];
-  applyA<double, BZ>(kB, z, q);
+  applyA<double, false>(kB, z, q);
 #pragma unroll
   for (int i = 0; i < 3; ++i) out[i] -= q[i];
 }
@@ -392,7 +401,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
     const double cpb = fma(fvb[1], is, hvb[0] * o.a.ct), spb = fma(-fvb[0], is, hvb[1] * o.a.ct);
     isb = fma(fvb[1], o.a.cp, fma(-fvb[0], o.a.sp, isb));
     const double ctb = fma(hvb[0], o.a.cp, hvb[1] * o.a.sp);
-    const double stb = -hvb[2] - isb * (is * is);
+    const double stb = fma(-isb, is * is, -hvb[2]);
     const double itn = fabs(o.inv_cos) > 0.0 ? inv_nT * rcp_any(o.inv_cos) : 0.0;  // 1 / |T|
     const double phib = (lxp[2] + fma(o.a.cp, spb, -o.a.sp * cpb)) * itn;
     const double thb = (lxp[3] + fma(o.a.ct, stb, -o.a.st * ctb)) * itn;
@@ -477,7 +486,7 @@ __device__ __forceinline__ void transport_reverse(const Surf& sa, const Surf& sb
       const double gg = fma(x, fma(x * (1.0 / 6.0), p2, c24 * p1), p0), gb = -dib * si;
       distb += dib;
       sbar = fma(-dib, gg, sbar);
-      p0b += gb + nTb2;
+      p0b += fma(-dib, si, nTb2);
       p1b = fma(gb, x * c24, fma(nTb2, x * t6, p1b));
       p2b = fma(gb, x * x * (1.0 / 6.0), fma(nTb2, x * x * c24, p2b));
       const double xb = fma(gb, fma(x * (1.0 / 3.0), p2, fma(y, -0.125, 0.5) * p1),
@@ -585,13 +594,18 @@ __device__ __forceinline__ void update_reverse(const Innov& q, const double Cp[2
   const double* Si = q.Si;
   const double* r = q.r;
   double Z[6][2], yb[2] = {0.0, 0.0};
-  double G00 = w * r[0] * r[0], G01 = w * r[0] * r[1], G11 = w * r[1] * r[1];
+  const double wr0 = w * r[0], wr1 = w * r[1];
+  double G00, G01, G11;
   if (SM) {
     yb[0] = sm.yb[0];
     yb[1] = sm.yb[1];
-    G00 += sm.G[0];
-    G01 += sm.G[1];
-    G11 += sm.G[2];
+    G00 = fma(wr0, r[0], sm.G[0]);
+    G01 = fma(wr0, r[1], sm.G[1]);
+    G11 = fma(wr1, r[1], sm.G[2]);
+  } else {
+    G00 = wr0 * r[0];
+    G01 = wr0 * r[1];
+    G11 = wr1 * r[1];
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -623,8 +637,8 @@ __device__ __forceinline__ void update_reverse(const Innov& q, const double Cp[2
   for (int i = 0; i < N; ++i) {
     const double P0 = fma(lf[i], q.y[0], -fma(Z[i][0], Si[0], Z[i][1] * Si[1]));
     const double P1 = fma(lf[i], q.y[1], -fma(Z[i][0], Si[1], Z[i][1] * Si[2]));
-    Lf[sym(i, 0)] += i == 0 ? P0 : 0.5 * P0;
-    Lf[sym(i, 1)] += i == 1 ? P1 : 0.5 * P1;
+    Lf[sym(i, 0)] = i == 0 ? Lf[sym(i, 0)] + P0 : fma(0.5, P0, Lf[sym(i, 0)]);
+    Lf[sym(i, 1)] = i == 1 ? Lf[sym(i, 1)] + P1 : fma(0.5, P1, Lf[sym(i, 1)]);
   }
   // adjoint of r: Si (yb + 2 w r)
   lf[0] -= fma(2.0 * w, q.y[0], fma(Si[0], yb[0], Si[1] * yb[1]));

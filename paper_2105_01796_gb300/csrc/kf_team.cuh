@@ -1,6 +1,10 @@
 // kf_team.cuh -- the FP64 fit of 32 tracks by a team of W warps (kf_team.cu
 // says why and how), shared by the team fit kernel and the adjoint's kernel
 // for small batches (kf_adjoint.cu), whose forward pass it is.
+// Each warp runs its own instance of this code on the state and takes the
+// discrete decisions (sub-steps, corrections, failures) by itself: the files
+// that include it are compiled with -fmad=false, so that every instance does
+// the same IEEE operations and all warps agree.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
