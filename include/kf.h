@@ -363,10 +363,11 @@ int kf_autotune(kf_handle* handle, const kf_tracks* tracks,
  *   grad_align[6][S]  dL/d align (optional); overwritten.
  * Method: reverse mode throughout: a forward pass that stores the filtered
  * states, then a reverse sweep over the states in which every transport is
- * run again and swept backwards.  Launch shape: one thread per track with
- * opt->block threads per CTA (a multiple of 32 up to 256; 0, and opt == NULL,
- * choose CTAs of the warp count that covers the batch in nearly full waves
- * of one CTA per SM); the other launch options do not apply.  Device pointers; asynchronous on `stream`.  Tracks that fail
+ * run again and swept backwards.  Launch shape: opt->team_warps as for
+ * kf_grad; one thread per track with opt->block threads per CTA (a multiple of
+ * 32 up to 256; 0, and opt == NULL, choose CTAs of the warp count that covers
+ * the batch in nearly full waves of one CTA per SM); the other launch options
+ * do not apply.  Device pointers; asynchronous on `stream`.  Tracks that fail
  * get NaN chi2 and gradients and do not contribute to grad_align. */
 int kf_chi2_grad(kf_handle* handle, const kf_tracks* tracks,
                  const kf_surfaces* surfaces, const double* align,
@@ -398,7 +399,7 @@ typedef struct {
  * filter step list and the smoother paragraph): the value and gradient of
  * L above with respect to the seed parameters and the per-surface alignment,
  * in FP64 whatever opt->precision says.  align as for kf_chi2_grad.
- * Method: reverse mode throughout, one thread per track.
+ * Method: reverse mode throughout.
  *   1. the forward filter with the smoothed state 0 carried along (the
  *      cross-covariance of state 0 and the current state); the filtered
  *      states, and with v or W those cross-covariances, are stored;
@@ -406,7 +407,14 @@ typedef struct {
  * Scratch per track: 176 B per state; charged with v or W 216 B per 5 states,
  * 216 B per 5 states and 216 B more, and 632 B per state; a batch whose
  * scratch exceeds opt->workspace_bytes (0: 32 GiB) runs as several launches.
- * opt->team_warps may be 0, 1 or 2 (no effect); others: KF_EUNSUPPORTED.
+ * Launch shape: opt->team_warps 1 = one thread per track (CTAs as for
+ * kf_chi2_grad); 2 = for batches too small to fill the GPU: four warps per 32
+ * tracks, which share the forward pass as a track team and run the reverse
+ * sweep as a pipeline (opt->block does not apply; the same results, up to the
+ * summation order of the alignment gradient; one thread per track above some
+ * 600 surfaces); 0 (the default, and opt == NULL) = the latter for up to 32
+ * tracks per SM when opt->block is 0, else one thread per track; others:
+ * KF_EUNSUPPORTED.
  * Failure behaviour as for kf_chi2_grad; a track whose smoother meets a
  * non-positive pivot gets NaN outputs and gradients.
  * Device pointers; asynchronous on `stream`. */

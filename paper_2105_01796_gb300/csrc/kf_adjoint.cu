@@ -1415,7 +1415,7 @@ size_t grad_scratch_doubles(int max_states, bool smoother_adjoint) {
 }
 
 cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tables, double* scratch, int block,
-                        int min_blocks, cudaStream_t stream) {
+                        int min_blocks, int team_warps, cudaStream_t stream) {
   GradParams g;
   g.f = f;
   g.f.surf = tables;
@@ -1430,15 +1430,18 @@ cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tab
   g.grad_align = a.grad_align;
   g.rec = scratch;
   const bool sm = (a.grad_seed || a.grad_align) && (a.dl_dparams || a.dl_dcov);
-  // a batch of at most one team per SM, with the launch shape left to the
-  // library (above that two teams would share an SM's pipes)
+  // teams where the caller asks for them, and for a batch of at most one team
+  // per SM with the launch shape left to the library (above that two teams
+  // would share an SM's pipes); one thread per track where a team's buffers do
+  // not fit beside the surface table (above some 600 surfaces)
   int dev = 0, nsm = 0, smem_max = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  if (block <= 0 && min_blocks <= 1 && f.n_tracks <= 32 * nsm &&
-      (long long)grad_team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
+  const bool team =
+      team_warps == 2 || (team_warps == 0 && block <= 0 && min_blocks <= 1 && f.n_tracks <= 32 * nsm);
+  if (team && (long long)grad_team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
     g.f.out_params = a.params;
     g.f.out_cov = a.cov;
     g.f.out_chi2 = a.chi2;

@@ -761,8 +761,10 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   // threads per CTA for min_blocks 1 / 3 / 4)
   const int grad_block = opt.block;
   if (grad_block < 0 || grad_block % 32 != 0 || grad_block > max_threads_of(opt.min_blocks)) return KF_EUNSUPPORTED;
-  // 0, 1 and 2 are accepted and run the same kernel
-  if (opt.team_warps != 0 && opt.team_warps != 1 && opt.team_warps != 2) return KF_EUNSUPPORTED;
+  // 1: one thread per track; 2: a team of warps per 32 tracks; 0: by the
+  // batch's size (launch_grad)
+  const int grad_team = opt.team_warps;
+  if (grad_team != 0 && grad_team != 1 && grad_team != 2) return KF_EUNSUPPORTED;
   opt.team_warps = 0;
   opt.block = 0;
   kf_outputs dummy;
@@ -851,7 +853,7 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
     p.track0 = (int32_t)t0;
     p.n_tracks = (int32_t)((tr->n_tracks - t0) < chunk ? (tr->n_tracks - t0) : chunk);
     e = launch_grad(p, a, (const double*)h->ckpt, (double*)((char*)h->ckpt + table_bytes), grad_block, opt.min_blocks,
-                    stream);
+                    grad_team, stream);
     if (e != cudaSuccess) return cuda_fail(e, "grad launch");
     ++launches;
   }

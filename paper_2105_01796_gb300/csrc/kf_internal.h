@@ -225,8 +225,10 @@ size_t grad_scratch_doubles(int max_states, bool smoother_adjoint);
 
 // One launch over tracks [f.track0, f.track0 + f.n_tracks) of
 // f.n_tracks_total; scratch holds grad_scratch_doubles(...) x f.n_tracks.
+// team_warps: 1 one thread per track, 2 a team of warps per 32 tracks (block
+// and min_blocks do not apply), 0 by the batch's size.
 cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tables, double* scratch, int block,
-                        int min_blocks, cudaStream_t stream);
+                        int min_blocks, int team_warps, cudaStream_t stream);
 
 // Counting sort of the tracks by state count, longest first:
 // order[0..n_tracks) receives track indices.  hist needs max_states + 2 ints.

@@ -49,3 +49,49 @@ def test_team_equals_one_thread(handle, field, h_max, n_iter, nonzero, objective
         for k in VALUES:
             assert np.array_equal(f[k][..., ok], team[k][..., ok]), k
             assert np.isnan(team[k][..., ~ok]).all(), k
+
+
+@pytest.mark.parametrize("objective", ["chi2", "whole"])
+def test_the_form_is_the_caller_s(handle, objective):  # noqa: F811
+    """team_warps 1 and 2 each start the form they name: on a batch that leaves
+    the GPU idle a team takes well under the time of one thread per track
+    (device times, best of ten), also with a block given; 0 starts the team
+    there, and one thread per track with a block given."""
+    import torch
+    ev = synth.make_event(synth.scaled(synth.WORKLOADS["align20_100k"], 320))
+    dev = kf.event_to_device(ev)
+    S = ev["center"].shape[1]
+    v, W = _smoother_weights(ev) if objective == "whole" else (None, None)
+    cu = lambda a: None if a is None else torch.from_numpy(a).cuda()  # noqa: E731
+    v, W = cu(v), cu(W)
+    gs = torch.empty((6, 320), dtype=torch.float64, device="cuda")
+    ga = torch.empty((6, S), dtype=torch.float64, device="cuda")
+
+    def best(**opt):
+        o, t = kf.kf_default_options(**opt), []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            kf.kf_grad(handle, dev, dl_dparams=v, dl_dcov=W, grad_seed=gs, grad_align=ga, opt=o)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t[2:])
+
+    one, team = best(block=0, team_warps=1), best(block=0, team_warps=2)
+    assert team < 0.8 * one, (team, one)
+    assert best(block=64, team_warps=2) < 0.8 * one
+    assert best(block=0) < 0.8 * one < best(block=64)
+
+
+def test_more_teams_than_sms(handle):  # noqa: F811
+    import torch
+    n = 32 * torch.cuda.get_device_properties(0).multi_processor_count + 33
+    ev = synth.make_event(synth.scaled(synth.WORKLOADS["tel10_1k"], n))
+    S = ev["center"].shape[1]
+    v, W = np.full((6, n), 0.5), np.full((21, n), 2.0)
+    one, team, auto = (_whole(handle, ev, np.zeros((6, S)), None, v, W,
+                              opt=kf.kf_default_options(block=0, team_warps=t)) for t in (1, 2, 0))
+    for k in VALUES + ("gs",):
+        assert np.array_equal(one[k], team[k]) and np.array_equal(one[k], auto[k]), k
+    assert np.allclose(team["ga"], one["ga"], rtol=1e-11, atol=1e-11 * np.abs(one["ga"]).max())
