@@ -442,9 +442,9 @@ const char* kf_last_cuda_error(void);
  * counts[6] (host memory) receives the mismatch counts: [0] float->double,
  * [1] double->float (round to nearest even), [2] 1/sqrt one step beyond 1e-13
  * relative, [3] 1/x one step beyond 1e-13, [4] two-step forms beyond 4 ulp,
- * [5] the full-range forms of the FP64 path (any normal double) beyond
- * 4 ulp, and its logarithm beyond 1.5e-14 |log m| (m the mantissa) plus
- * rounding.  All zero means the helpers behave as documented.  Synchronous. */
+ * [5] the full-range forms of the FP64 path (any normal double) and its
+ * logarithm beyond 4 ulp.  All zero means the helpers behave as documented.
+ * Synchronous. */
 int kf_selftest(int64_t n_patterns, uint64_t* counts);
 
 /* Diagnostic: device self-check of the mixed path's double-float arithmetic
