@@ -404,9 +404,11 @@ typedef struct {
  *      cross-covariance of state 0 and the current state); the filtered
  *      states, and with v or W those cross-covariances, are stored;
  *   2. the reverse sweep over the states.
- * Scratch per track: 176 B per state; charged with v or W 216 B per 5 states,
- * 216 B per 5 states and 216 B more, and 632 B per state; a batch whose
- * scratch exceeds opt->workspace_bytes (0: 32 GiB) runs as several launches.
+ * Scratch per track: 176 B per state, with v or W 416 B.  A batch that is
+ * charged more than opt->workspace_bytes (0: 32 GiB) runs as several launches.
+ * The charge per track is the 176 B per state; with v or W it is 632 B per
+ * state, 432 B for every 5 states begun and 216 B, so that a given cap splits
+ * a batch as it always has.
  * Launch shape: opt->team_warps 1 = one thread per track (CTAs as for
  * kf_chi2_grad); 2 = for batches too small to fill the GPU: four warps per 32
  * tracks, which share the forward pass as a track team and run the reverse

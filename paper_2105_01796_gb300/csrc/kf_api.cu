@@ -798,19 +798,18 @@ int kf_grad(kf_handle* h, const kf_tracks* tr, const kf_surfaces* su, const doub
   // as several launches over consecutive track ranges
   const bool want = a.grad_seed || a.grad_align;
   const bool sm_adj = want && (a.dl_dparams || a.dl_dcov);
-  // charged against the cap as the header documents it (at least what the
-  // kernel uses), so that a given cap splits a batch the same way always
+  // what the kernel uses, and what the header says a track is charged against
+  // the cap (more for the whole fit: callers' caps split their batches by it)
+  const size_t used = sizeof(double) * grad_scratch_doubles(tr->max_states, sm_adj);
   const size_t n_seg = ((size_t)tr->max_states + 4) / 5;
-  size_t per_track_d = sm_adj ? 27 * n_seg + 27 * (n_seg + 1) + 79 * (size_t)tr->max_states : 0;
-  if (per_track_d < grad_scratch_doubles(tr->max_states, sm_adj)) per_track_d = grad_scratch_doubles(tr->max_states, sm_adj);
-  const size_t per_track = sizeof(double) * per_track_d;
+  const size_t charged = sm_adj ? sizeof(double) * (27 * n_seg + 27 * (n_seg + 1) + 79 * (size_t)tr->max_states) : used;
   const int64_t cap = opt.workspace_bytes > 0 ? opt.workspace_bytes : kDefaultWorkspace;
-  int64_t chunk = cap / (int64_t)per_track;
+  int64_t chunk = cap / (int64_t)charged;
   if (chunk < 1) chunk = 1;
   if (chunk > tr->n_tracks) chunk = tr->n_tracks;
   // the surface tables ahead of the tracks' scratch
   const size_t table_bytes = align_up(sizeof(double) * grad_table_doubles(su->n_surfaces), 256);
-  const size_t need = table_bytes + per_track * (size_t)chunk;
+  const size_t need = table_bytes + used * (size_t)chunk;
   if (h->ckpt_bytes < need) {
     if (h->ckpt) cudaFree(h->ckpt);
     h->ckpt = nullptr;
