@@ -413,8 +413,7 @@ typedef struct {
  * kf_chi2_grad); 2 = for batches too small to fill the GPU: four warps per 32
  * tracks, which share the forward pass as a track team and run the reverse
  * sweep as a pipeline (opt->block does not apply; the same results, up to the
- * summation order of the alignment gradient; one thread per track above some
- * 600 surfaces); 0 (the default, and opt == NULL) = the latter for up to 32
+ * summation order of the alignment gradient); 0 (the default, and opt == NULL) = the latter for up to 32
  * tracks per SM when opt->block is 0, else one thread per track; others:
  * KF_EUNSUPPORTED.
  * Failure behaviour as for kf_chi2_grad; a track whose smoother meets a

@@ -1346,6 +1346,8 @@ __global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g
 // dynamic shared memory of one of its CTAs
 size_t grad_team_smem_bytes(int n_surfaces) {
   static_assert(kPipeFields >= kShFields, "the exchange buffers are reused");
+  static_assert((kMaxSurfaces * kSurfStride + kPipeFields * 32) * 8 + 1024 <= 227 * 1024,
+                "fits beside the largest surface table");
   return ((size_t)n_surfaces * kSurfStride + (size_t)kPipeFields * 32) * sizeof(double);
 }
 
@@ -1432,16 +1434,14 @@ cudaError_t launch_grad(const FitParams& f, const GradArgs& a, const double* tab
   const bool sm = (a.grad_seed || a.grad_align) && (a.dl_dparams || a.dl_dcov);
   // teams where the caller asks for them, and for a batch of at most one team
   // per SM with the launch shape left to the library (above that two teams
-  // would share an SM's pipes); one thread per track where a team's buffers do
-  // not fit beside the surface table (above some 600 surfaces)
-  int dev = 0, nsm = 0, smem_max = 0;
+  // would share an SM's pipes)
+  int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   const bool team =
       team_warps == 2 || (team_warps == 0 && block <= 0 && min_blocks <= 1 && f.n_tracks <= 32 * nsm);
-  if (team && (long long)grad_team_smem_bytes(f.n_surfaces) + 1024 <= smem_max) {
+  if (team) {
     g.f.out_params = a.params;
     g.f.out_cov = a.cov;
     g.f.out_chi2 = a.chi2;

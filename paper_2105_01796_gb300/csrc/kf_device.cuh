@@ -84,14 +84,6 @@ struct Surf {
   __device__ double v(int i) const { return R(i, 1); }
   __device__ double n(int i) const { return R(i, 2); }
   __device__ double xx0() const { return d[12]; }
-  __device__ double nc() const { return d[13]; }  // n . c
-  __device__ double uc() const { return d[14]; }  // u . c
-  __device__ double vc() const { return d[15]; }  // v . c
-  __device__ const float* f() const { return reinterpret_cast<const float*>(d + 16); }
-  __device__ float nf(int i) const { return f()[i]; }
-  __device__ float uf(int i) const { return f()[3 + i]; }
-  __device__ float vf(int i) const { return f()[6 + i]; }
-  __device__ float xx0f() const { return f()[9]; }
 };
 
 // out = v x bs, with bs = (q/p) kappa B: the operator A of dT/ds = A T

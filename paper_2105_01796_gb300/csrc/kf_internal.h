@@ -6,12 +6,9 @@
 
 namespace kfgb {
 
-// Packed surface record staged into shared memory: 24 doubles (192 B, a
+// Packed surface record staged into shared memory: 14 doubles (112 B, a
 // whole number of 16-byte units for the bulk copy):
-//   doubles [0..2] centre c, [3..11] R row-major (columns u, v, n), [12] x/X0,
-//           [13] n.c, [14] u.c, [15] v.c
-//   floats at double offset 16: [0..2] n, [3..5] u, [6..8] v, [9] x/X0
-//           (float copies)
+//   [0..2] centre c, [3..11] R row-major (columns u, v, n), [12] x/X0, [13] 0
 // The mixed kernel stages a table of its own, 32 floats (128 B) per surface,
 // packed after the FP64 table in the same buffer ([n_surfaces][kSurfStride]
 // doubles, then [n_surfaces][kSurfStrideM] doubles): every FP64 quantity as
@@ -21,10 +18,10 @@ namespace kfgb {
 //   [10..12] n lo, [13..15] u lo, [16..18] v lo,
 //   [19..21] (n.c, u.c, v.c) hi, [22..24] (n.c, u.c, v.c) lo,
 //   [25..27] c hi, [28..30] c lo, [31] 0
-constexpr int kSurfStride = 24;
+constexpr int kSurfStride = 14;
 constexpr int kSurfStrideM = 16;
 constexpr int kSurfPacked = kSurfStride + kSurfStrideM;  // doubles per surface in the packed buffer
-constexpr int kMaxSurfaces = 1024;  // 192 KiB of shared memory (FP64 table)
+constexpr int kMaxSurfaces = 1024;  // 112 KiB of shared memory (FP64 table), 128 KiB (mixed)
 
 // Per-state record the forward pass writes and the RTS pass reads back.
 // FP64 path, all in ws64: 90 doubles.  The fit itself writes none (its

@@ -133,17 +133,7 @@ __global__ void pack_surfaces_kernel(int n, const double* __restrict__ center, c
   for (int i = 0; i < 3; ++i) o[i] = center[(size_t)i * n + s];
   for (int i = 0; i < 9; ++i) o[3 + i] = rot[(size_t)i * n + s];
   o[12] = xx0[s];
-  // n.c, u.c, v.c (column j of R is o[3 + 3 i + j], i = 0..2)
-  for (int j = 0; j < 3; ++j) o[13 + (j + 1) % 3] = o[3 + j] * o[0] + o[6 + j] * o[1] + o[9 + j] * o[2];
-  // float copies of n, u, v and x/X0
-  float* f = reinterpret_cast<float*>(o + 16);
-  for (int i = 0; i < 3; ++i) {
-    f[i] = (float)o[3 + 3 * i + 2];
-    f[3 + i] = (float)o[3 + 3 * i + 0];
-    f[6 + i] = (float)o[3 + 3 * i + 1];
-  }
-  f[9] = (float)o[12];
-  for (int i = 10; i < 16; ++i) f[i] = 0.0f;
+  o[13] = 0.0;
   // the mixed kernel's table: each FP64 value v as hi = (float)v and
   // lo = (float)(v - hi)
   float* m = reinterpret_cast<float*>(out + (size_t)n * kSurfStride + (size_t)s * kSurfStrideM);
@@ -156,7 +146,8 @@ __global__ void pack_surfaces_kernel(int n, const double* __restrict__ center, c
     split(o[3 + 3 * i + 2], &m[i], &m[10 + i]);      // n
     split(o[3 + 3 * i + 0], &m[3 + i], &m[13 + i]);  // u
     split(o[3 + 3 * i + 1], &m[6 + i], &m[16 + i]);  // v
-    split(o[13 + i], &m[19 + i], &m[22 + i]);        // n.c, u.c, v.c
+    const int j = (i + 2) % 3;  // n.c, u.c, v.c: column j of R is o[3 + 3 k + j], k = 0..2
+    split(o[3 + j] * o[0] + o[6 + j] * o[1] + o[9 + j] * o[2], &m[19 + i], &m[22 + i]);
     split(o[i], &m[25 + i], &m[28 + i]);             // c
   }
   m[9] = (float)o[12];

@@ -95,3 +95,29 @@ def test_more_teams_than_sms(handle):  # noqa: F811
     for k in VALUES + ("gs",):
         assert np.array_equal(one[k], team[k]) and np.array_equal(one[k], auto[k]), k
     assert np.allclose(team["ga"], one["ga"], rtol=1e-11, atol=1e-11 * np.abs(one["ga"]).max())
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed", "grad"])
+def test_largest_surface_table(handle, prec):  # noqa: F811
+    """1024 surfaces, of which the tracks cross the last ones: the staged tables
+    at their largest, beside the teams' buffers."""
+    ev = dict(synth.make_event(synth.scaled(synth.WORKLOADS["tel10_1k"], 65)))
+    small = ev
+    S = ev["center"].shape[1]
+    pad = lambda a: np.concatenate([np.repeat(a[..., :1], 1024 - S, -1), a], -1)  # noqa: E731
+    ev = dict(ev, center=pad(ev["center"]), rot=pad(ev["rot"]), x_over_x0=pad(ev["x_over_x0"]),
+              surface_id=(ev["surface_id"] + (1024 - S)).astype(np.int32))
+    if prec == "grad":
+        v, W = np.full((6, 65), 0.5), np.full((21, 65), 2.0)
+        a, b = (_whole(handle, e, np.zeros((6, e["center"].shape[1])), None, v, W,
+                       opt=kf.kf_default_options(block=0, team_warps=t)) for e, t in ((small, 1), (ev, 2)))
+        for k in VALUES + ("gs",):
+            assert np.array_equal(a[k], b[k]), k
+        assert np.allclose(b["ga"][:, -S:], a["ga"], rtol=1e-12, atol=1e-12 * np.abs(a["ga"]).max())
+        assert not b["ga"][:, :-S].any()
+        return
+    from tests.test_gpu_parity import MIXED
+    for team in (1, 2, 4) if prec == "fp64" else (0,):
+        a, b = (gpu_fit(handle, e, FP64 if prec == "fp64" else MIXED, team_warps=team) for e in (small, ev))
+        for k in VALUES:
+            assert np.array_equal(a[k], b[k]), (team, k)
