@@ -106,16 +106,16 @@ static __device__ __noinline__ double log_call(double x) { return log(x); }
 // Natural logarithm of a positive normal double for 10 FP64 instructions where
 // the library's takes some 25: x = 2^e m with m in [0.7, 1.42),
 // z = (m - 1) / (m + 1),
-//   log m = 2 z + z w (2/3 + w (2/5 + ... + w (2/11 + w t(w)))),  w = z^2,
+//   log m = 2 z + z w (2/3 + w (2/5 + w (2/7 + w (2/9 + w t(w))))),  w = z^2,
 // the series of 2 atanh(z): z itself in FP64, the rest (at most 1 % of it) in
-// pairs of floats on the FP32 pipe and its last terms t (2/13 ... 2/21) in
+// pairs of floats on the FP32 pipe and its last terms t (2/11 ... 2/21) in
 // float; e ln 2 is added in FP64.  |z| <= 0.172: the terms left out are below
-// 1e-18 and t's rounding 1e-17 of log m; z's three roundings and the pairs'
-// (2^-46 of the 1 %) leave at most 5e-16 of the logarithm, with 2/9 and 2/11
-// in float as well 3.7e-15.  Those two levels cost the fit with energy loss
-// (three logarithms a state) 0.4 %, the others nothing.  Against the library's
-// function: FP64 fit of 100k tracks of 30 planes 5.39 -> 5.29 ms, energy loss
-// at 50k tracks 2.45 -> 2.31 ms.
+// 1e-18, t's rounding and that of w t 2e-16 of log m; z's three roundings and
+// the pairs' (2^-46 of the 1 %) bring it to at most 6e-16 of the logarithm.
+// With 2/9 in t as well it is 3.7e-15; with 2/11 a full pair too, 5e-16 for
+// 0.4 % of the fit with energy loss (three logarithms a state).  Against the
+// library's function: FP64 fit of 100k tracks of 30 planes 5.39 -> 5.29 ms,
+// energy loss at 50k tracks 2.45 -> 2.31 ms.
 __device__ __forceinline__ double log_df(double x) {
   const int h = __double2hiint(x);
   if (h < 0x00100000 || h >= 0x7ff00000) return log_call(x);
@@ -130,6 +130,7 @@ __device__ __forceinline__ double log_df(double x) {
   t = fmaf(f, t, 2.0f / 17.0f);
   t = fmaf(f, t, 2.0f / 15.0f);
   t = fmaf(f, t, 2.0f / 13.0f);
+  t = fmaf(f, t, 2.0f / 11.0f);
   // c + w * a with a constant pair c above the product
   auto level = [&](double c, DF a) {
     const float ch = (float)c, cl = (float)(c - (double)(float)c);
@@ -137,8 +138,10 @@ __device__ __forceinline__ double log_df(double x) {
     const DF s = fast_two_sum(ch, b.hi);
     return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(b.lo, cl)));
   };
-  DF a = level(2.0 / 11.0, DF{t, 0.0f});
-  a = level(2.0 / 9.0, a);
+  // 2/9 + w t: the product's rounding is 1e-9 of the sum
+  constexpr float c9 = (float)(2.0 / 9.0), c9l = (float)(2.0 / 9.0 - (double)c9);
+  DF a = fast_two_sum(c9, __fmul_rn(f, t));
+  a.lo = __fadd_rn(a.lo, c9l);
   a = level(2.0 / 7.0, a);
   a = level(2.0 / 5.0, a);
   a = level(2.0 / 3.0, a);
