@@ -21,7 +21,7 @@
  * Memory: every array pointer passed to kf_fit / kf_fit_ex is a DEVICE pointer
  * on the current CUDA device, owned by the caller; kf_fit_host takes HOST
  * pointers.  The library never frees caller memory.  A kf_handle owns its
- * workspace (the per-state record the smoother reads back) and staging
+ * workspace (per-state records, the gradients' scratch) and staging
  * buffers.
  *
  * Layouts (structure of arrays; T tracks, S surfaces, M states in total):
@@ -89,16 +89,23 @@ typedef enum {
 } kf_track_status;
 
 typedef enum {
-  KF_PRECISION_FP64 = 0, /* every step in double precision */
+  KF_PRECISION_FP64 = 0, /* every step in double precision; the logarithm of
+                            the scattering width and of the energy loss by a
+                            series whose small terms are pairs of floats (4
+                            ulp, see kf_selftest); whether a prediction is
+                            positive definite by a float factorisation where
+                            that proves it, else by the double one */
   KF_PRECISION_MIXED = 1 /* propagation, Jacobians, covariance transport and
-                            gain in float; Joseph covariance update (its
+                            gain in float; in pairs of floats (hi + lo, about
+                            48 bits, reciprocals to 2^-44): the track state
+                            between surfaces, the innovation and its LDL^T,
+                            chi2, the Joseph covariance update (its
                             second-order term K W, O(eps_float |Cp|), in
-                            float), chi2 and the smoother's inverse in
-                            double (the two columns of the inverse the
-                            smoother needs, by a 4x4 LDL^T of the non-angle
-                            block and the 2x2 Schur complement of the angle
-                            block); the track state between surfaces as
-                            double-float pairs (about 48 bits) */
+                            float) and the smoother's inverse (the two
+                            columns of it that the smoother needs, by a 4x4
+                            LDL^T of the non-angle block and the 2x2 Schur
+                            complement of the angle block); the update of a
+                            measured state 0 in double */
 } kf_precision;
 
 typedef struct {
@@ -233,7 +240,11 @@ typedef struct {
                                   but the schedule at their defaults (and a
                                   schedule other than waves) a last round
                                   that would fill at most half of the GPU
-                                  goes to teams; the same bits) */
+                                  goes to teams; the same bits.  Teams spend
+                                  twice the FP64 work of one thread per track
+                                  for a shorter latency: where fits on several
+                                  streams fill the GPU, 1 gives up to twice
+                                  the rate) */
   int32_t test_wait_timeout;   /* diagnostic of the timeout path (0 = off):
                                   1 announces the surface table's copy on
                                   each CTA's barrier without issuing it, so
@@ -313,8 +324,9 @@ int kf_fit_host(kf_handle* handle, const kf_tracks* tracks,
  * counterpart; it is an addition of this library.)
  * Scratch space is one fixed 64 MiB block of device memory per GPU, reserved
  * for the whole life of the process once the library is loaded.  It holds
- * the packed surface table (up to 1024 surfaces) and the per-state records;
- * larger batches run as several launches on `stream`.  Returns KF_ESIZE when
+ * the packed surface table (up to 1024 surfaces) and the per-state records
+ * (charged in full, also where a fit writes none); larger batches run as
+ * several launches on `stream`.  Returns KF_ESIZE when
  * n_surfaces > 1024 or when one track's records (max_states x 720 B in FP64,
  * max_states x 264 B in mixed precision) do not fit the block, and
  * KF_EUNSUPPORTED for schedules other than GRID and PERSISTENT and for the

@@ -15,7 +15,7 @@ namespace dev {
 
 // 1/sqrt(x) (x > 0) and 1/x (x != 0) for the whole double range: the
 // argument is scaled by a power of two into [1, 4) (resp. [1, 2)) on the
-// integer pipe, the two-step Newton form runs there, and the result is
+// integer pipe, the third-order Newton form runs there, and the result is
 // scaled back.  Arguments with extreme exponents (zero, subnormal, Inf, NaN)
 // take CUDA's double operations, so NaN and Inf propagate as usual.
 __device__ __forceinline__ double rsqrt_any(double x) {
@@ -268,9 +268,10 @@ __device__ __forceinline__ bool time_is_settled(const double C[21]) {
 // per state where the backward recursion with stored Jacobians (a Cholesky
 // factorisation, six pairs of triangular solves and A (Cs' - Cp') A^T) takes
 // 735, needs no inverse of Cp, and no record of the forward pass is written
-// to memory (720 B per state before).  Against an 80-bit evaluation of the
-// whole fit (ten shapes of 2000 tracks) the errors of parameters, covariances
-// and chi2 are 0.2 to 0.7 of those of the backward recursion it replaced.
+// to memory (720 B per state before).  Against an evaluation of the whole fit
+// in 80 bits (27 shapes of 1000 tracks over 5 to 30 planes) the rms errors of
+// parameters, covariances and chi2 are 0.10 to 0.32, 0.29 to 0.62 and 0.41 to
+// 0.89 of those of the backward recursion in plain double precision.
 // ---------------------------------------------------------------------------
 
 // row (v0..v4) -> row F^T over the columns 0..4, with F row 4 = g e4

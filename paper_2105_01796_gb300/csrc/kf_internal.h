@@ -23,7 +23,7 @@ constexpr int kSurfStrideM = 16;
 constexpr int kSurfPacked = kSurfStride + kSurfStrideM;  // doubles per surface in the packed buffer
 constexpr int kMaxSurfaces = 1024;  // 112 KiB of shared memory (FP64 table), 128 KiB (mixed)
 
-// Per-state record the forward pass writes and the RTS pass reads back.
+// Per-state record of a fit's workspace.
 // FP64 path, all in ws64: 90 doubles.  The fit itself writes none (its
 //   smoother runs along with the filter); with smoothed states wanted, what
 //   their backward pass reads (StateRec, kf_fp64.cuh).  The method variants
@@ -139,8 +139,6 @@ cudaError_t launch_fit(const FitParams& p, int precision, int block, int min_blo
 // The FP64 fit with each track's work shared by a team of 2 or 4 warps
 // (kf_team.cu): one CTA per 32 tracks, grid schedule.
 cudaError_t launch_fit_team(const FitParams& p, int team_warps, cudaStream_t stream, int* launched = nullptr);
-// dynamic shared memory of one of its CTAs
-size_t team_smem_bytes(int n_surfaces);
 
 // Whether the options leave the FP64 fit's launch shape to the library (every
 // launch option but the schedule at its default; the wave-split schedule
@@ -162,6 +160,11 @@ inline bool shape_is_default(bool waves, int block, int min_blocks, int resident
 // (kf_team.cu) a last wave of one or two warps per SM takes 0.62 or 0.74.
 // All tracks equally long is what the host can see (n_states = n_tracks x
 // max_states); uneven ones keep the work counter's order of smaller CTAs.
+// The costs are the FP64 kernel's with the field along z.  The other kernels
+// that follow them (a general field, every state output, the method variants
+// with and without a map: ten kinds, 1 to 20.6 warps per SM, 15 planes) take
+// 0.64 to 1.00 of the persistent grid's time, 1.02 to 1.03 (0.82 with a map)
+// at 12 warps per SM, where three even rounds leave nothing to gain.
 struct WavePlan {
   long long main = 0;  // 32-track units of the full waves
   int warps = 0, last = 0;

@@ -235,20 +235,18 @@ namespace {
 // states: 2.07-2.41 ms by the luck of the placement, 1.58-1.64 ms with them).
 cudaError_t launch_fp64_auto(const FitParams& p, int block, int min_blocks, bool bz, cudaStream_t stream,
                              int* launched) {
-  int dev = 0, nsm = 0, smem_max = 0;
+  int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   const long long units = ((long long)p.n_tracks + 31) / 32, round = 4LL * nsm;
   long long rest = units % round;
-  const bool teams = (long long)team_smem_bytes(p.n_surfaces) + 1024 <= smem_max;
-  int team = rest == 0 || !teams ? 1 : rest <= nsm ? 4 : rest <= 2 * nsm ? 2 : 1;
+  int team = rest == 0 ? 1 : rest <= nsm ? 4 : rest <= 2 * nsm ? 2 : 1;
   FitParams a = p;
   if (p.uniform() && !p.order) {
-    const WavePlan plan = plan_waves(units, nsm, teams);
+    const WavePlan plan = plan_waves(units, nsm, true);
     rest = units - plan.main;
-    team = plan.last == 1 && teams ? 4 : plan.last == 2 && teams ? 2 : 1;
+    team = plan.last == 1 ? 4 : plan.last == 2 ? 2 : 1;
     a.work_counter = nullptr;
     block = 32 * plan.warps;
     if (team == 1 && rest > 0) {

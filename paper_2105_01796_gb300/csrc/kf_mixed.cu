@@ -19,11 +19,12 @@
 //     left to launches that output every state, sums of products normalised
 //     once and the first state ahead of the loop; 1M uneven tracks 8.41 ->
 //     5.14 ms, one event of 3001 tracks 0.209 -> 0.121 ms.
-//     Against an 80-bit evaluation of the fit the rms errors are the same
-//     (0.9 to 1.04 times the former; ten shapes of 2000 tracks): the float
-//     quantities set them.  What bounds it now is issue: 4950 instructions per
-//     state and warp, 59 % of the issue slots used, the rest waits for the
-//     records and for dependent results (counted before the last of these).
+//     Against an evaluation of the fit in 80 bits the rms errors are the same
+//     (0.92 to 1.00 times the former for parameters, 0.96 to 1.02 for
+//     covariances, 0.96 to 1.05 for chi2; 24 shapes of 1000 tracks): the float
+//     quantities set them.  What bounds it now is issue: 4666 instructions
+//     per state and warp, 56 % of the issue slots used, the rest waits for
+//     the records and for dependent results.
 //   * FP64 only for the seed: its direction's sines and cosines, and the
 //     update of state 0 where that is measured.
 //   * float<->double conversions run on the integer pipe (dev::f2d/d2f,

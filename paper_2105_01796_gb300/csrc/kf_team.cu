@@ -7,26 +7,32 @@
 // cycles per DFMA warp instruction with 32, 16, 8, 4, 2 or 1 active lanes),
 // and one warp of the one-thread-per-track kernel keeps that pipe busy on its
 // own: a batch of fewer tracks than sub-partitions x 32 runs at one warp's
-// FP64 instruction count per state (about 2400).  Splitting a track over the
+// FP64 instruction count per state (887).  Splitting a track over the
 // lanes of one warp cannot shorten that; splitting it over W warps, each on
 // its own sub-partition, can.
 //
 // Lane l of each of a CTA's W warps works on track l of the CTA's 32.  The
-// warps all propagate the state (point, direction, time) and take the same
-// discrete decisions; they split
+// warps all propagate the state (point, direction) and take the same discrete
+// decisions; they split
 //   * the columns of F (the q/p column's derivatives along the path, the path
 //     correction and the free -> bound projection),
 //   * F C and F C F^T, the Joseph update (by row of C),
 //   * the fixed-point smoother (by row of S = Cov(x_0, x_k): every warp keeps
 //     its rows of S and P_0 in registers, they are never exchanged),
 // and exchange F, Cp, Cf and a few scalars through shared memory, three
-// barriers per state and no second pass.  The 32 tracks of a CTA step through
-// the states in lockstep (a track with fewer states, or one that failed,
-// idles at its barriers).  The arithmetic of every element is that of the
-// one-thread-per-track FP64 kernel (kf_kernels.cu), bit for bit: the shared
-// functions write their fused multiply-adds out.  1000 tracks of 11 states,
-// 4 warps: 0.535 ms with the backward smoother as a second pass of two
-// barriers per state, 0.213 ms now.
+// barriers per state and no second pass.  A team spends 1672 FP64 instructions
+// per state where one thread per track spends 887, on pipes that would idle:
+// where fits on several streams fill the GPU, one thread per track is the
+// better choice (events of 3000 tracks, 11 states: 223 us by teams against 347
+// on one stream, 112 against 49 us per event on sixteen).
+//
+// The 32 tracks of a CTA step through the states in lockstep (a track with
+// fewer states, or one that failed, idles at its barriers).  The arithmetic of
+// every element is that of the one-thread-per-track FP64 kernel
+// (kf_kernels.cu), bit for bit: the shared functions write their fused
+// multiply-adds out, and the compiler fuses nothing more.  1000 tracks of 11
+// states, 4 warps: 0.535 ms with the backward smoother as a second pass of two
+// barriers per state, 0.207 ms now.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -61,13 +67,12 @@ __global__ void __launch_bounds__(32 * W, 1) team_kernel(const FitParams p) {
   }
 }
 
-}  // namespace
-
+// dynamic shared memory of one of its CTAs
 size_t team_smem_bytes(int n_surfaces) {
+  static_assert((kMaxSurfaces * kSurfStride + kShFields * kTeamTracks) * 8 + 1024 <= 227 * 1024,
+                "fits beside the largest surface table");
   return (size_t)n_surfaces * kSurfStride * sizeof(double) + (size_t)kShFields * kTeamTracks * sizeof(double);
 }
-
-namespace {
 
 template <bool BZ, int W>
 cudaError_t launch_team_v(const FitParams& p, cudaStream_t stream) {
