@@ -40,16 +40,16 @@ FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12    # 80.5
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) and the flops the
 # hardware counted (2 x FMA + ADD + MUL thread instructions), per state, from
 # one ncu capture each: the mixed kernel's launch of a 100k-track, 3.1M-state
-# fit of the same workload, and the FP64 kernel's of its first 97 280 tracks
-# (3 015 680 states).  Both grow in proportion to the states.  They hold only
+# fit of the same workload, and the FP64 kernel's of its first 68 096 tracks
+# (2 110 976 states).  Both grow in proportion to the states.  They hold only
 # for the kernel sources and build flags that were captured: any change to them
 # makes the figures null.
-MIXED_TRAFFIC_BYTES_PER_STATE = (700.33e6 + 665.54e6) / 3.1e6
-MIXED_FLOPS_PER_STATE = (2 * 4189804071 + 5358001003 + 1848603186) / 3.1e6    # FP32
-MIXED_TRAFFIC_SOURCES_SHA256 = "d8c6abc03831e8bc3e9a52143ac687d07f35536d90eee69f32ac054619b64122"
-FP64_TRAFFIC_BYTES_PER_STATE = (161.02e6 + 12.50e6) / 3015680
-FP64_FLOPS_PER_STATE = (2 * 1830282709 + 70924384 + 730438129) / 3015680    # FP64
-FP64_TRAFFIC_SOURCES_SHA256 = "9def4ae28b9b04333262edb2678b912d8e1ae21f35c73a5c96614c18ed47ff27"
+MIXED_TRAFFIC_BYTES_PER_STATE = (696.49e6 + 664.96e6) / 3.1e6
+MIXED_FLOPS_PER_STATE = (2 * 4186804071 + 5331001003 + 1842603186) / 3.1e6    # FP32
+MIXED_TRAFFIC_SOURCES_SHA256 = "2016a9aae2b56d960b73dba96c6e7c25cee93074a519251791c21fdc8ce92aa3"
+FP64_TRAFFIC_BYTES_PER_STATE = (110.36e6 + 5.68e6) / 2110976
+FP64_FLOPS_PER_STATE = (2 * 1281198792 + 49647162 + 511307364) / 2110976    # FP64
+FP64_TRAFFIC_SOURCES_SHA256 = "3fabe10bbfa0466f30a19791432dcd4a2e6fb031ef1c4a6ff53e2f3b5930d0ad"
 
 
 # FP64 flops the hardware counted (ncu: 2 x DFMA + DADD + DMUL thread
@@ -58,9 +58,9 @@ FP64_TRAFFIC_SOURCES_SHA256 = "9def4ae28b9b04333262edb2678b912d8e1ae21f35c73a5c9
 # (align20, 21 states; the chi2 objective and the whole-fit objective);
 # reported while those kernels' sources match
 EXT_FLOPS_PER_TRACK = {"variants": (2 * 1998482340 + 463353310 + 886198499) / 3e4,
-                       "adjoint_chi2": (2 * 983610000 + 122860160 + 451470000) / 3e4,
-                       "adjoint_whole": (2 * 1482240000 + 126130080 + 492750000) / 3e4}
-EXT_SOURCES_SHA256 = "b0ee6640d6ec29f79cb8d89b60f4b8c28910eb1da23ff018769d18050bfaa075"
+                       "adjoint_chi2": (2 * 983610000 + 122860160 + 452070000) / 3e4,
+                       "adjoint_whole": (2 * 1482210000 + 125980080 + 493380000) / 3e4}
+EXT_SOURCES_SHA256 = "188ec174597d1a437400e5f4c8815ae4c39038ecba9a028b38a41c7976342660"
 
 
 def ext_kernel_sources_sha256():
