@@ -57,9 +57,9 @@ __device__ __forceinline__ int filter_first(const FitParams& p, int t, int64_t o
   f.nmeas = 0;
   f.spd = true;
   if (!p.is_hole[o0]) {
-    double m[2], V[3], K[6][2], Si[3], r[2];
+    double m[2], V[3], K[6][2], fs[3], r[2];
     hit_of(p, o0, m, V);
-    const int status = kalman_gain<6>(f.x, f.C, m, V, K, Si, r, f.xs, f.chi2);
+    const int status = kalman_gain<6>(f.x, f.C, m, V, K, fs, r, f.xs, f.chi2);
     if (status != ST_OK) return status;
     joseph_update<6>(f.C, V, K);
     f.nmeas = 1;
@@ -157,17 +157,16 @@ __device__ __forceinline__ int filter_states(const FitParams& p, const double* s
     // update
     double K[6][2], ir[2] = {0.0, 0.0};
     if (!p.is_hole[o0 + k]) {
-      double m[2], V[3], Si[3], r[2], dx[6], c2;
+      double m[2], V[3], fs[3], r[2], dx[6], c2;
       hit_of(p, o0 + k, m, V);
-      const int st = kalman_gain<N>(f.x, f.C, m, V, K, Si, r, dx, c2);
+      const int st = kalman_gain<N>(f.x, f.C, m, V, K, fs, r, dx, c2);
       if (st != ST_OK) return st;
       joseph_update<N>(f.C, V, K);
       f.chi2 += c2;
       ++f.nmeas;
 #pragma unroll
       for (int e = 0; e < N; ++e) f.x[e] += dx[e];
-      ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
-      ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+      innovation_solve(fs, r[0], r[1], ir[0], ir[1]);
       if (smooth) {
         double hall[6][2];
 #pragma unroll
@@ -176,7 +175,7 @@ __device__ __forceinline__ int filter_states(const FitParams& p, const double* s
           hall[e][1] = f.S[e][1];
         }
 #pragma unroll
-        for (int e = 0; e < 6; ++e) fixed_point_row(e, f.S[e], K, Si, r, hall, f.xs[e], f.P0);
+        for (int e = 0; e < 6; ++e) fixed_point_row(e, f.S[e], K, fs, r, hall, f.xs[e], f.P0);
       }
       turn(f.ang.cp, f.ang.sp, dx[2]);
       turn(f.ang.ct, f.ang.st, dx[3]);

@@ -201,9 +201,9 @@ __device__ __forceinline__ int team_states(const FitParams& p, const double* s_s
     const bool meas = act && !p.is_hole[o0 + k];
     double K[6][2] = {}, ir[2] = {0.0, 0.0}, dx[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if (meas) {
-      double m[2], V[3], Si[3], r[2], c2;
+      double m[2], V[3], fs[3], r[2], c2;
       hit_of(p, o0 + k, m, V);
-      status = kalman_gain<N>(f.x, f.C, m, V, K, Si, r, dx, c2);
+      status = kalman_gain<N>(f.x, f.C, m, V, K, fs, r, dx, c2);
       if (status == ST_OK) {
         f.chi2 += c2;
         ++f.nmeas;
@@ -225,11 +225,10 @@ __device__ __forceinline__ int team_states(const FitParams& p, const double* s_s
         }
 #pragma unroll
         for (int e = 0; e < 6; ++e)
-          if (srow_owner<W, N>(e) == w) fixed_point_row(e, f.S[e], K, Si, r, hall, f.xs[e], f.P0);
+          if (srow_owner<W, N>(e) == w) fixed_point_row(e, f.S[e], K, fs, r, hall, f.xs[e], f.P0);
 #pragma unroll
         for (int e = 0; e < N; ++e) f.x[e] += dx[e];
-        ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
-        ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+        innovation_solve(fs, r[0], r[1], ir[0], ir[1]);
       }
     }
     // the start angles' cosines and sines for the next transport

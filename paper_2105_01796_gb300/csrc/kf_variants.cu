@@ -519,17 +519,16 @@ __device__ __forceinline__ int variant_states(const FitParams& p, const double* 
     }
     double K[6][2], ir[2] = {0.0, 0.0};
     if (!p.is_hole[o0 + k]) {
-      double m[2], V[3], Si[3], r[2], dx[6], c2;
+      double m[2], V[3], fs[3], r[2], dx[6], c2;
       hit_of(p, o0 + k, m, V);
-      status = kalman_gain<N>(f.x, f.C, m, V, K, Si, r, dx, c2);
+      status = kalman_gain<N>(f.x, f.C, m, V, K, fs, r, dx, c2);
       if (status != ST_OK) return status;
       joseph_update<N>(f.C, V, K);
       f.chi2 += c2;
       ++f.nmeas;
 #pragma unroll
       for (int e = 0; e < N; ++e) f.x[e] += dx[e];
-      ir[0] = fma(Si[0], r[0], Si[1] * r[1]);
-      ir[1] = fma(Si[1], r[0], Si[2] * r[1]);
+      innovation_solve(fs, r[0], r[1], ir[0], ir[1]);
       if (MODE != kBackward) {
         double hall[6][2];
 #pragma unroll
@@ -538,7 +537,7 @@ __device__ __forceinline__ int variant_states(const FitParams& p, const double* 
           hall[e][1] = f.S[e][1];
         }
 #pragma unroll
-        for (int e = 0; e < 6; ++e) fixed_point_row(e, f.S[e], K, Si, r, hall, f.xs[e], f.P0);
+        for (int e = 0; e < 6; ++e) fixed_point_row(e, f.S[e], K, fs, r, hall, f.xs[e], f.P0);
       }
       turn(f.ang.cp, f.ang.sp, dx[2]);
       turn(f.ang.ct, f.ang.st, dx[3]);
@@ -640,8 +639,8 @@ __device__ __forceinline__ void fit_one_variants(const FitParams& p, const doubl
         if (!p.is_hole[o0 + k]) {
           const double m[2] = {p.loc[o0 + k], p.loc[p.n_states + o0 + k]};
           const double V[3] = {p.cov[o0 + k], p.cov[p.n_states + o0 + k], p.cov[2 * p.n_states + o0 + k]};
-          double c2, K[6][2], Si[3], r[2], dx[6];
-          status = kalman_gain<6>(x, C, m, V, K, Si, r, dx, c2);
+          double c2, K[6][2], fs[3], r[2], dx[6];
+          status = kalman_gain<6>(x, C, m, V, K, fs, r, dx, c2);
           if (status != ST_OK) break;
           joseph_update<6>(C, V, K);
 #pragma unroll
