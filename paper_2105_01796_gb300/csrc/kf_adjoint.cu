@@ -562,22 +562,21 @@ struct SmOut {
   double yb[2], G[3], Z[5][2], lF[4][5];
 };
 
-// Si and y = Si r of the update at a state
+// The factors of S at a state's update (innovation_solve: as in the filter, no
+// inverse of S is formed) and y = Si r.
 struct Innov {
-  double Si[3], r[2], y[2];
+  double f[3], r[2], y[2];
 };
 __device__ __forceinline__ Innov innovation(const double xp[2], const double Cp[21], const double m[2],
                                             const double V[3]) {
   const double S00 = V[0] + Cp[sy(0, 0)], S01 = V[1] + Cp[sy(1, 0)], S11 = V[2] + Cp[sy(1, 1)];
-  const double idet = rcp_any(fma(S00, S11, -S01 * S01));
   Innov q;
-  q.Si[0] = S11 * idet;
-  q.Si[1] = -S01 * idet;
-  q.Si[2] = S00 * idet;
+  q.f[0] = rcp_any(S00);
+  q.f[1] = S01 * q.f[0];
+  q.f[2] = rcp_any(fma(-q.f[1], S01, S11));
   q.r[0] = m[0] - xp[0];
   q.r[1] = m[1] - xp[1];
-  q.y[0] = fma(q.Si[0], q.r[0], q.Si[1] * q.r[1]);
-  q.y[1] = fma(q.Si[1], q.r[0], q.Si[2] * q.r[1]);
+  innovation_solve(q.f, q.r[0], q.r[1], q.y[0], q.y[1]);
   return q;
 }
 
@@ -591,7 +590,6 @@ template <bool SM, int N>
 __device__ __forceinline__ void update_reverse(const Innov& q, const double Cp[21], double w, const SmOut& sm,
                                                double lf[6], double Lf[21]) {
   // U = Lf P; yb = P^T lf (+ h^T v); G = adjoint of Si (symmetric)
-  const double* Si = q.Si;
   const double* r = q.r;
   double Z[6][2], yb[2] = {0.0, 0.0};
   const double wr0 = w * r[0], wr1 = w * r[1];
@@ -627,22 +625,29 @@ __device__ __forceinline__ void update_reverse(const Innov& q, const double Cp[2
   G11 = fma(yb[1], r[1], G11);
   G01 = fma(0.5, fma(yb[0], r[1], yb[1] * r[0]), G01);
   // adjoint of S: -Si G Si
-  const double t00 = fma(G00, Si[0], G01 * Si[1]), t01 = fma(G00, Si[1], G01 * Si[2]);
-  const double t10 = fma(G01, Si[0], G11 * Si[1]), t11 = fma(G01, Si[1], G11 * Si[2]);
-  Lf[sy(0, 0)] -= fma(Si[0], t00, Si[1] * t10);
-  Lf[sy(1, 0)] -= fma(Si[1], t00, Si[2] * t10);
-  Lf[sy(1, 1)] -= fma(Si[1], t01, Si[2] * t11);
+  double t00, t01, t10, t11, x00, x10, x01, x11;
+  innovation_solve(q.f, G00, G01, t00, t01);
+  innovation_solve(q.f, G01, G11, t10, t11);
+  innovation_solve(q.f, t00, t10, x00, x10);
+  innovation_solve(q.f, t01, t11, x01, x11);
+  Lf[sy(0, 0)] -= x00;
+  Lf[sy(1, 0)] -= x10;
+  Lf[sy(1, 1)] -= x11;
   // adjoint of P: lf y^T - Z Si, into columns 0 and 1 (symmetrised)
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const double P0 = fma(lf[i], q.y[0], -fma(Z[i][0], Si[0], Z[i][1] * Si[1]));
-    const double P1 = fma(lf[i], q.y[1], -fma(Z[i][0], Si[1], Z[i][1] * Si[2]));
+    double z0, z1;
+    innovation_solve(q.f, Z[i][0], Z[i][1], z0, z1);
+    const double P0 = fma(lf[i], q.y[0], -z0);
+    const double P1 = fma(lf[i], q.y[1], -z1);
     Lf[sym(i, 0)] = i == 0 ? Lf[sym(i, 0)] + P0 : fma(0.5, P0, Lf[sym(i, 0)]);
     Lf[sym(i, 1)] = i == 1 ? Lf[sym(i, 1)] + P1 : fma(0.5, P1, Lf[sym(i, 1)]);
   }
   // adjoint of r: Si (yb + 2 w r)
-  lf[0] -= fma(2.0 * w, q.y[0], fma(Si[0], yb[0], Si[1] * yb[1]));
-  lf[1] -= fma(2.0 * w, q.y[1], fma(Si[1], yb[0], Si[2] * yb[1]));
+  double s0, s1;
+  innovation_solve(q.f, yb[0], yb[1], s0, s1);
+  lf[0] -= fma(2.0 * w, q.y[0], s0);
+  lf[1] -= fma(2.0 * w, q.y[1], s1);
 }
 
 struct GradParams {
@@ -884,8 +889,10 @@ __device__ __forceinline__ void smoother_part(const TrackB<true>& t, int k, cons
       o.G[1] = fma(-0.5, fma(hm[i][0], b1, hm[i][1] * b0), o.G[1]);
       const double c0 = fma(2.0, a0, q0), c1 = fma(2.0, a1, q1);
       // adjoint of h: v y^T - (2 W h + LS P) Si
-      LS[i][0] += fma(v[i], q.y[0], -fma(c0, q.Si[0], c1 * q.Si[1]));
-      LS[i][1] += fma(v[i], q.y[1], -fma(c0, q.Si[1], c1 * q.Si[2]));
+      double s0, s1;
+      innovation_solve(q.f, c0, c1, s0, s1);
+      LS[i][0] += fma(v[i], q.y[0], -s0);
+      LS[i][1] += fma(v[i], q.y[1], -s1);
     }
   }
   // Sp = S F^T
