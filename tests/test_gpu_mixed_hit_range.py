@@ -9,7 +9,7 @@ import pytest
 import oracle
 from tests.test_gpu_fp64_path import _event
 from tests.test_gpu_mixed_path import SHAPES
-from tests.test_gpu_parity import MIXED, compare, gpu_fit, handle  # noqa: F401
+from tests.test_gpu_parity import FP64, MIXED, compare, gpu_fit, handle  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +31,17 @@ def test_hit_variances(handle, var, coords, shape):  # noqa: F811
     r = oracle.fit_batch(ev)
     assert (r["status"] == 0).all()
     compare(gpu_fit(handle, ev, MIXED, **shape), r, MIXED)
+
+
+@pytest.mark.parametrize("coords", [(0,), (1,), (0, 1)], ids=["loc0", "loc1", "both"])
+@pytest.mark.parametrize("prec,opt", [(FP64, dict(team_warps=1)), (FP64, dict(team_warps=4)), (FP64, dict(energy_loss=1)),
+                                      (MIXED, {})], ids=["one_thread", "team", "energy_loss", "mixed"])
+def test_infinite_variance_is_refused(handle, prec, opt, coords):  # noqa: F811
+    """An infinite variance fails its track, in either precision; the others fit."""
+    ev = _event(64)
+    ev["cov"] = ev["cov"].copy()
+    for c in coords:
+        ev["cov"][2 * c, 4::22] = np.inf  # every second track
+    g = gpu_fit(handle, ev, prec, **opt)
+    assert (g["status"][0::2] != 0).all() and (g["status"][1::2] == 0).all()
+    assert np.isnan(g["params"][:, 0::2]).all() and np.isnan(g["chi2"][0::2]).all()
