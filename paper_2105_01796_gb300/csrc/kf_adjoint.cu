@@ -853,15 +853,22 @@ __device__ __forceinline__ void forward_part(const TrackB<SM>& t, int k, const S
   f.xp[1] = fma(d0, sb.v(0), fma(d1, sb.v(1), d2 * sb.v(2)));
 }
 
+// the innovation of transition k run again (of a hole: not used)
+template <bool SM>
+__device__ __forceinline__ Innov innovation_at(const TrackB<SM>& t, int k, const FwdB& f) {
+  Innov q;
+  if (t.hole(k)) return q;
+  double m[2], V[3];
+  hit_of(t.g->f, t.o0 + k, m, V);
+  return innovation(f.xp, f.Cp, m, V);
+}
+
 // The smoother's part of the reverse of transition k: LS (adjoint of S_k)
 // becomes that of S_k-1; it depends on nothing else of the reverse.
 __device__ __forceinline__ void smoother_part(const TrackB<true>& t, int k, const double F[4][5], const double Cp[21],
-                                              const double xp[2], const double hm[6][2], const double v[6],
+                                              const Innov& q, const double hm[6][2], const double v[6],
                                               const double W[21], double LS[6][5], SmOut& o) {
   if (!t.hole(k)) {
-    double m[2], V[3];
-    hit_of(t.g->f, t.o0 + k, m, V);
-    const Innov q = innovation(xp, Cp, m, V);
     o.yb[0] = o.yb[1] = o.G[0] = o.G[1] = o.G[2] = 0.0;
 #pragma unroll
     for (int j = 0; j < 5; ++j) o.Z[j][0] = o.Z[j][1] = 0.0;
@@ -927,15 +934,11 @@ __device__ __forceinline__ void smoother_part(const TrackB<true>& t, int k, cons
 // that of k-1; ga receives surface k's alignment derivatives.
 template <bool BZ, bool SM>
 __device__ __forceinline__ void reverse_part(const TrackB<SM>& t, int k, double w, const StartB& st, const FwdB& f,
-                                             const Step* tape, const SmOut& sm, double lf[6], double Lf[21],
-                                             PlaneAdj& adj, double ga[6]) {
+                                             const Step* tape, const Innov& q, const SmOut& sm, double lf[6],
+                                             double Lf[21], PlaneAdj& adj, double ga[6]) {
   const FitParams& p = t.g->f;
   const Surf sa = t.surf(k - 1), sb = t.surf(k);
-  if (!t.hole(k)) {
-    double m[2], V[3];
-    hit_of(p, t.o0 + k, m, V);
-    update_reverse<SM, 5>(innovation(f.xp, f.Cp, m, V), f.Cp, w, sm, lf, Lf);
-  }
+  if (!t.hole(k)) update_reverse<SM, 5>(q, f.Cp, w, sm, lf, Lf);
   // reverse of Cp = F C F^T + Q (and Sp = S F^T):
   //   l_F = 2 Lp F C (+ LSp^T S), L_C = F^T Lp F
   double lF[4][5];  // rows loc0, loc1, phi, theta
@@ -1101,8 +1104,9 @@ __device__ __forceinline__ void grad_reverse(const GradParams& g, const double* 
       FwdB f;
       SmOut sm;
       forward_part<BZ, SM>(t, k, st, f, tape);
-      if constexpr (SM) smoother_part(t, k, f.F, f.Cp, f.xp, f.hm, v, W, LS, sm);
-      reverse_part<BZ, SM>(t, k, b.w, st, f, tape, sm, b.lf, b.Lf, b.adj, ga);
+      const Innov q = innovation_at(t, k, f);
+      if constexpr (SM) smoother_part(t, k, f.F, f.Cp, q, f.hm, v, W, LS, sm);
+      reverse_part<BZ, SM>(t, k, b.w, st, f, tape, q, sm, b.lf, b.Lf, b.adj, ga);
     }
     if (g.grad_align) add_align_grad(g.grad_align, g.f.n_surfaces, act ? g.f.surface_id[t.o0 + k] : 0, ga, act);
   }
@@ -1176,7 +1180,7 @@ __device__ __forceinline__ void grad_reverse_pipe(const GradParams& g, const dou
         SmOut o;
         int e = 0;
         visit<SM>(f, [&](double& x) { x = q[(e++) * 32]; });  // (what is not used is not loaded)
-        smoother_part(t, k, f.F, f.Cp, f.xp, f.hm, v, W, LS, o);
+        smoother_part(t, k, f.F, f.Cp, innovation_at(t, k, f), f.hm, v, W, LS, o);
 #pragma unroll
         for (int i = 0; i < 2; ++i) qs[i * 32] = o.yb[i];
 #pragma unroll
@@ -1220,7 +1224,7 @@ __device__ __forceinline__ void grad_reverse_pipe(const GradParams& g, const dou
 #pragma unroll
           for (int i = 0; i < 20; ++i) sm.lF[i / 5][i % 5] = qs[(15 + i) * 32];
         }
-        reverse_part<BZ, SM>(t, k, b.w, st, f, tape, sm, b.lf, b.Lf, b.adj, ga);
+        reverse_part<BZ, SM>(t, k, b.w, st, f, tape, innovation_at(t, k, f), sm, b.lf, b.Lf, b.adj, ga);
       }
       if (g.grad_align && go)
         add_align_grad(g.grad_align, g.f.n_surfaces, act ? g.f.surface_id[t.o0 + k] : 0, ga, act);
