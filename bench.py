@@ -44,12 +44,12 @@ FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12    # 80.5
 # (2 110 976 states).  Both grow in proportion to the states.  They hold only
 # for the kernel sources and build flags that were captured: any change to them
 # makes the figures null.
-MIXED_TRAFFIC_BYTES_PER_STATE = (696.49e6 + 664.96e6) / 3.1e6
+MIXED_TRAFFIC_BYTES_PER_STATE = (697.33e6 + 664.96e6) / 3.1e6
 MIXED_FLOPS_PER_STATE = (2 * 4186804071 + 5331001003 + 1842603186) / 3.1e6    # FP32
 MIXED_TRAFFIC_SOURCES_SHA256 = "2016a9aae2b56d960b73dba96c6e7c25cee93074a519251791c21fdc8ce92aa3"
-FP64_TRAFFIC_BYTES_PER_STATE = (110.36e6 + 5.68e6) / 2110976
-FP64_FLOPS_PER_STATE = (2 * 1281198792 + 49647162 + 511307364) / 2110976    # FP64
-FP64_TRAFFIC_SOURCES_SHA256 = "3fabe10bbfa0466f30a19791432dcd4a2e6fb031ef1c4a6ff53e2f3b5930d0ad"
+FP64_TRAFFIC_BYTES_PER_STATE = (110.33e6 + 5.76e6) / 2110976
+FP64_FLOPS_PER_STATE = (2 * 1287327432 + 47604282 + 505178724) / 2110976    # FP64
+FP64_TRAFFIC_SOURCES_SHA256 = "c3dcd1240e18dcdf01709cdbe6068f3dec53cfeed3c197d4cdda88aed2543ea6"
 
 
 # FP64 flops the hardware counted (ncu: 2 x DFMA + DADD + DMUL thread
@@ -57,10 +57,10 @@ FP64_TRAFFIC_SOURCES_SHA256 = "3fabe10bbfa0466f30a19791432dcd4a2e6fb031ef1c4a6ff
 # (fringe30, 31 states, all three variants) and of the adjoint kernel
 # (align20, 21 states; the chi2 objective and the whole-fit objective);
 # reported while those kernels' sources match
-EXT_FLOPS_PER_TRACK = {"variants": (2 * 1998482340 + 463353310 + 886198499) / 3e4,
-                       "adjoint_chi2": (2 * 983610000 + 122860160 + 452070000) / 3e4,
-                       "adjoint_whole": (2 * 1482210000 + 125980080 + 493380000) / 3e4}
-EXT_SOURCES_SHA256 = "188ec174597d1a437400e5f4c8815ae4c39038ecba9a028b38a41c7976342660"
+EXT_FLOPS_PER_TRACK = {"variants": (2 * 2003882340 + 462453310 + 880798499) / 3e4,
+                       "adjoint_chi2": (2 * 988410000 + 123460160 + 449670000) / 3e4,
+                       "adjoint_whole": (2 * 1482210000 + 122380080 + 486180000) / 3e4}
+EXT_SOURCES_SHA256 = "e98ae50a13e36c327e402625d1981f52ac4329cfb8399123f69e7c2f7ed6cc74"
 
 
 def ext_kernel_sources_sha256():

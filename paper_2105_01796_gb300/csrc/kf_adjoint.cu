@@ -37,7 +37,7 @@
 // checkpoints every 5 states and a separate smoother adjoint: chi2 gradient
 // of 100k tracks x 21 states 50.3 -> 10.8 ms (9.6 ms without the time row,
 // 9.4 ms with the cheaper logarithm), fit and whole gradient of 2000 tracks x
-// 21 states 14.8 -> 3.57 ms (there two warps shared 32 tracks; 1.89 ms with
+// 21 states 14.8 -> 3.57 ms (there two warps shared 32 tracks; 1.86 ms with
 // the team kernel below).
 // Storing every filtered state (176 B, whole fit 416 B) costs 0.14 ms of
 // memory traffic on the 100k tracks; recomputing them took a quarter of the
@@ -1319,7 +1319,7 @@ __global__ void __launch_bounds__(max_threads_of(MINB), 1) kf_grad_kernel(const 
 // warp's time) and whose pass B is a pipeline over its warps.  Up to one team
 // per SM.  2000 tracks x 21 states, forward and backward of the
 // differentiable fit: 3.57 -> 2.98 ms with the team's forward pass (2.66
-// without the time row), 1.90 ms with the pipeline.
+// without the time row), 1.86 ms with the pipeline.
 template <bool BZ, bool SM>
 __global__ void __launch_bounds__(128, 1) kf_grad_team_kernel(const GradParams g) {
   extern __shared__ __align__(128) unsigned char smem_raw[];

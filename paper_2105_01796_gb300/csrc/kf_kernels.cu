@@ -12,14 +12,14 @@
 // in global memory accessed once; constant field).
 //
 // The bound is the FP64 pipe (2 DFMA per clock and SM), so the design spends
-// as few FP64 instructions as the method allows: about 880 per state with the
+// as few FP64 instructions as the method allows: about 885 per state with the
 // field along z, where the stage-by-stage transport with the backward
 // smoother took 2370.  100k tracks of 31 states: 15.28 -> 6.47 ms with the
 // closed-form transport and the fixed-point smoother, 6.22 ms with teams for
 // the last round, 5.43 ms without the time row (kf_filter.cuh), 5.29 ms with
-// cheaper reciprocals and logarithms, 4.90 ms in waves of 7 warps per SM; 20k
+// cheaper reciprocals and logarithms, 4.88 ms in waves of 7 warps per SM; 20k
 // tracks of 24 tilted planes in a general field with every smoothed state 3.56
-// -> 1.57 ms.
+// -> 1.55 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

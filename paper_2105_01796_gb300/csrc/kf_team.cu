@@ -7,7 +7,7 @@
 // cycles per DFMA warp instruction with 32, 16, 8, 4, 2 or 1 active lanes),
 // and one warp of the one-thread-per-track kernel keeps that pipe busy on its
 // own: a batch of fewer tracks than sub-partitions x 32 runs at one warp's
-// FP64 instruction count per state (887).  Splitting a track over the
+// FP64 instruction count per state (885).  Splitting a track over the
 // lanes of one warp cannot shorten that; splitting it over W warps, each on
 // its own sub-partition, can.
 //
@@ -20,8 +20,8 @@
 //   * the fixed-point smoother (by row of S = Cov(x_0, x_k): every warp keeps
 //     its rows of S and P_0 in registers, they are never exchanged),
 // and exchange F, Cp, Cf and a few scalars through shared memory, three
-// barriers per state and no second pass.  A team spends 1672 FP64 instructions
-// per state where one thread per track spends 887, on pipes that would idle:
+// barriers per state and no second pass.  A team spends 1664 FP64 instructions
+// per state where one thread per track spends 885, on pipes that would idle:
 // where fits on several streams fill the GPU, one thread per track is the
 // better choice (events of 3000 tracks, 11 states: 223 us by teams against 347
 // on one stream, 112 against 49 us per event on sixteen).
@@ -32,7 +32,7 @@
 // (kf_kernels.cu), bit for bit: the shared functions write their fused
 // multiply-adds out, and the compiler fuses nothing more.  1000 tracks of 11
 // states, 4 warps: 0.535 ms with the backward smoother as a second pass of two
-// barriers per state, 0.207 ms now.
+// barriers per state, 0.201 ms now.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

@@ -19,8 +19,8 @@
 // stay stage by stage; the corrections after the first are tiny and take
 // their leading terms.  The backward filter's weighted mean (a 6x6
 // factorisation and six solves) is formed on the states that are output.
-// 50k tracks of 21 states with energy loss 7.54 -> 2.17 ms; 30k tracks of 31
-// states with map, energy loss and backward filter 16.9 -> 9.58 ms (4290 FP64
+// 50k tracks of 21 states with energy loss 7.54 -> 2.16 ms; 30k tracks of 31
+// states with map, energy loss and backward filter 16.9 -> 9.43 ms (4286 FP64
 // instructions per state; the 938 warps run as one wave of 7 per SM).
 #include <cuda_runtime.h>
 #include <math.h>
